@@ -5,75 +5,38 @@
 // The triangulation wanted is the unique one of the symbolically perturbed
 // point set (lifted heights |p_i|^2 + eps_i, eps_0 >> eps_1 >> ..., i = list
 // index), the same one the host routine builds.  Here every point builds its
-// own star, one warp per point:
-//   1. its nearest neighbour a0 (always a Delaunay edge: the circle with
-//      diameter p-a0 holds no other point, not even on its boundary);
-//   2. gift-wrapping counter-clockwise: the Delaunay triangle left of edge
-//      (p, a) has as third vertex the point left of p->a that no other such
-//      point lies inside the circle through p, a and it (exact predicate with
-//      the symbolic tie-break: a strict total order, so a warp min-reduction
-//      finds it); continue with (p, b) until the star closes at a0 or no
-//      point is left of the edge (p on the hull), then wrap clockwise from a0.
-// Pass 1 (a group of 16 lanes per point, 4 in batches) lists the points
-// within R = 24 pixels (18 in batches) of p from a 16-pixel grid and wraps
-// the star among them with the pencil key; it is accepted when every
-// triangle's circumdisc lies inside that disc (4 r^2 <= R^2 in exact
-// arithmetic, so no farther point can matter) and,
-// where the star stays open (p on the hull), nothing lies beyond either open
-// edge (checked against the extreme points of every image row).  In batches
-// of two or more pairs the other stars go through the same group pass twice
-// more: eight lanes and the points within 32 pixels, then one warp and the
-// points within 64.  The rest are rebuilt by one CTA per point: each step
-// takes the best of the points within 96 (then 192) pixels when its circle
-// fits that disc, else scans the grid cells its circle (or, with no
-// candidate, its half-plane) meets, which is exact.  Each triangle
-// is emitted once, by its lowest-index vertex, at an offset from an
-// exclusive scan of the per-point counts, so the output order is
-// deterministic.
+// own star (the triangles around it) by gift-wrapping: the third vertex of a
+// directed edge (p, a) is the point on its left that no other such point lies
+// inside the circle through p, a and it (a strict total order with the
+// symbolic tie-break, so a warp reduction finds it).  A triangle is emitted
+// once, by its lowest-index vertex, so of a star only the fan of triangles
+// that p owns and one more on either side are needed (dt_warp_star).
+//   1. Warp pass: one warp per point, the points within 24 pixels from a
+//      16-pixel grid; a star counts when the circles of its triangles fit
+//      that disc (2r <= R, so no farther point can matter), 93-95 % of them.
+//   2. Middle pass (batches): the others again, with 64 pixels.
+//   3. CTA pass: one CTA per star left (the hull, the rims of empty areas):
+//      the star over the points within 96 pixels, then scans of the cells
+//      that its wide circles meet until they are empty (dt_block_item).
+// The output order is deterministic: an exclusive scan of the per-point
+// counts, and within a star counter-clockwise from the nearest neighbour (an
+// open star then clockwise from it).
+//
+// One step of the earlier design (4 or 16 lanes per star, the whole star,
+// 64-bit key comparisons, one region scan per step of a wide star) against
+// this one: 640x480 172 -> 96 us, 1920x1080 590 -> 276 us, 64 x 1242x375
+// 3.44 -> 1.82 ms for all triangulation kernels.
 #include "launch.cuh"
 
 namespace elas {
 
 constexpr int kDtCell = 16;
-constexpr int kDtMaxStar = 4096;  // wrap steps per star
 
 __device__ __forceinline__ int dt_ncell(const DtArgs &a) { return a.gw * a.gh; }
 
 __device__ __forceinline__ int dt_cell(const DtArgs &a, int x, int y) {
     const int cx = min(max(x, 0) / kDtCell, a.gw - 1), cy = min(max(y, 0) / kDtCell, a.gh - 1);
     return cy * a.gw + cx;
-}
-
-// -------------------------------------------------------------------------
-// Exact predicates (coordinates below 2^15, products in 64 bits)
-// -------------------------------------------------------------------------
-
-__device__ __forceinline__ int64_t dt_orient(int ax, int ay, int bx, int by, int cx, int cy) {
-    return (int64_t)(bx - ax) * (cy - ay) - (int64_t)(by - ay) * (cx - ax);
-}
-
-// Sign of "C strictly inside the circle through P, A, B" (P, A, B
-// counter-clockwise), with the symbolic tie-break on the list indices.  T is
-// the arithmetic type of the determinant: int is exact while every coordinate
-// differs from P's by at most 64 (6 terms of at most 64*64*8192), int64_t
-// always (differences below 2^15).
-template <typename T>
-__device__ __forceinline__ int dt_incircle(const int4 &P, const int4 &A, const int4 &B, const int4 &C) {
-    const T ax = A.x - P.x, ay = A.y - P.y, bx = B.x - P.x, by = B.y - P.y, cx = C.x - P.x, cy = C.y - P.y;
-    const T al = ax * ax + ay * ay, bl = bx * bx + by * by, cl = cx * cx + cy * cy;
-    // value = -det[[a, |a|^2], [b, |b|^2], [c, |c|^2]] (relative to P)
-    const T det = ax * (by * cl - bl * cy) - ay * (bx * cl - bl * cx) + al * (bx * cy - by * cx);
-    if (det != 0) return det < 0 ? 1 : -1;
-    // raising lift i by eps_i adds eps_P*orient(A,B,C) + eps_A*orient(B,P,C)
-    // + eps_B*orient(P,A,C) - eps_C*orient(P,A,B); the lowest index decides
-    const int who[4] = {P.z, A.z, B.z, C.z};
-    const int64_t coef[4] = {dt_orient(A.x, A.y, B.x, B.y, C.x, C.y), dt_orient(B.x, B.y, P.x, P.y, C.x, C.y),
-                             dt_orient(P.x, P.y, A.x, A.y, C.x, C.y), -dt_orient(P.x, P.y, A.x, A.y, B.x, B.y)};
-    int best = -1;
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-        if (coef[k] != 0 && (best < 0 || who[k] < who[best])) best = k;
-    return best < 0 ? 0 : (coef[best] > 0 ? 1 : -1);
 }
 
 // -------------------------------------------------------------------------
@@ -88,8 +51,8 @@ __device__ __forceinline__ void dt_points_body(const DtArgs &a, const VB &vb) {
         const int x = S.right ? u - d : u;
         S.X[i] = x;
         S.Y[i] = v;
-        S.status[i] = 0;
         S.owned[i] = 0;
+        if (i > 0 && a.list[3 * i - 2] > v) atomicOr(S.err, 8);  // not in raster order
         atomicAdd(S.cell_cnt + dt_cell(a, x, v), 1);
         if (v >= 0 && v < a.h) {
             atomicMin(S.rowmin + v, x);
@@ -190,10 +153,7 @@ __device__ __forceinline__ void dt_dedup_body(const DtArgs &a, const VB &vb) {
             const int4 q = S.pts[k];
             if (q.x == x && q.y == y && q.z < i) dup = true;
         }
-        if (dup) {
-            S.status[i] = -1;
-            S.pts[S.slot[i]].w = 0;
-        }
+        if (dup) S.pts[S.slot[i]].w = 0;
     }
 }
 
@@ -207,857 +167,1080 @@ __global__ void dt_dedup_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
 // Stars
 // -------------------------------------------------------------------------
 
-constexpr int kDtRadius = 24;     // pass-1 search radius (one pair)
-constexpr int kDtRadiusBatch = 18;  // pass-1 search radius in batched launches
-constexpr int kDtSlots = 32;      // owned triangles kept per point
+constexpr int kDtSlots = 16;       // owned triangles kept per point; larger fans go to the pool
+constexpr int kDtRadius = 24;      // warp pass: candidates within this many pixels
+constexpr int kDtListCap = 128;    // its list (a radius-24 disc holds about 75 points of a full step-5 lattice)
+constexpr int kDtRadiusM = 64;     // middle pass (batches)
+constexpr int kDtListCapM = 640;   // a radius-64 disc holds about 520 lattice points
+constexpr int kDtWarps = 8;        // stars per CTA of the warp pass
+constexpr int kDtWarpsM = 4;       // stars per CTA of the middle pass
+constexpr float kDtInf = 3.402823466e38f;  // "no candidate" key (every real key is far below)
 
-__device__ __forceinline__ int4 shfl4(const int4 &v, int src_xor) {
-    return make_int4(__shfl_xor_sync(0xFFFFFFFFu, v.x, src_xor), __shfl_xor_sync(0xFFFFFFFFu, v.y, src_xor),
-                     __shfl_xor_sync(0xFFFFFFFFu, v.z, src_xor), __shfl_xor_sync(0xFFFFFFFFu, v.w, src_xor));
+__device__ __forceinline__ float dt_warp_min(float v) {
+    float r;
+    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
 }
 
-__device__ __forceinline__ unsigned long long dt_nn_key(const int4 &p, const int4 &q) {
-    const int64_t dx = q.x - p.x, dy = q.y - p.y;
-    return ((unsigned long long)(dx * dx + dy * dy) << 32) | (unsigned)q.z;
+// The Delaunay third vertex of directed edge (p, e) on side s (+1 left, -1
+// right) is the candidate c with s*cross(e, c) > 0 (coordinates relative to
+// p) that minimises t(c) = N/D, N = |c|^2 - e.c, D = s*cross(e, c): the
+// circles through p and e are nested on each side in the order of t.  Every
+// step below finds the least t in FP32 (one approximate division per
+// candidate, one warp reduction), takes the candidates within a band that
+// covers the rounding, and, when the band has several members, orders those
+// exactly in integers.
+//
+// Equal t means that p, e and both candidates are cocircular: of the four,
+// the one with the lowest list index (raised the most by the symbolic
+// perturbation) gets the ear, so the diagonal joins its two neighbours on
+// the circle.  With x the first candidate after e (going round from p over
+// e) and y the second, y wins iff the lowest index is p's or x's.
+// Does the second candidate beat the first?  o = s*cross(c1, c2).
+__device__ __forceinline__ bool dt_tie_second(int pz, int ez, int z1, int z2, bool first_is_x) {
+    const int xz = first_is_x ? z1 : z2, yz = first_is_x ? z2 : z1;
+    const bool ywins = min(pz, xz) < min(ez, yz);
+    return first_is_x == ywins;
 }
 
-__device__ __forceinline__ unsigned long long warp_min64(unsigned long long k) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long other = __shfl_xor_sync(0xFFFFFFFFu, k, o);
-        k = other < k ? other : k;
-    }
-    return k;
-}
-
-// Is the circle through p, a, b no wider than R (2r <= R, r its radius)?
-// With 4 r^2 = |pa|^2 |pb|^2 |ab|^2 / orient(p, a, b)^2 this is
-// |pa|^2 |pb|^2 |ab|^2 <= R^2 orient^2, in exact integer arithmetic.  A point
-// farther than R from p makes the diameter exceed R at once, so the products
-// only see points within R: below R^4 * 4 R^2 < 2^63 for R <= 1024.
-__device__ __forceinline__ bool dt_small_circle(const int4 &p, const int4 &a, const int4 &b, int R) {
-    const int64_t R2 = (int64_t)R * R;
-    const int64_t pa = (int64_t)(a.x - p.x) * (a.x - p.x) + (int64_t)(a.y - p.y) * (a.y - p.y);
-    const int64_t pb = (int64_t)(b.x - p.x) * (b.x - p.x) + (int64_t)(b.y - p.y) * (b.y - p.y);
-    if (pa > R2 || pb > R2) return false;
-    const int64_t ab = (int64_t)(b.x - a.x) * (b.x - a.x) + (int64_t)(b.y - a.y) * (b.y - a.y);
-    const int64_t ar = dt_orient(p.x, p.y, a.x, a.y, b.x, b.y);
-    return pa * pb * ab <= R2 * ar * ar;
-}
-
-// The same test in 32-bit integers for discs of radius R <= 24: once pa and
-// pb are at most R^2, pa * pb * ab <= 4 R^6 < 2^31 and R^2 * ar^2 <= R^6
-// (|ar| <= sqrt(pa pb)); coordinate differences below 2^15 keep pa and pb
-// themselves within 31 bits.
-template <int R>
-__device__ __forceinline__ bool dt_small_circle32(const int4 &p, const int4 &a, const int4 &b) {
-    static_assert(R <= 24, "4 R^6 must fit in 31 bits");
-    const int ax = a.x - p.x, ay = a.y - p.y, bx = b.x - p.x, by = b.y - p.y;
-    const int pa = ax * ax + ay * ay, pb = bx * bx + by * by;
-    if (pa > R * R || pb > R * R) return false;
+// Is the circle through the origin, a and b no wider than R (2r <= R)?
+// |a|^2 |b|^2 |a-b|^2 <= R^2 cross(a, b)^2, in FP32 with a margin far above
+// its rounding: a false answer only sends a star to the next pass.
+__device__ __forceinline__ bool dt_small_circle(int ax, int ay, int bx, int by, float R2) {
+    const float pa = (float)(ax * ax + ay * ay), pb = (float)(bx * bx + by * by);
     const int dx = bx - ax, dy = by - ay;
-    const int ab = dx * dx + dy * dy;
-    const int ar = ax * by - ay * bx;
-    return pa * pb * ab <= R * R * ar * ar;
+    const float ab = (float)dx * (float)dx + (float)dy * (float)dy, ar = (float)(ax * by - ay * bx);
+    return pa * pb * ab * 1.00001f <= R2 * ar * ar;
 }
 
-template <int R>
-__device__ __forceinline__ bool dt_small_circle_r(const int4 &p, const int4 &a, const int4 &b) {
-    if constexpr (R <= 24)
-        return dt_small_circle32<R>(p, a, b);
-    else
-        return dt_small_circle(p, a, b, R);
-}
-
-// Records triangle (p, a, b) if p owns it (lowest index).
-__device__ __forceinline__ void dt_record(const DtSide &S, int i, int &written, const int4 &p, const int4 &a,
-                                          const int4 &b, bool leader) {
-    if (p.z < a.z && p.z < b.z) {
-        if (leader && written < kDtSlots) {
-            int32_t *slot = S.slots + ((size_t)i * kDtSlots + written) * 2;
-            slot[0] = a.z;
-            slot[1] = b.z;
-        }
-        ++written;
-    }
-}
-
-// The Delaunay third vertex of directed edge (p, e) on side s (+1 left,
-// -1 right) is the candidate c with s*orient(p,e,c) > 0 that minimises the
-// pencil parameter t(c) = N/D, N = |c-p|^2 - (e-p).(c-p), D = 2 s orient(p,e,c)
-// (the circles through p and e are nested on each side in the order of t).
-// Equal t means cocircular: the symbolic tie-break decides.  T: arithmetic
-// type of the cross-multiplied comparison.
-template <typename T>
-struct DtKey {
-    T N, D;
+struct DtPt {
+    int x, y, z;  // relative to the star's point; list index
 };
 
-template <typename T>
-__device__ __forceinline__ DtKey<T> dt_key(const int4 &p, const int4 &e, const int4 &c, int side) {
-    const T ex = e.x - p.x, ey = e.y - p.y, cx = c.x - p.x, cy = c.y - p.y;
-    DtKey<T> k;
-    k.N = cx * cx + cy * cy - (ex * cx + ey * cy);
-    k.D = 2 * side * (ex * cy - ey * cx);
-    return k;
-}
-
-// Does c2 (key k2) beat c1 (key k1) for edge (p, e) on side s?
-template <typename T>
-__device__ __forceinline__ bool dt_key_better(const DtKey<T> &k1, const DtKey<T> &k2, const int4 &p, const int4 &e,
-                                              const int4 &c1, const int4 &c2, int side) {
-    const T l = k2.N * k1.D, r = k1.N * k2.D;
-    if (l != r) return l < r;
-    const int s = side > 0 ? dt_incircle<int64_t>(p, e, c1, c2) : dt_incircle<int64_t>(p, c1, e, c2);
-    return s > 0 || (s == 0 && c2.z < c1.z);
-}
-
-// Pass 1: one group of kDtGroup lanes (kDtGroupOne for one pair) per point.
-// The group lists the points within R of p (kDtRadius for one pair,
-// kDtRadiusBatch in batches; indices into the grid-sorted array, in shared
-// memory), then wraps the star: each lane keeps the best candidate of its
-// share of the list under the pencil key (32-bit integers are exact: every
-// difference is at most R <= 64) and the group reduces with shuffles.  A
-// star is accepted when every triangle's circumdisc lies inside the radius
-// (4 r^2 <= R^2, exact) and, for an open star (p on the hull), nothing lies
-// beyond either open edge (checked against the extreme points of every image
-// row).  Other stars are queued for the next pass.
-constexpr int kDtGroup = 4;       // lanes per star in batched launches (issue-bound: less divergence waste)
-constexpr int kDtGroupOne = 16;   // lanes per star for one pair (latency-bound: shorter star chains)
-constexpr int kDtGroupThreads = 256;
-constexpr int kDtListCap = 128;  // candidates per point (a radius-24 disc holds at most ~75 lattice points at step 5)
-constexpr int kDtRadiusB = 64;   // warp pass (batches): one warp per star left by the middle pass
-constexpr int kDtListCapB = 640; // the radius-64 disc holds at most ~520 lattice points
-
-// Group reduction of (best, key) under the pencil order of edge (p, e).
-template <int G>
-__device__ __forceinline__ int4 dt_group_best(unsigned m, int4 best, DtKey<int> bk, const int4 &p, const int4 &e,
-                                              int side) {
-#pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) {
-        int4 ob;
-        ob.x = __shfl_xor_sync(m, best.x, o);
-        ob.y = __shfl_xor_sync(m, best.y, o);
-        ob.z = __shfl_xor_sync(m, best.z, o);
-        ob.w = __shfl_xor_sync(m, best.w, o);
-        DtKey<int> ok;
-        ok.N = __shfl_xor_sync(m, bk.N, o);
-        ok.D = __shfl_xor_sync(m, bk.D, o);
-        bool take = false;
-        if (ob.w) {
-            if (!best.w) {
-                take = true;
-            } else {
-                // the same decision on both lanes of the pair: compare in a
-                // fixed order (lower index first)
-                const bool mine_first = best.z < ob.z;
-                const bool second_wins = mine_first ? dt_key_better<int>(bk, ok, p, e, best, ob, side)
-                                                    : dt_key_better<int>(ok, bk, p, e, ob, best, side);
-                take = mine_first ? second_wins : !second_wins;
-            }
-        }
-        if (take) {
-            best = ob;
-            bk = ok;
-        }
+// Candidates of a star as packed relative coordinates and list index.
+struct DtListSrc {
+    const int2 *list;
+    int k;
+    __device__ __forceinline__ DtPt get(int c) const {
+        const int2 v = list[c];
+        return DtPt{(int)(int16_t)(v.x & 0xFFFF), v.x >> 16, v.y};
     }
-    return best;
-}
+};
+__device__ __forceinline__ int2 dt_pack(int x, int y, int z) { return make_int2((y << 16) | (x & 0xFFFF), z); }
 
-// Star queues of a side: 1 = (pending, npending), 2 = (pending2,
-// npending2), 3 = (pending, npending3) (batches: the third pass's output,
-// written after the second pass has read `pending`).
-__device__ __forceinline__ const int32_t *dt_queue(const DtSide &S, int q) { return q == 2 ? S.pending2 : S.pending; }
-__device__ __forceinline__ int32_t *dt_queue_len(const DtSide &S, int q) {
-    return q == 2 ? S.npending2 : (q == 3 ? S.npending3 : S.npending);
-}
-
-// G lanes per star, candidates within R (list capacity CAP).  QIN: 0 =
-// every point, else the stars of that queue; failures go to queue QOUT.
-template <int G, int R, int CAP, int QIN, int QOUT>
-__device__ __forceinline__ void dt_group_pass_body(const DtArgs &a, const VB &vb) {
-    constexpr bool QUEUE = QIN != 0;
-    static_assert(2 * R / kDtCell + 2 <= G, "the group's lanes fetch the cell rows of the disc");
-    static_assert(R <= 64, "32-bit pencil keys are exact for coordinates within 64 of p");
-    __shared__ int s_list[kDtGroupThreads / G][CAP];
-    const DtSide S = vb.y ? a.s[1] : a.s[0];
-    const int n = min(max(*a.count, 0), a.cap);
-    const int lane = threadIdx.x & 31, gl = lane & (G - 1), gbase = lane & ~(G - 1);
-    const unsigned gm = G == 32 ? 0xFFFFFFFFu : ((1u << (G & 31)) - 1u) << gbase;
-    int *list = s_list[threadIdx.x / G];
-    const int groups = vb.gx * (kDtGroupThreads / G);
-    const int njobs = QUEUE ? *dt_queue_len(S, QIN) : n;
-    const int32_t *qin = dt_queue(S, QIN);
-    for (int j = vb.x * (kDtGroupThreads / G) + threadIdx.x / G; j < njobs; j += groups) {
-        const int4 p = QUEUE ? S.pts[S.slot[qin[j]]] : S.pts[j];
-        if (!p.w || (!QUEUE && S.status[p.z] != 0)) continue;
-        // candidates: lanes fetch the cell rows' ranges, then stride over them
-        const int cx0 = max(0, p.x - R) / kDtCell, cx1 = min(a.gw - 1, max(0, p.x + R) / kDtCell);
-        const int cy0 = max(0, p.y - R) / kDtCell, cy1 = min(a.gh - 1, max(0, p.y + R) / kDtCell);
-        const int nrows = cy1 - cy0 + 1;  // at most 2R/16 + 2
-        int rs = 0, re = 0;
-        if (gl < nrows) {
-            rs = S.cell_start[(cy0 + gl) * a.gw + cx0];
-            re = S.cell_start[(cy0 + gl) * a.gw + cx1 + 1];
-        }
-        int k = 0;
-        unsigned long long key = ~0ull;
-        int nn = -1;
-        for (int r = 0; r < nrows; ++r) {
-            const int s0 = __shfl_sync(gm, rs, gbase + r), e0 = __shfl_sync(gm, re, gbase + r);
-            for (int c = s0; c < e0; c += G) {
-                bool take = false;
-                if (c + gl < e0) {
-                    const int4 q = S.pts[c + gl];
-                    const int dx = q.x - p.x, dy = q.y - p.y, d2 = dx * dx + dy * dy;
-                    take = q.w && q.z != p.z && d2 <= R * R;
-                    if (take) {
-                        const unsigned long long kk = ((unsigned long long)d2 << 32) | (unsigned)q.z;
-                        if (kk < key) {
-                            key = kk;
-                            nn = c + gl;
-                        }
-                    }
-                }
-                const unsigned b = __ballot_sync(gm, take) >> gbase;
-                const int pos = k + __popc(b & ((1u << gl) - 1u));
-                if (take && pos < CAP) list[pos] = c + gl;
-                k += __popc(b);
-            }
-        }
-        __syncwarp(gm);
-        bool certified = k > 0 && k <= CAP;
-        int written = 0;
-        bool open_l = false, open_r = false;
-        int4 e_l = p, e_r = p;
-        if (certified) {
-            // nearest neighbour of the group
-            unsigned long long kmin = key;
-#pragma unroll
-            for (int o = G / 2; o > 0; o >>= 1) {
-                const unsigned long long other = __shfl_xor_sync(gm, kmin, o);
-                kmin = other < kmin ? other : kmin;
-            }
-            const int src = __ffs(__ballot_sync(gm, key == kmin) >> gbase) - 1;
-            const int first_slot = __shfl_sync(gm, nn, gbase + src);
-            const int4 first = S.pts[first_slot];
-            int4 cur = first;
-            bool closed = false;
-            for (int step = 0; step <= k && certified; ++step) {  // counter-clockwise
-                int4 best = make_int4(0, 0, 0, 0);
-                DtKey<int> bk{0, 1};
-                for (int c = gl; c < k; c += G) {
-                    const int4 q = S.pts[list[c]];
-                    if (q.z == cur.z) continue;
-                    const DtKey<int> qk = dt_key<int>(p, cur, q, +1);
-                    if (qk.D <= 0) continue;
-                    if (!best.w || dt_key_better<int>(bk, qk, p, cur, best, q, +1)) {
-                        best = q;
-                        bk = qk;
-                    }
-                }
-                best = dt_group_best<G>(gm, best, bk, p, cur, +1);
-                if (!best.w) {
-                    open_l = true;
-                    e_l = cur;
-                    break;
-                }
-                if (!dt_small_circle_r<R>(p, cur, best)) {
-                    certified = false;
-                    break;
-                }
-                dt_record(S, p.z, written, p, cur, best, gl == 0);
-                if (best.z == first.z) {
-                    closed = true;
-                    break;
-                }
-                cur = best;
-            }
-            if (certified && !closed) {
-                if (!open_l) certified = false;  // ran out of steps
-                cur = first;
-                for (int step = 0; step <= k && certified; ++step) {  // clockwise
-                    int4 best = make_int4(0, 0, 0, 0);
-                    DtKey<int> bk{0, 1};
-                    for (int c = gl; c < k; c += G) {
-                        const int4 q = S.pts[list[c]];
-                        if (q.z == cur.z) continue;
-                        const DtKey<int> qk = dt_key<int>(p, cur, q, -1);
-                        if (qk.D <= 0) continue;
-                        if (!best.w || dt_key_better<int>(bk, qk, p, cur, best, q, -1)) {
-                            best = q;
-                            bk = qk;
-                        }
-                    }
-                    best = dt_group_best<G>(gm, best, bk, p, cur, -1);
-                    if (!best.w) {
-                        open_r = true;
-                        e_r = cur;
-                        break;
-                    }
-                    if (!dt_small_circle_r<R>(p, best, cur)) {
-                        certified = false;
-                        break;
-                    }
-                    dt_record(S, p.z, written, p, best, cur, gl == 0);
-                    cur = best;
-                }
-                if (!open_r) certified = false;
-            }
-            // open edges (p on the hull): nothing may lie beyond them
-            for (int side = 0; side < 2 && certified; ++side) {
-                const bool open = side ? open_r : open_l;
-                if (!open) continue;
-                const int4 e = side ? e_r : e_l;
-                bool bad = false;
-                for (int y = gl; y < a.h && !bad; y += G) {
-                    const int x0 = S.rowmin[y], x1 = S.rowmax[y];
-                    if (x0 > x1) continue;
-                    const int64_t o0 = dt_orient(p.x, p.y, e.x, e.y, x0, y);
-                    const int64_t o1 = dt_orient(p.x, p.y, e.x, e.y, x1, y);
-                    bad = side ? (o0 < 0 || o1 < 0) : (o0 > 0 || o1 > 0);
-                }
-                if (__ballot_sync(gm, bad) & gm) certified = false;
-            }
-        }
-        if (gl == 0) {
-            if (certified) {
-                S.status[p.z] = 1;
-                S.owned[p.z] = written;
-                if (written > kDtSlots) atomicOr(S.err, 4);
-            } else {
-                const_cast<int32_t *>(dt_queue(S, QOUT))[atomicAdd(dt_queue_len(S, QOUT), 1)] = p.z;
-            }
-        }
-        __syncwarp(gm);
+// A quarter of the grid-sorted points (the exact pass over every point).
+struct DtAllSrc {
+    const int4 *pts;
+    int k, part, px, py, pz;
+    __device__ __forceinline__ DtPt get(int c) const {
+        const int4 q = pts[4 * c + part];
+        if (!q.w || q.z == pz) return DtPt{0, 0, pz};  // D = 0: never a candidate
+        return DtPt{q.x - px, q.y - py, q.z};
     }
-}
-
-
-template <int G, int R> __device__ __forceinline__ void dt_pass1_body(const DtArgs &a, const VB &vb) {
-    dt_group_pass_body<G, R, kDtListCap, 0, 1>(a, vb);
-}
-
-// Batches: the stars left by the first pass go through a middle pass (eight
-// lanes, the 32-pixel disc) and those left again through the warp pass
-// (the 64-pixel disc); the CTA pass takes the third queue.
-constexpr int kDtRadiusM = 32;
-constexpr int kDtListCapM = 192;  // the radius-32 disc holds at most ~130 lattice points
-constexpr int kDtGroupM = 8;
-
-__global__ void __launch_bounds__(kDtGroupThreads, 4) dt_pass1m_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
-    const VB vb = vb_batch(vm);
-    dt_group_pass_body<kDtGroupM, kDtRadiusM, kDtListCapM, 1, 2>(slot_entry(tab, vm.stride, vb.slot), vb);
-}
-__global__ void __launch_bounds__(kDtGroupThreads, 3) dt_pass1b_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
-    const VB vb = vb_batch(vm);
-    dt_group_pass_body<32, kDtRadiusB, kDtListCapB, 2, 3>(slot_entry(tab, vm.stride, vb.slot), vb);
-}
-
-__global__ void __launch_bounds__(kDtGroupThreads, 4) dt_pass1_kernel(DtArgs a) {
-    dt_pass1_body<kDtGroupOne, kDtRadius>(a, vb_single());
-}
-// A batch of one pair takes the one-pair group pass (wider groups, larger disc).
-__global__ void __launch_bounds__(kDtGroupThreads, 4) dt_pass1_kernel_b1(const DtArgs *__restrict__ tab, VMap vm) {
-    const VB vb = vb_batch(vm);
-    dt_pass1_body<kDtGroupOne, kDtRadius>(slot_entry(tab, vm.stride, vb.slot), vb);
-}
-__global__ void __launch_bounds__(kDtGroupThreads, 4) dt_pass1_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
-    const VB vb = vb_batch(vm);
-    dt_pass1_body<kDtGroup, kDtRadiusBatch>(slot_entry(tab, vm.stride, vb.slot), vb);
-}
-
-// CTA pass: one CTA per star left by the group passes.  The points within
-// kDtRadius1 are cached in shared memory; every wrap step first takes the
-// best cached candidate and keeps it when its circumdisc lies inside the
-// cached disc (then no other point can beat it); the first step that does
-// not fit refills the cache with the points within kDtRadius2, and a step
-// that fits neither (large circle, no cached candidate on that side, or the
-// cache overflowed) scans the grid cells its disc or half-plane meets, which
-// is exact.  So every queued star comes out exact.
-constexpr int kDtRadius1 = 96;     // first cache radius of the CTA pass
-constexpr int kDtRadius2 = 192;    // its second, when a step's circle does not fit the first
-constexpr int kDtCandCap2 = 3072;  // candidates cached per CTA (48 KB)
-constexpr int kDtMaxRows = 64;     // cell rows a radius-192 disc spans, with margin
-constexpr int kDtBlockThreads = 256;  // threads of a CTA-pass CTA (one pair: its longest star sets the pass)
-constexpr int kDtBlocksPerSM = 3;     // CTA-pass CTAs resident per SM (85 registers a thread)
-// batches of two or more pairs: smaller CTAs, one more per SM (more stars at
-// once across the pairs; a step's selection takes a little longer)
-constexpr int kDtBlockThreadsB = 192;
-constexpr int kDtBlocksPerSMB = 4;
-static_assert(2 * kDtRadius2 / kDtCell + 2 <= kDtMaxRows, "the CTA pass's disc must fit the row table");
-
-// CTA reduction of the threads' (best, key) under the pencil order: each
-// warp reduces with shuffles, warp 0 reduces the warps' results, and every
-// thread reads the winner from shared memory.
-template <int UNUSED = 0>
-__device__ __forceinline__ int4 dt_warp_key_best(int4 best, DtKey<int64_t> &bk, const int4 &p, const int4 &e,
-                                                 int side) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const int4 ob = shfl4(best, o);
-        DtKey<int64_t> ok;
-        ok.N = __shfl_xor_sync(0xFFFFFFFFu, bk.N, o);
-        ok.D = __shfl_xor_sync(0xFFFFFFFFu, bk.D, o);
-        if (ob.w && (!best.w || dt_key_better<int64_t>(bk, ok, p, e, best, ob, side))) {
-            best = ob;
-            bk = ok;
-        }
-    }
-    return best;
-}
-
-__device__ __forceinline__ int4 dt_block_best(int4 best, DtKey<int64_t> bk, const int4 &p, const int4 &e, int side,
-                                              int4 *s_red, int64_t *s_n, int64_t *s_d) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    best = dt_warp_key_best(best, bk, p, e, side);
-    __syncthreads();
-    if (lane == 0) {
-        s_red[warp] = best;
-        s_n[warp] = bk.N;
-        s_d[warp] = bk.D;
-    }
-    __syncthreads();
-    if (warp == 0) {
-        int4 b = lane < nw ? s_red[lane] : make_int4(0, 0, 0, 0);
-        DtKey<int64_t> k{lane < nw ? s_n[lane] : 0, lane < nw ? s_d[lane] : 1};
-        b = dt_warp_key_best(b, k, p, e, side);
-        if (lane == 0) s_red[32] = b;
-    }
-    __syncthreads();
-    return s_red[32];
-}
-
-struct DtBlockShared {
-    int4 red[33];
-    int64_t rn[32], rd[32];
-    unsigned long long key[32];
-    int rs[kDtMaxRows], rlen[kDtMaxRows + 1], cnt;
-    unsigned fmin[3];  // least float key of a selection (three buffers, used in turn)
-    int nband[3];      // band members listed by a selection
-    int4 win;          // winner of an exactly ordered band
-    int small;         // the first band member's circle fits the disc of radius R (selections with R > 0)
 };
 
-// Float filter of the pencil order (CTA pass).  With coordinates below 2^14
-// the key (N, D) of every candidate fits in 32 bits (|N|, |D| < 2^31) and
-// two keys compare exactly through 64-bit products.  The float
-// f = fl(N) / fl(D) (two conversions rounded to nearest, one division within
-// 2 ulp) is within 2^-21 |t| of t = N / D, so the exact winner w (least t)
-// has f_w - f_min <= 2^-21 (|f_w| + |f_min|) + rounding, f_min the least f
-// over the candidates: every candidate that can win lies in the band
-// f - f_min <= 2^-17 (|f| + |f_min|).  A band of one is the winner; a larger
-// band (cocircular candidates, or nearly) is ordered exactly.
-constexpr int kDtBandCap = 32;
-
-__device__ __forceinline__ unsigned dt_fbits(float f) {  // monotone in f (no NaN)
-    const unsigned u = __float_as_uint(f);
-    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-__device__ __forceinline__ float dt_fbits_value(unsigned k) {
-    return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);
-}
-__device__ __forceinline__ float dt_fkey(const DtKey<int> &k) { return __fdividef((float)k.N, (float)k.D); }
-__device__ __forceinline__ bool dt_in_band(float f, float fmin) {
-    return f - fmin <= 0x1p-17f * (fabsf(f) + fabsf(fmin));
-}
-
-// Does c2 (key k2) beat c1 (key k1)?  32-bit keys, 64-bit products.
-__device__ __forceinline__ bool dt_key_better_w(const DtKey<int> &k1, const DtKey<int> &k2, const int4 &p,
-                                                const int4 &e, const int4 &c1, const int4 &c2, int side) {
-    const int64_t l = (int64_t)k2.N * k1.D, r = (int64_t)k1.N * k2.D;
+// Does c2 beat c1 for edge (p, e) on `side`, exactly?
+__device__ __forceinline__ bool dt_beats(const DtPt &e, int pz, const DtPt &c1, const DtPt &c2, int side) {
+    const int D1 = side * (e.x * c1.y - e.y * c1.x), D2 = side * (e.x * c2.y - e.y * c2.x);
+    const int N1 = c1.x * c1.x + c1.y * c1.y - (e.x * c1.x + e.y * c1.y);
+    const int N2 = c2.x * c2.x + c2.y * c2.y - (e.x * c2.x + e.y * c2.y);
+    const int64_t l = (int64_t)N2 * D1, r = (int64_t)N1 * D2;
     if (l != r) return l < r;
-    const int s = side > 0 ? dt_incircle<int64_t>(p, e, c1, c2) : dt_incircle<int64_t>(p, c1, e, c2);
-    return s > 0 || (s == 0 && c2.z < c1.z);
+    if (c1.z == c2.z) return false;
+    return dt_tie_second(pz, e.z, c1.z, c2.z, side * ((int64_t)c1.x * c2.y - (int64_t)c1.y * c2.x) > 0);
 }
 
-// CTA-wide Delaunay third vertex of edge (p, e) on `side`: each thread
-// offers its candidates through each(visit) (called twice), thread 0 also
-// the seed (w = 0: none).  Pass 1 finds the least float key (one warp
-// reduction and a shared atomic), pass 2 has every thread take the exact
-// best of its candidates in the band (its least one, unless its second
-// least is in the band too) and list it; a single listed candidate
-// is the winner, else warp 0 orders the list exactly (the whole CTA when it
-// overflows).  par: the caller's turn counter (the same on every thread).
-// With R > 0, small tells whether the winner's circumdisc lies inside the
-// disc of radius R about p (dt_small_circle): the thread that lists the
-// first band member tests it before the second barrier, which is the answer
-// when the band has one member, so the other threads skip the 64-bit test.
-// Thread 0 resets the next call's buffers before this call's first barrier:
-// their last readers (two calls back) have passed the previous call's first
-// barrier, and the next call writes them only after this call's.
-template <typename Each>
-__device__ int4 dt_block_select(Each each, const int4 &p, const int4 &e, int side, const int4 &seed,
-                                DtBlockShared &sh, int &par, int R, bool &small) {
-    const int tid = threadIdx.x, lane = tid & 31;
-    const int b = par, nxt = par == 2 ? 0 : par + 1;
-    par = nxt;
-    small = false;
-    if (tid == 0) {
-        sh.fmin[nxt] = 0xFFFFFFFFu;
-        sh.nband[nxt] = 0;
-    }
-    auto usable = [&](const int4 &q) { return q.w && q.z != e.z && q.z != p.z; };
-    // each thread keeps its least float key (with its candidate) and its
-    // second least
-    const float inf = __int_as_float(0x7F800000);
-    float fl = inf, f2 = inf;
-    int4 q1 = make_int4(0, 0, 0, 0);
-    auto offer = [&](const int4 &q) {
-        if (!usable(q)) return;
-        const DtKey<int> k = dt_key<int>(p, e, q, side);
-        if (k.D <= 0) return;
-        const float f = dt_fkey(k);
-        if (f < fl) {
-            f2 = fl;
-            fl = f;
-            q1 = q;
-        } else if (f < f2) {
-            f2 = f;
-        }
-    };
-    each(offer);
-    if (tid == 0) offer(seed);
-    const unsigned kb = __reduce_min_sync(0xFFFFFFFFu, fl == __int_as_float(0x7F800000) ? 0xFFFFFFFFu : dt_fbits(fl));
-    if (lane == 0 && kb != 0xFFFFFFFFu) atomicMin(&sh.fmin[b], kb);
-    __syncthreads();
-    const unsigned kmin = sh.fmin[b];
-    if (kmin == 0xFFFFFFFFu) return make_int4(0, 0, 0, 0);  // uniform: no candidate on this side
-    const float fmin = dt_fbits_value(kmin);
-    int4 best = make_int4(0, 0, 0, 0);
-    DtKey<int> bk{0, 1};
-    // the band test is increasing in f: with the second least key outside
-    // the band only the least can be in it; else the thread offers again
-    if (q1.w && dt_in_band(fl, fmin)) {
-        if (f2 != inf && dt_in_band(f2, fmin)) {
-            auto visit = [&](const int4 &q) {
-                if (!usable(q)) return;
-                const DtKey<int> k = dt_key<int>(p, e, q, side);
-                if (k.D <= 0 || !dt_in_band(dt_fkey(k), fmin)) return;
-                if (!best.w || dt_key_better_w(bk, k, p, e, best, q, side)) {
-                    best = q;
-                    bk = k;
-                }
-            };
-            each(visit);
-            if (tid == 0) visit(seed);
-        } else {
-            best = q1;
-            bk = dt_key<int>(p, e, q1, side);
+// One wrap step by a warp over src's candidates, exact while every
+// coordinate difference stays below 2^14.5 (N and D fit 32 bits; their
+// rounding to FP32 and the division leave a relative error below 2^-20).
+template <class Src>
+__device__ __forceinline__ bool dt_step(const Src &src, int lane, const DtPt &e, int pz, int side, DtPt &w) {
+    float f1 = kDtInf, f2 = kDtInf;
+    int c1 = 0;
+    const int sx = side * e.x, sy = side * e.y;
+#pragma unroll 4
+    for (int c = lane; c < src.k; c += 32) {
+        const DtPt q = src.get(c);
+        const int D = sx * q.y - sy * q.x, N = q.x * q.x + q.y * q.y - (e.x * q.x + e.y * q.y);
+        const float f = D > 0 ? __fdividef((float)N, (float)D) : kDtInf;
+        f2 = fminf(f2, fmaxf(f1, f));
+        if (f < f1) {
+            f1 = f;
+            c1 = c;
         }
     }
-    auto fits = [&](const int4 &c) {
-        return c.w && (side > 0 ? dt_small_circle(p, e, c, R) : dt_small_circle(p, c, e, R));
-    };
-    if (best.w) {
-        const int pos = atomicAdd(&sh.nband[b], 1);
-        if (pos < kDtBandCap) {
-            sh.red[pos] = best;
-            sh.rn[pos] = bk.N;
-            sh.rd[pos] = bk.D;
-            if (pos == 0 && R > 0) sh.small = fits(best);
-        }
-    }
-    __syncthreads();
-    const int nb = sh.nband[b];
-    if (nb == 1) {
-        small = R > 0 && sh.small;
-        return sh.red[0];
-    }
-    int4 w;
-    if (nb > kDtBandCap) {
-        w = dt_block_best(best, DtKey<int64_t>{bk.N, bk.D}, p, e, side, sh.red, sh.rn, sh.rd);
-    } else {
-        if (tid < 32) {
-            int4 c = lane < nb ? sh.red[lane] : make_int4(0, 0, 0, 0);
-            DtKey<int64_t> k{lane < nb ? sh.rn[lane] : 0, lane < nb ? sh.rd[lane] : 1};
-            c = dt_warp_key_best(c, k, p, e, side);
-            if (lane == 0) sh.win = c;
-        }
-        __syncthreads();
-        w = sh.win;
-    }
-    small = R > 0 && fits(w);
-    return w;
-}
-
-// Best third vertex for edge (p, cur) on `side`, over the cache (cand, k) or,
-// with cand == NULL, over every alive point.
-__device__ __forceinline__ int4 dt_block_step(const DtSide &S, const int4 &p, const int4 &cur, int side,
-                                              const int4 *cand, int k, int n, DtBlockShared &sh, int &par, int R,
-                                              bool &small) {
-    const int tid = threadIdx.x, nth = blockDim.x;
-    const int4 none = make_int4(0, 0, 0, 0);
-    if (cand)
-        return dt_block_select(
-            [&](auto &&v) {
-                for (int j = tid; j < k; j += nth) v(cand[j]);
-            },
-            p, cur, side, none, sh, par, R, small);
-    return dt_block_select(
-        [&](auto &&v) {
-            for (int j = tid; j < n; j += nth) v(S.pts[j]);
-        },
-        p, cur, side, none, sh, par, R, small);
-}
-
-// Exact step for edge (p, cur) on `side` without the radius limit.  Only
-// points strictly inside the closed circumdisc of (p, cur, bc) can beat the
-// cached best bc, and with no cached candidate only the open half-plane on
-// that side matters; so the CTA scans the grid cells that meet that region,
-// taking each cell row's cells as one contiguous range.  The region is
-// widened so that float rounding cannot lose a cell: the circle's centre
-// comes from exact integer numerators (one rounding each in the division),
-// its radius is padded by 4 pixels plus 1e-4 of itself, each cell row band
-// by 2 pixels and each x-range by a cell; a circle wider than 1e6 pixels is
-// replaced by its half-plane (the part of the disc beyond the chord p-cur
-// is then thinner than a pixel, and only that side's points are candidates).
-__device__ int4 dt_block_region_step(const DtArgs &a, const DtSide &S, const int4 &p, const int4 &cur, int side,
-                                     const int4 &bc, DtBlockShared &sh, int *r_start, int *r_len, int &par) {
-    const int tid = threadIdx.x, nth = blockDim.x;
-    float ccx = 0.0f, ccy = 0.0f, rad = 0.0f;
-    bool disc = false;
-    if (bc.w) {
-        const int64_t ax = cur.x - p.x, ay = cur.y - p.y, bx = bc.x - p.x, by = bc.y - p.y;
-        const int64_t d = 2 * (ax * by - ay * bx);  // nonzero: bc lies strictly on `side`
-        const int64_t a2 = ax * ax + ay * ay, b2 = bx * bx + by * by;
-        const float fd = (float)d;
-        const float ux = (float)(by * a2 - ay * b2) / fd, uy = (float)(ax * b2 - bx * a2) / fd;
-        const float r = sqrtf(ux * ux + uy * uy);
-        if (r <= 1e6f) {
-            disc = true;
-            ccx = (float)p.x + ux;
-            ccy = (float)p.y + uy;
-            rad = r * 1.0001f + 4.0f;
-        }
-    }
-    // half-plane: side * ((cur.x-p.x)(y-p.y) - (cur.y-p.y)(x-p.x)) > 0
-    const int ex = cur.x - p.x, ey = cur.y - p.y;
-    for (int cy = tid; cy < a.gh; cy += nth) {
-        const int y0 = cy * kDtCell - 2, y1 = cy * kDtCell + kDtCell + 1;
-        float xlo = -1e30f, xhi = 1e30f;
-        bool any = true;
-        if (disc) {
-            const float dy = ccy < (float)y0 ? (float)y0 - ccy : (ccy > (float)y1 ? ccy - (float)y1 : 0.0f);
-            if (dy > rad) {
-                any = false;
-            } else {
-                const float hc = sqrtf(rad * rad - dy * dy) + 2.0f;
-                xlo = ccx - hc;
-                xhi = ccx + hc;
+    const float fm = dt_warp_min(f1);
+    if (fm == kDtInf) return false;
+    const float thr = fm + 0x1p-17f * fabsf(fm);
+    bool in = f1 <= thr;
+    if (in && f2 <= thr) {  // several of this lane's candidates: keep the exact best
+        int best = -1;
+        DtPt bq{0, 0, 0};
+        for (int c = lane; c < src.k; c += 32) {
+            const DtPt q = src.get(c);
+            const int D = sx * q.y - sy * q.x, N = q.x * q.x + q.y * q.y - (e.x * q.x + e.y * q.y);
+            if (D <= 0 || __fdividef((float)N, (float)D) > thr) continue;
+            if (best < 0 || dt_beats(e, pz, bq, q, side)) {
+                best = c;
+                bq = q;
             }
-        } else if (ey != 0) {
-            // boundary x at the band's two edges (exact products, one rounding
-            // in each division); the admissible side of x
-            const float xa = (float)p.x + (float)(ex * (y0 - p.y)) / (float)ey;
-            const float xb = (float)p.x + (float)(ex * (y1 - p.y)) / (float)ey;
-            const float xm = fminf(xa, xb), xM = fmaxf(xa, xb);
-            // side*(ex*(y-py) - ey*(x-px)) > 0  <=>  x < boundary if side*ey > 0
-            if (side * ey > 0)
-                xhi = xM + 2.0f;
-            else
-                xlo = xm - 2.0f;
-        } else {
-            // horizontal edge: the whole row is in or out
-            any = side * ex * (y0 + y1 - 2 * p.y) > 0 || (y0 <= p.y && p.y <= y1);
         }
-        int c0 = 0, c1 = a.gw - 1;
-        if (any) {
-            c0 = xlo < 0.0f ? 0 : (int)fminf((float)(a.gw - 1), floorf(xlo / kDtCell) - 1.0f);
-            c1 = xhi >= 1e29f ? a.gw - 1 : (int)fmaxf(0.0f, fminf((float)(a.gw - 1), floorf(xhi / kDtCell) + 1.0f));
-            c0 = max(0, c0);
-        }
-        const int s0 = any && c0 <= c1 ? S.cell_start[cy * a.gw + c0] : 0;
-        const int e0 = any && c0 <= c1 ? S.cell_start[cy * a.gw + c1 + 1] : 0;
-        r_start[cy] = s0;
-        r_len[cy] = e0 - s0;  // the row's range length
+        c1 = best;
     }
-    __syncthreads();
-    // each warp takes cell rows in turn; its lanes stride over the row's
-    // contiguous range of the grid-sorted points
-    const int lane = tid & 31, warp = tid >> 5, nwarps = nth >> 5;
-    bool unused;
-    return dt_block_select(
-        [&](auto &&v) {
-            for (int cy = warp; cy < a.gh; cy += nwarps) {
-                const int s0 = r_start[cy], len = r_len[cy];
-                int j = lane;
-                for (; j + 96 < len; j += 128) {  // four loads in flight
-                    const int4 q0 = S.pts[s0 + j], q1 = S.pts[s0 + j + 32], q2 = S.pts[s0 + j + 64],
-                               q3 = S.pts[s0 + j + 96];
-                    v(q0);
-                    v(q1);
-                    v(q2);
-                    v(q3);
-                }
-                for (; j < len; j += 32) v(S.pts[s0 + j]);
-            }
-        },
-        p, cur, side, bc, sh, par, 0, unused);
+    unsigned b = __ballot_sync(0xFFFFFFFFu, in);
+    int ch = __shfl_sync(0xFFFFFFFFu, c1, __ffs(b) - 1);
+    w = src.get(ch);
+    if (b & (b - 1)) {
+        const DtPt mine = in ? src.get(c1) : w;
+        while (b & (b - 1)) {
+            in = in && c1 != ch && dt_beats(e, pz, w, mine, side);
+            b = __ballot_sync(0xFFFFFFFFu, in);
+            if (!b) break;
+            ch = __shfl_sync(0xFFFFFFFFu, c1, __ffs(b) - 1);
+            w = src.get(ch);
+        }
+    }
+    return true;
 }
 
-__device__ int dt_block_gather(const DtArgs &a, const DtSide &S, const int4 &p, int R, int4 *cand,
-                               DtBlockShared &sh);
-
-// Exact star of p, CTA-wide.  cand: shared cache (capacity kDtCandCap2)
-// holding the k points within R of p (k > kDtCandCap2: unusable), or NULL.
-// A step is taken from the cache when the winner's circle lies inside the
-// disc of radius R (2r <= R: no point outside the cache can be inside it);
-// otherwise the cache is refilled once at kDtRadius2 and, if that still does
-// not hold the circle, the step scans the cells its disc or half-plane meets
-// (every point without the region tables).  Writes the owned triangles to the
-// slots or, with out != NULL, to out.  Returns 1, or -1 if it exceeded
-// kDtMaxStar.
-__device__ int dt_block_star(const DtArgs &a, const DtSide &S, int i, const int4 &p, int n, int4 *cand, int R, int k,
-                             int *written, int32_t *out, DtBlockShared &sh, int *r_start, int *r_len) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nth = blockDim.x;
-    int par = 0;  // selection buffers: cleared here, before the barriers below
-    if (tid == 0) {
-        sh.fmin[0] = sh.fmin[1] = sh.fmin[2] = 0xFFFFFFFFu;
-        sh.nband[0] = sh.nband[1] = sh.nband[2] = 0;
-    }
-    // nearest neighbour: a cached point is nearer than every point outside
-    // the cache, so a non-empty cache holds it; else one pass over all points
-    unsigned long long key = ~0ull;
-    const bool nn_cached = cand && k > 0 && k <= kDtCandCap2;
-    const int nn_n = nn_cached ? k : n;
-    for (int j = tid; j < nn_n; j += nth) {
-        const int4 q = nn_cached ? cand[j] : S.pts[j];
-        if (q.w && q.z != p.z) {
-            const unsigned long long kk = dt_nn_key(p, q);
-            key = kk < key ? kk : key;
-        }
-    }
-    key = warp_min64(key);
-    __syncthreads();
-    if (lane == 0) sh.key[warp] = key;
-    __syncthreads();
-    key = lane < (nth >> 5) ? sh.key[lane] : ~0ull;
-    key = warp_min64(key);
-    *written = 0;
-    if (key == ~0ull) return 1;  // p is the only point
-    const int4 first = S.pts[S.slot[(int)(unsigned)(key & 0xFFFFFFFFu)]];
-    int wr = 0;
-    auto emit = [&](const int4 &u, const int4 &v) {  // triangle (p, u, v), ccw
-        if (p.z < u.z && p.z < v.z) {
-            if (tid == 0) {
-                if (out) {
-                    out[3 * wr] = p.z;
-                    out[3 * wr + 1] = u.z;
-                    out[3 * wr + 2] = v.z;
-                } else if (wr < kDtSlots) {
-                    int32_t *slot = S.slots + ((size_t)i * kDtSlots + wr) * 2;
-                    slot[0] = u.z;
-                    slot[1] = v.z;
-                }
-            }
-            ++wr;
-        }
+// First vertex of a fan (see dt_warp_star): the candidate below p (y > 0)
+// that a circle through p growing straight down touches first, least
+// |c|^2 / y; of several on that circle the first one counter-clockwise.
+template <class Src> __device__ __forceinline__ bool dt_fan_start(const Src &src, int lane, DtPt &w) {
+    auto better = [](const DtPt &c1, const DtPt &c2) {  // c2 before c1
+        const int64_t l = (int64_t)(c2.x * c2.x + c2.y * c2.y) * c1.y, r = (int64_t)(c1.x * c1.x + c1.y * c1.y) * c2.y;
+        if (l != r) return l < r;
+        return (int64_t)c2.x * c1.y - (int64_t)c2.y * c1.x > 0;
     };
-    auto next = [&](const int4 &cur, int side) {
-        int4 b = make_int4(0, 0, 0, 0);
+    float f1 = kDtInf, f2 = kDtInf;
+    int c1 = 0;
+    for (int c = lane; c < src.k; c += 32) {
+        const DtPt q = src.get(c);
+        const float f = q.y > 0 ? __fdividef((float)(q.x * q.x + q.y * q.y), (float)q.y) : kDtInf;
+        f2 = fminf(f2, fmaxf(f1, f));
+        if (f < f1) {
+            f1 = f;
+            c1 = c;
+        }
+    }
+    const float fm = dt_warp_min(f1);
+    if (fm == kDtInf) return false;
+    const float thr = fm + 0x1p-17f * fm;
+    bool in = f1 <= thr;
+    if (in && f2 <= thr) {
+        DtPt bq = src.get(c1);
+        for (int c = lane; c < src.k; c += 32) {
+            const DtPt q = src.get(c);
+            if (q.y > 0 && better(bq, q)) {
+                bq = q;
+                c1 = c;
+            }
+        }
+    }
+    unsigned b = __ballot_sync(0xFFFFFFFFu, in);
+    int ch = __shfl_sync(0xFFFFFFFFu, c1, __ffs(b) - 1);
+    w = src.get(ch);
+    if (b & (b - 1)) {
+        const DtPt mine = in ? src.get(c1) : w;
+        while (b & (b - 1)) {
+            in = in && c1 != ch && better(w, mine);
+            b = __ballot_sync(0xFFFFFFFFu, in);
+            if (!b) break;
+            ch = __shfl_sync(0xFFFFFFFFu, c1, __ffs(b) - 1);
+            w = src.get(ch);
+        }
+    }
+    return true;
+}
+
+// The warp pass's candidates: within 24 pixels of p, so every key is a small
+// integer and FP32 arithmetic on it is exact (N and D below 2^11, their
+// cross products below 2^24).  Each lane keeps two of them (x, y, |c|^2,
+// index) in registers; a list of more than 64 reads the rest from shared
+// memory.
+struct DtNearSrc {
+    const float4 *list;
+    int k;
+    float4 c0, c1;
+
+    __device__ __forceinline__ void load(int lane) {
+        const float4 none = make_float4(0.0f, 0.0f, 0.0f, 0.0f);  // D = 0 and y = 0: never a candidate
+        c0 = lane < k ? list[lane] : none;
+        c1 = lane + 32 < k ? list[lane + 32] : none;
+    }
+    __device__ __forceinline__ float4 far_cand(int c) const {
+        return c < k ? list[c] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    }
+    __device__ __forceinline__ DtPt point(const float4 &v) const {
+        return DtPt{(int)v.x, (int)v.y, __float_as_int(v.z == 0.0f ? 0.0f : v.w)};
+    }
+    // Least key over the slots, then the exact order among its band:
+    // key(c) (kDtInf: not a candidate), beats(c1, c2): c2 before c1.
+    template <class Key, class Beats>
+    __device__ __forceinline__ bool select(int lane, Key key, Beats beats, float4 &w) const {
+        const float f0 = key(c0), f1 = key(c1);
+        float f2 = kDtInf, f3 = kDtInf;
+        if (k > 64) {
+            f2 = key(far_cand(lane + 64));
+            f3 = key(far_cand(lane + 96));
+        }
+        const float fm = dt_warp_min(fminf(fminf(f0, f1), fminf(f2, f3)));
+        if (fm == kDtInf) return false;
+        const float thr = fm + 0x1p-18f * fabsf(fm);
+        unsigned b0 = __ballot_sync(0xFFFFFFFFu, f0 <= thr), b1 = __ballot_sync(0xFFFFFFFFu, f1 <= thr);
+        unsigned b2 = 0, b3 = 0;
+        if (k > 64) {
+            b2 = __ballot_sync(0xFFFFFFFFu, f2 <= thr);
+            b3 = __ballot_sync(0xFFFFFFFFu, f3 <= thr);
+        }
         for (;;) {
-            if (!cand || k > kDtCandCap2) break;
-            bool small;
-            b = dt_block_step(S, p, cur, side, cand, k, n, sh, par, R, small);
-            if (small) return b;
-            if (R >= kDtRadius2) break;
-            R = kDtRadius2;  // refill the cache once with the larger disc
-            k = dt_block_gather(a, S, p, R, cand, sh);
+            const int ch = b0   ? __ffs(b0) - 1
+                           : b1 ? __ffs(b1) + 31
+                           : b2 ? __ffs(b2) + 63
+                                : __ffs(b3) + 95;
+            w = list[ch];
+            if (__popc(b0) + __popc(b1) + __popc(b2) + __popc(b3) == 1) return true;
+            const unsigned me = 1u << lane;
+            // the champion itself never beats itself
+            const unsigned n0 = __ballot_sync(0xFFFFFFFFu, (b0 & me) && beats(w, c0));
+            const unsigned n1 = __ballot_sync(0xFFFFFFFFu, (b1 & me) && beats(w, c1));
+            unsigned n2 = 0, n3 = 0;
+            if (k > 64) {
+                n2 = __ballot_sync(0xFFFFFFFFu, (b2 & me) && beats(w, far_cand(lane + 64)));
+                n3 = __ballot_sync(0xFFFFFFFFu, (b3 & me) && beats(w, far_cand(lane + 96)));
+            }
+            if (!(n0 | n1 | n2 | n3)) return true;
+            b0 = n0;
+            b1 = n1;
+            b2 = n2;
+            b3 = n3;
         }
-        if (r_start) return dt_block_region_step(a, S, p, cur, side, b, sh, r_start, r_len, par);
-        bool unused;
-        return dt_block_step(S, p, cur, side, nullptr, 0, n, sh, par, 0, unused);
+    }
+};
+
+__device__ __forceinline__ bool dt_step(const DtNearSrc &src, int lane, const float4 &e, int pz, float side,
+                                        float4 &w) {
+    const float sx = side * e.x, sy = side * e.y;
+    auto dkey = [&](const float4 &c) { return __fmaf_rn(sx, c.y, -(sy * c.x)); };
+    auto nkey = [&](const float4 &c) { return __fmaf_rn(-e.x, c.x, __fmaf_rn(-e.y, c.y, c.z)); };
+    return src.select(
+        lane,
+        [&](const float4 &c) {
+            const float D = dkey(c);
+            return D > 0.0f ? __fdividef(nkey(c), D) : kDtInf;
+        },
+        [&](const float4 &c1, const float4 &c2) {
+            const float l = nkey(c2) * dkey(c1), r = nkey(c1) * dkey(c2);
+            if (l != r) return l < r;
+            const int z1 = __float_as_int(c1.w), z2 = __float_as_int(c2.w);
+            return z1 != z2 &&
+                   dt_tie_second(pz, __float_as_int(e.w), z1, z2, side * (c1.x * c2.y - c1.y * c2.x) > 0.0f);
+        },
+        w);
+}
+
+__device__ __forceinline__ bool dt_fan_start(const DtNearSrc &src, int lane, float4 &w) {
+    return src.select(
+        lane, [&](const float4 &c) { return c.y > 0.0f ? __fdividef(c.z, c.y) : kDtInf; },
+        [&](const float4 &c1, const float4 &c2) {
+            const float l = c2.z * c1.y, r = c1.z * c2.y;
+            if (l != r) return l < r;
+            return c2.x * c1.y - c2.y * c1.x > 0.0f;
+        },
+        w);
+}
+
+// Views of a candidate for the star driver.
+__device__ __forceinline__ int dt_z(const DtPt &c) { return c.z; }
+__device__ __forceinline__ int dt_z(const float4 &c) { return __float_as_int(c.w); }
+__device__ __forceinline__ int dt_ix(const DtPt &c) { return c.x; }
+__device__ __forceinline__ int dt_ix(const float4 &c) { return (int)c.x; }
+__device__ __forceinline__ int dt_iy(const DtPt &c) { return c.y; }
+__device__ __forceinline__ int dt_iy(const float4 &c) { return (int)c.y; }
+
+// Nearest candidate (least |c|^2, then least index) and the open quadrants
+// that hold candidates (bit 2*(y>0) + (x>0)).
+__device__ __forceinline__ unsigned dt_quadrant(int x, int y) {
+    return x && y ? 1u << ((x > 0) | ((y > 0) << 1)) : 0u;
+}
+__device__ __forceinline__ float4 dt_nearest(const DtNearSrc &src, int lane, unsigned &quads) {
+    unsigned d = 0x7FFFFFFFu, q = 0;
+    int z = 0x7FFFFFFF, c = 0;
+    auto offer = [&](const float4 &v, int at) {
+        if (v.z == 0.0f) return;
+        const unsigned vd = __float_as_uint(v.z);  // positive: ordered as integers
+        const int vz = __float_as_int(v.w);
+        if (vd < d || (vd == d && vz < z)) {
+            d = vd;
+            z = vz;
+            c = at;
+        }
+        q |= dt_quadrant((int)v.x, (int)v.y);
     };
-    int4 cur = first;
-    bool closed = false;
-    int step = 0;
-    for (; step < kDtMaxStar; ++step) {  // counter-clockwise
-        const int4 best = next(cur, +1);
-        if (!best.w) break;  // hull edge
-        emit(cur, best);
-        if (best.z == first.z) {
+    offer(src.c0, lane);
+    offer(src.c1, lane + 32);
+    if (src.k > 64) {
+        offer(src.far_cand(lane + 64), lane + 64);
+        offer(src.far_cand(lane + 96), lane + 96);
+    }
+    quads = __reduce_or_sync(0xFFFFFFFFu, q);
+    const unsigned dm = __reduce_min_sync(0xFFFFFFFFu, d);
+    const int zm = __reduce_min_sync(0xFFFFFFFFu, d == dm ? z : 0x7FFFFFFF);
+    const unsigned b = __ballot_sync(0xFFFFFFFFu, d == dm && z == zm);
+    return src.list[__shfl_sync(0xFFFFFFFFu, c, __ffs(b) - 1)];
+}
+__device__ __forceinline__ DtPt dt_nearest(const DtListSrc &src, int lane, unsigned &quads) {
+    unsigned d = 0xFFFFFFFFu, q = 0;
+    int z = 0x7FFFFFFF, c = 0;
+    for (int j = lane; j < src.k; j += 32) {
+        const DtPt v = src.get(j);
+        const unsigned vd = (unsigned)(v.x * v.x + v.y * v.y);
+        if (vd < d || (vd == d && v.z < z)) {
+            d = vd;
+            z = v.z;
+            c = j;
+        }
+        q |= dt_quadrant(v.x, v.y);
+    }
+    quads = __reduce_or_sync(0xFFFFFFFFu, q);
+    const unsigned dm = __reduce_min_sync(0xFFFFFFFFu, d);
+    const int zm = __reduce_min_sync(0xFFFFFFFFu, d == dm ? z : 0x7FFFFFFF);
+    const unsigned b = __ballot_sync(0xFFFFFFFFu, d == dm && z == zm);
+    return src.get(__shfl_sync(0xFFFFFFFFu, c, __ffs(b) - 1));
+}
+
+// Where triangle t of a fan of m goes in the output: the owned triangles of a
+// star are written counter-clockwise from its nearest neighbour, which is
+// vertex r of the fan (0 when it is none of its vertices).
+__device__ __forceinline__ int dt_fan_pos(int t, int m, int r) { return t >= r ? t - r : t + m - r; }
+
+// The owned triangles of a star whose vertices sit one per lane: a[0..na]
+// counter-clockwise from the first vertex, b[0..nb] clockwise from it.
+__device__ __forceinline__ void dt_warp_write(const DtSide &S, int pz, int lane, bool fan, int va, int vb, int na,
+                                              int nb, int nnz) {
+    const int va1 = __shfl_down_sync(0xFFFFFFFFu, va, 1), vb1 = __shfl_down_sync(0xFFFFFFFFu, vb, 1);
+    const bool oa = lane < na && pz < va && pz < va1, ob = lane < nb && pz < vb && pz < vb1;
+    const unsigned ba = __ballot_sync(0xFFFFFFFFu, oa), bb = __ballot_sync(0xFFFFFFFFu, ob);
+    const int ma = __popc(ba), mb = __popc(bb), m = ma + mb;
+    int pa = __popc(ba & ((1u << lane) - 1u)), pb = ma + __popc(bb & ((1u << lane) - 1u));
+    if (fan) {
+        const unsigned ra = __ballot_sync(0xFFFFFFFFu, lane <= ma && va == nnz);
+        const unsigned rb = __ballot_sync(0xFFFFFFFFu, lane <= mb && vb == nnz);
+        const int r = ra ? mb + __ffs(ra) - 1 : (rb ? mb - (__ffs(rb) - 1) : 0);
+        pa = dt_fan_pos(mb + lane, m, r);
+        pb = dt_fan_pos(mb - 1 - lane, m, r);
+    }
+    int2 *out = S.slots + (size_t)pz * kDtSlots;
+    if (m > kDtSlots) {
+        int base = 0;
+        if (lane == 0) {
+            base = atomicAdd(S.npool, m);
+            *out = make_int2(base, 0);
+        }
+        out = S.pool + __shfl_sync(0xFFFFFFFFu, base, 0);
+    }
+    if (oa) out[pa] = make_int2(va, va1);
+    if (ob) out[pb] = make_int2(vb1, vb);
+    if (lane == 0) S.owned[pz] = m;
+}
+
+// One star by a warp over the candidates within R of p; true if it came out
+// certified (its owned triangles are then written).
+//
+// Triangles are emitted by their lowest-index vertex.  A list in raster order
+// (v never decreases) puts the two others of an owned triangle level with p
+// or below it, so the owned triangles are one run of consecutive sectors in
+// the lower half of the star, and only that fan is wrapped: from the vertex
+// that the circle growing straight down from p meets first, both ways until
+// a vertex is not below p.  That is 4 steps per star on average instead of
+// the whole star's 6.  It needs p strictly inside the hull (candidates in all
+// four open quadrants show that); other stars, and every star of an
+// unordered list, are wrapped whole from the nearest neighbour,
+// counter-clockwise and, when that meets the hull, clockwise from it again.
+//
+// A triangle is certain when its circle, which passes through p, is no wider
+// than R: no point farther than R from p is inside it.  Where a whole star
+// stays open (p on the hull), nothing may lie beyond either open edge, tested
+// against the extreme points of every image row.
+template <class Src>
+__device__ __forceinline__ bool dt_warp_star(const DtArgs &a, const DtSide &S, const int4 &p, const Src &src, int R,
+                                             bool ordered, int lane) {
+    unsigned quads;
+    auto nn = dt_nearest(src, lane, quads);
+    auto first = nn;
+    const bool fan = ordered && quads == 15u;
+    if (fan && !dt_fan_start(src, lane, first)) return false;
+    const float R2 = (float)(R * R);
+    int va = dt_z(first), vb = va, na = 0, nb = 0;
+    bool closed = false, open_l = false, open_r = false;
+    auto cur = first;
+    for (;;) {  // counter-clockwise
+        auto w = cur;
+        if (!dt_step(src, lane, cur, p.z, 1, w)) {
+            open_l = true;
+            break;
+        }
+        if (na == 30 || !dt_small_circle(dt_ix(cur), dt_iy(cur), dt_ix(w), dt_iy(w), R2)) return false;
+        ++na;
+        if (lane == na) va = dt_z(w);
+        if (fan && dt_iy(w) <= 0) break;
+        if (!fan && dt_z(w) == dt_z(first)) {
             closed = true;
             break;
         }
-        cur = best;
+        cur = w;
     }
-    if (step >= kDtMaxStar) return -1;
-    if (!closed) {  // clockwise from the first edge
-        cur = first;
-        for (step = 0; step < kDtMaxStar; ++step) {
-            const int4 best = next(cur, -1);
-            if (!best.w) break;
-            emit(best, cur);
-            cur = best;
+    if (fan && open_l) return false;
+    const auto e_l = cur;
+    cur = first;
+    while (!closed) {  // clockwise
+        auto w = cur;
+        if (!dt_step(src, lane, cur, p.z, -1, w)) {
+            open_r = true;
+            break;
         }
-        if (step >= kDtMaxStar) return -1;
+        if (nb == 30 || !dt_small_circle(dt_ix(w), dt_iy(w), dt_ix(cur), dt_iy(cur), R2)) return false;
+        ++nb;
+        if (lane == nb) vb = dt_z(w);
+        if (fan && dt_iy(w) <= 0) break;
+        cur = w;
     }
-    *written = wr;
-    return 1;
+    if (fan && open_r) return false;
+    if (open_l || open_r) {
+        const int lx = dt_ix(e_l), ly = dt_iy(e_l), rx = dt_ix(cur), ry = dt_iy(cur);
+        bool bad = false;
+        for (int y = lane; y < a.h; y += 32) {
+            const int x0 = S.rowmin[y], x1 = S.rowmax[y];
+            if (x0 > x1) continue;
+            const int dy = y - p.y, d0 = x0 - p.x, d1 = x1 - p.x;
+            bad |= lx * dy - ly * d0 > 0 || lx * dy - ly * d1 > 0;
+            bad |= rx * dy - ry * d0 < 0 || rx * dy - ry * d1 < 0;
+        }
+        if (__any_sync(0xFFFFFFFFu, bad)) return false;
+    }
+    dt_warp_write(S, p.z, lane, fan, va, vb, na, nb, dt_z(nn));
+    return true;
 }
 
-// Gathers the points within R of p into the shared cache; returns their
-// number (more than kDtCandCap2 means the cache overflowed).  The cell rows'
-// ranges are fetched at once, the candidates read as one flat index space,
-// and each warp places its hits with one atomic.
-__device__ int dt_block_gather(const DtArgs &a, const DtSide &S, const int4 &p, int R, int4 *cand,
-                               DtBlockShared &sh) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
-    const int cx0 = max(0, p.x - R) / kDtCell, cx1 = min(a.gw - 1, max(0, p.x + R) / kDtCell);
+// Calls visit(q, inside) for the points of the grid cells that the square of
+// half-size R around p meets, 32 at a time: the cell rows' ranges, up to
+// 2^LOG2 of them, are walked as one index space (a binary search over the
+// lanes' prefix sums), two loads in flight.
+template <int LOG2, class Visit>
+__device__ __forceinline__ void dt_warp_window(const DtArgs &a, const DtSide &S, const int4 &p, int R, int lane,
+                                               Visit visit) {
+    const int cx0 = min(a.gw - 1, max(0, p.x - R) / kDtCell), cx1 = min(a.gw - 1, max(0, p.x + R) / kDtCell);
     const int cy0 = max(0, p.y - R) / kDtCell, cy1 = min(a.gh - 1, max(0, p.y + R) / kDtCell);
-    const int nrows = min(kDtMaxRows, cy1 - cy0 + 1);
+    int rs = 0, len = 0;
+    if (lane <= cy1 - cy0) {
+        const int *row = S.cell_start + (cy0 + lane) * a.gw;
+        rs = row[cx0];
+        len = row[cx1 + 1] - rs;
+    }
+    int incl = len;
+#pragma unroll
+    for (int o = 1; o < (1 << LOG2); o <<= 1) {
+        const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    const int total = __shfl_sync(0xFFFFFFFFu, incl, (1 << LOG2) - 1);
+    const int excl = incl - len, off = rs - excl;
+    for (int t0 = 0; t0 < total; t0 += 64) {
+        int4 q[2];
+        bool in[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int t = t0 + 32 * u + lane;
+            int lo = 0;
+#pragma unroll
+            for (int s = 1 << (LOG2 - 1); s > 0; s >>= 1)
+                if (t >= __shfl_sync(0xFFFFFFFFu, excl, lo + s)) lo += s;
+            in[u] = t < total;
+            const int at = t + __shfl_sync(0xFFFFFFFFu, off, lo);
+            q[u] = in[u] ? S.pts[at] : make_int4(0, 0, 0, 0);
+        }
+        visit(q[0], in[0]);
+        if (t0 + 32 < total) visit(q[1], in[1]);
+    }
+}
+
+// Warp pass: one warp per point, the candidates within 24 pixels (12 or 6
+// where the list is full).  Bound by instruction issue: about 400 warp
+// instructions per star.
+__device__ __forceinline__ void dt_pass1_body(const DtArgs &a, const VB &vb) {
+    __shared__ float4 s_list[kDtWarps][kDtListCap];
+    const DtSide &S = a.s[vb.y];
+    const int n = min(max(*a.count, 0), a.cap);
+    const int lane = threadIdx.x & 31;
+    float4 *list = s_list[threadIdx.x >> 5];
+    const bool ordered = !(*S.err & 8);
+    for (int j = vb.x * kDtWarps + (threadIdx.x >> 5); j < n; j += vb.gx * kDtWarps) {
+        const int4 p = S.pts[j];
+        if (!p.w) continue;
+        int k = 0;
+        auto gather = [&](int R) {
+            k = 0;
+            dt_warp_window<2>(a, S, p, R, lane, [&](const int4 &q, bool inside) {
+                const int dx = q.x - p.x, dy = q.y - p.y, d2 = dx * dx + dy * dy;
+                const bool take = inside && q.w && q.z != p.z && d2 <= R * R;
+                const unsigned b = __ballot_sync(0xFFFFFFFFu, take);
+                const int pos = k + __popc(b & ((1u << lane) - 1u));
+                if (take && pos < kDtListCap)
+                    list[pos] = make_float4((float)dx, (float)dy, (float)d2, __int_as_float(q.z));
+                k += __popc(b);
+            });
+        };
+        int R = kDtRadius;
+        gather(R);
+        while (k > kDtListCap && R > 6) {
+            R >>= 1;
+            __syncwarp();
+            gather(R);
+        }
+        __syncwarp();
+        bool done = false;
+        if (k > 0 && k <= kDtListCap) {
+            DtNearSrc src{list, k};
+            src.load(lane);
+            done = dt_warp_star(a, S, p, src, R, ordered, lane);
+        }
+        if (!done && lane == 0) S.pending[atomicAdd(S.npending, 1)] = p.z;
+        __syncwarp();
+    }
+}
+
+__global__ void __launch_bounds__(kDtWarps * 32, 5) dt_pass1_kernel(DtArgs a) { dt_pass1_body(a, vb_single()); }
+__global__ void __launch_bounds__(kDtWarps * 32, 5) dt_pass1_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
+    const VB vb = vb_batch(vm);
+    dt_pass1_body(slot_entry(tab, vm.stride, vb.slot), vb);
+}
+
+// Middle pass (batches): the stars left by the warp pass, again a warp each,
+// with the candidates within 64 pixels.
+__device__ __forceinline__ void dt_pass1m_body(const DtArgs &a, const VB &vb) {
+    __shared__ int2 s_list[kDtWarpsM][kDtListCapM];
+    const DtSide &S = a.s[vb.y];
+    const int lane = threadIdx.x & 31;
+    int2 *list = s_list[threadIdx.x >> 5];
+    const bool ordered = !(*S.err & 8);
+    const int njobs = *S.npending;
+    for (int j = vb.x * kDtWarpsM + (threadIdx.x >> 5); j < njobs; j += vb.gx * kDtWarpsM) {
+        const int4 p = S.pts[S.slot[S.pending[j]]];
+        int k = 0;
+        dt_warp_window<4>(a, S, p, kDtRadiusM, lane, [&](const int4 &q, bool inside) {
+            const int dx = q.x - p.x, dy = q.y - p.y;
+            const bool take = inside && q.w && q.z != p.z && dx * dx + dy * dy <= kDtRadiusM * kDtRadiusM;
+            const unsigned b = __ballot_sync(0xFFFFFFFFu, take);
+            const int pos = k + __popc(b & ((1u << lane) - 1u));
+            if (take && pos < kDtListCapM) list[pos] = dt_pack(dx, dy, q.z);
+            k += __popc(b);
+        });
+        __syncwarp();
+        bool done = false;
+        if (k > 0 && k <= kDtListCapM) {
+            const DtListSrc src{list, k};
+            done = dt_warp_star(a, S, p, src, kDtRadiusM, ordered, lane);
+        }
+        if (!done && lane == 0) S.pending2[atomicAdd(S.npending2, 1)] = p.z;
+        __syncwarp();
+    }
+}
+static_assert(2 * kDtRadius / kDtCell + 1 <= 4 && 2 * kDtRadiusM / kDtCell + 2 <= 16, "cell rows of a disc");
+
+__global__ void __launch_bounds__(kDtWarpsM * 32) dt_pass1m_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
+    const VB vb = vb_batch(vm);
+    dt_pass1m_body(slot_entry(tab, vm.stride, vb.slot), vb);
+}
+
+// -------------------------------------------------------------------------
+// CTA pass: the stars whose circles do not fit the listed discs (the hull,
+// the rims of empty areas)
+// -------------------------------------------------------------------------
+// One CTA per star.  The points within kDtRadiusC are cached in shared
+// memory and the star is wrapped over the cache (warp 0 counter-clockwise,
+// warp 1 clockwise).  Triangles whose circle is no wider than the disc are
+// certain; for all the others at once the CTA scans the grid cells that their
+// circles (and, at an open end, the half-plane beyond the edge) meet, adds
+// every point found inside to the cache, and the star is wrapped again.  The
+// star is done when a scan finds no point: each of its triangles then has an
+// empty circle.  Most stars take one scan, the widest three; a step-by-step
+// search would scan once per triangle (up to 50).  A large region is first
+// scanned with a stride, which finds points that shrink the circles to a
+// small part of it.  A full cache keeps only the star's own vertices and
+// goes on with the whole star (its region can only shrink, so that ends).
+constexpr int kDtRadiusC = 96;
+constexpr int kDtCacheCap = 2048;   // cached points (16 KB)
+constexpr int kDtBlockThreads = 128;
+constexpr int kDtBlocksPerSM = 8;
+constexpr int kDtVertCap = 256;     // star vertices per direction
+constexpr int kDtBadCap = 32;       // circles scanned for at a time (a warp's triangles)
+constexpr int kDtMaxRounds = 64;
+constexpr int kDtSampleMin = 2048;  // regions of more points are sampled first
+
+// Triangle (p, a, b), counter-clockwise, coordinates relative to p: q lies
+// inside its circle iff |q|^2 W - U q.x - V q.y < 0 (below 2^60).
+struct DtCircle {
+    DtPt a, b;
+    int W;
+    int64_t U, V;
+};
+
+__device__ __forceinline__ DtCircle dt_circle(const DtPt &a, const DtPt &b) {
+    DtCircle c;
+    c.a = a;
+    c.b = b;
+    const int64_t a2 = a.x * a.x + a.y * a.y, b2 = b.x * b.x + b.y * b.y;
+    c.W = a.x * b.y - a.y * b.x;
+    c.U = b.y * a2 - a.y * b2;
+    c.V = a.x * b2 - b.x * a2;
+    return c;
+}
+
+// Does q invalidate the triangle: inside its circle or, on it, favoured by
+// the symbolic order?  On the circle the triangle stays iff the lowest index
+// of the four is q's or that of the vertex opposite to it (the diagonal then
+// joins the two others).
+__device__ __forceinline__ bool dt_violates(const DtCircle &c, int pz, const DtPt &q) {
+    const int64_t q2 = q.x * q.x + q.y * q.y;
+    const int64_t s = q2 * c.W - c.U * q.x - c.V * q.y;
+    if (s != 0) return s < 0;
+    if (q.z == pz || q.z == c.a.z || q.z == c.b.z) return false;
+    const int64_t oa = (int64_t)c.a.x * q.y - (int64_t)c.a.y * q.x, ob = (int64_t)c.b.x * q.y - (int64_t)c.b.y * q.x;
+    const int opp = oa < 0 ? c.b.z : (ob > 0 ? c.a.z : pz);
+    const int m1 = oa < 0 || ob > 0 ? pz : c.a.z, m2 = oa < 0 ? c.a.z : c.b.z;
+    return min(m1, m2) < min(opp, q.z);
+}
+
+struct DtStarShared {
+    DtCircle bad[kDtBadCap];
+    int2 vert[2][kDtVertCap];  // the star: counter-clockwise, clockwise from the first vertex
+    int nv[2];                 // triangles in each direction
+    int open[2];
+    int over;                  // more vertices than the lists hold
+    int closed;
+    unsigned long long nn;     // |c|^2 and index of the nearest point
+    unsigned quads;
+    int k, nbad, next, found, total;
+    int rs[16], rlen[16];
+    DtPt win[4];
+    int won[4];
+};
+
+// Cell range of image rows [cy*16, cy*16+15] that a region meets, widened so
+// that FP32 rounding cannot lose a cell (two pixels in y, one cell and more
+// in x).  A disc (rad >= 0) or the half-plane nx*x + ny*y >= 0 about (x0, y0).
+__device__ __forceinline__ bool dt_row_range(int cy, float x0, float y0, float rad, float nx, float ny, int gw,
+                                             int &c0, int &c1) {
+    const float ya = (float)(cy * kDtCell - 2) - y0, yb = (float)(cy * kDtCell + kDtCell + 1) - y0;
+    float xlo = -1e9f, xhi = 1e9f;
+    if (rad >= 0.0f) {
+        const float dy = ya > 0.0f ? ya : (yb < 0.0f ? -yb : 0.0f);
+        if (dy > rad) return false;
+        const float hc = sqrtf(rad * rad - dy * dy) + 2.0f;
+        xlo = x0 - hc;
+        xhi = x0 + hc;
+    } else {
+        // x >= or <= the boundary of the band's more permissive edge, 4 pixels wider
+        const float m = fmaxf(ny * ya, ny * yb) + 4.0f;
+        if (fabsf(nx) < 1e-4f) {
+            if (m < -4.0f) return false;
+        } else if (nx > 0.0f) {
+            xlo = x0 - m / nx - 4.0f;
+        } else {
+            xhi = x0 - m / nx + 4.0f;
+        }
+    }
+    c0 = (int)fmaxf(0.0f, fminf((float)(gw - 1), floorf(xlo / kDtCell) - 1.0f));
+    c1 = (int)fmaxf(0.0f, fminf((float)(gw - 1), floorf(xhi / kDtCell) + 1.0f));
+    return true;
+}
+
+// Gathers the points within R of p into the cache (their number, even past
+// the capacity, in sh.k), with the nearest one and the quadrants.
+__device__ __forceinline__ void dt_block_gather(const DtArgs &a, const DtSide &S, const int4 &p, int R, int2 *cand,
+                                                DtStarShared &sh) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int cx0 = min(a.gw - 1, max(0, p.x - R) / kDtCell), cx1 = min(a.gw - 1, max(0, p.x + R) / kDtCell);
+    const int cy0 = max(0, p.y - R) / kDtCell, cy1 = min(a.gh - 1, max(0, p.y + R) / kDtCell);
+    const int nrows = cy1 - cy0 + 1;
     __syncthreads();
     if (tid < nrows) {
-        const int r0 = S.cell_start[(cy0 + tid) * a.gw + cx0], r1 = S.cell_start[(cy0 + tid) * a.gw + cx1 + 1];
+        const int *row = S.cell_start + (cy0 + tid) * a.gw;
+        const int r0 = row[cx0], r1 = row[cx1 + 1];
         sh.rs[tid] = r0;
         sh.rlen[tid] = r1 - r0;
     }
-    if (tid == 0) sh.cnt = 0;
+    if (tid == 0) {
+        sh.k = 0;
+        sh.nn = ~0ull;
+        sh.quads = 0;
+    }
     __syncthreads();
-    // each warp takes cell rows in turn; its lanes stride over the row's
-    // contiguous range and the warp places its hits with one atomic
-    const int64_t R2 = (int64_t)R * R;
-    for (int r = warp; r < nrows; r += nwarps) {
+    unsigned long long nn = ~0ull;
+    unsigned quads = 0;
+    for (int r = warp; r < nrows; r += kDtBlockThreads / 32) {
         const int s0 = sh.rs[r], len = sh.rlen[r];
-        for (int j0 = 0; j0 < len; j0 += 32) {
-            const int j = j0 + lane;
-            bool take = false;
-            int4 q = make_int4(0, 0, 0, 0);
-            if (j < len) {
-                q = S.pts[s0 + j];
-                const int64_t dx = q.x - p.x, dy = q.y - p.y;
-                take = q.w && q.z != p.z && dx * dx + dy * dy <= R2;
+        for (int j0 = 0; j0 < len; j0 += 64) {
+            int4 q[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int j = j0 + 32 * u + lane;
+                q[u] = j < len ? S.pts[s0 + j] : make_int4(0, 0, 0, 0);
             }
-            const unsigned m = __ballot_sync(0xFFFFFFFFu, take);
-            int base = 0;
-            if (lane == 0 && m) base = atomicAdd(&sh.cnt, __popc(m));
-            base = __shfl_sync(0xFFFFFFFFu, base, 0);
-            const int pos = base + __popc(m & ((1u << lane) - 1u));
-            if (take && pos < kDtCandCap2) cand[pos] = q;
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int dx = q[u].x - p.x, dy = q[u].y - p.y, d2 = dx * dx + dy * dy;
+                const bool take = q[u].w && q[u].z != p.z && abs(dx) <= R && abs(dy) <= R && d2 <= R * R;
+                const unsigned m = __ballot_sync(0xFFFFFFFFu, take);
+                int base = 0;
+                if (lane == 0 && m) base = atomicAdd(&sh.k, __popc(m));
+                const int pos = __shfl_sync(0xFFFFFFFFu, base, 0) + __popc(m & ((1u << lane) - 1u));
+                if (take) {
+                    if (pos < kDtCacheCap) cand[pos] = dt_pack(dx, dy, q[u].z);
+                    nn = min(nn, ((unsigned long long)d2 << 32) | (unsigned)q[u].z);
+                    quads |= dt_quadrant(dx, dy);
+                }
+            }
+        }
+    }
+    if (nn != ~0ull) {
+        atomicMin(&sh.nn, nn);
+        atomicOr(&sh.quads, quads);
+    }
+    __syncthreads();
+}
+static_assert(2 * kDtRadiusC / kDtCell + 2 <= 16, "cell rows of the cached disc");
+
+// Wraps the star over the cache: warp 0 counter-clockwise, warp 1 clockwise.
+__device__ __forceinline__ void dt_block_wrap(const int2 *cand, int k, int pz, bool fan, const DtPt &nn,
+                                              DtStarShared &sh) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __syncthreads();
+    if (warp < 2) {
+        const DtListSrc src{cand, k};
+        const int side = warp ? -1 : 1;
+        DtPt first = nn;
+        bool ok = !fan || dt_fan_start(src, lane, first);
+        DtPt cur = first;
+        int nv = 0;
+        bool open = false, closed = false;
+        if (lane == 0) sh.vert[warp][0] = dt_pack(first.x, first.y, first.z);
+        while (ok) {
+            DtPt w;
+            if (!dt_step(src, lane, cur, pz, side, w)) {
+                open = true;
+                break;
+            }
+            if (nv == kDtVertCap - 1) {
+                ok = false;
+                break;
+            }
+            ++nv;
+            if (lane == 0) sh.vert[warp][nv] = dt_pack(w.x, w.y, w.z);
+            if (fan && w.y <= 0) break;
+            if (!fan && w.z == first.z) {
+                closed = true;
+                break;
+            }
+            cur = w;
+        }
+        if (lane == 0) {
+            sh.nv[warp] = nv;
+            sh.open[warp] = open;
+            if (!ok || (fan && open)) sh.over = 1;
+            if (closed) sh.closed = 1;  // both warps meet the first vertex again
         }
     }
     __syncthreads();
-    return sh.cnt;
+    if (threadIdx.x == 0 && sh.closed) sh.nv[1] = 0;
+    __syncthreads();
 }
 
-// One queued star rebuilt by the whole CTA (exact): cached steps among the
-// points within kDtRadius1 (then kDtRadius2), region scans otherwise.
-__device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, int i, int n, int4 *s_cand,
-                                              DtBlockShared &sh, int *r_start, int *r_len) {
-    const int4 p = S.pts[S.slot[i]];
-    const int k = dt_block_gather(a, S, p, kDtRadius1, s_cand, sh);
-    int written = 0;
-    const int r = dt_block_star(a, S, i, p, n, s_cand, kDtRadius1, k, &written, nullptr, sh, r_start, r_len);
-    if (threadIdx.x == 0) {
-        if (r == 1) {
-            S.status[i] = 2;
-            S.owned[i] = written;
-            if (written > kDtSlots) atomicOr(S.err, 4);
-        } else {
-            atomicOr(S.err, 1);
+// Triangle t of the star in sh (counter-clockwise run first), as (a, b).
+__device__ __forceinline__ void dt_star_tri(const DtStarShared &sh, int t, DtPt &a, DtPt &b) {
+    const int na = sh.nv[0];
+    const DtListSrc src{sh.vert[t < na ? 0 : 1] + (t < na ? t : t - na), 2};
+    a = src.get(t < na ? 0 : 1);
+    b = src.get(t < na ? 1 : 0);
+}
+
+// Writes the owned triangles of the star in sh (warp 0).
+__device__ __forceinline__ void dt_block_write(const DtSide &S, int pz, bool fan, int nnz, const DtStarShared &sh) {
+    const int lane = threadIdx.x & 31;
+    const int na = sh.nv[0], nt = na + sh.nv[1];
+    int ma = 0, mb = 0, r = -1;
+    for (int t0 = 0; t0 < nt; t0 += 32) {
+        DtPt u{0, 0, 0}, v{0, 0, 0};
+        if (t0 + lane < nt) dt_star_tri(sh, t0 + lane, u, v);
+        const bool own = t0 + lane < nt && pz < u.z && pz < v.z;
+        ma += __popc(__ballot_sync(0xFFFFFFFFu, own && t0 + lane < na));
+        mb += __popc(__ballot_sync(0xFFFFFFFFu, own && t0 + lane >= na));
+    }
+    const int m = ma + mb;
+    if (fan) {
+        for (int i = lane; i <= ma; i += 32)
+            if (sh.vert[0][i].y == nnz) r = mb + i;
+        for (int i = lane; i <= mb; i += 32)
+            if (sh.vert[1][i].y == nnz) r = mb - i;
+        r = max(0, __reduce_max_sync(0xFFFFFFFFu, r));
+    }
+    int2 *out = S.slots + (size_t)pz * kDtSlots;
+    if (m > kDtSlots) {
+        int base = 0;
+        if (lane == 0) {
+            base = atomicAdd(S.npool, m);
+            *out = make_int2(base, 0);
+        }
+        out = S.pool + __shfl_sync(0xFFFFFFFFu, base, 0);
+    }
+    int done = 0;
+    for (int t0 = 0; t0 < nt; t0 += 32) {
+        const int t = t0 + lane;
+        DtPt u{0, 0, 0}, v{0, 0, 0};
+        if (t < nt) dt_star_tri(sh, t, u, v);
+        const bool own = t < nt && pz < u.z && pz < v.z;
+        const unsigned b = __ballot_sync(0xFFFFFFFFu, own);
+        int pos = done + __popc(b & ((1u << lane) - 1u));
+        if (fan) pos = dt_fan_pos(t < na ? mb + t : mb - 1 - (t - na), m, r);
+        if (own) out[pos] = make_int2(u.z, v.z);
+        done += __popc(b);
+    }
+    if (lane == 0) S.owned[pz] = m;
+}
+
+// The whole star of p over every point, one exact step after the other (more
+// vertices than the lists hold, e.g. the apex of a huge fan): counted first,
+// then written.
+__device__ void dt_block_star_all(const DtSide &S, const int4 &p, int n, const DtPt &nn, DtStarShared &sh) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int2 *out = nullptr;
+    int m = 0;
+    for (int pass = 0; pass < 2; ++pass) {
+        int written = 0;
+        bool closed = false;
+        for (int side = 1; side >= -1 && !closed; side -= 2) {
+            DtPt cur = nn;
+            for (int step = 0; step <= n; ++step) {
+                const DtAllSrc src{S.pts, (n - warp + 3) / 4, warp, p.x, p.y, p.z};
+                DtPt w{0, 0, 0};
+                const bool any = dt_step(src, lane, cur, p.z, side, w);
+                __syncthreads();
+                if (lane == 0) {
+                    sh.win[warp] = w;
+                    sh.won[warp] = any;
+                }
+                __syncthreads();
+                bool got = false;
+                for (int i = 0; i < 4; ++i)
+                    if (sh.won[i] && (!got || dt_beats(cur, p.z, w, sh.win[i], side))) {
+                        w = sh.win[i];
+                        got = true;
+                    }
+                if (!got) break;
+                if (p.z < cur.z && p.z < w.z) {
+                    if (out && threadIdx.x == 0) out[written] = side > 0 ? make_int2(cur.z, w.z) : make_int2(w.z, cur.z);
+                    ++written;
+                }
+                if (w.z == nn.z) {
+                    closed = true;
+                    break;
+                }
+                cur = w;
+            }
+        }
+        if (pass == 0) {
+            m = written;
+            out = S.slots + (size_t)p.z * kDtSlots;
+            if (m > kDtSlots) {
+                if (threadIdx.x == 0) {
+                    sh.total = atomicAdd(S.npool, m);
+                    *out = make_int2(sh.total, 0);
+                }
+                __syncthreads();
+                out = S.pool + sh.total;
+            }
         }
     }
+    if (threadIdx.x == 0) S.owned[p.z] = m;
+    __syncthreads();
+}
+
+__device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, int i, int n, bool ordered,
+                                              int2 *cand, int *r_start, int *r_len, DtStarShared &sh) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int4 p = S.pts[S.slot[i]];
+    int R = kDtRadiusC;
+    dt_block_gather(a, S, p, R, cand, sh);
+    while (sh.k > kDtCacheCap && R > 1) {
+        R >>= 1;
+        dt_block_gather(a, S, p, R, cand, sh);
+    }
+    int k = sh.k;
+    if (k == 0) {  // nothing near: the nearest of all points
+        unsigned long long key = ~0ull;
+        for (int j = tid; j < n; j += kDtBlockThreads) {
+            const int4 q = S.pts[j];
+            const int64_t dx = q.x - p.x, dy = q.y - p.y;
+            if (q.w && q.z != p.z) key = min(key, ((unsigned long long)(dx * dx + dy * dy) << 32) | (unsigned)q.z);
+        }
+        if (key != ~0ull) atomicMin(&sh.nn, key);
+        __syncthreads();
+        if (sh.nn == ~0ull) {  // p is the only point
+            if (tid == 0) S.owned[p.z] = 0;
+            __syncthreads();
+            return;
+        }
+    }
+    const int4 nq = S.pts[S.slot[(int)(unsigned)(sh.nn & 0xFFFFFFFFu)]];
+    const DtPt nn{nq.x - p.x, nq.y - p.y, nq.z};
+    bool fan = ordered && sh.quads == 15u;
+    if (k == 0) {
+        if (tid == 0) cand[0] = dt_pack(nn.x, nn.y, nn.z);
+        k = 1;
+    }
+    for (int round = 0;; ++round) {
+        if (tid == 0) {
+            sh.over = 0;
+            sh.closed = 0;
+            sh.found = 0;
+        }
+        dt_block_wrap(cand, k, p.z, fan, nn, sh);
+        if (sh.over || round == kDtMaxRounds) {
+            dt_block_star_all(S, p, n, nn, sh);
+            return;
+        }
+        const int nt = sh.nv[0] + sh.nv[1];
+        const bool open_l = sh.open[0], open_r = !sh.closed && sh.open[1];
+        const float R2 = (float)(R * R);
+        bool first = true;  // the open ends go with the first group of circles
+        int found = 0;
+        for (int t0 = 0; t0 < nt || first;) {
+            // the next circles that the disc does not certify
+            __syncthreads();
+            if (warp == 0) {
+                int nb = 0;
+                for (; t0 < nt && nb == 0; t0 += 32) {
+                    DtPt u{0, 0, 0}, v{0, 0, 0};
+                    if (t0 + lane < nt) dt_star_tri(sh, t0 + lane, u, v);
+                    const bool bad = t0 + lane < nt && !dt_small_circle(u.x, u.y, v.x, v.y, R2);
+                    const unsigned b = __ballot_sync(0xFFFFFFFFu, bad);
+                    if (bad) sh.bad[__popc(b & ((1u << lane) - 1u))] = dt_circle(u, v);
+                    nb = __popc(b);
+                }
+                if (lane == 0) {
+                    sh.nbad = nb;
+                    sh.next = t0;
+                    sh.total = 0;
+                }
+            }
+            const bool ends = first && (open_l || open_r);
+            first = false;
+            __syncthreads();
+            const int nbad = sh.nbad;
+            t0 = sh.next;
+            if (nbad == 0 && !ends) continue;
+            const DtListSrc v0{sh.vert[0], 0}, v1{sh.vert[1], 0};
+            const DtPt el = v0.get(sh.nv[0]), er = v1.get(sh.nv[1]);
+            int tot = 0;
+            for (int cy = tid; cy < a.gh; cy += kDtBlockThreads) {
+                int lo = a.gw, hi = -1, c0, c1;
+                for (int b = 0; b < nbad; ++b) {
+                    const DtCircle &c = sh.bad[b];
+                    const float U = (float)c.U, V = (float)c.V, W2 = 2.0f * (float)c.W;
+                    const float ux = U / W2, uy = V / W2, r = sqrtf(ux * ux + uy * uy);
+                    bool any;
+                    if (r <= 1e6f) {
+                        any = dt_row_range(cy, (float)p.x + ux, (float)p.y + uy, r * 1.0001f + 4.0f, 0.0f, 0.0f, a.gw,
+                                           c0, c1);
+                    } else {  // the half-plane beyond the circle's tangent at p holds the disc
+                        const float l = rsqrtf(U * U + V * V);
+                        any = dt_row_range(cy, (float)p.x, (float)p.y, -1.0f, U * l, V * l, a.gw, c0, c1);
+                    }
+                    if (any) {
+                        lo = min(lo, c0);
+                        hi = max(hi, c1);
+                    }
+                }
+                if (ends) {
+                    for (int s = 0; s < 2; ++s) {
+                        if (!(s ? open_r : open_l)) continue;
+                        const float ex = (float)(s ? -er.x : el.x), ey = (float)(s ? -er.y : el.y);
+                        const float l = rsqrtf(ex * ex + ey * ey);
+                        if (dt_row_range(cy, (float)p.x, (float)p.y, -1.0f, -ey * l, ex * l, a.gw, c0, c1)) {
+                            lo = min(lo, c0);
+                            hi = max(hi, c1);
+                        }
+                    }
+                }
+                const int *row = S.cell_start + cy * a.gw;
+                const int s0 = lo <= hi ? row[lo] : 0, e0 = lo <= hi ? row[hi + 1] : 0;
+                r_start[cy] = s0;
+                r_len[cy] = e0 - s0;
+                tot += e0 - s0;
+            }
+            tot = __reduce_add_sync(0xFFFFFFFFu, tot);
+            if (lane == 0 && tot) atomicAdd(&sh.total, tot);
+            __syncthreads();
+            int stride = sh.total > kDtSampleMin && round < 4 ? sh.total / (kDtSampleMin / 4) : 1;
+            for (;;) {
+                for (int cy = warp; cy < a.gh; cy += kDtBlockThreads / 32) {
+                    const int s0 = r_start[cy], len = r_len[cy];
+                    for (int j0 = stride > 1 ? (cy * 5) % stride : 0; j0 < len; j0 += 32 * stride) {
+                        const int j = j0 + lane * stride;
+                        bool hit = false;
+                        DtPt q{0, 0, 0};
+                        if (j < len) {
+                            const int4 t = S.pts[s0 + j];
+                            if (t.w && t.z != p.z) {
+                                q = DtPt{t.x - p.x, t.y - p.y, t.z};
+                                for (int b = 0; b < nbad && !hit; ++b) hit = dt_violates(sh.bad[b], p.z, q);
+                                if (ends) {
+                                    hit = hit || (open_l && el.x * q.y - el.y * q.x > 0);
+                                    hit = hit || (open_r && er.x * q.y - er.y * q.x < 0);
+                                }
+                            }
+                        }
+                        const unsigned m = __ballot_sync(0xFFFFFFFFu, hit);
+                        if (!m) continue;
+                        int base = 0;
+                        if (lane == 0) base = atomicAdd(&sh.found, __popc(m));
+                        const int pos = k + __shfl_sync(0xFFFFFFFFu, base, 0) + __popc(m & ((1u << lane) - 1u));
+                        if (hit && pos < kDtCacheCap) cand[pos] = dt_pack(q.x, q.y, q.z);
+                    }
+                }
+                __syncthreads();
+                found = sh.found;
+                __syncthreads();
+                if (stride == 1 || found > 0) break;
+                stride = 1;
+            }
+            if (found) break;  // wrap again before the other circles
+        }
+        if (found == 0) break;
+        if (k + found <= kDtCacheCap) {
+            k += found;
+            continue;
+        }
+        // full: wrap the whole star over the cache and keep only its vertices
+        // (no disc certifies its circles any more)
+        fan = false;
+        R = 0;
+        if (tid == 0) {
+            sh.over = 0;
+            sh.closed = 0;
+        }
+        dt_block_wrap(cand, kDtCacheCap, p.z, false, nn, sh);
+        if (sh.over) {
+            dt_block_star_all(S, p, n, nn, sh);
+            return;
+        }
+        const int na = sh.nv[0] + (sh.closed ? 0 : 1);
+        for (int j = tid; j < na; j += kDtBlockThreads) cand[j] = sh.vert[0][j];
+        for (int j = tid; j < sh.nv[1]; j += kDtBlockThreads) cand[na + j] = sh.vert[1][j + 1];
+        k = na + sh.nv[1];
+        __syncthreads();
+    }
+    if (warp == 0) dt_block_write(S, p.z, fan, nn.z, sh);
     __syncthreads();
 }
 
@@ -1068,11 +1251,10 @@ __device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, 
 // counter is side 0's npending2, which dt_init_kernel zeroes and the one-pair
 // passes leave unused.
 __global__ void __launch_bounds__(kDtBlockThreads, kDtBlocksPerSM) dt_pass_block_kernel(DtArgs a, int nsides) {
-    extern __shared__ int4 s_cand[];  // [kDtCandCap2], then the region rows
-    __shared__ DtBlockShared sh;
+    extern __shared__ int2 s_cand[];  // [kDtCacheCap], then the region rows
+    __shared__ DtStarShared sh;
     __shared__ int s_item;
-    int *r_start = reinterpret_cast<int *>(s_cand + kDtCandCap2);
-    int *r_len = r_start + a.gh;
+    int *r_start = reinterpret_cast<int *>(s_cand + kDtCacheCap);
     const int n = min(max(*a.count, 0), a.cap);
     const int nq0 = *a.s[0].npending, nq1 = nsides > 1 ? *a.s[1].npending : 0;
     const int m = min(nq0, nq1), total = nq0 + nq1;
@@ -1086,22 +1268,21 @@ __global__ void __launch_bounds__(kDtBlockThreads, kDtBlocksPerSM) dt_pass_block
         const bool two = item < 2 * m;
         const int side = two ? (item & 1) : (nq0 > nq1 ? 0 : 1);
         const int idx = two ? (item >> 1) : item - m;
-        const DtSide S = side ? a.s[1] : a.s[0];
-        dt_block_item(a, S, S.pending[idx], n, s_cand, sh, r_start, r_len);
+        const DtSide &S = a.s[side];
+        dt_block_item(a, S, S.pending[idx], n, !(*S.err & 8), s_cand, r_start, r_start + a.gh, sh);
     }
 }
 
 // Many pairs, persistent: the queues of every (pair, side) of the launch are
 // concatenated in launch order and the CTAs take their entries one at a
 // time from one atomic counter (zeroed by dt_init_kernel_b), so the long
-// stars of one pair overlap the work of all the others.  queue_id 1: the
-// warp pass's queues; 0: the group pass's (a batch of one pair, which skips
-// the middle and warp passes).
-template <int THREADS, int PER_SM>
-__global__ void __launch_bounds__(THREADS, PER_SM)
-    dt_pass_block_kernel_b(const DtArgs *__restrict__ tab, VMap vm, int nsides, int32_t *counter, int queue_id) {
-    extern __shared__ int4 s_cand[];
-    __shared__ DtBlockShared sh;
+// stars of one pair overlap the work of all the others.  second: the middle
+// pass's queues; else the warp pass's (a batch of one pair, which skips the
+// middle pass).
+__global__ void __launch_bounds__(kDtBlockThreads, kDtBlocksPerSM)
+    dt_pass_block_kernel_b(const DtArgs *__restrict__ tab, VMap vm, int nsides, int32_t *counter, int second) {
+    extern __shared__ int2 s_cand[];
+    __shared__ DtStarShared sh;
     __shared__ int s_pre[2 * kMaxBatch + 1];
     __shared__ int s_item;
     const int tid = threadIdx.x, lane = tid & 31;
@@ -1116,7 +1297,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
             v[j] = 0;
             if (q < nq_all) {
                 const DtSide &Q = slot_entry(tab, vm.stride, vm.slot[q / nsides]).s[q % nsides];
-                v[j] = max(0, *dt_queue_len(Q, queue_id ? 3 : 1));
+                v[j] = max(0, second ? *Q.npending2 : *Q.npending);
             }
             sum += v[j];
         }
@@ -1136,7 +1317,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
     }
     __syncthreads();
     const int total = s_pre[nq_all];
-    int *r_start = reinterpret_cast<int *>(s_cand + kDtCandCap2);
+    int *r_start = reinterpret_cast<int *>(s_cand + kDtCacheCap);
     for (;;) {
         if (tid == 0) s_item = atomicAdd(counter, 1);
         __syncthreads();
@@ -1155,8 +1336,8 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
         const DtArgs &a = slot_entry(tab, vm.stride, vm.slot[lo / nsides]);
         const DtSide &S = a.s[lo % nsides];
         const int n = min(max(*a.count, 0), a.cap);
-        dt_block_item(a, S, dt_queue(S, queue_id ? 3 : 1)[item - s_pre[lo]], n, s_cand, sh, r_start,
-                      r_start + a.gh);
+        const int i = (second ? S.pending2 : S.pending)[item - s_pre[lo]];
+        dt_block_item(a, S, i, n, !(*S.err & 8), s_cand, r_start, r_start + a.gh, sh);
     }
 }
 
@@ -1209,7 +1390,7 @@ __device__ __forceinline__ void dt_tri_scan_body(const DtArgs &a, const VB &vb) 
     }
     if (tid == 0) {
         if (s_carry > a.cap_tri) atomicOr(S.err, 2);
-        *S.ntri = (*S.err & 3) ? -1 : s_carry;  // -1: the triangulation failed
+        *S.ntri = (*S.err & 2) ? -1 : s_carry;  // -1: the triangulation failed
     }
 }
 
@@ -1221,17 +1402,19 @@ __global__ void __launch_bounds__(1024) dt_tri_scan_kernel_b(const DtArgs *__res
 
 // One thread per point: copy the owned triangles to their offset.
 __device__ __forceinline__ void dt_emit_body(const DtArgs &a, const VB &vb) {
-    const DtSide S = vb.y ? a.s[1] : a.s[0];
+    const DtSide &S = a.s[vb.y];
     const int n = min(max(*a.count, 0), a.cap);
     if (*S.ntri < 0) return;
     for (int i = vb.x * blockDim.x + threadIdx.x; i < n; i += vb.gx * blockDim.x) {
-        const int m = min(S.owned[i], kDtSlots);
+        const int m = S.owned[i];
         int32_t *out = S.tri + 3 * (size_t)S.offset[i];
-        const int32_t *sl = S.slots + (size_t)i * kDtSlots * 2;
+        const int2 *sl = S.slots + (size_t)i * kDtSlots;
+        if (m > kDtSlots) sl = S.pool + sl->x;
         for (int k = 0; k < m; ++k) {
+            const int2 t = sl[k];
             out[3 * k + 0] = i;
-            out[3 * k + 1] = sl[2 * k];
-            out[3 * k + 2] = sl[2 * k + 1];
+            out[3 * k + 1] = t.x;
+            out[3 * k + 2] = t.y;
         }
     }
 }
@@ -1242,32 +1425,11 @@ __global__ void dt_emit_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
     dt_emit_body(slot_entry(tab, vm.stride, vb.slot), vb);
 }
 
-// Points that own more than kDtSlots triangles (fan apexes): one CTA each
-// rebuilds its star over every point and writes the owned triangles in order.
-__device__ __forceinline__ void dt_emit_big_body(const DtArgs &a, const VB &vb) {
-    __shared__ DtBlockShared sh;
-    const DtSide S = vb.y ? a.s[1] : a.s[0];
-    const int n = min(max(*a.count, 0), a.cap);
-    if (*S.ntri < 0 || !(*S.err & 4)) return;
-    for (int i = vb.x; i < n; i += vb.gx) {
-        if (S.owned[i] <= kDtSlots) continue;
-        const int4 p = S.pts[S.slot[i]];
-        int written = 0;
-        dt_block_star(a, S, i, p, n, nullptr, 0, 0, &written, S.tri + 3 * (size_t)S.offset[i], sh, nullptr,
-                      nullptr);
-        __syncthreads();
-    }
-}
-
-__global__ void __launch_bounds__(256) dt_emit_big_kernel(DtArgs a) { dt_emit_big_body(a, vb_single()); }
-__global__ void __launch_bounds__(256) dt_emit_big_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
-    const VB vb = vb_batch(vm);
-    dt_emit_big_body(slot_entry(tab, vm.stride, vb.slot), vb);
-}
-
 // -------------------------------------------------------------------------
 // Host side
 // -------------------------------------------------------------------------
+
+constexpr int kDtCounters = 4;  // err, npending, npending2, npool
 
 static void dt_geom(int w, int h, int &gw, int &gh) {
     gw = (w + kDtCell - 1) / kDtCell;
@@ -1280,8 +1442,8 @@ size_t dt_side_bytes(int cap, int w, int h) {
     const size_t c = (size_t)(cap > 0 ? cap : 1);
     const size_t cells = (size_t)gw * gh + 1;
     return 2 * align_up(c * 4, 256) + align_up(c * 16, 256) + align_up(c * 4, 256) + 3 * align_up(cells * 4, 256) +
-           3 * align_up(c * 4, 256) + align_up(c * kDtSlots * 8, 256) + 2 * align_up(c * 4, 256) +
-           2 * align_up((size_t)h * 4, 256) + align_up(16, 256);
+           2 * align_up(c * 4, 256) + align_up(c * kDtSlots * 8, 256) + align_up(2 * c * 8, 256) +
+           2 * align_up(c * 4, 256) + 2 * align_up((size_t)h * 4, 256) + align_up(kDtCounters * 4, 256);
 }
 
 static DtSide dt_carve(void *ws, int cap, int w, int h) {
@@ -1303,19 +1465,19 @@ static DtSide dt_carve(void *ws, int cap, int w, int h) {
     s.cell_cnt = reinterpret_cast<int32_t *>(take(cells * 4));
     s.cell_start = reinterpret_cast<int32_t *>(take(cells * 4));
     s.cell_fill = reinterpret_cast<int32_t *>(take(cells * 4));
-    s.status = reinterpret_cast<int32_t *>(take(c * 4));
     s.owned = reinterpret_cast<int32_t *>(take(c * 4));
     s.offset = reinterpret_cast<int32_t *>(take(c * 4));
-    s.slots = reinterpret_cast<int32_t *>(take(c * kDtSlots * 8));
+    s.slots = reinterpret_cast<int2 *>(take(c * kDtSlots * 8));
+    s.pool = reinterpret_cast<int2 *>(take(2 * c * 8));  // a mesh has fewer than 2n triangles
     s.pending = reinterpret_cast<int32_t *>(take(c * 4));
     s.pending2 = reinterpret_cast<int32_t *>(take(c * 4));
     s.rowmin = reinterpret_cast<int32_t *>(take((size_t)h * 4));
     s.rowmax = reinterpret_cast<int32_t *>(take((size_t)h * 4));
-    int32_t *small = reinterpret_cast<int32_t *>(take(16));
-    s.err = small;
-    s.npending = small + 1;
-    s.npending2 = small + 2;
-    s.npending3 = small + 3;
+    int32_t *counters = reinterpret_cast<int32_t *>(take(kDtCounters * 4));
+    s.err = counters;
+    s.npending = counters + 1;
+    s.npending2 = counters + 2;
+    s.npool = counters + 3;
     return s;
 }
 
@@ -1341,7 +1503,7 @@ elas_status launch_triangulate_device(const int16_t *list, const int32_t *count,
         a.s[i].ntri = ntri[i];
     }
     // counters, cell counts and row extremes of both sides: one kernel
-    const int nall = a.gw * a.gh + 1 + 2 * h + 4;
+    const int nall = a.gw * a.gh + 1 + 2 * h + kDtCounters;
     dt_init_kernel<<<dim3((nall + 255) / 256, nsides), 256, 0, st>>>(a);
     const int tb = 256;
     const int pblocks = max(1, min((cap + tb - 1) / tb, sm_count() * 8));
@@ -1349,21 +1511,16 @@ elas_status launch_triangulate_device(const int16_t *list, const int32_t *count,
     dt_cell_scan_kernel<<<dim3(1, nsides), 1024, 0, st>>>(a);
     dt_scatter_kernel<<<dim3(pblocks, nsides), tb, 0, st>>>(a);
     dt_dedup_kernel<<<dim3(pblocks, nsides), tb, 0, st>>>(a);
-    const int gblocks =
-        max(1, min((cap + kDtGroupThreads / kDtGroupOne - 1) / (kDtGroupThreads / kDtGroupOne), sm_count() * 16));
-    // one pair: the CTA pass takes the group pass's queue directly (its time
-    // is that of the longest star, which the warp pass would not shorten)
-    dt_pass1_kernel<<<dim3(gblocks, nsides), kDtGroupThreads, 0, st>>>(a);
-    const int smem2 = kDtCandCap2 * (int)sizeof(int4);
-    const int smem3 = smem2 + (2 * a.gh + 1) * (int)sizeof(int);
-    if (smem3 > 227 * 1024) return fail(ELAS_ERR_INVALID_ARG, "image too tall for the triangulation grid");
-    if (cudaFuncSetAttribute(dt_pass_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem3) != cudaSuccess)
+    // one pair: the CTA pass takes the warp pass's queue directly (its time is
+    // that of its longest star, which a middle pass would not shorten)
+    dt_pass1_kernel<<<dim3(max(1, min((cap + kDtWarps - 1) / kDtWarps, sm_count() * 16)), nsides), kDtWarps * 32, 0,
+                      st>>>(a);
+    const int smem = kDtCacheCap * (int)sizeof(int2) + 2 * a.gh * (int)sizeof(int);
+    if (cudaFuncSetAttribute(dt_pass_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
         return launch_status("dt_pass_block_kernel shared memory attribute");
-    (void)smem2;
-    dt_pass_block_kernel<<<sm_count() * kDtBlocksPerSM, kDtBlockThreads, smem3, st>>>(a, nsides);
+    dt_pass_block_kernel<<<sm_count() * kDtBlocksPerSM, kDtBlockThreads, smem, st>>>(a, nsides);
     dt_tri_scan_kernel<<<dim3(1, nsides), 1024, 0, st>>>(a);
     dt_emit_kernel<<<dim3(pblocks, nsides), tb, 0, st>>>(a);
-    dt_emit_big_kernel<<<dim3(sm_count(), nsides), 256, 0, st>>>(a);
     return launch_status("triangulation kernels");
 }
 
@@ -1372,7 +1529,7 @@ elas_status launch_triangulate_device(const int16_t *list, const int32_t *count,
 __device__ __forceinline__ void dt_init_body(const DtArgs &a, const VB &vb, int32_t *counter) {
     const DtSide &S = a.s[vb.y];
     const int ncell1 = a.gw * a.gh + 1;
-    const int nall = ncell1 + 2 * a.h + 4;
+    const int nall = ncell1 + 2 * a.h + kDtCounters;
     if (counter && blockIdx.x == 0 && threadIdx.x == 0) *counter = 0;
     for (int k = vb.x * blockDim.x + threadIdx.x; k < nall; k += vb.gx * blockDim.x) {
         if (k < ncell1)
@@ -1382,7 +1539,7 @@ __device__ __forceinline__ void dt_init_body(const DtArgs &a, const VB &vb, int3
         else if (k < ncell1 + 2 * a.h)
             S.rowmax[k - ncell1 - a.h] = (int32_t)0x80808080u;
         else
-            S.err[k - ncell1 - 2 * a.h] = 0;  // err, npending, npending2, npending3
+            S.err[k - ncell1 - 2 * a.h] = 0;
     }
 }
 
@@ -1404,62 +1561,41 @@ elas_status launch_triangulate_b(const DtArgs *tab, const DtArgs *host, const VM
                                  int32_t *counter, cudaStream_t st) {
     if (pairs.n == 0) return ELAS_OK;
     if (nsides < 1 || nsides > 2) return fail(ELAS_ERR_INVALID_ARG, "nsides %d", nsides);
-    VMap m_init, m_pts, m_scan, m_grp, m_grp2, m_big;
+    VMap m_init, m_pts, m_scan, m_grp, m_grp2;
     vmap_clear(m_init, pairs.stride);
     vmap_clear(m_pts, pairs.stride);
     vmap_clear(m_scan, pairs.stride);
     vmap_clear(m_grp, pairs.stride);
     vmap_clear(m_grp2, pairs.stride);
-    vmap_clear(m_big, pairs.stride);
     int max_gh = 1;
     for (int i = 0; i < pairs.n; ++i) {
         const int slot = pairs.slot[i];
         const DtArgs &a = slot_entry(host, pairs.stride, slot);
-        const int nall = a.gw * a.gh + 1 + 2 * a.h + 4;
+        const int nall = a.gw * a.gh + 1 + 2 * a.h + kDtCounters;
         vmap_add(m_init, slot, dim3((nall + 255) / 256, nsides));
         vmap_add(m_pts, slot, dim3(dt_point_blocks(a.cap, 256, pairs.n), nsides));
         vmap_add(m_scan, slot, dim3(1, nsides));
-        const int gthreads = kDtGroupThreads / (pairs.n == 1 ? kDtGroupOne : kDtGroup);
-        vmap_add(m_grp, slot, dim3(dt_point_blocks(a.cap, gthreads, pairs.n), nsides));
-        // the middle and warp passes get their queues of a few percent of
-        // the points (grid-stride over the queue)
-        vmap_add(m_grp2, slot, dim3(max(1, min(sm_count(), a.cap / 256)), nsides));
-        vmap_add(m_big, slot, dim3(pairs.n == 1 ? sm_count() : 64, nsides));
+        vmap_add(m_grp, slot, dim3(dt_point_blocks(a.cap, kDtWarps, pairs.n), nsides));
+        // the middle pass gets a few percent of the points (grid-stride over
+        // the queue)
+        vmap_add(m_grp2, slot, dim3(max(1, min(sm_count(), a.cap / 128)), nsides));
         max_gh = max(max_gh, a.gh);
     }
-    const int smem3 = kDtCandCap2 * (int)sizeof(int4) + (2 * max_gh + 1) * (int)sizeof(int);
-    if (smem3 > 200 * 1024) return fail(ELAS_ERR_INVALID_ARG, "image too tall for the triangulation grid");
-    if (cudaFuncSetAttribute(dt_pass_block_kernel_b<kDtBlockThreads, kDtBlocksPerSM>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem3) != cudaSuccess ||
-        cudaFuncSetAttribute(dt_pass_block_kernel_b<kDtBlockThreadsB, kDtBlocksPerSMB>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem3) != cudaSuccess)
+    const int smem = kDtCacheCap * (int)sizeof(int2) + 2 * max_gh * (int)sizeof(int);
+    if (cudaFuncSetAttribute(dt_pass_block_kernel_b, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
         return launch_status("dt_pass_block_kernel_b shared memory attribute");
     dt_init_kernel_b<<<vmap_total(m_init), 256, 0, st>>>(tab, m_init, counter);
     dt_points_kernel_b<<<vmap_total(m_pts), 256, 0, st>>>(tab, m_pts);
     dt_cell_scan_kernel_b<<<vmap_total(m_scan), 1024, 0, st>>>(tab, m_scan);
     dt_scatter_kernel_b<<<vmap_total(m_pts), 256, 0, st>>>(tab, m_pts);
     dt_dedup_kernel_b<<<vmap_total(m_pts), 256, 0, st>>>(tab, m_pts);
-    // one pair: the one-pair group pass, then the CTA pass on its queue (as
-    // in launch_triangulate_device); several: the batch group pass and the
-    // warp pass
-    const bool one = pairs.n == 1;
-    if (one) {
-        dt_pass1_kernel_b1<<<vmap_total(m_grp), kDtGroupThreads, 0, st>>>(tab, m_grp);
-    } else {
-        dt_pass1_kernel_b<<<vmap_total(m_grp), kDtGroupThreads, 0, st>>>(tab, m_grp);
-        dt_pass1m_kernel_b<<<vmap_total(m_grp2), kDtGroupThreads, 0, st>>>(tab, m_grp2);
-        dt_pass1b_kernel_b<<<vmap_total(m_grp2), kDtGroupThreads, 0, st>>>(tab, m_grp2);
-    }
-    const int nsm = sm_count();
-    if (one)
-        dt_pass_block_kernel_b<kDtBlockThreads, kDtBlocksPerSM>
-            <<<nsm * kDtBlocksPerSM, kDtBlockThreads, smem3, st>>>(tab, pairs, nsides, counter, 0);
-    else
-        dt_pass_block_kernel_b<kDtBlockThreadsB, kDtBlocksPerSMB>
-            <<<nsm * kDtBlocksPerSMB, kDtBlockThreadsB, smem3, st>>>(tab, pairs, nsides, counter, 1);
+    dt_pass1_kernel_b<<<vmap_total(m_grp), kDtWarps * 32, 0, st>>>(tab, m_grp);
+    const int middle = pairs.n > 1;
+    if (middle) dt_pass1m_kernel_b<<<vmap_total(m_grp2), kDtWarpsM * 32, 0, st>>>(tab, m_grp2);
+    dt_pass_block_kernel_b<<<sm_count() * kDtBlocksPerSM, kDtBlockThreads, smem, st>>>(tab, pairs, nsides, counter,
+                                                                                       middle);
     dt_tri_scan_kernel_b<<<vmap_total(m_scan), 1024, 0, st>>>(tab, m_scan);
     dt_emit_kernel_b<<<vmap_total(m_pts), 256, 0, st>>>(tab, m_pts);
-    dt_emit_big_kernel_b<<<vmap_total(m_big), 256, 0, st>>>(tab, m_big);
     return launch_status("batched triangulation kernels");
 }
 

@@ -105,19 +105,19 @@ struct DtSide {
     int32_t *cell_cnt;         // [ncell + 1]
     int32_t *cell_start;       // [ncell + 1]
     int32_t *cell_fill;        // [ncell + 1]
-    int32_t *status;           // [cap] 0 pending, k: star done in pass k, -1 duplicate
     int32_t *owned;            // [cap] triangles owned (lowest-index vertex)
     int32_t *offset;           // [cap] exclusive scan of owned
-    int32_t *slots;            // [cap][kDtSlots][2] owned triangles (the other two vertices)
-    int32_t *pending;          // [cap] points queued for the CTA pass
+    int2 *slots;               // [cap][kDtSlots] owned triangles (the other two vertices), or where they are in pool
+    int2 *pool;                // [2 * cap] the owned triangles of larger fans
+    int32_t *npool;            // pool entries taken
+    int32_t *pending;          // [cap] points queued by the warp pass
     int32_t *npending;         // queue length
-    int32_t *pending2;         // [cap] points queued again
+    int32_t *pending2;         // [cap] points queued by the middle pass (batches)
     int32_t *npending2;        // its length (one pair: side 0's is the CTA pass's work counter)
-    int32_t *npending3;        // batches: the third queue's length (its entries reuse `pending`)
     int32_t *rowmin, *rowmax;  // [h] extreme x of the points of each image row
     int32_t *tri;              // output [cap_tri][3]
     int32_t *ntri;             // output count
-    int32_t *err;              // bit 0: a star failed, bit 1: capacity, bit 2: slots overflowed
+    int32_t *err;              // bit 1: triangle capacity, bit 3: the list is not in raster order
 };
 
 struct DtArgs {

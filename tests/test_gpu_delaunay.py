@@ -104,6 +104,38 @@ def test_right_coordinates_with_many_duplicates():
     _check(pts, 210, 70)
 
 
+def _dense_block(x0, y0, nx, ny, rng, keep):
+    return [(x0 + i, y0 + j, int(rng.integers(0, 8))) for j in range(ny) for i in range(nx) if rng.random() < keep]
+
+
+@pytest.mark.parametrize("case", ["fan17", "fan255", "fan256", "fan700", "unordered", "every_pixel", "far_blocks",
+                                  "one_row_apart"])
+def test_star_list_limits(case):
+    """Where a star outgrows its lists: owned triangles past a point's slots (16), star vertices
+    past the CTA's (256 a side), candidates past the warp's (128) and the cache's (2,048), and
+    lists that are not in raster order (whole stars)."""
+    rng = np.random.default_rng(11)
+    if case.startswith("fan"):
+        n = int(case[3:])
+        # the apex sees every point of a distant row: n + 1 neighbours
+        pts = [(2, 3, 1)] + [(10 + 5 * i, 900, 1 + i % 7) for i in range(n)]
+        w, h = 5 * n + 20, 910
+    elif case == "unordered":
+        pts = [(5 * i + 5, 5 * j + 5, int(rng.integers(0, 40))) for j in range(25) for i in range(30)
+               if rng.random() < 0.4]
+        pts = [pts[i] for i in rng.permutation(len(pts))]
+        w, h = 165, 140
+    elif case == "every_pixel":
+        pts, w, h = _dense_block(4, 4, 60, 50, rng, 0.9), 70, 60
+    elif case == "far_blocks":  # every point of the other block lies beyond an open edge
+        a, b = _dense_block(4, 4, 56, 50, rng, 0.95), _dense_block(700, 500, 56, 50, rng, 0.95)
+        pts, w, h = a + b, 800, 600
+    else:  # two rows far apart: each point's circle reaches the other row
+        pts = [(5 * i + 5, y, int(rng.integers(0, 3))) for y in (5, 400) for i in range(60)]
+        w, h = 320, 410
+    _check(pts, w, h)
+
+
 @pytest.mark.parametrize("gpu", [True, False])
 def test_pipeline_both_triangulation_modes(gpu):
     from paper_1802_07210_gb300 import binding as B
