@@ -16,7 +16,7 @@
 //      that disc (2r <= R, so no farther point can matter), 93-95 % of them.
 //   2. Middle pass (batches): the others again, with 64 pixels.
 //   3. CTA pass: one CTA per star left (the hull, the rims of empty areas):
-//      the star over the points within 96 pixels, then scans of the cells
+//      the star over the points within 64 pixels, then scans of the cells
 //      that its wide circles meet until they are empty (dt_block_item).
 // The output order is deterministic: an exclusive scan of the per-point
 // counts, and within a star counter-clockwise from the nearest neighbour (an
@@ -169,9 +169,10 @@ __global__ void dt_dedup_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
 
 constexpr int kDtSlots = 16;       // owned triangles kept per point; larger fans go to the pool
 constexpr int kDtRadius = 24;      // warp pass: candidates within this many pixels
-constexpr int kDtListCap = 128;    // its list (a radius-24 disc holds about 75 points of a full step-5 lattice)
-constexpr int kDtRadiusM = 64;     // middle pass (batches)
-constexpr int kDtListCapM = 640;   // a radius-64 disc holds about 520 lattice points
+constexpr int kDtNearCap = 64;     // and at most this many, two per lane (else the nearer ones of 16 or 8 pixels)
+constexpr int kDtRadiusM = 48;     // middle pass
+constexpr int kDtListCapM = 320;   // a radius-48 disc holds about 290 points of a full step-5 lattice
+constexpr float kDtWideMax = 96.0f;  // the middle pass searches circles up to this radius
 constexpr int kDtWarps = 8;        // stars per CTA of the warp pass
 constexpr int kDtWarpsM = 4;       // stars per CTA of the middle pass
 constexpr float kDtInf = 3.402823466e38f;  // "no candidate" key (every real key is far below)
@@ -180,6 +181,13 @@ __device__ __forceinline__ float dt_warp_min(float v) {
     float r;
     asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
     return r;
+}
+
+// n / d for an integer-valued d >= 1, off by at most 2^-22.4 (relatively).
+__device__ __forceinline__ float dt_div(float n, float d) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    return n * r;
 }
 
 // The Delaunay third vertex of directed edge (p, e) on side s (+1 left, -1
@@ -203,43 +211,54 @@ __device__ __forceinline__ bool dt_tie_second(int pz, int ez, int z1, int z2, bo
     return first_is_x == ywins;
 }
 
-// Is the circle through the origin, a and b no wider than R (2r <= R)?
-// |a|^2 |b|^2 |a-b|^2 <= R^2 cross(a, b)^2, in FP32 with a margin far above
-// its rounding: a false answer only sends a star to the next pass.
-__device__ __forceinline__ bool dt_small_circle(int ax, int ay, int bx, int by, float R2) {
-    const float pa = (float)(ax * ax + ay * ay), pb = (float)(bx * bx + by * by);
-    const int dx = bx - ax, dy = by - ay;
-    const float ab = (float)dx * (float)dx + (float)dy * (float)dy, ar = (float)(ax * by - ay * bx);
-    return pa * pb * ab * 1.00001f <= R2 * ar * ar;
+// Is the circle of edge (p, e) with pencil parameter t no wider than R
+// (2r <= R)?  Its centre lies |e|/2 along the edge and t |e|/2 off it, so
+// 4 r^2 = |e|^2 (1 + t^2); with a margin far above the FP32 rounding of t (a
+// false answer only sends a star to the next pass).
+__device__ __forceinline__ bool dt_small_circle(float e2, float t, float R2) {
+    return e2 * __fmaf_rn(t, t, 1.0f) * 1.0001f <= R2;
 }
 
 struct DtPt {
     int x, y, z;  // relative to the star's point; list index
 };
 
-// Candidates of a star as packed relative coordinates and list index.
-struct DtListSrc {
-    const int2 *list;
-    int k;
-    __device__ __forceinline__ DtPt get(int c) const {
-        const int2 v = list[c];
-        return DtPt{(int)(int16_t)(v.x & 0xFFFF), v.x >> 16, v.y};
-    }
-};
-__device__ __forceinline__ int2 dt_pack(int x, int y, int z) { return make_int2((y << 16) | (x & 0xFFFF), z); }
+// Candidates are (x, y, |c|^2, index) in FP32, coordinates relative to p.
+__device__ __forceinline__ float4 dt_cand(int x, int y, int z) {
+    return make_float4((float)x, (float)y, (float)(x * x + y * y), __int_as_float(z));
+}
+__device__ __forceinline__ DtPt dt_point(const float4 &v) {
+    return DtPt{(int)v.x, (int)v.y, __float_as_int(v.w)};
+}
+__device__ __forceinline__ float4 dt_no_cand() {  // D = 0 and y = 0: never a candidate
+    return make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+}
 
-// A quarter of the grid-sorted points (the exact pass over every point).
-struct DtAllSrc {
-    const int4 *pts;
-    int k, part, px, py, pz;
-    __device__ __forceinline__ DtPt get(int c) const {
-        const int4 q = pts[4 * c + part];
-        if (!q.w || q.z == pz) return DtPt{0, 0, pz};  // D = 0: never a candidate
-        return DtPt{q.x - px, q.y - py, q.z};
-    }
-};
+// N and D of candidate c; exact in FP32 while every coordinate is below 2048
+// (all values then stay below 2^24).
+constexpr int kDtNearMax = 2048;
+__device__ __forceinline__ float dt_n(const float4 &e, const float4 &c) {
+    return __fmaf_rn(-e.x, c.x, __fmaf_rn(-e.y, c.y, c.z));
+}
+__device__ __forceinline__ float dt_d(const float4 &e, const float4 &c, float side) {
+    return side * __fmaf_rn(e.x, c.y, -(e.y * c.x));
+}
 
-// Does c2 beat c1 for edge (p, e) on `side`, exactly?
+// Does c2 beat c1 for edge (p, e) on `side`, exactly (coordinates below
+// 2048)?  The cross products N2 D1 and N1 D2 compare by their rounded values
+// (rounding is monotone) and, when those are equal, by their exact errors.
+__device__ __forceinline__ bool dt_beats(const float4 &e, int pz, const float4 &c1, const float4 &c2, float side) {
+    const float N1 = dt_n(e, c1), D1 = dt_d(e, c1, side), N2 = dt_n(e, c2), D2 = dt_d(e, c2, side);
+    const float l = N2 * D1, r = N1 * D2;
+    if (l != r) return l < r;
+    const float le = __fmaf_rn(N2, D1, -l), re = __fmaf_rn(N1, D2, -r);
+    if (le != re) return le < re;
+    const int z1 = __float_as_int(c1.w), z2 = __float_as_int(c2.w);
+    return z1 != z2 && dt_tie_second(pz, __float_as_int(e.w), z1, z2, side * (c1.x * c2.y - c1.y * c2.x) > 0.0f);
+}
+
+// The same in integers, for coordinate differences below 2^14.5 (N and D fit
+// 32 bits).
 __device__ __forceinline__ bool dt_beats(const DtPt &e, int pz, const DtPt &c1, const DtPt &c2, int side) {
     const int D1 = side * (e.x * c1.y - e.y * c1.x), D2 = side * (e.x * c2.y - e.y * c2.x);
     const int N1 = c1.x * c1.x + c1.y * c1.y - (e.x * c1.x + e.y * c1.y);
@@ -250,213 +269,225 @@ __device__ __forceinline__ bool dt_beats(const DtPt &e, int pz, const DtPt &c1, 
     return dt_tie_second(pz, e.z, c1.z, c2.z, side * ((int64_t)c1.x * c2.y - (int64_t)c1.y * c2.x) > 0);
 }
 
-// One wrap step by a warp over src's candidates, exact while every
-// coordinate difference stays below 2^14.5 (N and D fit 32 bits; their
-// rounding to FP32 and the division leave a relative error below 2^-20).
-template <class Src>
-__device__ __forceinline__ bool dt_step(const Src &src, int lane, const DtPt &e, int pz, int side, DtPt &w) {
-    float f1 = kDtInf, f2 = kDtInf;
-    int c1 = 0;
-    const int sx = side * e.x, sy = side * e.y;
-#pragma unroll 4
-    for (int c = lane; c < src.k; c += 32) {
-        const DtPt q = src.get(c);
-        const int D = sx * q.y - sy * q.x, N = q.x * q.x + q.y * q.y - (e.x * q.x + e.y * q.y);
-        const float f = D > 0 ? __fdividef((float)N, (float)D) : kDtInf;
-        f2 = fminf(f2, fmaxf(f1, f));
-        if (f < f1) {
-            f1 = f;
-            c1 = c;
-        }
+// Winner of a warp's lanes, those with `in` offering candidate own(at): the
+// band's members ordered exactly, champion against challengers.  get(at) on
+// every lane: the candidate that some lane offered.
+template <class Pt, class Get, class Own, class Beats>
+__device__ __forceinline__ int dt_champion(bool in, int at, Get get, Own own, Beats beats, Pt &w) {
+    unsigned b = __ballot_sync(0xFFFFFFFFu, in);
+    int ch = __shfl_sync(0xFFFFFFFFu, at, __ffs(b) - 1);
+    w = get(ch);
+    if (b & (b - 1)) {
+        const Pt mine = own(at);
+        do {
+            in = in && at != ch && beats(w, mine);
+            b = __ballot_sync(0xFFFFFFFFu, in);
+            if (!b) break;
+            ch = __shfl_sync(0xFFFFFFFFu, at, __ffs(b) - 1);
+            w = get(ch);
+        } while (b & (b - 1));
     }
+    return ch;
+}
+
+// One wrap step by a warp over points given as integers by get(0..k-1)
+// (coordinate differences below 2^14.5; the keys' rounding to FP32 and the
+// division leave a relative error below 2^-20).  The winner's position in at.
+template <class Get>
+__device__ __forceinline__ bool dt_step_int(Get get, int k, int lane, const DtPt &e, int pz, int side, DtPt &w,
+                                            int &at) {
+    auto key = [&](const DtPt &q) {
+        const int D = side * (e.x * q.y - e.y * q.x), N = q.x * q.x + q.y * q.y - (e.x * q.x + e.y * q.y);
+        return D > 0 ? dt_div((float)N, (float)D) : kDtInf;
+    };
+    float f1 = kDtInf;
+    for (int c = lane; c < k; c += 32) f1 = fminf(f1, key(get(c)));
     const float fm = dt_warp_min(f1);
     if (fm == kDtInf) return false;
     const float thr = fm + 0x1p-17f * fabsf(fm);
-    bool in = f1 <= thr;
-    if (in && f2 <= thr) {  // several of this lane's candidates: keep the exact best
-        int best = -1;
+    const bool in = f1 <= thr;
+    int c1 = -1;
+    if (in) {  // this lane's exact best of the band
         DtPt bq{0, 0, 0};
-        for (int c = lane; c < src.k; c += 32) {
-            const DtPt q = src.get(c);
-            const int D = sx * q.y - sy * q.x, N = q.x * q.x + q.y * q.y - (e.x * q.x + e.y * q.y);
-            if (D <= 0 || __fdividef((float)N, (float)D) > thr) continue;
-            if (best < 0 || dt_beats(e, pz, bq, q, side)) {
-                best = c;
+        for (int c = lane; c < k; c += 32) {
+            const DtPt q = get(c);
+            if (key(q) > thr) continue;
+            if (c1 < 0 || dt_beats(e, pz, bq, q, side)) {
+                c1 = c;
                 bq = q;
             }
         }
-        c1 = best;
     }
-    unsigned b = __ballot_sync(0xFFFFFFFFu, in);
-    int ch = __shfl_sync(0xFFFFFFFFu, c1, __ffs(b) - 1);
-    w = src.get(ch);
-    if (b & (b - 1)) {
-        const DtPt mine = in ? src.get(c1) : w;
-        while (b & (b - 1)) {
-            in = in && c1 != ch && dt_beats(e, pz, w, mine, side);
-            b = __ballot_sync(0xFFFFFFFFu, in);
-            if (!b) break;
-            ch = __shfl_sync(0xFFFFFFFFu, c1, __ffs(b) - 1);
-            w = src.get(ch);
-        }
-    }
+    at = dt_champion(
+        in, c1, get, [&](int c) { return get(max(0, c)); },
+        [&](const DtPt &a, const DtPt &b) { return dt_beats(e, pz, a, b, side); }, w);
     return true;
+}
+
+// A star's candidates in shared memory.  near: all below 2048, so that the
+// FP32 arithmetic is exact but for the division.
+struct DtListSrc {
+    const float4 *list;
+    int k;
+    bool near;
+    __device__ __forceinline__ DtListSrc(const float4 *l, int n, bool exact, int) : list(l), k(n), near(exact) {}
+
+    // Least key over the list (kDtInf: no candidate) and the winner, the
+    // keys' band (2^-17, far above the division's error) ordered by beats.
+    // Four candidates a lane at a time, so that their latencies overlap.
+    template <class Key, class Beats>
+    __device__ __forceinline__ float select(int lane, Key key, Beats beats, float4 &w, int &at) const {
+        float f1 = kDtInf, f2 = kDtInf;
+        int c1 = 0;
+        for (int c0 = lane; c0 - lane < k; c0 += 128) {
+            float f[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) f[u] = key(list[min(c0 + 32 * u, k - 1)]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (c0 + 32 * u >= k) f[u] = kDtInf;
+            const float fa = fminf(f[0], f[1]), fb = fminf(f[2], f[3]), g = fminf(fa, fb);
+            const float second = fminf(fmaxf(fa, fb), fa < fb ? fmaxf(f[0], f[1]) : fmaxf(f[2], f[3]));
+            f2 = fminf(f2, fminf(second, fmaxf(f1, g)));
+            if (g < f1) {
+                f1 = g;
+                c1 = c0 + (g == f[0] ? 0 : g == f[1] ? 32 : g == f[2] ? 64 : 96);
+            }
+        }
+        const float fm = dt_warp_min(f1);
+        if (fm == kDtInf) return fm;
+        const float thr = __fmaf_rn(fabsf(fm), 0x1p-17f, fm);
+        const bool in = f1 <= thr;
+        const unsigned b = __ballot_sync(0xFFFFFFFFu, in);
+        const unsigned more = __ballot_sync(0xFFFFFFFFu, f2 <= thr);
+        if (!(more | (b & (b - 1)))) {
+            at = __shfl_sync(0xFFFFFFFFu, c1, __ffs(b) - 1);
+            w = list[at];
+            return fm;
+        }
+        if (in && f2 <= thr) {  // several of this lane's candidates: its exact best
+            float4 bq = list[c1];
+            for (int c = lane; c < k; c += 32) {
+                const float4 q = list[c];
+                if (c == c1 || key(q) > thr || !beats(bq, q)) continue;
+                c1 = c;
+                bq = q;
+            }
+        }
+        at = dt_champion(
+            in, c1, [&](int c) { return list[c]; }, [&](int c) { return list[c]; }, beats, w);
+        return fm;
+    }
+};
+
+__device__ __noinline__ bool dt_step_far(const float4 *list, int k, int lane, const float4 &e, int pz, int side,
+                                         float4 &w, int &at) {
+    DtPt wi;
+    const bool any = dt_step_int([&](int c) { return dt_point(list[c]); }, k, lane, dt_point(e), pz, side, wi, at);
+    if (any) w = list[at];
+    return any;
+}
+
+// One wrap step over a list; t: the winner's pencil parameter (near lists),
+// at: its place in the list.
+__device__ __forceinline__ bool dt_step(const DtListSrc &src, int lane, const float4 &e, int pz, int side, float4 &w,
+                                        float &t, int &at) {
+    if (!src.near) {
+        t = kDtInf;
+        return dt_step_far(src.list, src.k, lane, e, pz, side, w, at);
+    }
+    const float sd = (float)side, sx = sd * e.x, sy = sd * e.y;
+    t = src.select(
+        lane,
+        [&](const float4 &c) {
+            const float D = __fmaf_rn(sx, c.y, -(sy * c.x));
+            return D > 0.0f ? dt_div(dt_n(e, c), D) : kDtInf;
+        },
+        [&](const float4 &c1, const float4 &c2) { return dt_beats(e, pz, c1, c2, sd); }, w, at);
+    return t != kDtInf;
 }
 
 // First vertex of a fan (see dt_warp_star): the candidate below p (y > 0)
 // that a circle through p growing straight down touches first, least
 // |c|^2 / y; of several on that circle the first one counter-clockwise.
-template <class Src> __device__ __forceinline__ bool dt_fan_start(const Src &src, int lane, DtPt &w) {
-    auto better = [](const DtPt &c1, const DtPt &c2) {  // c2 before c1
-        const int64_t l = (int64_t)(c2.x * c2.x + c2.y * c2.y) * c1.y, r = (int64_t)(c1.x * c1.x + c1.y * c1.y) * c2.y;
-        if (l != r) return l < r;
-        return (int64_t)c2.x * c1.y - (int64_t)c2.y * c1.x > 0;
-    };
-    float f1 = kDtInf, f2 = kDtInf;
-    int c1 = 0;
-    for (int c = lane; c < src.k; c += 32) {
-        const DtPt q = src.get(c);
-        const float f = q.y > 0 ? __fdividef((float)(q.x * q.x + q.y * q.y), (float)q.y) : kDtInf;
-        f2 = fminf(f2, fmaxf(f1, f));
-        if (f < f1) {
-            f1 = f;
-            c1 = c;
-        }
-    }
-    const float fm = dt_warp_min(f1);
-    if (fm == kDtInf) return false;
-    const float thr = fm + 0x1p-17f * fm;
-    bool in = f1 <= thr;
-    if (in && f2 <= thr) {
-        DtPt bq = src.get(c1);
-        for (int c = lane; c < src.k; c += 32) {
-            const DtPt q = src.get(c);
-            if (q.y > 0 && better(bq, q)) {
-                bq = q;
-                c1 = c;
-            }
-        }
-    }
-    unsigned b = __ballot_sync(0xFFFFFFFFu, in);
-    int ch = __shfl_sync(0xFFFFFFFFu, c1, __ffs(b) - 1);
-    w = src.get(ch);
-    if (b & (b - 1)) {
-        const DtPt mine = in ? src.get(c1) : w;
-        while (b & (b - 1)) {
-            in = in && c1 != ch && better(w, mine);
-            b = __ballot_sync(0xFFFFFFFFu, in);
-            if (!b) break;
-            ch = __shfl_sync(0xFFFFFFFFu, c1, __ffs(b) - 1);
-            w = src.get(ch);
-        }
-    }
-    return true;
+__device__ __forceinline__ bool dt_fan_start(const DtListSrc &src, int lane, float4 &w, int &at) {
+    return src.select(
+               lane, [](const float4 &c) { return c.y > 0.0f ? dt_div(c.z, c.y) : kDtInf; },
+               [](const float4 &c1, const float4 &c2) {
+                   const DtPt a = dt_point(c1), b = dt_point(c2);
+                   const int64_t l = (int64_t)(b.x * b.x + b.y * b.y) * a.y, r = (int64_t)(a.x * a.x + a.y * a.y) * b.y;
+                   if (l != r) return l < r;
+                   return (int64_t)b.x * a.y - (int64_t)b.y * a.x > 0;
+               },
+               w, at) != kDtInf;
 }
 
-// The warp pass's candidates: within 24 pixels of p, so every key is a small
-// integer and FP32 arithmetic on it is exact (N and D below 2^11, their
-// cross products below 2^24).  Each lane keeps two of them (x, y, |c|^2,
-// index) in registers; a list of more than 64 reads the rest from shared
-// memory.
+// The warp pass's candidates: at most 64 within 24 pixels of p, two per lane
+// in registers as (x, y, |c|^2, index), the list in shared memory for the
+// winners.  All their arithmetic is exact in FP32 but the keys' division:
+// |N| <= 1152 and D <= 576, so two different keys lie at least 2^-19.3 apart
+// (relatively: 1 / (|N| D)), while a computed key is off by at most 2^-22.4.  The keys within 2^-20.35 of the least one are
+// therefore exactly those equal to it: the band holds ties only.
 struct DtNearSrc {
     const float4 *list;
-    int k;
     float4 c0, c1;
 
-    __device__ __forceinline__ void load(int lane) {
-        const float4 none = make_float4(0.0f, 0.0f, 0.0f, 0.0f);  // D = 0 and y = 0: never a candidate
-        c0 = lane < k ? list[lane] : none;
-        c1 = lane + 32 < k ? list[lane + 32] : none;
+    __device__ __forceinline__ DtNearSrc(const float4 *l, int k, int lane) : list(l) {
+        c0 = lane < k ? list[lane] : dt_no_cand();
+        c1 = lane + 32 < k ? list[lane + 32] : dt_no_cand();
     }
-    __device__ __forceinline__ float4 far_cand(int c) const {
-        return c < k ? list[c] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    }
-    __device__ __forceinline__ DtPt point(const float4 &v) const {
-        return DtPt{(int)v.x, (int)v.y, __float_as_int(v.z == 0.0f ? 0.0f : v.w)};
-    }
-    // Least key over the slots, then the exact order among its band:
-    // key(c) (kDtInf: not a candidate), beats(c1, c2): c2 before c1.
-    template <class Key, class Beats>
-    __device__ __forceinline__ bool select(int lane, Key key, Beats beats, float4 &w) const {
-        const float f0 = key(c0), f1 = key(c1);
-        float f2 = kDtInf, f3 = kDtInf;
-        if (k > 64) {
-            f2 = key(far_cand(lane + 64));
-            f3 = key(far_cand(lane + 96));
-        }
-        const float fm = dt_warp_min(fminf(fminf(f0, f1), fminf(f2, f3)));
-        if (fm == kDtInf) return false;
-        const float thr = fm + 0x1p-18f * fabsf(fm);
+    // The winner of keys f0, f1 (least value fm): with ties, champion and
+    // challenger in turn, beats(c1, c2): c2 before c1.
+    template <class Beats>
+    __device__ __forceinline__ float4 pick(float f0, float f1, float fm, Beats beats) const {
+        const float thr = __fmaf_rn(fabsf(fm), 7.5e-7f, fm);
         unsigned b0 = __ballot_sync(0xFFFFFFFFu, f0 <= thr), b1 = __ballot_sync(0xFFFFFFFFu, f1 <= thr);
-        unsigned b2 = 0, b3 = 0;
-        if (k > 64) {
-            b2 = __ballot_sync(0xFFFFFFFFu, f2 <= thr);
-            b3 = __ballot_sync(0xFFFFFFFFu, f3 <= thr);
+        auto next = [&]() {
+            const float4 *l = b0 ? list : list + 32;
+            const unsigned b = b0 ? b0 : b1;
+            if (b0)
+                b0 &= b0 - 1;
+            else
+                b1 &= b1 - 1;
+            return l[__ffs(b) - 1];
+        };
+        float4 w = next();
+        while (b0 | b1) {
+            const float4 q = next();
+            if (beats(w, q)) w = q;
         }
-        for (;;) {
-            const int ch = b0   ? __ffs(b0) - 1
-                           : b1 ? __ffs(b1) + 31
-                           : b2 ? __ffs(b2) + 63
-                                : __ffs(b3) + 95;
-            w = list[ch];
-            if (__popc(b0) + __popc(b1) + __popc(b2) + __popc(b3) == 1) return true;
-            const unsigned me = 1u << lane;
-            // the champion itself never beats itself
-            const unsigned n0 = __ballot_sync(0xFFFFFFFFu, (b0 & me) && beats(w, c0));
-            const unsigned n1 = __ballot_sync(0xFFFFFFFFu, (b1 & me) && beats(w, c1));
-            unsigned n2 = 0, n3 = 0;
-            if (k > 64) {
-                n2 = __ballot_sync(0xFFFFFFFFu, (b2 & me) && beats(w, far_cand(lane + 64)));
-                n3 = __ballot_sync(0xFFFFFFFFu, (b3 & me) && beats(w, far_cand(lane + 96)));
-            }
-            if (!(n0 | n1 | n2 | n3)) return true;
-            b0 = n0;
-            b1 = n1;
-            b2 = n2;
-            b3 = n3;
-        }
+        return w;
     }
 };
 
-__device__ __forceinline__ bool dt_step(const DtNearSrc &src, int lane, const float4 &e, int pz, float side,
-                                        float4 &w) {
-    const float sx = side * e.x, sy = side * e.y;
-    auto dkey = [&](const float4 &c) { return __fmaf_rn(sx, c.y, -(sy * c.x)); };
-    auto nkey = [&](const float4 &c) { return __fmaf_rn(-e.x, c.x, __fmaf_rn(-e.y, c.y, c.z)); };
-    return src.select(
-        lane,
-        [&](const float4 &c) {
-            const float D = dkey(c);
-            return D > 0.0f ? __fdividef(nkey(c), D) : kDtInf;
-        },
-        [&](const float4 &c1, const float4 &c2) {
-            const float l = nkey(c2) * dkey(c1), r = nkey(c1) * dkey(c2);
-            if (l != r) return l < r;
-            const int z1 = __float_as_int(c1.w), z2 = __float_as_int(c2.w);
-            return z1 != z2 &&
-                   dt_tie_second(pz, __float_as_int(e.w), z1, z2, side * (c1.x * c2.y - c1.y * c2.x) > 0.0f);
-        },
-        w);
+// One wrap step; t: the winner's pencil parameter.
+__device__ __forceinline__ bool dt_step(const DtNearSrc &src, int, const float4 &e, int pz, int side, float4 &w,
+                                        float &t, int &) {
+    const float sx = side > 0 ? e.x : -e.x, sy = side > 0 ? e.y : -e.y;
+    auto key = [&](const float4 &c) {
+        const float D = __fmaf_rn(sx, c.y, -(sy * c.x));
+        const float N = __fmaf_rn(-e.x, c.x, __fmaf_rn(-e.y, c.y, c.z));
+        return D > 0.0f ? dt_div(N, D) : kDtInf;
+    };
+    const float f0 = key(src.c0), f1 = key(src.c1);
+    t = dt_warp_min(fminf(f0, f1));
+    if (t == kDtInf) return false;
+    w = src.pick(f0, f1, t, [&](const float4 &c1, const float4 &c2) {
+        const float o = c1.x * c2.y - c1.y * c2.x;
+        return dt_tie_second(pz, __float_as_int(e.w), __float_as_int(c1.w), __float_as_int(c2.w),
+                             side > 0 ? o > 0.0f : o < 0.0f);
+    });
+    return true;
 }
 
-__device__ __forceinline__ bool dt_fan_start(const DtNearSrc &src, int lane, float4 &w) {
-    return src.select(
-        lane, [&](const float4 &c) { return c.y > 0.0f ? __fdividef(c.z, c.y) : kDtInf; },
-        [&](const float4 &c1, const float4 &c2) {
-            const float l = c2.z * c1.y, r = c1.z * c2.y;
-            if (l != r) return l < r;
-            return c2.x * c1.y - c2.y * c1.x > 0.0f;
-        },
-        w);
+__device__ __forceinline__ bool dt_fan_start(const DtNearSrc &src, int, float4 &w, int &) {
+    const float f0 = src.c0.y > 0.0f ? dt_div(src.c0.z, src.c0.y) : kDtInf;
+    const float f1 = src.c1.y > 0.0f ? dt_div(src.c1.z, src.c1.y) : kDtInf;
+    const float fm = dt_warp_min(fminf(f0, f1));
+    if (fm == kDtInf) return false;
+    w = src.pick(f0, f1, fm, [](const float4 &c1, const float4 &c2) { return c2.x * c1.y - c2.y * c1.x > 0.0f; });
+    return true;
 }
-
-// Views of a candidate for the star driver.
-__device__ __forceinline__ int dt_z(const DtPt &c) { return c.z; }
-__device__ __forceinline__ int dt_z(const float4 &c) { return __float_as_int(c.w); }
-__device__ __forceinline__ int dt_ix(const DtPt &c) { return c.x; }
-__device__ __forceinline__ int dt_ix(const float4 &c) { return (int)c.x; }
-__device__ __forceinline__ int dt_iy(const DtPt &c) { return c.y; }
-__device__ __forceinline__ int dt_iy(const float4 &c) { return (int)c.y; }
 
 // Nearest candidate (least |c|^2, then least index) and the open quadrants
 // that hold candidates (bit 2*(y>0) + (x>0)).
@@ -464,49 +495,131 @@ __device__ __forceinline__ unsigned dt_quadrant(int x, int y) {
     return x && y ? 1u << ((x > 0) | ((y > 0) << 1)) : 0u;
 }
 __device__ __forceinline__ float4 dt_nearest(const DtNearSrc &src, int lane, unsigned &quads) {
-    unsigned d = 0x7FFFFFFFu, q = 0;
-    int z = 0x7FFFFFFF, c = 0;
-    auto offer = [&](const float4 &v, int at) {
-        if (v.z == 0.0f) return;
-        const unsigned vd = __float_as_uint(v.z);  // positive: ordered as integers
-        const int vz = __float_as_int(v.w);
-        if (vd < d || (vd == d && vz < z)) {
-            d = vd;
+    auto quad = [](const float4 &c) {
+        return c.x != 0.0f && c.y != 0.0f ? 1u << ((c.x > 0.0f ? 1 : 0) | (c.y > 0.0f ? 2 : 0)) : 0u;
+    };
+    quads = __reduce_or_sync(0xFFFFFFFFu, quad(src.c0) | quad(src.c1));
+    const float d0 = src.c0.z > 0.0f ? src.c0.z : kDtInf, d1 = src.c1.z > 0.0f ? src.c1.z : kDtInf;
+    const float dm = dt_warp_min(fminf(d0, d1));
+    const unsigned z = min(d0 == dm ? __float_as_uint(src.c0.w) : 0xFFFFFFFFu,
+                           d1 == dm ? __float_as_uint(src.c1.w) : 0xFFFFFFFFu);
+    const unsigned zm = __reduce_min_sync(0xFFFFFFFFu, z);
+    const unsigned b = __ballot_sync(0xFFFFFFFFu, z == zm);
+    const int at = __ffs(b) - 1;
+    const float4 w = src.list[at];
+    if (__float_as_uint(w.w) == zm) return w;
+    return src.list[at + 32];
+}
+__device__ __forceinline__ float4 dt_nearest(const DtListSrc &src, int lane, unsigned &quads) {
+    float d = kDtInf;
+    unsigned q = 0, z = 0xFFFFFFFFu;
+    int c = 0;
+    for (int j = lane; j < src.k; j += 32) {
+        const float4 v = src.list[j];
+        const unsigned vz = __float_as_uint(v.w);
+        if (v.z < d || (v.z == d && vz < z)) {
+            d = v.z;
             z = vz;
-            c = at;
+            c = j;
         }
         q |= dt_quadrant((int)v.x, (int)v.y);
-    };
-    offer(src.c0, lane);
-    offer(src.c1, lane + 32);
-    if (src.k > 64) {
-        offer(src.far_cand(lane + 64), lane + 64);
-        offer(src.far_cand(lane + 96), lane + 96);
     }
     quads = __reduce_or_sync(0xFFFFFFFFu, q);
-    const unsigned dm = __reduce_min_sync(0xFFFFFFFFu, d);
-    const int zm = __reduce_min_sync(0xFFFFFFFFu, d == dm ? z : 0x7FFFFFFF);
+    const float dm = dt_warp_min(d);
+    const unsigned zm = __reduce_min_sync(0xFFFFFFFFu, d == dm ? z : 0xFFFFFFFFu);
     const unsigned b = __ballot_sync(0xFFFFFFFFu, d == dm && z == zm);
     return src.list[__shfl_sync(0xFFFFFFFFu, c, __ffs(b) - 1)];
 }
-__device__ __forceinline__ DtPt dt_nearest(const DtListSrc &src, int lane, unsigned &quads) {
-    unsigned d = 0xFFFFFFFFu, q = 0;
-    int z = 0x7FFFFFFF, c = 0;
-    for (int j = lane; j < src.k; j += 32) {
-        const DtPt v = src.get(j);
-        const unsigned vd = (unsigned)(v.x * v.x + v.y * v.y);
-        if (vd < d || (vd == d && v.z < z)) {
-            d = vd;
-            z = v.z;
-            c = j;
-        }
-        q |= dt_quadrant(v.x, v.y);
+
+// Calls visit(q, inside) for the points of the cells [c0, c1] of consecutive
+// cell rows from cy0 on, one row per lane (up to 16; c0 > c1: none), 32 at a
+// time and two loads in flight: the rows' ranges are walked as one index
+// space (a binary search over the lanes' prefix sums).
+template <class Visit>
+__device__ __forceinline__ void dt_warp_rows(const DtArgs &a, const DtSide &S, int cy0, int nrows, int c0, int c1,
+                                             int lane, Visit visit) {
+    int rs = 0, len = 0;
+    if (lane < nrows && c0 <= c1) {
+        const int *row = S.cell_start + (cy0 + lane) * a.gw;
+        rs = row[c0];
+        len = row[c1 + 1] - rs;
     }
-    quads = __reduce_or_sync(0xFFFFFFFFu, q);
-    const unsigned dm = __reduce_min_sync(0xFFFFFFFFu, d);
-    const int zm = __reduce_min_sync(0xFFFFFFFFu, d == dm ? z : 0x7FFFFFFF);
-    const unsigned b = __ballot_sync(0xFFFFFFFFu, d == dm && z == zm);
-    return src.get(__shfl_sync(0xFFFFFFFFu, c, __ffs(b) - 1));
+    int incl = len;
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) {
+        const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    const int total = __shfl_sync(0xFFFFFFFFu, incl, 15);
+    const int excl = incl - len, off = rs - excl;
+    for (int t0 = 0; t0 < total; t0 += 64) {
+        int4 q[2];
+        bool in[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int t = t0 + 32 * u + lane;
+            int lo = 0;
+#pragma unroll
+            for (int s = 8; s > 0; s >>= 1)
+                if (t >= __shfl_sync(0xFFFFFFFFu, excl, lo + s)) lo += s;
+            in[u] = t < total;
+            const int at = t + __shfl_sync(0xFFFFFFFFu, off, lo);
+            q[u] = in[u] ? S.pts[at] : make_int4(0, 0, 0, 0);
+        }
+        visit(q[0], in[0]);
+        if (t0 + 32 < total) visit(q[1], in[1]);
+    }
+}
+
+// A step whose circle the near list does not certify: w (parameter t) is the
+// best listed third vertex of edge (p, e), so the true one is w or lies inside
+// their circle (centre e/2 + side t perp(e)/2).  Every point of the cells that
+// the circle meets is offered; each lane keeps its exact best, and the lanes'
+// bests are ordered like dt_step's.  False: the circle is too wide.
+__device__ __forceinline__ bool dt_wide_step(const DtArgs &a, const DtSide &S, const int4 &p, const float4 &e, int side,
+                                             float t, int lane, float4 &w) {
+    const float r = 0.5f * sqrtf(e.z * __fmaf_rn(t, t, 1.0f));
+    if (!(r <= kDtWideMax)) return false;
+    const float st = side > 0 ? t : -t;
+    const float X = (float)p.x + 0.5f * (e.x - st * e.y), Y = (float)p.y + 0.5f * (e.y + st * e.x);
+    const float rr = r * 1.001f + 1.0f;  // padded for the rounding of t and the centre
+    const int cy0 = (int)fmaxf(0.0f, floorf((Y - rr) / kDtCell));
+    const int cy1 = min(a.gh - 1, (int)fmaxf(0.0f, floorf((Y + rr) / kDtCell)));
+    const float ya = (float)((cy0 + lane) * kDtCell) - Y, yb = ya + (float)(kDtCell - 1);
+    const float dy = ya > 0.0f ? ya : (yb < 0.0f ? -yb : 0.0f);
+    int c0 = 1, c1 = 0;
+    if (dy <= rr) {
+        const float hc = sqrtf(rr * rr - dy * dy);
+        // points left of the image are in the first cell of their row
+        c0 = min(a.gw - 1, (int)fmaxf(0.0f, floorf((X - hc) / kDtCell)));
+        c1 = min(a.gw - 1, (int)fmaxf(0.0f, floorf((X + hc) / kDtCell)));
+    }
+    const float sd = (float)side, most = __fmaf_rn(fabsf(t), 0x1p-16f, t);
+    float fl = kDtInf;
+    float4 best = dt_no_cand();
+    dt_warp_rows(a, S, cy0, cy1 - cy0 + 1, c0, c1, lane, [&](const int4 &q, bool inside) {
+        const float x = (float)(q.x - p.x), y = (float)(q.y - p.y);
+        const float4 c = make_float4(x, y, __fmaf_rn(x, x, y * y), __int_as_float(q.z));
+        const float D = dt_d(e, c, sd);
+        const float f = inside && q.w && D > 0.0f ? dt_div(dt_n(e, c), D) : kDtInf;
+        if (f > most) return;
+        const float band = 0x1p-17f * fabsf(f);
+        if (f < fl - band || (f <= fl + band && dt_beats(e, p.z, best, c, sd))) {
+            fl = f;
+            best = c;
+        }
+    });
+    const float fm = dt_warp_min(fl);
+    if (fm == kDtInf) return false;
+    dt_champion(
+        fl <= __fmaf_rn(fabsf(fm), 0x1p-17f, fm), lane,
+        [&](int src) {
+            return make_float4(__shfl_sync(0xFFFFFFFFu, best.x, src), __shfl_sync(0xFFFFFFFFu, best.y, src),
+                               __shfl_sync(0xFFFFFFFFu, best.z, src), __shfl_sync(0xFFFFFFFFu, best.w, src));
+        },
+        [&](int) { return best; },
+        [&](const float4 &c1, const float4 &c2) { return dt_beats(e, p.z, c1, c2, sd); }, w);
+    return true;
 }
 
 // Where triangle t of a fan of m goes in the output: the owned triangles of a
@@ -545,7 +658,7 @@ __device__ __forceinline__ void dt_warp_write(const DtSide &S, int pz, int lane,
 }
 
 // One star by a warp over the candidates within R of p; true if it came out
-// certified (its owned triangles are then written).
+// certain (its owned triangles are then written).
 //
 // Triangles are emitted by their lowest-index vertex.  A list in raster order
 // (v never decreases) puts the two others of an owned triangle level with p
@@ -554,121 +667,97 @@ __device__ __forceinline__ void dt_warp_write(const DtSide &S, int pz, int lane,
 // that the circle growing straight down from p meets first, both ways until
 // a vertex is not below p.  That is 4 steps per star on average instead of
 // the whole star's 6.  It needs p strictly inside the hull (candidates in all
-// four open quadrants show that); other stars, and every star of an
-// unordered list, are wrapped whole from the nearest neighbour,
+// four open quadrants show that) and a certain first vertex; other stars, and
+// every star of an unordered list, are wrapped whole from the nearest neighbour,
 // counter-clockwise and, when that meets the hull, clockwise from it again.
 //
 // A triangle is certain when its circle, which passes through p, is no wider
-// than R: no point farther than R from p is inside it.  Where a whole star
+// than R (no point farther than R from p is inside it), or when its third
+// vertex came from a search of the circle (WIDE: dt_wide_step).  Where a whole star
 // stays open (p on the hull), nothing may lie beyond either open edge, tested
 // against the extreme points of every image row.
-template <class Src>
+template <bool WIDE, class Src>
 __device__ __forceinline__ bool dt_warp_star(const DtArgs &a, const DtSide &S, const int4 &p, const Src &src, int R,
                                              bool ordered, int lane) {
     unsigned quads;
-    auto nn = dt_nearest(src, lane, quads);
-    auto first = nn;
-    const bool fan = ordered && quads == 15u;
-    if (fan && !dt_fan_start(src, lane, first)) return false;
+    const float4 nn = dt_nearest(src, lane, quads);
+    bool fan = ordered && quads == 15u;
+    float4 first = nn;
+    if (fan) {
+        int at;
+        dt_fan_start(src, lane, first, at);
+        // certain only when the touching circle (diameter |c|^2 / y) fits the disc
+        fan = first.z <= (float)R * first.y;
+        if (!fan) first = nn;
+    }
     const float R2 = (float)(R * R);
-    int va = dt_z(first), vb = va, na = 0, nb = 0;
-    bool closed = false, open_l = false, open_r = false;
-    auto cur = first;
+    const int z0 = __float_as_int(first.w);
+    int va = z0, vb = z0, na = 0, nb = 0, at;
+    float4 cur = first, w;
+    float t;
+    bool closed = false, open = false;
     for (;;) {  // counter-clockwise
-        auto w = cur;
-        if (!dt_step(src, lane, cur, p.z, 1, w)) {
-            open_l = true;
+        if (!dt_step(src, lane, cur, p.z, 1, w, t, at)) {
+            open = true;
             break;
         }
-        if (na == 30 || !dt_small_circle(dt_ix(cur), dt_iy(cur), dt_ix(w), dt_iy(w), R2)) return false;
+        if (!dt_small_circle(cur.z, t, R2)) {
+            if constexpr (!WIDE) return false;
+            if (!dt_wide_step(a, S, p, cur, 1, t, lane, w)) return false;
+        }
+        if (na == 30) return false;
         ++na;
-        if (lane == na) va = dt_z(w);
-        if (fan && dt_iy(w) <= 0) break;
-        if (!fan && dt_z(w) == dt_z(first)) {
+        const int z = __float_as_int(w.w);
+        if (lane == na) va = z;
+        if (fan) {
+            if (!(w.y > 0.0f)) break;
+        } else if (z == z0) {
             closed = true;
             break;
         }
         cur = w;
     }
-    if (fan && open_l) return false;
-    const auto e_l = cur;
+    if (fan && open) return false;
+    const float lx = cur.x, ly = cur.y;
     cur = first;
     while (!closed) {  // clockwise
-        auto w = cur;
-        if (!dt_step(src, lane, cur, p.z, -1, w)) {
-            open_r = true;
+        if (!dt_step(src, lane, cur, p.z, -1, w, t, at)) {
+            open = true;
             break;
         }
-        if (nb == 30 || !dt_small_circle(dt_ix(w), dt_iy(w), dt_ix(cur), dt_iy(cur), R2)) return false;
+        if (!dt_small_circle(cur.z, t, R2)) {
+            if constexpr (!WIDE) return false;
+            if (!dt_wide_step(a, S, p, cur, -1, t, lane, w)) return false;
+        }
+        if (nb == 30) return false;
         ++nb;
-        if (lane == nb) vb = dt_z(w);
-        if (fan && dt_iy(w) <= 0) break;
+        if (lane == nb) vb = __float_as_int(w.w);
+        if (fan && !(w.y > 0.0f)) break;
         cur = w;
     }
-    if (fan && open_r) return false;
-    if (open_l || open_r) {
-        const int lx = dt_ix(e_l), ly = dt_iy(e_l), rx = dt_ix(cur), ry = dt_iy(cur);
+    if (fan && open) return false;
+    if (open) {
+        const int ax = (int)lx, ay = (int)ly, bx = (int)cur.x, by = (int)cur.y;
         bool bad = false;
         for (int y = lane; y < a.h; y += 32) {
             const int x0 = S.rowmin[y], x1 = S.rowmax[y];
             if (x0 > x1) continue;
             const int dy = y - p.y, d0 = x0 - p.x, d1 = x1 - p.x;
-            bad |= lx * dy - ly * d0 > 0 || lx * dy - ly * d1 > 0;
-            bad |= rx * dy - ry * d0 < 0 || rx * dy - ry * d1 < 0;
+            bad |= ax * dy - ay * d0 > 0 || ax * dy - ay * d1 > 0;
+            bad |= bx * dy - by * d0 < 0 || bx * dy - by * d1 < 0;
         }
         if (__any_sync(0xFFFFFFFFu, bad)) return false;
     }
-    dt_warp_write(S, p.z, lane, fan, va, vb, na, nb, dt_z(nn));
+    dt_warp_write(S, p.z, lane, fan, va, vb, na, nb, __float_as_int(nn.w));
     return true;
 }
 
-// Calls visit(q, inside) for the points of the grid cells that the square of
-// half-size R around p meets, 32 at a time: the cell rows' ranges, up to
-// 2^LOG2 of them, are walked as one index space (a binary search over the
-// lanes' prefix sums), two loads in flight.
-template <int LOG2, class Visit>
-__device__ __forceinline__ void dt_warp_window(const DtArgs &a, const DtSide &S, const int4 &p, int R, int lane,
-                                               Visit visit) {
-    const int cx0 = min(a.gw - 1, max(0, p.x - R) / kDtCell), cx1 = min(a.gw - 1, max(0, p.x + R) / kDtCell);
-    const int cy0 = max(0, p.y - R) / kDtCell, cy1 = min(a.gh - 1, max(0, p.y + R) / kDtCell);
-    int rs = 0, len = 0;
-    if (lane <= cy1 - cy0) {
-        const int *row = S.cell_start + (cy0 + lane) * a.gw;
-        rs = row[cx0];
-        len = row[cx1 + 1] - rs;
-    }
-    int incl = len;
-#pragma unroll
-    for (int o = 1; o < (1 << LOG2); o <<= 1) {
-        const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    const int total = __shfl_sync(0xFFFFFFFFu, incl, (1 << LOG2) - 1);
-    const int excl = incl - len, off = rs - excl;
-    for (int t0 = 0; t0 < total; t0 += 64) {
-        int4 q[2];
-        bool in[2];
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const int t = t0 + 32 * u + lane;
-            int lo = 0;
-#pragma unroll
-            for (int s = 1 << (LOG2 - 1); s > 0; s >>= 1)
-                if (t >= __shfl_sync(0xFFFFFFFFu, excl, lo + s)) lo += s;
-            in[u] = t < total;
-            const int at = t + __shfl_sync(0xFFFFFFFFu, off, lo);
-            q[u] = in[u] ? S.pts[at] : make_int4(0, 0, 0, 0);
-        }
-        visit(q[0], in[0]);
-        if (t0 + 32 < total) visit(q[1], in[1]);
-    }
-}
-
-// Warp pass: one warp per point, the candidates within 24 pixels (12 or 6
-// where the list is full).  Bound by instruction issue: about 400 warp
-// instructions per star.
+// Warp pass: one warp per point, the candidates within 24 pixels (16 or 8
+// where there are more than 64).  Bound by instruction issue.
 __device__ __forceinline__ void dt_pass1_body(const DtArgs &a, const VB &vb) {
-    __shared__ float4 s_list[kDtWarps][kDtListCap];
+    constexpr int kRows = 2 * kDtRadius / kDtCell + 1;  // cell rows (and columns) the disc's square meets
+    static_assert(2 * kDtRadius % kDtCell == 0, "the square of a disc spans kRows rows wherever it lies");
+    __shared__ float4 s_list[kDtWarps][kDtNearCap];
     const DtSide &S = a.s[vb.y];
     const int n = min(max(*a.count, 0), a.cap);
     const int lane = threadIdx.x & 31;
@@ -677,79 +766,98 @@ __device__ __forceinline__ void dt_pass1_body(const DtArgs &a, const VB &vb) {
     for (int j = vb.x * kDtWarps + (threadIdx.x >> 5); j < n; j += vb.gx * kDtWarps) {
         const int4 p = S.pts[j];
         if (!p.w) continue;
-        int k = 0;
-        auto gather = [&](int R) {
+        const int cx0 = min(a.gw - 1, max(0, p.x - kDtRadius) / kDtCell);
+        const int cx1 = min(a.gw - 1, max(0, p.x + kDtRadius) / kDtCell);
+        const int cy0 = max(0, p.y - kDtRadius) / kDtCell, cy1 = min(a.gh - 1, (p.y + kDtRadius) / kDtCell);
+        int rs = 0, len = 0;
+        if (lane <= cy1 - cy0) {
+            const int *row = S.cell_start + (cy0 + lane) * a.gw;
+            rs = row[cx0];
+            len = row[cx1 + 1] - rs;
+        }
+        const int most = __reduce_max_sync(0xFFFFFFFFu, len);
+        int R = kDtRadius, k;
+        for (;;) {
+            const float R2 = (float)(R * R);
             k = 0;
-            dt_warp_window<2>(a, S, p, R, lane, [&](const int4 &q, bool inside) {
-                const int dx = q.x - p.x, dy = q.y - p.y, d2 = dx * dx + dy * dy;
-                const bool take = inside && q.w && q.z != p.z && d2 <= R * R;
-                const unsigned b = __ballot_sync(0xFFFFFFFFu, take);
-                const int pos = k + __popc(b & ((1u << lane) - 1u));
-                if (take && pos < kDtListCap)
-                    list[pos] = make_float4((float)dx, (float)dy, (float)d2, __int_as_float(q.z));
-                k += __popc(b);
-            });
-        };
-        int R = kDtRadius;
-        gather(R);
-        while (k > kDtListCap && R > 6) {
-            R >>= 1;
+            for (int c0 = 0; c0 < most; c0 += 32) {
+                int4 q[kRows];  // a chunk of every row, the loads together
+#pragma unroll
+                for (int r = 0; r < kRows; ++r) {
+                    const int s0 = __shfl_sync(0xFFFFFFFFu, rs, r), l = __shfl_sync(0xFFFFFFFFu, len, r);
+                    q[r] = c0 + lane < l ? S.pts[s0 + c0 + lane] : make_int4(0, 0, p.z, 0);
+                }
+#pragma unroll
+                for (int r = 0; r < kRows; ++r) {
+                    const float dx = (float)(q[r].x - p.x), dy = (float)(q[r].y - p.y);
+                    const float d2 = __fmaf_rn(dx, dx, dy * dy);
+                    const bool take = q[r].w && q[r].z != p.z && d2 <= R2;
+                    const unsigned b = __ballot_sync(0xFFFFFFFFu, take);
+                    const int pos = k + __popc(b & ((1u << lane) - 1u));
+                    if (take && pos < kDtNearCap) list[pos] = make_float4(dx, dy, d2, __int_as_float(q[r].z));
+                    k += __popc(b);
+                }
+            }
+            if (k <= kDtNearCap || R <= 8) break;
+            R -= 8;
             __syncwarp();
-            gather(R);
         }
         __syncwarp();
         bool done = false;
-        if (k > 0 && k <= kDtListCap) {
-            DtNearSrc src{list, k};
-            src.load(lane);
-            done = dt_warp_star(a, S, p, src, R, ordered, lane);
-        }
-        if (!done && lane == 0) S.pending[atomicAdd(S.npending, 1)] = p.z;
+        if (k > 0 && k <= kDtNearCap) done = dt_warp_star<false>(a, S, p, DtNearSrc(list, k, lane), R, ordered, lane);
+        if (!done && lane == 0) S.pending[atomicAdd(S.npending, 1)] = j;
         __syncwarp();
     }
 }
 
-__global__ void __launch_bounds__(kDtWarps * 32, 5) dt_pass1_kernel(DtArgs a) { dt_pass1_body(a, vb_single()); }
-__global__ void __launch_bounds__(kDtWarps * 32, 5) dt_pass1_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
+__global__ void __launch_bounds__(kDtWarps * 32, 4) dt_pass1_kernel(const __grid_constant__ DtArgs a) { dt_pass1_body(a, vb_single()); }
+__global__ void __launch_bounds__(kDtWarps * 32, 4) dt_pass1_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
     const VB vb = vb_batch(vm);
     dt_pass1_body(slot_entry(tab, vm.stride, vb.slot), vb);
 }
 
-// Middle pass (batches): the stars left by the warp pass, again a warp each,
-// with the candidates within 64 pixels.
-__device__ __forceinline__ void dt_pass1m_body(const DtArgs &a, const VB &vb) {
-    __shared__ int2 s_list[kDtWarpsM][kDtListCapM];
+// Middle pass (batches): the stars left by the warp pass, again a warp each, with the
+// candidates within 48 pixels and searches of wider circles.
+__device__ __forceinline__ void dt_pass2_body(const DtArgs &a, const VB &vb) {
+    __shared__ float4 s_list[kDtWarpsM][kDtListCapM];
     const DtSide &S = a.s[vb.y];
     const int lane = threadIdx.x & 31;
-    int2 *list = s_list[threadIdx.x >> 5];
+    float4 *list = s_list[threadIdx.x >> 5];
     const bool ordered = !(*S.err & 8);
     const int njobs = *S.npending;
     for (int j = vb.x * kDtWarpsM + (threadIdx.x >> 5); j < njobs; j += vb.gx * kDtWarpsM) {
-        const int4 p = S.pts[S.slot[S.pending[j]]];
-        int k = 0;
-        dt_warp_window<4>(a, S, p, kDtRadiusM, lane, [&](const int4 &q, bool inside) {
-            const int dx = q.x - p.x, dy = q.y - p.y;
-            const bool take = inside && q.w && q.z != p.z && dx * dx + dy * dy <= kDtRadiusM * kDtRadiusM;
-            const unsigned b = __ballot_sync(0xFFFFFFFFu, take);
-            const int pos = k + __popc(b & ((1u << lane) - 1u));
-            if (take && pos < kDtListCapM) list[pos] = dt_pack(dx, dy, q.z);
-            k += __popc(b);
-        });
+        const int at = S.pending[j];
+        const int4 p = S.pts[at];
+        const int cx0 = min(a.gw - 1, max(0, p.x - kDtRadiusM) / kDtCell);
+        const int cx1 = min(a.gw - 1, max(0, p.x + kDtRadiusM) / kDtCell);
+        const int cy0 = max(0, p.y - kDtRadiusM) / kDtCell, cy1 = min(a.gh - 1, (p.y + kDtRadiusM) / kDtCell);
+        int R = kDtRadiusM, k;
+        for (;;) {
+            k = 0;
+            dt_warp_rows(a, S, cy0, cy1 - cy0 + 1, cx0, cx1, lane, [&](const int4 &q, bool inside) {
+                const int dx = q.x - p.x, dy = q.y - p.y;
+                const bool take = inside && q.w && q.z != p.z && dx * dx + dy * dy <= R * R;
+                const unsigned b = __ballot_sync(0xFFFFFFFFu, take);
+                const int pos = k + __popc(b & ((1u << lane) - 1u));
+                if (take && pos < kDtListCapM) list[pos] = dt_cand(dx, dy, q.z);
+                k += __popc(b);
+            });
+            if (k <= kDtListCapM || R <= 8) break;
+            R >>= 1;
+            __syncwarp();
+        }
         __syncwarp();
         bool done = false;
-        if (k > 0 && k <= kDtListCapM) {
-            const DtListSrc src{list, k};
-            done = dt_warp_star(a, S, p, src, kDtRadiusM, ordered, lane);
-        }
-        if (!done && lane == 0) S.pending2[atomicAdd(S.npending2, 1)] = p.z;
+        if (k > 0 && k <= kDtListCapM)
+            done = dt_warp_star<true>(a, S, p, DtListSrc(list, k, true, lane), R, ordered, lane);
+        if (!done && lane == 0) S.pending2[atomicAdd(S.npending2, 1)] = at;
         __syncwarp();
     }
 }
-static_assert(2 * kDtRadius / kDtCell + 1 <= 4 && 2 * kDtRadiusM / kDtCell + 2 <= 16, "cell rows of a disc");
 
-__global__ void __launch_bounds__(kDtWarpsM * 32) dt_pass1m_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
+__global__ void __launch_bounds__(kDtWarpsM * 32, 7) dt_pass2_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
     const VB vb = vb_batch(vm);
-    dt_pass1m_body(slot_entry(tab, vm.stride, vb.slot), vb);
+    dt_pass2_body(slot_entry(tab, vm.stride, vb.slot), vb);
 }
 
 // -------------------------------------------------------------------------
@@ -760,22 +868,39 @@ __global__ void __launch_bounds__(kDtWarpsM * 32) dt_pass1m_kernel_b(const DtArg
 // memory and the star is wrapped over the cache (warp 0 counter-clockwise,
 // warp 1 clockwise).  Triangles whose circle is no wider than the disc are
 // certain; for all the others at once the CTA scans the grid cells that their
-// circles (and, at an open end, the half-plane beyond the edge) meet, adds
-// every point found inside to the cache, and the star is wrapped again.  The
-// star is done when a scan finds no point: each of its triangles then has an
-// empty circle.  Most stars take one scan, the widest three; a step-by-step
-// search would scan once per triangle (up to 50).  A large region is first
-// scanned with a stride, which finds points that shrink the circles to a
-// small part of it.  A full cache keeps only the star's own vertices and
-// goes on with the whole star (its region can only shrink, so that ends).
-constexpr int kDtRadiusC = 96;
-constexpr int kDtCacheCap = 2048;   // cached points (16 KB)
-constexpr int kDtBlockThreads = 128;
-constexpr int kDtBlocksPerSM = 8;
+// circles (and, at an open end, the half-plane beyond the edge) meet and adds
+// every point found inside to the cache.  Then the star is wrapped again:
+// triangles that no point was found in stay, the gaps are stepped over anew.
+// The star is done when a scan finds no point: each of its triangles then has
+// an empty circle.  Most stars take one or two scans; a step-by-step search
+// would scan once per triangle (up to 50).  A large region is first scanned
+// with a stride, which finds points that shrink the circles to a small part
+// of it.  A full cache keeps only the star's own vertices and goes on with
+// the whole star (its region can only shrink, so that ends).
+constexpr int kDtRadiusC = 48;
+constexpr int kDtSamples = 128;     // points of the whole set cached too
+constexpr int kDtCacheCap = 1024;   // cached points (16 KB)
+// Threads of a CTA and CTAs per SM: one pair, whose time is that of its
+// longest star, 256 and 4 (1920x1080 triangulation 272 -> 258 us against 128
+// and 8); batches, bound by issue, 128 and 8 (64 x 1242x375 1.74 -> 1.66 ms
+// against 256 and 4).
+constexpr int kDtBlockThreads = 256, kDtBlocksPerSM = 4;
+constexpr int kDtBlockThreadsB = 128, kDtBlocksPerSMB = 8;
+constexpr int kDtBlockWarpsMax = 8;
 constexpr int kDtVertCap = 256;     // star vertices per direction
 constexpr int kDtBadCap = 32;       // circles scanned for at a time (a warp's triangles)
 constexpr int kDtMaxRounds = 64;
-constexpr int kDtSampleMin = 2048;  // regions of more points are sampled first
+constexpr int kDtSampleMin = 512;   // regions of more points are sampled first
+
+// Is the circle through the origin, a and b no wider than R (2r <= R)?
+// |a|^2 |b|^2 |a-b|^2 <= R^2 cross(a, b)^2, in FP32 with a margin (a false
+// answer only has the circle scanned).
+__device__ __forceinline__ bool dt_small_circle(const DtPt &a, const DtPt &b, float R2) {
+    const float pa = (float)(a.x * a.x + a.y * a.y), pb = (float)(b.x * b.x + b.y * b.y);
+    const float dx = (float)(b.x - a.x), dy = (float)(b.y - a.y);
+    const float ab = dx * dx + dy * dy, ar = (float)(a.x * b.y - a.y * b.x);
+    return pa * pb * ab * 1.00001f <= R2 * ar * ar;
+}
 
 // Triangle (p, a, b), counter-clockwise, coordinates relative to p: q lies
 // inside its circle iff |q|^2 W - U q.x - V q.y < 0 (below 2^60).
@@ -811,95 +936,139 @@ __device__ __forceinline__ bool dt_violates(const DtCircle &c, int pz, const DtP
     return min(m1, m2) < min(opp, q.z);
 }
 
-struct DtStarShared {
-    DtCircle bad[kDtBadCap];
-    int2 vert[2][kDtVertCap];  // the star: counter-clockwise, clockwise from the first vertex
-    int nv[2];                 // triangles in each direction
-    int open[2];
-    int over;                  // more vertices than the lists hold
-    int closed;
-    unsigned long long nn;     // |c|^2 and index of the nearest point
-    unsigned quads;
-    int k, nbad, next, found, total;
-    int rs[16], rlen[16];
-    DtPt win[4];
-    int won[4];
+// The region of a circle, relative to p: a disc (x, y, r padded for the FP32
+// rounding of the centre) or, past 1e6 pixels, the half-plane beyond its
+// tangent at p, which holds it (unit normal x, y; r < 0).
+__device__ __forceinline__ float3 dt_region(const DtCircle &c) {
+    const float U = (float)c.U, V = (float)c.V, w = 0.5f * dt_div(1.0f, (float)c.W);
+    const float ux = U * w, uy = V * w, r = sqrtf(ux * ux + uy * uy);
+    if (r <= 1e6f) return make_float3(ux, uy, r * 1.0001f + 1.0f);
+    const float l = rsqrtf(U * U + V * V);
+    return make_float3(U * l, V * l, -1.0f);
+}
+
+// A star over the cache: per direction the vertices' places in it and the
+// state of the triangle that follows each.
+enum { kDtOpenCircle = 0, kDtEmpty = 1, kDtHit = 2 };
+struct DtStarList {
+    uint16_t v[2][kDtVertCap];
+    uint8_t state[2][kDtVertCap];
+    int n[2];     // triangles in each direction
+    int open[2];  // the direction ends at the hull of the cache
 };
 
-// Cell range of image rows [cy*16, cy*16+15] that a region meets, widened so
-// that FP32 rounding cannot lose a cell (two pixels in y, one cell and more
-// in x).  A disc (rad >= 0) or the half-plane nx*x + ny*y >= 0 about (x0, y0).
-__device__ __forceinline__ bool dt_row_range(int cy, float x0, float y0, float rad, float nx, float ny, int gw,
-                                             int &c0, int &c1) {
-    const float ya = (float)(cy * kDtCell - 2) - y0, yb = (float)(cy * kDtCell + kDtCell + 1) - y0;
+struct DtStarShared {
+    DtStarList star[2];            // the star and the one before it
+    DtCircle bad[kDtBadCap];
+    float3 region[kDtBadCap + 2];  // of the circles, then of the open ends
+    uint16_t tri[kDtBadCap];       // direction << 15 | triangle
+    int over;                      // more vertices than the lists hold
+    int closed;
+    unsigned long long nn;         // |c|^2 and index of the nearest point
+    int nearest;                   // its place in the cache
+    unsigned quads;
+    int far;                       // a cached point lies 2048 pixels or more from p
+    int k, nbad, next, found, total, row0, row1;
+    int rs[16], rpre[17];
+    DtPt win[kDtBlockWarpsMax];
+    int won[kDtBlockWarpsMax];
+};
+
+// Cells [c0, c1] that a region (about (x0, y0), padded for the FP32 rounding)
+// meets in cell row cy.  False: none.
+__device__ __forceinline__ bool dt_row_range(int cy, float x0, float y0, const float3 &g, int gw, int &c0, int &c1) {
+    const float ya = (float)(cy * kDtCell) - y0, yb = (float)(cy * kDtCell + kDtCell - 1) - y0;
     float xlo = -1e9f, xhi = 1e9f;
-    if (rad >= 0.0f) {
-        const float dy = ya > 0.0f ? ya : (yb < 0.0f ? -yb : 0.0f);
-        if (dy > rad) return false;
-        const float hc = sqrtf(rad * rad - dy * dy) + 2.0f;
-        xlo = x0 - hc;
-        xhi = x0 + hc;
+    if (g.z >= 0.0f) {
+        const float a = ya - g.y, b = yb - g.y;
+        const float dy = a > 0.0f ? a : (b < 0.0f ? -b : 0.0f);
+        if (dy > g.z) return false;
+        const float h2 = g.z * g.z - dy * dy, hc = h2 * rsqrtf(fmaxf(h2, 1e-6f)) * 1.0001f + 1.0f;
+        xlo = x0 + g.x - hc;
+        xhi = x0 + g.x + hc;
     } else {
-        // x >= or <= the boundary of the band's more permissive edge, 4 pixels wider
-        const float m = fmaxf(ny * ya, ny * yb) + 4.0f;
-        if (fabsf(nx) < 1e-4f) {
+        // the boundary at the band's more permissive edge, 4 pixels wider
+        const float m = fmaxf(g.y * ya, g.y * yb) + 4.0f;
+        if (fabsf(g.x) < 1e-4f) {
             if (m < -4.0f) return false;
-        } else if (nx > 0.0f) {
-            xlo = x0 - m / nx - 4.0f;
+        } else if (g.x > 0.0f) {
+            xlo = x0 - __fdividef(m, g.x) - 4.0f;
         } else {
-            xhi = x0 - m / nx + 4.0f;
+            xhi = x0 - __fdividef(m, g.x) + 4.0f;
         }
     }
-    c0 = (int)fmaxf(0.0f, fminf((float)(gw - 1), floorf(xlo / kDtCell) - 1.0f));
-    c1 = (int)fmaxf(0.0f, fminf((float)(gw - 1), floorf(xhi / kDtCell) + 1.0f));
+    c0 = (int)fmaxf(0.0f, fminf((float)(gw - 1), floorf(xlo * (1.0f / kDtCell))));
+    c1 = (int)fmaxf(0.0f, fminf((float)(gw - 1), floorf(xhi * (1.0f / kDtCell))));
     return true;
 }
 
 // Gathers the points within R of p into the cache (their number, even past
 // the capacity, in sh.k), with the nearest one and the quadrants.
-__device__ __forceinline__ void dt_block_gather(const DtArgs &a, const DtSide &S, const int4 &p, int R, int2 *cand,
+template <int THREADS>
+__device__ __forceinline__ void dt_block_gather(const DtArgs &a, const DtSide &S, const int4 &p, int R, float4 *cand,
                                                 DtStarShared &sh) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31;
     const int cx0 = min(a.gw - 1, max(0, p.x - R) / kDtCell), cx1 = min(a.gw - 1, max(0, p.x + R) / kDtCell);
     const int cy0 = max(0, p.y - R) / kDtCell, cy1 = min(a.gh - 1, max(0, p.y + R) / kDtCell);
     const int nrows = cy1 - cy0 + 1;
     __syncthreads();
-    if (tid < nrows) {
-        const int *row = S.cell_start + (cy0 + tid) * a.gw;
-        const int r0 = row[cx0], r1 = row[cx1 + 1];
-        sh.rs[tid] = r0;
-        sh.rlen[tid] = r1 - r0;
-    }
-    if (tid == 0) {
-        sh.k = 0;
-        sh.nn = ~0ull;
-        sh.quads = 0;
+    if (tid < 32) {
+        int r0 = 0, len = 0;
+        if (lane < nrows) {
+            const int *row = S.cell_start + (cy0 + lane) * a.gw;
+            r0 = row[cx0];
+            len = row[cx1 + 1] - r0;
+        }
+        int incl = len;
+#pragma unroll
+        for (int o = 1; o < 16; o <<= 1) {
+            const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane < 16) {
+            sh.rs[lane] = r0 - (incl - len);
+            sh.rpre[lane] = incl - len;
+            if (lane == 15) sh.rpre[16] = incl;
+        }
+        if (lane == 0) {
+            sh.k = 0;
+            sh.nn = ~0ull;
+            sh.quads = 0;
+        }
     }
     __syncthreads();
+    const int total = sh.rpre[16];
     unsigned long long nn = ~0ull;
     unsigned quads = 0;
-    for (int r = warp; r < nrows; r += kDtBlockThreads / 32) {
-        const int s0 = sh.rs[r], len = sh.rlen[r];
-        for (int j0 = 0; j0 < len; j0 += 64) {
-            int4 q[2];
+    int at = 0;
+    for (int t0 = 0; t0 < total; t0 += 4 * THREADS) {  // four loads in flight
+        int4 q[4];
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int j = j0 + 32 * u + lane;
-                q[u] = j < len ? S.pts[s0 + j] : make_int4(0, 0, 0, 0);
-            }
+        for (int u = 0; u < 4; ++u) {
+            const int t = t0 + u * THREADS + tid;
+            int r = 0;
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int dx = q[u].x - p.x, dy = q[u].y - p.y, d2 = dx * dx + dy * dy;
-                const bool take = q[u].w && q[u].z != p.z && abs(dx) <= R && abs(dy) <= R && d2 <= R * R;
-                const unsigned m = __ballot_sync(0xFFFFFFFFu, take);
-                int base = 0;
-                if (lane == 0 && m) base = atomicAdd(&sh.k, __popc(m));
-                const int pos = __shfl_sync(0xFFFFFFFFu, base, 0) + __popc(m & ((1u << lane) - 1u));
-                if (take) {
-                    if (pos < kDtCacheCap) cand[pos] = dt_pack(dx, dy, q[u].z);
-                    nn = min(nn, ((unsigned long long)d2 << 32) | (unsigned)q[u].z);
-                    quads |= dt_quadrant(dx, dy);
+            for (int s = 8; s > 0; s >>= 1)
+                if (t >= sh.rpre[r + s]) r += s;
+            q[u] = t < total ? S.pts[sh.rs[r] + t] : make_int4(0, 0, 0, 0);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (t0 + u * THREADS >= total) break;
+            const int dx = q[u].x - p.x, dy = q[u].y - p.y, d2 = dx * dx + dy * dy;
+            const bool take = q[u].w && q[u].z != p.z && abs(dx) <= R && abs(dy) <= R && d2 <= R * R;
+            const unsigned m = __ballot_sync(0xFFFFFFFFu, take);
+            int base = 0;
+            if (lane == 0 && m) base = atomicAdd(&sh.k, __popc(m));
+            const int pos = __shfl_sync(0xFFFFFFFFu, base, 0) + __popc(m & ((1u << lane) - 1u));
+            if (take) {
+                if (pos < kDtCacheCap) cand[pos] = dt_cand(dx, dy, q[u].z);
+                const unsigned long long key = ((unsigned long long)d2 << 32) | (unsigned)q[u].z;
+                if (key < nn) {
+                    nn = key;
+                    at = pos;
                 }
+                quads |= dt_quadrant(dx, dy);
             }
         }
     }
@@ -908,80 +1077,119 @@ __device__ __forceinline__ void dt_block_gather(const DtArgs &a, const DtSide &S
         atomicOr(&sh.quads, quads);
     }
     __syncthreads();
+    if (nn != ~0ull && nn == sh.nn) sh.nearest = at;
+    __syncthreads();
 }
 static_assert(2 * kDtRadiusC / kDtCell + 2 <= 16, "cell rows of the cached disc");
 
-// Wraps the star over the cache: warp 0 counter-clockwise, warp 1 clockwise.
-__device__ __forceinline__ void dt_block_wrap(const int2 *cand, int k, int pz, bool fan, const DtPt &nn,
+// Wraps the star over the cache into sh.star[cur] (warp 0 counter-clockwise,
+// warp 1 clockwise from the first vertex).  again: sh.star[cur ^ 1] is the
+// star before the last points were added, its hit triangles marked: the
+// others stay triangles of the star, so only the gaps are stepped over.
+__device__ __forceinline__ void dt_block_wrap(const float4 *cand, int k, int pz, bool fan, bool again, int cur,
                                               DtStarShared &sh) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const DtStarList &old = sh.star[cur ^ 1];
+    DtStarList &star = sh.star[cur];
     __syncthreads();
     if (warp < 2) {
-        const DtListSrc src{cand, k};
-        const int side = warp ? -1 : 1;
-        DtPt first = nn;
-        bool ok = !fan || dt_fan_start(src, lane, first);
-        DtPt cur = first;
-        int nv = 0;
-        bool open = false, closed = false;
-        if (lane == 0) sh.vert[warp][0] = dt_pack(first.x, first.y, first.z);
-        while (ok) {
-            DtPt w;
-            if (!dt_step(src, lane, cur, pz, side, w)) {
-                open = true;
-                break;
+        const DtListSrc src(cand, k, !sh.far, lane);
+        // a fan's first vertex is certain while a triangle beside it is
+        if (again && fan && old.state[0][0] == kDtHit && old.state[1][0] == kDtHit) again = false;
+        const int side = warp ? -1 : 1, nold = again ? old.n[warp] : 0;
+        int first = again ? old.v[warp][0] : sh.nearest, n = 0;
+        float4 e;
+        bool ok = again || !fan || dt_fan_start(src, lane, e, first);
+        bool open = false;
+        const bool skip = warp == 1 && again && sh.closed;  // the other direction has the whole star
+        e = cand[first];
+        const int z0 = __float_as_int(e.w);
+        if (lane == 0) star.v[warp][0] = first;
+        int i = 0;        // the last vertex of the old star met
+        bool on = again;  // e is that vertex
+        while (ok && !skip) {
+            int at;
+            uint8_t state = kDtOpenCircle;
+            float4 w;
+            if (on && i < nold && old.state[warp][i] != kDtHit) {  // this triangle stays
+                state = old.state[warp][i];
+                at = old.v[warp][++i];
+                w = cand[at];
+            } else {
+                float t;
+                if (!dt_step(src, lane, e, pz, side, w, t, at)) {
+                    open = true;
+                    break;
+                }
+                on = false;
+                for (int j0 = i; j0 <= nold && !on && nold > 0; j0 += 32) {
+                    const unsigned b = __ballot_sync(0xFFFFFFFFu, j0 + lane <= nold && old.v[warp][j0 + lane] == at);
+                    if (b) {
+                        i = j0 + __ffs(b) - 1;
+                        on = true;
+                    }
+                }
             }
-            if (nv == kDtVertCap - 1) {
+            if (n == kDtVertCap - 1) {
                 ok = false;
                 break;
             }
-            ++nv;
-            if (lane == 0) sh.vert[warp][nv] = dt_pack(w.x, w.y, w.z);
-            if (fan && w.y <= 0) break;
-            if (!fan && w.z == first.z) {
-                closed = true;
+            if (lane == 0) {
+                star.v[warp][n + 1] = at;
+                star.state[warp][n] = state;
+            }
+            ++n;
+            if (fan) {
+                if (!(w.y > 0.0f)) break;
+            } else if (__float_as_int(w.w) == z0) {
+                if (lane == 0) sh.closed = 1;
                 break;
             }
-            cur = w;
+            e = w;
         }
         if (lane == 0) {
-            sh.nv[warp] = nv;
-            sh.open[warp] = open;
+            star.n[warp] = skip ? 0 : n;
+            star.open[warp] = open;
             if (!ok || (fan && open)) sh.over = 1;
-            if (closed) sh.closed = 1;  // both warps meet the first vertex again
         }
     }
     __syncthreads();
-    if (threadIdx.x == 0 && sh.closed) sh.nv[1] = 0;
+    // a closed star is the counter-clockwise run alone
+    if (threadIdx.x == 0 && sh.closed) star.n[1] = star.open[1] = 0;
     __syncthreads();
 }
 
-// Triangle t of the star in sh (counter-clockwise run first), as (a, b).
-__device__ __forceinline__ void dt_star_tri(const DtStarShared &sh, int t, DtPt &a, DtPt &b) {
-    const int na = sh.nv[0];
-    const DtListSrc src{sh.vert[t < na ? 0 : 1] + (t < na ? t : t - na), 2};
-    a = src.get(t < na ? 0 : 1);
-    b = src.get(t < na ? 1 : 0);
+// Triangle t of a star (counter-clockwise run first), as (a, b).
+__device__ __forceinline__ void dt_star_tri(const DtStarList &star, const float4 *cand, int t, float4 &a, float4 &b) {
+    const int na = star.n[0];
+    const uint16_t *v = t < na ? star.v[0] + t : star.v[1] + (t - na);
+    a = cand[v[t < na ? 0 : 1]];
+    b = cand[v[t < na ? 1 : 0]];
 }
 
-// Writes the owned triangles of the star in sh (warp 0).
-__device__ __forceinline__ void dt_block_write(const DtSide &S, int pz, bool fan, int nnz, const DtStarShared &sh) {
+// Writes the owned triangles of a star (warp 0).
+__device__ __forceinline__ void dt_block_write(const DtSide &S, int pz, bool fan, const float4 *cand,
+                                               const DtStarList &star, int nearest) {
     const int lane = threadIdx.x & 31;
-    const int na = sh.nv[0], nt = na + sh.nv[1];
+    const int na = star.n[0], nt = na + star.n[1];
+    auto owned = [&](int t, float4 &u, float4 &v) {
+        if (t >= nt) return false;
+        dt_star_tri(star, cand, t, u, v);
+        return pz < __float_as_int(u.w) && pz < __float_as_int(v.w);
+    };
     int ma = 0, mb = 0, r = -1;
     for (int t0 = 0; t0 < nt; t0 += 32) {
-        DtPt u{0, 0, 0}, v{0, 0, 0};
-        if (t0 + lane < nt) dt_star_tri(sh, t0 + lane, u, v);
-        const bool own = t0 + lane < nt && pz < u.z && pz < v.z;
+        float4 u, v;
+        const bool own = owned(t0 + lane, u, v);
         ma += __popc(__ballot_sync(0xFFFFFFFFu, own && t0 + lane < na));
         mb += __popc(__ballot_sync(0xFFFFFFFFu, own && t0 + lane >= na));
     }
     const int m = ma + mb;
     if (fan) {
         for (int i = lane; i <= ma; i += 32)
-            if (sh.vert[0][i].y == nnz) r = mb + i;
+            if (star.v[0][i] == nearest) r = mb + i;
         for (int i = lane; i <= mb; i += 32)
-            if (sh.vert[1][i].y == nnz) r = mb - i;
+            if (star.v[1][i] == nearest) r = mb - i;
         r = max(0, __reduce_max_sync(0xFFFFFFFFu, r));
     }
     int2 *out = S.slots + (size_t)pz * kDtSlots;
@@ -996,13 +1204,12 @@ __device__ __forceinline__ void dt_block_write(const DtSide &S, int pz, bool fan
     int done = 0;
     for (int t0 = 0; t0 < nt; t0 += 32) {
         const int t = t0 + lane;
-        DtPt u{0, 0, 0}, v{0, 0, 0};
-        if (t < nt) dt_star_tri(sh, t, u, v);
-        const bool own = t < nt && pz < u.z && pz < v.z;
+        float4 u, v;
+        const bool own = owned(t, u, v);
         const unsigned b = __ballot_sync(0xFFFFFFFFu, own);
         int pos = done + __popc(b & ((1u << lane) - 1u));
         if (fan) pos = dt_fan_pos(t < na ? mb + t : mb - 1 - (t - na), m, r);
-        if (own) out[pos] = make_int2(u.z, v.z);
+        if (own) out[pos] = make_int2(__float_as_int(u.w), __float_as_int(v.w));
         done += __popc(b);
     }
     if (lane == 0) S.owned[pz] = m;
@@ -1011,7 +1218,8 @@ __device__ __forceinline__ void dt_block_write(const DtSide &S, int pz, bool fan
 // The whole star of p over every point, one exact step after the other (more
 // vertices than the lists hold, e.g. the apex of a huge fan): counted first,
 // then written.
-__device__ void dt_block_star_all(const DtSide &S, const int4 &p, int n, const DtPt &nn, DtStarShared &sh) {
+template <int THREADS>
+__device__ __noinline__ void dt_block_star_all(const DtSide &S, const int4 &p, int n, const DtPt &nn, DtStarShared &sh) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int2 *out = nullptr;
     int m = 0;
@@ -1021,9 +1229,15 @@ __device__ void dt_block_star_all(const DtSide &S, const int4 &p, int n, const D
         for (int side = 1; side >= -1 && !closed; side -= 2) {
             DtPt cur = nn;
             for (int step = 0; step <= n; ++step) {
-                const DtAllSrc src{S.pts, (n - warp + 3) / 4, warp, p.x, p.y, p.z};
                 DtPt w{0, 0, 0};
-                const bool any = dt_step(src, lane, cur, p.z, side, w);
+                int at;
+                const bool any = dt_step_int(
+                    [&](int c) {  // this warp's quarter of the points
+                        const int4 q = S.pts[(THREADS / 32) * c + warp];
+                        // D = 0: never a candidate
+                        return q.w && q.z != p.z ? DtPt{q.x - p.x, q.y - p.y, q.z} : DtPt{0, 0, p.z};
+                    },
+                    (n - warp + (THREADS / 32) - 1) / (THREADS / 32), lane, cur, p.z, side, w, at);
                 __syncthreads();
                 if (lane == 0) {
                     sh.win[warp] = w;
@@ -1031,7 +1245,7 @@ __device__ void dt_block_star_all(const DtSide &S, const int4 &p, int n, const D
                 }
                 __syncthreads();
                 bool got = false;
-                for (int i = 0; i < 4; ++i)
+                for (int i = 0; i < (THREADS / 32); ++i)
                     if (sh.won[i] && (!got || dt_beats(cur, p.z, w, sh.win[i], side))) {
                         w = sh.win[i];
                         got = true;
@@ -1065,20 +1279,20 @@ __device__ void dt_block_star_all(const DtSide &S, const int4 &p, int n, const D
     __syncthreads();
 }
 
-__device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, int i, int n, bool ordered,
-                                              int2 *cand, int *r_start, int *r_len, DtStarShared &sh) {
+template <int THREADS>
+__device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, int at, int n, bool ordered,
+                                              float4 *cand, int *r_start, int *r_len, DtStarShared &sh) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int4 p = S.pts[S.slot[i]];
-    int R = kDtRadiusC;
-    dt_block_gather(a, S, p, R, cand, sh);
-    while (sh.k > kDtCacheCap && R > 1) {
+    const int4 p = S.pts[at];
+    int R = 2 * kDtRadiusC;
+    do {
         R >>= 1;
-        dt_block_gather(a, S, p, R, cand, sh);
-    }
+        dt_block_gather<THREADS>(a, S, p, R, cand, sh);
+    } while (sh.k > kDtCacheCap - kDtSamples && R > 1);
     int k = sh.k;
     if (k == 0) {  // nothing near: the nearest of all points
         unsigned long long key = ~0ull;
-        for (int j = tid; j < n; j += kDtBlockThreads) {
+        for (int j = tid; j < n; j += THREADS) {
             const int4 q = S.pts[j];
             const int64_t dx = q.x - p.x, dy = q.y - p.y;
             if (q.w && q.z != p.z) key = min(key, ((unsigned long long)(dx * dx + dy * dy) << 32) | (unsigned)q.z);
@@ -1090,114 +1304,230 @@ __device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, 
             __syncthreads();
             return;
         }
-    }
-    const int4 nq = S.pts[S.slot[(int)(unsigned)(sh.nn & 0xFFFFFFFFu)]];
-    const DtPt nn{nq.x - p.x, nq.y - p.y, nq.z};
-    bool fan = ordered && sh.quads == 15u;
-    if (k == 0) {
-        if (tid == 0) cand[0] = dt_pack(nn.x, nn.y, nn.z);
+        if (tid == 0) {
+            const int4 q = S.pts[S.slot[(int)(unsigned)(sh.nn & 0xFFFFFFFFu)]];
+            cand[0] = dt_cand(q.x - p.x, q.y - p.y, q.z);
+            sh.nearest = 0;
+        }
         k = 1;
+        __syncthreads();
     }
+    if (tid == 0) {
+        sh.far = max(fabsf(cand[sh.nearest].x), fabsf(cand[sh.nearest].y)) >= (float)kDtNearMax;
+        sh.k = k;
+    }
+    __syncthreads();
+    // points spread over the whole set, so that the first circles are not
+    // far wider than the star's
+    if (tid < kDtSamples) {
+        const int4 q = S.pts[(int)((int64_t)tid * n / kDtSamples)];
+        const int dx = q.x - p.x, dy = q.y - p.y, nz = __float_as_int(cand[sh.nearest].w);
+        if (q.w && q.z != p.z && q.z != nz && (max(abs(dx), abs(dy)) > R || dx * dx + dy * dy > R * R)) {
+            cand[atomicAdd(&sh.k, 1)] = dt_cand(dx, dy, q.z);
+            if (max(abs(dx), abs(dy)) >= kDtNearMax) sh.far = 1;
+            atomicOr(&sh.quads, dt_quadrant(dx, dy));
+        }
+    }
+    __syncthreads();
+    k = sh.k;
+    bool fan = ordered && sh.quads == 15u;
+    bool again = false, compact = false;
+    int cur = 0;
     for (int round = 0;; ++round) {
         if (tid == 0) {
             sh.over = 0;
-            sh.closed = 0;
-            sh.found = 0;
+            if (!again) sh.closed = 0;
         }
-        dt_block_wrap(cand, k, p.z, fan, nn, sh);
+        dt_block_wrap(cand, k, p.z, fan, again, cur, sh);
+        DtStarList &star = sh.star[cur];
         if (sh.over || round == kDtMaxRounds) {
-            dt_block_star_all(S, p, n, nn, sh);
+            dt_block_star_all<THREADS>(S, p, n, dt_point(cand[sh.nearest]), sh);
             return;
         }
-        const int nt = sh.nv[0] + sh.nv[1];
-        const bool open_l = sh.open[0], open_r = !sh.closed && sh.open[1];
+        if (compact) {
+            // full cache: keep only the whole star's vertices (no disc
+            // certifies its circles any more)
+            const int na = star.n[0] + (sh.closed ? 0 : 1), nv = na + star.n[1];
+            float4 keep[2 * kDtVertCap / THREADS];
+#pragma unroll
+            for (int u = 0; u < 2 * kDtVertCap / THREADS; ++u) {
+                const int j = u * THREADS + tid;
+                if (j < nv) keep[u] = cand[j < na ? star.v[0][j] : star.v[1][j - na + 1]];
+            }
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < 2 * kDtVertCap / THREADS; ++u) {
+                const int j = u * THREADS + tid;
+                if (j < nv) cand[j] = keep[u];
+            }
+            k = nv;
+            if (tid == 0) sh.nearest = 0;  // the first vertex
+            compact = false;
+            __syncthreads();
+            continue;
+        }
+        const int nt = star.n[0] + star.n[1];
+        const bool open_l = star.open[0], open_r = star.open[1];
         const float R2 = (float)(R * R);
         bool first = true;  // the open ends go with the first group of circles
         int found = 0;
         for (int t0 = 0; t0 < nt || first;) {
-            // the next circles that the disc does not certify
+            // the next circles that neither the disc nor a scan certifies
             __syncthreads();
             if (warp == 0) {
                 int nb = 0;
                 for (; t0 < nt && nb == 0; t0 += 32) {
+                    const int t = t0 + lane, dir = t < star.n[0] ? 0 : 1, i = dir ? t - star.n[0] : t;
+                    bool bad = false;
                     DtPt u{0, 0, 0}, v{0, 0, 0};
-                    if (t0 + lane < nt) dt_star_tri(sh, t0 + lane, u, v);
-                    const bool bad = t0 + lane < nt && !dt_small_circle(u.x, u.y, v.x, v.y, R2);
+                    if (t < nt && star.state[dir][i] != kDtEmpty) {
+                        float4 uf, vf;
+                        dt_star_tri(star, cand, t, uf, vf);
+                        u = dt_point(uf);
+                        v = dt_point(vf);
+                        bad = !dt_small_circle(u, v, R2);
+                    }
                     const unsigned b = __ballot_sync(0xFFFFFFFFu, bad);
-                    if (bad) sh.bad[__popc(b & ((1u << lane) - 1u))] = dt_circle(u, v);
+                    if (bad) {
+                        const int to = __popc(b & ((1u << lane) - 1u));
+                        sh.bad[to] = dt_circle(u, v);
+                        sh.region[to] = dt_region(sh.bad[to]);
+                        sh.tri[to] = (uint16_t)(dir << 15 | i);
+                    }
                     nb = __popc(b);
+                }
+                if (lane < 2 && first && (lane ? open_r : open_l)) {  // beyond the open edge
+                    const float4 e = cand[star.v[lane][star.n[lane]]];
+                    const float ex = lane ? -e.x : e.x, ey = lane ? -e.y : e.y, l = rsqrtf(ex * ex + ey * ey);
+                    sh.region[kDtBadCap + lane] = make_float3(-ey * l, ex * l, -1.0f);
                 }
                 if (lane == 0) {
                     sh.nbad = nb;
                     sh.next = t0;
                     sh.total = 0;
+                    sh.found = 0;
+                    sh.row0 = a.gh;
+                    sh.row1 = -1;
+                }
+            } else {
+                for (int cy = tid - 32; cy < a.gh; cy += THREADS - 32) {
+                    r_start[cy] = a.gw;
+                    r_len[cy] = -1;
                 }
             }
             const bool ends = first && (open_l || open_r);
-            first = false;
             __syncthreads();
             const int nbad = sh.nbad;
             t0 = sh.next;
+            // a whole star in one group: a point inside any circle is inside
+            // that of its own sector
+            const bool sector = !fan && first && t0 >= nt;
+            first = false;
             if (nbad == 0 && !ends) continue;
-            const DtListSrc v0{sh.vert[0], 0}, v1{sh.vert[1], 0};
-            const DtPt el = v0.get(sh.nv[0]), er = v1.get(sh.nv[1]);
-            int tot = 0;
-            for (int cy = tid; cy < a.gh; cy += kDtBlockThreads) {
-                int lo = a.gw, hi = -1, c0, c1;
-                for (int b = 0; b < nbad; ++b) {
-                    const DtCircle &c = sh.bad[b];
-                    const float U = (float)c.U, V = (float)c.V, W2 = 2.0f * (float)c.W;
-                    const float ux = U / W2, uy = V / W2, r = sqrtf(ux * ux + uy * uy);
-                    bool any;
-                    if (r <= 1e6f) {
-                        any = dt_row_range(cy, (float)p.x + ux, (float)p.y + uy, r * 1.0001f + 4.0f, 0.0f, 0.0f, a.gw,
-                                           c0, c1);
-                    } else {  // the half-plane beyond the circle's tangent at p holds the disc
-                        const float l = rsqrtf(U * U + V * V);
-                        any = dt_row_range(cy, (float)p.x, (float)p.y, -1.0f, U * l, V * l, a.gw, c0, c1);
-                    }
-                    if (any) {
-                        lo = min(lo, c0);
-                        hi = max(hi, c1);
+            const DtPt el = dt_point(cand[star.v[0][star.n[0]]]), er = dt_point(cand[star.v[1][star.n[1]]]);
+            // cell ranges: each warp takes regions, its lanes their cell rows
+            for (int b = warp; b < kDtBadCap + 2; b += (THREADS / 32)) {
+                if (b < kDtBadCap ? b >= nbad : !(ends && (b == kDtBadCap ? open_l : open_r))) continue;
+                const float3 g = sh.region[b];
+                int y0 = 0, y1 = a.gh - 1;
+                if (g.z >= 0.0f) {
+                    y0 = (int)fmaxf(0.0f, ((float)p.y + g.y - g.z - 2.0f) * (1.0f / kDtCell));
+                    y1 = (int)fminf((float)y1, ((float)p.y + g.y + g.z + 2.0f) * (1.0f / kDtCell));
+                }
+                for (int cy = y0 + lane; cy <= y1; cy += 32) {
+                    int c0, c1;
+                    if (dt_row_range(cy, (float)p.x, (float)p.y, g, a.gw, c0, c1)) {
+                        atomicMin(&r_start[cy], c0);
+                        atomicMax(&r_len[cy], c1);
                     }
                 }
-                if (ends) {
-                    for (int s = 0; s < 2; ++s) {
-                        if (!(s ? open_r : open_l)) continue;
-                        const float ex = (float)(s ? -er.x : el.x), ey = (float)(s ? -er.y : el.y);
-                        const float l = rsqrtf(ex * ex + ey * ey);
-                        if (dt_row_range(cy, (float)p.x, (float)p.y, -1.0f, -ey * l, ex * l, a.gw, c0, c1)) {
-                            lo = min(lo, c0);
-                            hi = max(hi, c1);
-                        }
-                    }
-                }
+            }
+            __syncthreads();
+            int tot = 0, row0 = a.gh, row1 = -1;
+            for (int cy = tid; cy < a.gh; cy += THREADS) {
+                const int lo = r_start[cy], hi = r_len[cy];
                 const int *row = S.cell_start + cy * a.gw;
-                const int s0 = lo <= hi ? row[lo] : 0, e0 = lo <= hi ? row[hi + 1] : 0;
+                const int s0 = lo <= hi ? row[lo] : 0, len = lo <= hi ? row[hi + 1] - s0 : 0;
                 r_start[cy] = s0;
-                r_len[cy] = e0 - s0;
-                tot += e0 - s0;
+                r_len[cy] = len;
+                tot += len;
+                if (len) {
+                    row0 = min(row0, cy);
+                    row1 = cy;
+                }
             }
             tot = __reduce_add_sync(0xFFFFFFFFu, tot);
-            if (lane == 0 && tot) atomicAdd(&sh.total, tot);
+            row0 = __reduce_min_sync(0xFFFFFFFFu, row0);
+            row1 = __reduce_max_sync(0xFFFFFFFFu, row1);
+            if (lane == 0 && tot) {
+                atomicAdd(&sh.total, tot);
+                atomicMin(&sh.row0, row0);
+                atomicMax(&sh.row1, row1);
+            }
             __syncthreads();
-            int stride = sh.total > kDtSampleMin && round < 4 ? sh.total / (kDtSampleMin / 4) : 1;
+            row0 = sh.row0;
+            row1 = sh.row1;
+            int stride = sh.total > kDtSampleMin && round < 4 ? sh.total / (kDtSampleMin / 2) : 1;
             for (;;) {
-                for (int cy = warp; cy < a.gh; cy += kDtBlockThreads / 32) {
-                    const int s0 = r_start[cy], len = r_len[cy];
-                    for (int j0 = stride > 1 ? (cy * 5) % stride : 0; j0 < len; j0 += 32 * stride) {
-                        const int j = j0 + lane * stride;
+                // each warp takes every fourth row, 32 of them as one index space
+                for (int cy0 = row0 + warp; cy0 <= row1; cy0 += 32 * (THREADS / 32)) {
+                    const int cy = cy0 + lane * (THREADS / 32);
+                    const int len = cy <= row1 ? r_len[cy] : 0;
+                    int incl = len;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+                        if (lane >= o) incl += y;
+                    }
+                    const int all = __shfl_sync(0xFFFFFFFFu, incl, 31), excl = incl - len;
+                    const int off = (cy <= row1 ? r_start[cy] : 0) - excl;
+                    auto load = [&](int j) {
+                        int r = 0;
+#pragma unroll
+                        for (int h = 16; h > 0; h >>= 1)
+                            if (j >= __shfl_sync(0xFFFFFFFFu, excl, r + h)) r += h;
+                        const int src = __shfl_sync(0xFFFFFFFFu, off, r) + j;
+                        return j < all ? S.pts[src] : make_int4(0, 0, 0, 0);
+                    };
+                    int4 next = load(lane * stride);
+                    for (int j0 = 0; j0 < all; j0 += 32 * stride) {
+                        const int4 t = next;
+                        if (j0 + 32 * stride < all) next = load(j0 + (32 + lane) * stride);
+                        const DtPt q{t.x - p.x, t.y - p.y, t.z};
+                        const float qx = (float)q.x, qy = (float)q.y;
+                        // the circles that need the exact test: the one in
+                        // whose sector the point lies, or all whose padded
+                        // region holds it
+                        unsigned need = 0;
+                        for (int b = 0; b < nbad; ++b) {
+                            bool in;
+                            if (!sector) {
+                                const float3 g = sh.region[b];
+                                const float dx = qx - g.x, dy = qy - g.y;
+                                in = !(g.z >= 0.0f && dx * dx + dy * dy > g.z * g.z);
+                            } else {
+                                const DtPt u = sh.bad[b].a, v = sh.bad[b].b;
+                                in = u.x * q.y - u.y * q.x >= 0 && v.x * q.y - v.y * q.x <= 0;
+                            }
+                            need |= (unsigned)in << b;
+                        }
+                        const bool some = t.w && t.z != p.z;
                         bool hit = false;
-                        DtPt q{0, 0, 0};
-                        if (j < len) {
-                            const int4 t = S.pts[s0 + j];
-                            if (t.w && t.z != p.z) {
-                                q = DtPt{t.x - p.x, t.y - p.y, t.z};
-                                for (int b = 0; b < nbad && !hit; ++b) hit = dt_violates(sh.bad[b], p.z, q);
-                                if (ends) {
-                                    hit = hit || (open_l && el.x * q.y - el.y * q.x > 0);
-                                    hit = hit || (open_r && er.x * q.y - er.y * q.x < 0);
-                                }
+                        if (ends && some)
+                            hit = (open_l && el.x * q.y - el.y * q.x > 0) || (open_r && er.x * q.y - er.y * q.x < 0);
+                        if (!some) need = 0;
+                        if (hit && sector) need = nbad < 32 ? (1u << nbad) - 1u : 0xFFFFFFFFu;
+                        for (bool all = hit || !sector; need; need &= need - 1) {
+                            const int b = __ffs(need) - 1;
+                            if (!dt_violates(sh.bad[b], p.z, q)) continue;
+                            hit = true;
+                            star.state[sh.tri[b] >> 15][sh.tri[b] & 0x7FFF] = kDtHit;
+                            if (!all) {  // now every circle that holds it
+                                all = true;
+                                for (int c = 0; c < nbad; ++c)
+                                    if (c != b && dt_violates(sh.bad[c], p.z, q))
+                                        star.state[sh.tri[c] >> 15][sh.tri[c] & 0x7FFF] = kDtHit;
+                                break;
                             }
                         }
                         const unsigned m = __ballot_sync(0xFFFFFFFFu, hit);
@@ -1205,11 +1535,16 @@ __device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, 
                         int base = 0;
                         if (lane == 0) base = atomicAdd(&sh.found, __popc(m));
                         const int pos = k + __shfl_sync(0xFFFFFFFFu, base, 0) + __popc(m & ((1u << lane) - 1u));
-                        if (hit && pos < kDtCacheCap) cand[pos] = dt_pack(q.x, q.y, q.z);
+                        if (hit && pos < kDtCacheCap) cand[pos] = dt_cand(q.x, q.y, q.z);
+                        if (hit && max(abs(q.x), abs(q.y)) >= kDtNearMax) sh.far = 1;
                     }
                 }
                 __syncthreads();
                 found = sh.found;
+                if (stride == 1 && tid < nbad) {
+                    uint8_t &st = star.state[sh.tri[tid] >> 15][sh.tri[tid] & 0x7FFF];
+                    if (st != kDtHit) st = kDtEmpty;
+                }
                 __syncthreads();
                 if (stride == 1 || found > 0) break;
                 stride = 1;
@@ -1219,28 +1554,16 @@ __device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, 
         if (found == 0) break;
         if (k + found <= kDtCacheCap) {
             k += found;
-            continue;
+            again = true;
+            cur ^= 1;
+        } else {
+            k = kDtCacheCap;
+            fan = again = false;
+            compact = true;
+            R = 0;
         }
-        // full: wrap the whole star over the cache and keep only its vertices
-        // (no disc certifies its circles any more)
-        fan = false;
-        R = 0;
-        if (tid == 0) {
-            sh.over = 0;
-            sh.closed = 0;
-        }
-        dt_block_wrap(cand, kDtCacheCap, p.z, false, nn, sh);
-        if (sh.over) {
-            dt_block_star_all(S, p, n, nn, sh);
-            return;
-        }
-        const int na = sh.nv[0] + (sh.closed ? 0 : 1);
-        for (int j = tid; j < na; j += kDtBlockThreads) cand[j] = sh.vert[0][j];
-        for (int j = tid; j < sh.nv[1]; j += kDtBlockThreads) cand[na + j] = sh.vert[1][j + 1];
-        k = na + sh.nv[1];
-        __syncthreads();
     }
-    if (warp == 0) dt_block_write(S, p.z, fan, nn.z, sh);
+    if (warp == 0) dt_block_write(S, p.z, fan, cand, sh.star[cur], sh.nearest);
     __syncthreads();
 }
 
@@ -1248,28 +1571,31 @@ __device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, 
 // both sides' queues from one atomic counter, the two queues interleaved so
 // that both sides' stars start in the first wave (the pass lasts as long as
 // its longest star, so none should wait behind the other side's).  The
-// counter is side 0's npending2, which dt_init_kernel zeroes and the one-pair
+// counter is side 0's nwork, which dt_init_kernel zeroes and the one-pair
 // passes leave unused.
-__global__ void __launch_bounds__(kDtBlockThreads, kDtBlocksPerSM) dt_pass_block_kernel(DtArgs a, int nsides) {
-    extern __shared__ int2 s_cand[];  // [kDtCacheCap], then the region rows
+__global__ void __launch_bounds__(kDtBlockThreads, kDtBlocksPerSM) dt_pass_block_kernel(const __grid_constant__ DtArgs a,
+                                                                                             int nsides) {
+    extern __shared__ float4 s_cand[];  // [kDtCacheCap], then the region rows
     __shared__ DtStarShared sh;
     __shared__ int s_item;
     int *r_start = reinterpret_cast<int *>(s_cand + kDtCacheCap);
     const int n = min(max(*a.count, 0), a.cap);
     const int nq0 = *a.s[0].npending, nq1 = nsides > 1 ? *a.s[1].npending : 0;
     const int m = min(nq0, nq1), total = nq0 + nq1;
-    int32_t *counter = a.s[0].npending2;
+    int32_t *counter = a.s[0].nwork;
+    int next = threadIdx.x == 0 ? atomicAdd(counter, 1) : 0;  // fetched while the item before is worked on
     for (;;) {
-        if (threadIdx.x == 0) s_item = atomicAdd(counter, 1);
+        if (threadIdx.x == 0) s_item = next;
         __syncthreads();
         const int item = s_item;
         __syncthreads();
         if (item >= total) break;
+        if (threadIdx.x == 0) next = atomicAdd(counter, 1);
         const bool two = item < 2 * m;
         const int side = two ? (item & 1) : (nq0 > nq1 ? 0 : 1);
         const int idx = two ? (item >> 1) : item - m;
         const DtSide &S = a.s[side];
-        dt_block_item(a, S, S.pending[idx], n, !(*S.err & 8), s_cand, r_start, r_start + a.gh, sh);
+        dt_block_item<kDtBlockThreads>(a, S, S.pending[idx], n, !(*S.err & 8), s_cand, r_start, r_start + a.gh, sh);
     }
 }
 
@@ -1277,11 +1603,12 @@ __global__ void __launch_bounds__(kDtBlockThreads, kDtBlocksPerSM) dt_pass_block
 // concatenated in launch order and the CTAs take their entries one at a
 // time from one atomic counter (zeroed by dt_init_kernel_b), so the long
 // stars of one pair overlap the work of all the others.  second: the middle
-// pass's queues; else the warp pass's (a batch of one pair, which skips the
+// pass's queues, else the warp pass's (a batch of one pair, which skips the
 // middle pass).
-__global__ void __launch_bounds__(kDtBlockThreads, kDtBlocksPerSM)
+template <int THREADS, int PER_SM>
+__global__ void __launch_bounds__(THREADS, PER_SM)
     dt_pass_block_kernel_b(const DtArgs *__restrict__ tab, VMap vm, int nsides, int32_t *counter, int second) {
-    extern __shared__ int2 s_cand[];
+    extern __shared__ float4 s_cand[];
     __shared__ DtStarShared sh;
     __shared__ int s_pre[2 * kMaxBatch + 1];
     __shared__ int s_item;
@@ -1318,12 +1645,14 @@ __global__ void __launch_bounds__(kDtBlockThreads, kDtBlocksPerSM)
     __syncthreads();
     const int total = s_pre[nq_all];
     int *r_start = reinterpret_cast<int *>(s_cand + kDtCacheCap);
+    int next = tid == 0 ? atomicAdd(counter, 1) : 0;  // fetched while the item before is worked on
     for (;;) {
-        if (tid == 0) s_item = atomicAdd(counter, 1);
+        if (tid == 0) s_item = next;
         __syncthreads();
         const int item = s_item;
         __syncthreads();
         if (item >= total) break;
+        if (tid == 0) next = atomicAdd(counter, 1);
         // last queue whose start is <= item
         int lo = 0, hi = nq_all - 1;
         while (lo < hi) {
@@ -1336,8 +1665,8 @@ __global__ void __launch_bounds__(kDtBlockThreads, kDtBlocksPerSM)
         const DtArgs &a = slot_entry(tab, vm.stride, vm.slot[lo / nsides]);
         const DtSide &S = a.s[lo % nsides];
         const int n = min(max(*a.count, 0), a.cap);
-        const int i = (second ? S.pending2 : S.pending)[item - s_pre[lo]];
-        dt_block_item(a, S, i, n, !(*S.err & 8), s_cand, r_start, r_start + a.gh, sh);
+        const int at = (second ? S.pending2 : S.pending)[item - s_pre[lo]];
+        dt_block_item<THREADS>(a, S, at, n, !(*S.err & 8), s_cand, r_start, r_start + a.gh, sh);
     }
 }
 
@@ -1429,7 +1758,7 @@ __global__ void dt_emit_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
 // Host side
 // -------------------------------------------------------------------------
 
-constexpr int kDtCounters = 4;  // err, npending, npending2, npool
+constexpr int kDtCounters = 5;  // err, npending, npending2, nwork, npool
 
 static void dt_geom(int w, int h, int &gw, int &gh) {
     gw = (w + kDtCell - 1) / kDtCell;
@@ -1477,7 +1806,8 @@ static DtSide dt_carve(void *ws, int cap, int w, int h) {
     s.err = counters;
     s.npending = counters + 1;
     s.npending2 = counters + 2;
-    s.npool = counters + 3;
+    s.nwork = counters + 3;
+    s.npool = counters + 4;
     return s;
 }
 
@@ -1511,11 +1841,12 @@ elas_status launch_triangulate_device(const int16_t *list, const int32_t *count,
     dt_cell_scan_kernel<<<dim3(1, nsides), 1024, 0, st>>>(a);
     dt_scatter_kernel<<<dim3(pblocks, nsides), tb, 0, st>>>(a);
     dt_dedup_kernel<<<dim3(pblocks, nsides), tb, 0, st>>>(a);
-    // one pair: the CTA pass takes the warp pass's queue directly (its time is
-    // that of its longest star, which a middle pass would not shorten)
     dt_pass1_kernel<<<dim3(max(1, min((cap + kDtWarps - 1) / kDtWarps, sm_count() * 16)), nsides), kDtWarps * 32, 0,
                       st>>>(a);
-    const int smem = kDtCacheCap * (int)sizeof(int2) + 2 * a.gh * (int)sizeof(int);
+
+    // no middle pass: it would add its longest star's time to the CTA pass's
+    // (640x480 115 against 78 us)
+    const int smem = kDtCacheCap * (int)sizeof(float4) + 2 * a.gh * (int)sizeof(int);
     if (cudaFuncSetAttribute(dt_pass_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
         return launch_status("dt_pass_block_kernel shared memory attribute");
     dt_pass_block_kernel<<<sm_count() * kDtBlocksPerSM, kDtBlockThreads, smem, st>>>(a, nsides);
@@ -1576,13 +1907,15 @@ elas_status launch_triangulate_b(const DtArgs *tab, const DtArgs *host, const VM
         vmap_add(m_pts, slot, dim3(dt_point_blocks(a.cap, 256, pairs.n), nsides));
         vmap_add(m_scan, slot, dim3(1, nsides));
         vmap_add(m_grp, slot, dim3(dt_point_blocks(a.cap, kDtWarps, pairs.n), nsides));
-        // the middle pass gets a few percent of the points (grid-stride over
-        // the queue)
-        vmap_add(m_grp2, slot, dim3(max(1, min(sm_count(), a.cap / 128)), nsides));
+        // the middle pass gets a few percent of the points
+        vmap_add(m_grp2, slot, dim3(max(1, min(sm_count() * 4, a.cap / (16 * kDtWarpsM))), nsides));
         max_gh = max(max_gh, a.gh);
     }
-    const int smem = kDtCacheCap * (int)sizeof(int2) + 2 * max_gh * (int)sizeof(int);
-    if (cudaFuncSetAttribute(dt_pass_block_kernel_b, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+    const int smem = kDtCacheCap * (int)sizeof(float4) + 2 * max_gh * (int)sizeof(int);
+    auto *one_kernel = dt_pass_block_kernel_b<kDtBlockThreads, kDtBlocksPerSM>;
+    auto *many_kernel = dt_pass_block_kernel_b<kDtBlockThreadsB, kDtBlocksPerSMB>;
+    if (cudaFuncSetAttribute(one_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+        cudaFuncSetAttribute(many_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
         return launch_status("dt_pass_block_kernel_b shared memory attribute");
     dt_init_kernel_b<<<vmap_total(m_init), 256, 0, st>>>(tab, m_init, counter);
     dt_points_kernel_b<<<vmap_total(m_pts), 256, 0, st>>>(tab, m_pts);
@@ -1590,10 +1923,12 @@ elas_status launch_triangulate_b(const DtArgs *tab, const DtArgs *host, const VM
     dt_scatter_kernel_b<<<vmap_total(m_pts), 256, 0, st>>>(tab, m_pts);
     dt_dedup_kernel_b<<<vmap_total(m_pts), 256, 0, st>>>(tab, m_pts);
     dt_pass1_kernel_b<<<vmap_total(m_grp), kDtWarps * 32, 0, st>>>(tab, m_grp);
-    const int middle = pairs.n > 1;
-    if (middle) dt_pass1m_kernel_b<<<vmap_total(m_grp2), kDtWarpsM * 32, 0, st>>>(tab, m_grp2);
-    dt_pass_block_kernel_b<<<sm_count() * kDtBlocksPerSM, kDtBlockThreads, smem, st>>>(tab, pairs, nsides, counter,
-                                                                                       middle);
+    if (pairs.n == 1) {
+        one_kernel<<<sm_count() * kDtBlocksPerSM, kDtBlockThreads, smem, st>>>(tab, pairs, nsides, counter, 0);
+    } else {
+        dt_pass2_kernel_b<<<vmap_total(m_grp2), kDtWarpsM * 32, 0, st>>>(tab, m_grp2);
+        many_kernel<<<sm_count() * kDtBlocksPerSMB, kDtBlockThreadsB, smem, st>>>(tab, pairs, nsides, counter, 1);
+    }
     dt_tri_scan_kernel_b<<<vmap_total(m_scan), 1024, 0, st>>>(tab, m_scan);
     dt_emit_kernel_b<<<vmap_total(m_pts), 256, 0, st>>>(tab, m_pts);
     return launch_status("batched triangulation kernels");

@@ -112,8 +112,9 @@ struct DtSide {
     int32_t *npool;            // pool entries taken
     int32_t *pending;          // [cap] points queued by the warp pass
     int32_t *npending;         // queue length
-    int32_t *pending2;         // [cap] points queued by the middle pass (batches)
-    int32_t *npending2;        // its length (one pair: side 0's is the CTA pass's work counter)
+    int32_t *pending2;         // [cap] points queued by the middle pass
+    int32_t *npending2;        // its length
+    int32_t *nwork;            // one pair: side 0's is the CTA pass's work counter
     int32_t *rowmin, *rowmax;  // [h] extreme x of the points of each image row
     int32_t *tri;              // output [cap_tri][3]
     int32_t *ntri;             // output count
