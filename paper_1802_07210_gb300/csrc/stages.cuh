@@ -118,7 +118,7 @@ struct DtSide {
     int32_t *rowmin, *rowmax;  // [h] extreme x of the points of each image row
     int32_t *tri;              // output [cap_tri][3]
     int32_t *ntri;             // output count
-    int32_t *err;              // bit 1: triangle capacity, bit 3: the list is not in raster order
+    int32_t *err;              // bit 3: the list is not in raster order
 };
 
 struct DtArgs {
