@@ -302,16 +302,13 @@ constexpr int kKeyMul = 2047;
 // GLIST: the cell's candidate list was expanded into global memory by the
 // prior's list kernel (the CTA only waits for the prior table, at its
 // start); else warp 0 expands the mask into shared memory first.
-// PF: the reference descriptor and prior of a thread's next pixel are
-// loaded while the current one is matched (batches, where a thread walks
-// many pixels; one pair has one pixel per thread).
 // WARPC: the cell belongs to one warp of the CTA (the persistent prior and
 // argmin kernel runs kFusedCellWarps cells per CTA): the warp keeps its own
 // list and prior table in shared memory and synchronises alone.
 constexpr int kFusedThreads = 256;
 constexpr int kFusedCellWarps = kFusedThreads / 32;
 
-template <int TPP, bool CENSUS, bool GLIST, bool PF, bool WARPC = false>
+template <int TPP, bool CENSUS, bool GLIST, bool WARPC = false>
 __device__ __forceinline__ void cell_body(const CellArgs &a, const VB &vb) {
     constexpr int NG = WARPC ? kFusedCellWarps : 1;  // cell groups of the CTA
     __shared__ __align__(16) uint16_t s_list_g[NG][GLIST ? 1 : kMaxDisp + 1 + kListPad];
@@ -360,36 +357,24 @@ __device__ __forceinline__ void cell_body(const CellArgs &a, const VB &vb) {
     const int sdy = ppb / cw, sdx = ppb - sdy * cw;
     int px = (tid / TPP) % cw, py = (tid / TPP) / cw;
     auto inner = [&](int qx, int qy) { return qx >= 2 && qx <= W - 3 && qy >= 2 && qy <= H - 3; };
-    uint4 r_nx = make_uint4(0u, 0u, 0u, 0u);
-    int dp_nx = -1;
-    if (PF && tid / TPP < npx && inner(x0 + px, y0 + py)) {
-        const size_t i0 = (size_t)(y0 + py) * W + x0 + px;
-        r_nx = __ldg(ref + i0);
-        if (!full) dp_nx = (int)__ldcg(S.dplane + i0);
-    }
     for (int pb = 0; pb < npx; pb += ppb) {
         const int p = pb + tid / TPP;
         const bool live = p < npx;
         const int x = x0 + px, y = y0 + py;
         const size_t row = (size_t)y * W;
         const bool in = live && inner(x, y);
-        uint4 r = r_nx;
-        int dp = full ? -1 : dp_nx;
-        if (!PF && in) {
+        uint4 r = make_uint4(0u, 0u, 0u, 0u);
+        int dp = -1;
+        if (in) {
             r = __ldg(ref + row + x);
             if (!full) dp = (int)__ldcg(S.dplane + row + x);
         }
-        // the next pixel's position and loads
+        // the next pixel's position
         px += sdx;
         py += sdy;
         if (px >= cw) {
             px -= cw;
             ++py;
-        }
-        if (PF && p + ppb < npx && inner(x0 + px, y0 + py)) {
-            const size_t i1 = (size_t)(y0 + py) * W + x0 + px;
-            r_nx = __ldg(ref + i1);
-            if (!full) dp_nx = (int)__ldcg(S.dplane + i1);
         }
         int best = 0x7FFFFFFF;
         // the list length, read after the pixel's own loads so that they are
@@ -425,7 +410,7 @@ __device__ __forceinline__ void cell_body(const CellArgs &a, const VB &vb) {
                     }
                     cnt = lo;
                 }
-#pragma unroll 8
+#pragma unroll 4
                 for (int k = sub; k < cnt; k += TPP) {
                     const int d = list_at(k);
                     if (kBisect || d <= dlim)
@@ -447,14 +432,18 @@ __device__ __forceinline__ void cell_body(const CellArgs &a, const VB &vb) {
 }
 
 template <bool CENSUS, bool GLIST> __global__ void __launch_bounds__(1024, 2) cell_kernel(CellArgs a) {
-    cell_body<1, CENSUS, GLIST, false>(a, vb_single());
+    cell_body<1, CENSUS, GLIST>(a, vb_single());
 }
 
-// Batched launches: one launch per cost kind among the pairs.
+// Batched launches: one launch per cost kind among the pairs.  Bound by the
+// gathers' latency, so the SM is filled: 32 registers a thread (2,048 threads
+// an SM), four candidates in flight each.  Loading a thread's next pixel ahead
+// with eight in flight took 62 registers and half the warps: 64 x 1242x375
+// 1.36 ms, now 1.02.
 template <int TPP, bool CENSUS>
-__global__ void __launch_bounds__(1024) cell_kernel_b(const CellArgs *__restrict__ tab, VMap vm) {
+__global__ void __launch_bounds__(1024, 2) cell_kernel_b(const CellArgs *__restrict__ tab, VMap vm) {
     const VB vb = vb_batch(vm);
-    cell_body<TPP, CENSUS, false, true>(slot_entry(tab, vm.stride, vb.slot), vb);
+    cell_body<TPP, CENSUS, false>(slot_entry(tab, vm.stride, vb.slot), vb);
 }
 
 template <bool CENSUS>
@@ -502,7 +491,7 @@ __device__ __forceinline__ void fused_cells(const DenseFusedArgs &f, const VMap 
     w.gx = a.gw;
     w.gy = gh;
     w.gz = 2;
-    cell_body<TPP, CENSUS, false, true, true>(a, w);
+    cell_body<TPP, CENSUS, false, true>(a, w);
 }
 
 template <int TPP> __global__ void __launch_bounds__(kFusedThreads, 4) dense_fused_kernel_b(DenseFusedArgs f) {
