@@ -13,7 +13,7 @@
 // raster_list_kernel   one thread per triangle: the chunks after the first
 //                      of a box go to the mesh's list of extra units (one
 //                      atomicAdd per triangle of more than one chunk);
-// raster_draw_kernel   one warp per unit (grid-stride; unit t < ntri is
+// raster_draw_kernel   half a warp per unit (grid-stride; unit t < ntri is
 //                      the first chunk of triangle t, the rest come from the
 //                      list), its lanes on 32 pixels of the box at a time: a
 //                      pixel owned by the triangle (at most one owner: the
@@ -224,17 +224,28 @@ __global__ void __launch_bounds__(256) raster_list_kernel_b(const RasterArgs *__
     raster_list_body(slot_entry(tab, vm.stride, vb.slot), vb);
 }
 
-// Pixels [p0, p1) of the box of record r (row-major in the box), 32 at a
-// time across the warp.
+// Lanes per unit in the draw kernel.  Boxes hold about 65 pixels, so a warp
+// per unit spent most of its instructions on the unit's constants; two units
+// a warp share them, and the edge functions step along with the pixel (64 x
+// 1242x375 prior stage 0.617 -> 0.531 ms, 1920x1080 63 -> 55 us; eight lanes
+// are as good in batches but slower at one 640x480 pair, 24 against 22 us).
+constexpr int kDrawLanes = 16;
+
+// Pixels [p0, p1) of the box of record r (row-major in the box), kDrawLanes
+// at a time across the unit's lanes.
 __device__ __forceinline__ void raster_span(const RasterArgs &a, const RasterSide &S, const TriRec &r, const int4 &b,
                                             int p0, int p1, int lane) {
     const int bw = b.y - b.x + 1;
     int p = p0 + lane;
     int y = b.z + p / bw, x = b.x + (p - (p / bw) * bw);
-    const int dy = 32 / bw, dx = 32 - dy * bw;
-    for (; p < p1; p += 32) {
-        if (r.A[0] * x + r.B[0] * y + r.C[0] > 0 && r.A[1] * x + r.B[1] * y + r.C[1] > 0 &&
-            r.A[2] * x + r.B[2] * y + r.C[2] > 0) {
+    const int dy = kDrawLanes / bw, dx = kDrawLanes - dy * bw;
+    // the edge functions step along with the pixel
+    int e0 = r.A[0] * x + r.B[0] * y + r.C[0], e1 = r.A[1] * x + r.B[1] * y + r.C[1],
+        e2 = r.A[2] * x + r.B[2] * y + r.C[2];
+    const int s0 = r.A[0] * dx + r.B[0] * dy, s1 = r.A[1] * dx + r.B[1] * dy, s2 = r.A[2] * dx + r.B[2] * dy;
+    const int w0 = r.B[0] - r.A[0] * bw, w1 = r.B[1] - r.A[1] * bw, w2 = r.B[2] - r.A[2] * bw;
+    for (; p < p1; p += kDrawLanes) {
+        if (min(e0, min(e1, e2)) > 0) {
             const float t1 = __fmul_rn(r.fa, __int2float_rn(x));
             const float t2 = __fmul_rn(r.fb, __int2float_rn(y));
             const float mu = __fadd_rn(__fadd_rn(t1, t2), r.fc);
@@ -243,22 +254,28 @@ __device__ __forceinline__ void raster_span(const RasterArgs &a, const RasterSid
         }
         x += dx;
         y += dy;
+        e0 += s0;
+        e1 += s1;
+        e2 += s2;
         if (x > b.y) {
             x -= bw;
             ++y;
+            e0 += w0;
+            e1 += w1;
+            e2 += w2;
         }
     }
 }
 
 __device__ __forceinline__ void raster_draw_body(const RasterArgs &a, const VB &vb) {
     const RasterSide &S = a.s[vb.y];
-    const int lane = threadIdx.x & 31;
-    const int wid = vb.x * (blockDim.x >> 5) + (threadIdx.x >> 5), nwarps = vb.gx * (blockDim.x >> 5);
+    const int lane = threadIdx.x & (kDrawLanes - 1);
+    const int gid = (vb.x * blockDim.x + threadIdx.x) / kDrawLanes, ngroups = vb.gx * blockDim.x / kDrawLanes;
     const int ntri = side_ntri(S);
     const unsigned long long nextra = *S.nunits;
     const bool whole = nextra > (unsigned long long)a.unit_cap;  // the list is incomplete
     const int nunits = ntri + (whole ? 0 : (int)nextra);
-    for (int u = wid; u < nunits; u += nwarps) {
+    for (int u = gid; u < nunits; u += ngroups) {
         int t = u, c = 0;
         if (u >= ntri) {
             const int2 e = S.ulist[u - ntri];
