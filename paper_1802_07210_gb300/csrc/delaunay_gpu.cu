@@ -1488,9 +1488,10 @@ __device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, 
             row1 = sh.row1;
             int stride = sh.total > kDtSampleMin && round < 4 ? sh.total / (kDtSampleMin / 2) : 1;
             for (;;) {
-                // each warp takes every fourth row, 32 of them as one index space
-                for (int cy0 = row0 + warp; cy0 <= row1; cy0 += 32 * (THREADS / 32)) {
-                    const int cy = cy0 + lane * (THREADS / 32);
+                // 32 rows at a time as one index space, which the warps share
+                // out evenly (a hull point's region is often one long row)
+                for (int cy0 = row0; cy0 <= row1; cy0 += 32) {
+                    const int cy = cy0 + lane;
                     const int len = cy <= row1 ? r_len[cy] : 0;
                     int incl = len;
 #pragma unroll
@@ -1508,10 +1509,10 @@ __device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, 
                         const int src = __shfl_sync(0xFFFFFFFFu, off, r) + j;
                         return j < all ? S.pts[src] : make_int4(0, 0, 0, 0);
                     };
-                    int4 next = load(lane * stride);
-                    for (int j0 = 0; j0 < all; j0 += 32 * stride) {
+                    int4 next = load(tid * stride);
+                    for (int j0 = 32 * warp * stride; j0 < all; j0 += THREADS * stride) {
                         const int4 t = next;
-                        if (j0 + 32 * stride < all) next = load(j0 + (32 + lane) * stride);
+                        if (j0 + THREADS * stride < all) next = load(j0 + (THREADS + lane) * stride);
                         const DtPt q{t.x - p.x, t.y - p.y, t.z};
                         const float qx = (float)q.x, qy = (float)q.y;
                         // the circles that need the exact test: the one in
