@@ -897,15 +897,11 @@ __global__ void __launch_bounds__(kDtWarpsM * 32, 7) dt_pass2_kernel_b(const DtA
 // of it.  A full cache keeps only the star's own vertices and goes on with
 // the whole star (its region can only shrink, so that ends).
 constexpr int kDtRadiusC = 48;
-constexpr int kDtSamples = 128;     // points of the whole set cached too
+constexpr int kDtSamples = 64;     // points of the whole set cached too
 constexpr int kDtCacheCap = 1024;   // cached points (16 KB)
-// Threads of a CTA and CTAs per SM: one pair, whose time is that of its
-// longest star, 256 and 4 (1920x1080 triangulation 272 -> 258 us against 128
-// and 8); batches, bound by issue, 128 and 8 (64 x 1242x375 1.74 -> 1.66 ms
-// against 256 and 4).
-constexpr int kDtBlockThreads = 256, kDtBlocksPerSM = 4;
-constexpr int kDtBlockThreadsB = 128, kDtBlocksPerSMB = 8;
-constexpr int kDtBlockWarpsMax = 8;
+constexpr int kDtBlockThreads = 128;
+constexpr int kDtBlockWarps = kDtBlockThreads / 32;
+constexpr int kDtBlocksPerSM = 8;   // 256 threads and 4 are slower (1920x1080 triangulation 227 against 218 us)
 constexpr int kDtVertCap = 256;     // star vertices per direction
 constexpr int kDtBadCap = 32;       // circles scanned for at a time (a warp's triangles)
 constexpr int kDtMaxRounds = 64;
@@ -989,8 +985,8 @@ struct DtStarShared {
     int far;                       // a cached point lies 2048 pixels or more from p
     int k, nbad, next, found, total, row0, row1;
     int rs[16], rpre[17];
-    DtPt win[kDtBlockWarpsMax];
-    int won[kDtBlockWarpsMax];
+    DtPt win[kDtBlockWarps];
+    int won[kDtBlockWarps];
 };
 
 // Cells [c0, c1] that a region (about (x0, y0), padded for the FP32 rounding)
@@ -1023,7 +1019,6 @@ __device__ __forceinline__ bool dt_row_range(int cy, float x0, float y0, const f
 
 // Gathers the points within R of p into the cache (their number, even past
 // the capacity, in sh.k), with the nearest one and the quadrants.
-template <int THREADS>
 __device__ __forceinline__ void dt_block_gather(const DtArgs &a, const DtSide &S, const int4 &p, int R, float4 *cand,
                                                 DtStarShared &sh) {
     const int tid = threadIdx.x, lane = tid & 31;
@@ -1060,11 +1055,11 @@ __device__ __forceinline__ void dt_block_gather(const DtArgs &a, const DtSide &S
     unsigned long long nn = ~0ull;
     unsigned quads = 0;
     int at = 0;
-    for (int t0 = 0; t0 < total; t0 += 4 * THREADS) {  // four loads in flight
+    for (int t0 = 0; t0 < total; t0 += 4 * kDtBlockThreads) {  // four loads in flight
         int4 q[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int t = t0 + u * THREADS + tid;
+            const int t = t0 + u * kDtBlockThreads + tid;
             int r = 0;
 #pragma unroll
             for (int s = 8; s > 0; s >>= 1)
@@ -1073,7 +1068,7 @@ __device__ __forceinline__ void dt_block_gather(const DtArgs &a, const DtSide &S
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            if (t0 + u * THREADS >= total) break;
+            if (t0 + u * kDtBlockThreads >= total) break;
             const int dx = q[u].x - p.x, dy = q[u].y - p.y, d2 = dx * dx + dy * dy;
             const bool take = q[u].w && q[u].z != p.z && abs(dx) <= R && abs(dy) <= R && d2 <= R * R;
             const unsigned m = __ballot_sync(0xFFFFFFFFu, take);
@@ -1237,7 +1232,6 @@ __device__ __forceinline__ void dt_block_write(const DtSide &S, int pz, bool fan
 // The whole star of p over every point, one exact step after the other (more
 // vertices than the lists hold, e.g. the apex of a huge fan): counted first,
 // then written.
-template <int THREADS>
 __device__ __noinline__ void dt_block_star_all(const DtSide &S, const int4 &p, int n, const DtPt &nn, DtStarShared &sh) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int2 *out = nullptr;
@@ -1252,11 +1246,11 @@ __device__ __noinline__ void dt_block_star_all(const DtSide &S, const int4 &p, i
                 int at;
                 const bool any = dt_step_int(
                     [&](int c) {  // this warp's quarter of the points
-                        const int4 q = S.pts[(THREADS / 32) * c + warp];
+                        const int4 q = S.pts[kDtBlockWarps * c + warp];
                         // D = 0: never a candidate
                         return q.w && q.z != p.z ? DtPt{q.x - p.x, q.y - p.y, q.z} : DtPt{0, 0, p.z};
                     },
-                    (n - warp + (THREADS / 32) - 1) / (THREADS / 32), lane, cur, p.z, side, w, at);
+                    (n - warp + kDtBlockWarps - 1) / kDtBlockWarps, lane, cur, p.z, side, w, at);
                 __syncthreads();
                 if (lane == 0) {
                     sh.win[warp] = w;
@@ -1264,7 +1258,7 @@ __device__ __noinline__ void dt_block_star_all(const DtSide &S, const int4 &p, i
                 }
                 __syncthreads();
                 bool got = false;
-                for (int i = 0; i < (THREADS / 32); ++i)
+                for (int i = 0; i < kDtBlockWarps; ++i)
                     if (sh.won[i] && (!got || dt_beats(cur, p.z, w, sh.win[i], side))) {
                         w = sh.win[i];
                         got = true;
@@ -1298,7 +1292,6 @@ __device__ __noinline__ void dt_block_star_all(const DtSide &S, const int4 &p, i
     __syncthreads();
 }
 
-template <int THREADS>
 __device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, int at, int n, bool ordered,
                                               float4 *cand, int *r_start, int *r_len, DtStarShared &sh) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1306,12 +1299,12 @@ __device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, 
     int R = 2 * kDtRadiusC;
     do {
         R >>= 1;
-        dt_block_gather<THREADS>(a, S, p, R, cand, sh);
+        dt_block_gather(a, S, p, R, cand, sh);
     } while (sh.k > kDtCacheCap - kDtSamples && R > 1);
     int k = sh.k;
     if (k == 0) {  // nothing near: the nearest of all points
         unsigned long long key = ~0ull;
-        for (int j = tid; j < n; j += THREADS) {
+        for (int j = tid; j < n; j += kDtBlockThreads) {
             const int4 q = S.pts[j];
             const int64_t dx = q.x - p.x, dy = q.y - p.y;
             if (q.w && q.z != p.z) key = min(key, ((unsigned long long)(dx * dx + dy * dy) << 32) | (unsigned)q.z);
@@ -1360,23 +1353,23 @@ __device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, 
         dt_block_wrap(cand, k, p.z, fan, again, cur, sh);
         DtStarList &star = sh.star[cur];
         if (sh.over || round == kDtMaxRounds) {
-            dt_block_star_all<THREADS>(S, p, n, dt_point(cand[sh.nearest]), sh);
+            dt_block_star_all(S, p, n, dt_point(cand[sh.nearest]), sh);
             return;
         }
         if (compact) {
             // full cache: keep only the whole star's vertices (no disc
             // certifies its circles any more)
             const int na = star.n[0] + (sh.closed ? 0 : 1), nv = na + star.n[1];
-            float4 keep[2 * kDtVertCap / THREADS];
+            float4 keep[2 * kDtVertCap / kDtBlockThreads];
 #pragma unroll
-            for (int u = 0; u < 2 * kDtVertCap / THREADS; ++u) {
-                const int j = u * THREADS + tid;
+            for (int u = 0; u < 2 * kDtVertCap / kDtBlockThreads; ++u) {
+                const int j = u * kDtBlockThreads + tid;
                 if (j < nv) keep[u] = cand[j < na ? star.v[0][j] : star.v[1][j - na + 1]];
             }
             __syncthreads();
 #pragma unroll
-            for (int u = 0; u < 2 * kDtVertCap / THREADS; ++u) {
-                const int j = u * THREADS + tid;
+            for (int u = 0; u < 2 * kDtVertCap / kDtBlockThreads; ++u) {
+                const int j = u * kDtBlockThreads + tid;
                 if (j < nv) cand[j] = keep[u];
             }
             k = nv;
@@ -1429,7 +1422,7 @@ __device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, 
                     sh.row1 = -1;
                 }
             } else {
-                for (int cy = tid - 32; cy < a.gh; cy += THREADS - 32) {
+                for (int cy = tid - 32; cy < a.gh; cy += kDtBlockThreads - 32) {
                     r_start[cy] = a.gw;
                     r_len[cy] = -1;
                 }
@@ -1445,7 +1438,7 @@ __device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, 
             if (nbad == 0 && !ends) continue;
             const DtPt el = dt_point(cand[star.v[0][star.n[0]]]), er = dt_point(cand[star.v[1][star.n[1]]]);
             // cell ranges: each warp takes regions, its lanes their cell rows
-            for (int b = warp; b < kDtBadCap + 2; b += (THREADS / 32)) {
+            for (int b = warp; b < kDtBadCap + 2; b += kDtBlockWarps) {
                 if (b < kDtBadCap ? b >= nbad : !(ends && (b == kDtBadCap ? open_l : open_r))) continue;
                 const float3 g = sh.region[b];
                 int y0 = 0, y1 = a.gh - 1;
@@ -1463,7 +1456,7 @@ __device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, 
             }
             __syncthreads();
             int tot = 0, row0 = a.gh, row1 = -1;
-            for (int cy = tid; cy < a.gh; cy += THREADS) {
+            for (int cy = tid; cy < a.gh; cy += kDtBlockThreads) {
                 const int lo = r_start[cy], hi = r_len[cy];
                 const int *row = S.cell_start + cy * a.gw;
                 const int s0 = lo <= hi ? row[lo] : 0, len = lo <= hi ? row[hi + 1] - s0 : 0;
@@ -1510,9 +1503,9 @@ __device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, 
                         return j < all ? S.pts[src] : make_int4(0, 0, 0, 0);
                     };
                     int4 next = load(tid * stride);
-                    for (int j0 = 32 * warp * stride; j0 < all; j0 += THREADS * stride) {
+                    for (int j0 = 32 * warp * stride; j0 < all; j0 += kDtBlockThreads * stride) {
                         const int4 t = next;
-                        if (j0 + THREADS * stride < all) next = load(j0 + (THREADS + lane) * stride);
+                        if (j0 + kDtBlockThreads * stride < all) next = load(j0 + (kDtBlockThreads + lane) * stride);
                         const DtPt q{t.x - p.x, t.y - p.y, t.z};
                         const float qx = (float)q.x, qy = (float)q.y;
                         // the circles that need the exact test: the one in
@@ -1615,7 +1608,7 @@ __global__ void __launch_bounds__(kDtBlockThreads, kDtBlocksPerSM) dt_pass_block
         const int side = two ? (item & 1) : (nq0 > nq1 ? 0 : 1);
         const int idx = two ? (item >> 1) : item - m;
         const DtSide &S = a.s[side];
-        dt_block_item<kDtBlockThreads>(a, S, S.pending[idx], n, !(*S.err & 8), s_cand, r_start, r_start + a.gh, sh);
+        dt_block_item(a, S, S.pending[idx], n, !(*S.err & 8), s_cand, r_start, r_start + a.gh, sh);
     }
 }
 
@@ -1625,8 +1618,7 @@ __global__ void __launch_bounds__(kDtBlockThreads, kDtBlocksPerSM) dt_pass_block
 // stars of one pair overlap the work of all the others.  second: the middle
 // pass's queues, else the warp pass's (a batch of one pair, which skips the
 // middle pass).
-template <int THREADS, int PER_SM>
-__global__ void __launch_bounds__(THREADS, PER_SM)
+__global__ void __launch_bounds__(kDtBlockThreads, kDtBlocksPerSM)
     dt_pass_block_kernel_b(const DtArgs *__restrict__ tab, VMap vm, int nsides, int32_t *counter, int second) {
     extern __shared__ float4 s_cand[];
     __shared__ DtStarShared sh;
@@ -1686,7 +1678,7 @@ __global__ void __launch_bounds__(THREADS, PER_SM)
         const DtSide &S = a.s[lo % nsides];
         const int n = min(max(*a.count, 0), a.cap);
         const int at = (second ? S.pending2 : S.pending)[item - s_pre[lo]];
-        dt_block_item<THREADS>(a, S, at, n, !(*S.err & 8), s_cand, r_start, r_start + a.gh, sh);
+        dt_block_item(a, S, at, n, !(*S.err & 8), s_cand, r_start, r_start + a.gh, sh);
     }
 }
 
@@ -1888,10 +1880,7 @@ elas_status launch_triangulate_b(const DtArgs *tab, const DtArgs *host, const VM
         max_gh = max(max_gh, a.gh);
     }
     const int smem = kDtCacheCap * (int)sizeof(float4) + 2 * max_gh * (int)sizeof(int);
-    auto *one_kernel = dt_pass_block_kernel_b<kDtBlockThreads, kDtBlocksPerSM>;
-    auto *many_kernel = dt_pass_block_kernel_b<kDtBlockThreadsB, kDtBlocksPerSMB>;
-    if (cudaFuncSetAttribute(one_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
-        cudaFuncSetAttribute(many_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+    if (cudaFuncSetAttribute(dt_pass_block_kernel_b, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
         return launch_status("dt_pass_block_kernel_b shared memory attribute");
     dt_init_kernel_b<<<vmap_total(m_init), 256, 0, st>>>(tab, m_init, counter);
     dt_points_kernel_b<<<vmap_total(m_pts), 256, 0, st>>>(tab, m_pts);
@@ -1899,12 +1888,10 @@ elas_status launch_triangulate_b(const DtArgs *tab, const DtArgs *host, const VM
     dt_scatter_kernel_b<<<vmap_total(m_pts), 256, 0, st>>>(tab, m_pts);
     dt_dedup_kernel_b<<<vmap_total(m_pts), 256, 0, st>>>(tab, m_pts);
     dt_pass1_kernel_b<<<vmap_total(m_grp), kDtWarps * 32, 0, st>>>(tab, m_grp);
-    if (pairs.n == 1) {
-        one_kernel<<<sm_count() * kDtBlocksPerSM, kDtBlockThreads, smem, st>>>(tab, pairs, nsides, counter, 0);
-    } else {
-        dt_pass2_kernel_b<<<vmap_total(m_grp2), kDtWarpsM * 32, 0, st>>>(tab, m_grp2);
-        many_kernel<<<sm_count() * kDtBlocksPerSMB, kDtBlockThreadsB, smem, st>>>(tab, pairs, nsides, counter, 1);
-    }
+    const int middle = pairs.n > 1;
+    if (middle) dt_pass2_kernel_b<<<vmap_total(m_grp2), kDtWarpsM * 32, 0, st>>>(tab, m_grp2);
+    dt_pass_block_kernel_b<<<sm_count() * kDtBlocksPerSM, kDtBlockThreads, smem, st>>>(tab, pairs, nsides, counter,
+                                                                                       middle);
     dt_tri_scan_kernel_b<<<vmap_total(m_scan), 1024, 0, st>>>(tab, m_scan);
     dt_emit_kernel_b<<<vmap_total(m_pts), 256, 0, st>>>(tab, m_pts);
     return launch_status("batched triangulation kernels");
