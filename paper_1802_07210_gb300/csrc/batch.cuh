@@ -98,6 +98,12 @@ inline bool vmap_add(VMap &m, int slot, dim3 g) {
     ++m.n;
     return true;
 }
+// Host: a pair's part of about `blocks` CTAs of a grid-stride kernel, by its
+// share of the work (`work` of `all`), at least one.
+inline int vmap_share(long long work, long long all, int blocks) {
+    const long long n = all > 0 ? (work * blocks + all - 1) / all : 1;
+    return (int)(n > 1 ? n : 1);
+}
 __host__ __device__ inline int vmap_total(const VMap &m) { return m.off[m.n]; }
 
 }  // namespace elas

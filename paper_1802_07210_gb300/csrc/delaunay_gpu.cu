@@ -1856,14 +1856,6 @@ static int dt_point_blocks(int cap, int threads, int npairs) {
     return max(1, min((full + 2) / 3, sm_count() * 8));
 }
 
-// A pair's part of about `blocks` CTAs, by its capacity in points.  The star
-// passes' warps take their points in turn: with a CTA for every eight points
-// of the capacity, finding its pair and loading the argument block cost a
-// warp 140 instructions for little more than one star (a third of the pass).
-static int dt_share(int cap, long long caps, int blocks) {
-    return (int)max(1LL, ((long long)cap * blocks + caps - 1) / max(1LL, caps));
-}
-
 elas_status launch_triangulate_b(const DtArgs *tab, const DtArgs *host, const VMap &pairs, int nsides,
                                  int32_t *counter, cudaStream_t st) {
     if (pairs.n == 0) return ELAS_OK;
@@ -1875,6 +1867,10 @@ elas_status launch_triangulate_b(const DtArgs *tab, const DtArgs *host, const VM
     vmap_clear(m_grp, pairs.stride);
     vmap_clear(m_grp2, pairs.stride);
     int max_gh = 1;
+    // the star passes' warps take their points in turn: with a CTA for every
+    // eight points of the capacity, finding its pair and loading the argument
+    // block cost a warp 140 instructions for little more than one star (a
+    // third of the pass)
     long long caps = 0;
     for (int i = 0; i < pairs.n; ++i) caps += slot_entry(host, pairs.stride, pairs.slot[i]).cap;
     for (int i = 0; i < pairs.n; ++i) {
@@ -1884,8 +1880,8 @@ elas_status launch_triangulate_b(const DtArgs *tab, const DtArgs *host, const VM
         vmap_add(m_init, slot, dim3((nall + 255) / 256, nsides));
         vmap_add(m_pts, slot, dim3(dt_point_blocks(a.cap, 256, pairs.n), nsides));
         vmap_add(m_scan, slot, dim3(1, nsides));
-        vmap_add(m_grp, slot, dim3(dt_share(a.cap, caps, sm_count() * 4 * 8 / nsides), nsides));
-        vmap_add(m_grp2, slot, dim3(dt_share(a.cap, caps, sm_count() * 7 * 4 / nsides), nsides));
+        vmap_add(m_grp, slot, dim3(vmap_share(a.cap, caps, sm_count() * 4 * 8 / nsides), nsides));
+        vmap_add(m_grp2, slot, dim3(vmap_share(a.cap, caps, sm_count() * 7 * 4 / nsides), nsides));
         max_gh = max(max_gh, a.gh);
     }
     const int smem = kDtCacheCap * (int)sizeof(float4) + 2 * max_gh * (int)sizeof(int);

@@ -825,16 +825,28 @@ elas_status launch_dense_b(const DenseTables &t, const DenseStage *host, const V
     vmap_clear(m_draw, pairs.stride);
     vmap_clear(m_cell[0], pairs.stride);
     vmap_clear(m_cell[1], pairs.stride);
-    // per pair: the one-pair grids shared out among the pairs, at least 16 CTAs
-    const int per_pair = max(16, sm_count() * 4 / pairs.n);
+    // the prior's grid-stride kernels: four sets of resident CTAs, shared out
+    // by the pairs' pixels and triangle capacities (as many CTAs for a small
+    // pair as for a large one, and 1.7 sets in all, ended unevenly)
+    long long pixels = 0, tris = 0;
+    for (int i = 0; i < pairs.n; ++i) {
+        const RasterArgs &r = slot_entry(host, pairs.stride, pairs.slot[i]).raster;
+        pixels += (long long)r.w * r.h;
+        tris += raster_max_ntri(r);
+    }
     int threads = 32;
     for (int i = 0; i < pairs.n; ++i) {
         const int slot = pairs.slot[i];
         const DenseStage &d = slot_entry(host, pairs.stride, slot);
         const RasterArgs &r = d.raster;
-        vmap_add(m_setup, slot, dim3(raster_setup_blocks(r, per_pair), r.nsides));
-        vmap_add(m_list, slot, dim3(raster_setup_blocks(r, per_pair), r.nsides));
-        vmap_add(m_draw, slot, dim3(per_pair, r.nsides));
+        const long long px = (long long)r.w * r.h;
+        const int nt = raster_max_ntri(r), all = sm_count() * 8 * 4 / 2;
+        // no more CTAs than two 16-byte stores of the fill a thread, or one for
+        // every 256 triangles
+        const int by_pixels = (int)min((long long)vmap_share(px, pixels, all), px / 4096 + 1);
+        vmap_add(m_setup, slot, dim3(by_pixels, r.nsides));
+        vmap_add(m_list, slot, dim3(by_pixels, r.nsides));
+        vmap_add(m_draw, slot, dim3(min(vmap_share(nt, tris, all), nt / 256 + 1), r.nsides));
         vmap_add(m_cell[d.cell.census ? 1 : 0], slot, cell_grid(d.cell, 2));
         threads = max(threads, cell_threads(d.cell.G, tpp, ppt));
     }
