@@ -155,7 +155,7 @@ template <bool CENSUS> __global__ void __launch_bounds__(512) support_match_kern
     support_match_body<CENSUS>(m, vb_single());
 }
 
-// The same matching with one CTA per lattice row, organised around the
+// The same matching with one CTA per lattice row or part of one, organised around the
 // right-image positions: a right window s meets the candidates u = s + d of
 // every disparity d, so a warp holds the windows of 32 consecutive s in
 // registers and walks the row's candidates once: per candidate each lane
@@ -175,14 +175,15 @@ struct SupRowSmem {
     size_t total;
 };
 
-__host__ __device__ __forceinline__ SupRowSmem sup_row_smem(int wc, int dmin, int dmax) {
+// For nc candidates.
+__host__ __device__ __forceinline__ SupRowSmem sup_row_smem(int nc, int dmin, int dmax) {
     SupRowSmem o;
     o.slots = (dmax - dmin + 1 + 31) / 32 + 1;
     o.desc = 0;
-    o.res = o.desc + (size_t)wc * 4 * sizeof(uint4);
-    o.lohi = o.res + (size_t)wc * o.slots * sizeof(uint2);
-    o.d1 = o.lohi + (size_t)wc * sizeof(int2);
-    o.total = o.d1 + (((size_t)wc * sizeof(int) + 15) & ~(size_t)15);
+    o.res = o.desc + (size_t)nc * 4 * sizeof(uint4);
+    o.lohi = o.res + (size_t)nc * o.slots * sizeof(uint2);
+    o.d1 = o.lohi + (size_t)nc * sizeof(int2);
+    o.total = o.d1 + (((size_t)nc * sizeof(int) + 15) & ~(size_t)15);
     return o;
 }
 
@@ -194,15 +195,17 @@ template <bool CENSUS> __device__ __forceinline__ void support_match_row_body(co
     const int ic = vb.x, v = ic * step;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     extern __shared__ __align__(16) unsigned char s_raw[];
-    const SupRowSmem L = sup_row_smem(wc, dmin, dmax);
+    // the candidates [ka, kb) of the row; in shared memory from 0
+    const int ka = (int)((long long)vb.y * wc / vb.gy), kb = (int)((long long)(vb.y + 1) * wc / vb.gy), nc = kb - ka;
+    const SupRowSmem L = sup_row_smem((wc + vb.gy - 1) / vb.gy, dmin, dmax);
     uint4 *s_desc = reinterpret_cast<uint4 *>(s_raw + L.desc);
     uint2 *s_res = reinterpret_cast<uint2 *>(s_raw + L.res);
     int2 *s_lohi = reinterpret_cast<int2 *>(s_raw + L.lohi);
     int *s_d1 = reinterpret_cast<int *>(s_raw + L.d1);
     const bool row_ok = v >= 4 && v <= a.h - 5;
     // candidates: left windows, texture, disparity range (lo > hi: none)
-    for (int k = tid; k < wc; k += blockDim.x) {
-        const int u = k * step;
+    for (int k = tid; k < nc; k += blockDim.x) {
+        const int u = (ka + k) * step;
         int lo = 1, hi = 0;
         if (row_ok && u >= 4 && u <= w - 5) {
             const Win l = load_win<CENSUS>(dL, w, u, v);
@@ -218,9 +221,11 @@ template <bool CENSUS> __device__ __forceinline__ void support_match_row_body(co
         for (int j = 0; j < L.slots; ++j) s_res[k * L.slots + j] = make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
     }
     __syncthreads();
-    // right windows s = 4 + 32 j + lane, 4 <= s <= w - 5
+    // right windows s = 4 + 32 j + lane, 4 <= s <= w - 5, that some u - d meets
     const int nwin = row_ok ? (w - 8 + 31) / 32 : 0;
-    for (int j = warp; j < nwin; j += nwarps) {
+    const int j0 = max(0, ka * step - dmax - 4) / 32;
+    const int j1 = min(nwin - 1, ((kb - 1) * step - dmin - 4) >> 5);
+    for (int j = j0 + warp; j <= j1; j += nwarps) {
         const int s0 = 4 + 32 * j, sl = s0 + lane;
         const bool s_ok = sl <= w - 5;
         Win r;
@@ -231,14 +236,14 @@ template <bool CENSUS> __device__ __forceinline__ void support_match_row_body(co
             for (int i = 0; i < 4; ++i) r.q[i] = make_uint4(0u, 0u, 0u, 0u);
         }
         // candidates u = s + d with d in [dmin, dmax] for some s of the window
-        const int k0 = max(0, (s0 + dmin + step - 1) / step), k1 = min(wc - 1, (s0 + 31 + dmax) / step);
+        const int k0 = max(0, (s0 + dmin + step - 1) / step - ka), k1 = min(nc - 1, (s0 + 31 + dmax) / step - ka);
         const int slot = j % L.slots;
         // two candidates per step: their chains (window load, cost, the two
         // reductions) are independent, so they overlap
         for (int k = k0; k <= k1; k += 2) {
             const bool has1 = k + 1 <= k1;
             const int2 lh0 = s_lohi[k], lh1 = has1 ? s_lohi[k + 1] : make_int2(1, 0);
-            const int d0 = k * step - sl, d1 = d0 + step;
+            const int d0 = (ka + k) * step - sl, d1 = d0 + step;
             const bool in0 = s_ok && d0 >= lh0.x && d0 <= lh0.y;
             const bool in1 = s_ok && d1 >= lh1.x && d1 <= lh1.y;
             Win lw0, lw1;
@@ -261,7 +266,7 @@ template <bool CENSUS> __device__ __forceinline__ void support_match_row_body(co
     }
     __syncthreads();
     // merge the windows of each candidate; ratio test
-    for (int k = tid; k < wc; k += blockDim.x) {
+    for (int k = tid; k < nc; k += blockDim.x) {
         uint32_t best = 0xFFFFFFFFu;
         int bj = -1;
         for (int j = 0; j < L.slots; ++j) {
@@ -284,21 +289,21 @@ template <bool CENSUS> __device__ __forceinline__ void support_match_row_body(co
                 d1 = (int)(best & 0xFFFFu);
         }
         s_d1[k] = d1;
-        if (d1 < 0) m.raw[ic * wc + k] = (int16_t)-1;
+        if (d1 < 0) m.raw[ic * wc + ka + k] = (int16_t)-1;
     }
     __syncthreads();
     // right-to-left re-match, one warp per candidate that passed
-    for (int k = warp; k < wc; k += nwarps) {
+    for (int k = warp; k < nc; k += nwarps) {
         const int d1 = s_d1[k];
         if (d1 < 0) continue;
-        const int ur = k * step - d1;
+        const int ur = (ka + k) * step - d1;
         const Win r = load_win<CENSUS>(dR, w, ur, v);
         int out = -1;
         if (win_textured<CENSUS>(r, a.support_texture)) {
             const int d2 = warp_best_disparity<CENSUS>(dL, w, r, ur, v, +1, dmin, dmax, a.thr, a.shift_sum, lane);
             if (d2 >= 0 && abs(d1 - d2) <= a.lr_threshold) out = d1;
         }
-        if (lane == 0) m.raw[ic * wc + k] = (int16_t)out;
+        if (lane == 0) m.raw[ic * wc + ka + k] = (int16_t)out;
     }
 }
 
@@ -612,10 +617,25 @@ static elas_status red_smem_attr(const void *fn, size_t smem) {
 }
 
 // Shared memory of the row-organised matcher; wider rows take the
-// per-candidate kernel, and so do launches of fewer lattice rows than two
-// per SM (one CTA per row would leave SMs idle).
+// per-candidate kernel.
 constexpr size_t kSupRowSmemMax = 160 * 1024;
-inline int sup_row_min_rows() { return 2 * sm_count(); }
+
+// The row-organised matcher or the one with a warp per candidate?  The rows
+// need two CTAs per SM to be worth it, by lattice rows or, with Sobel
+// descriptors, by the parts that a row can be split into: with 8 CTAs an SM
+// in all they are as fast at 1013x547 (22,000 candidates, 28 us) and faster
+// from 1280x720 on (36,800 candidates 51 -> 45 us, 1920x1080 115 -> 92); with
+// census records 1920x1080 takes 84 us in parts and 78 by candidates.
+constexpr int kSupRowMinCand = 32768;
+inline bool sup_by_rows(long long rows, long long cand, bool census, size_t smem) {
+    return smem <= kSupRowSmemMax && (rows >= 2 * sm_count() || (!census && cand >= kSupRowMinCand));
+}
+// CTAs per lattice row of wc candidates in a launch of `all` candidates: 8
+// per SM in the whole launch, no fewer than 16 candidates each.
+inline int sup_row_segments(int wc, long long all) {
+    const long long want = (8LL * sm_count() * wc + all - 1) / (all > 0 ? all : 1);
+    return (int)max(1LL, min(want, (long long)(wc / 16)));
+}
 
 static elas_status sup_row_smem_attr(const void *fn, size_t smem) {
     if (smem > 48 * 1024 &&
@@ -647,17 +667,18 @@ elas_status launch_support(const uint8_t *descL, const uint8_t *descR, int w, in
         return ELAS_OK;
     }
     const int warps_per_block = 8;
-    const size_t row_smem = sup_row_smem(sa.match.a.wc, sa.match.a.dmin, sa.match.a.dmax).total;
+    const int nseg = sup_row_segments(sa.match.a.wc, nc);
+    const size_t row_smem = sup_row_smem((sa.match.a.wc + nseg - 1) / nseg, sa.match.a.dmin, sa.match.a.dmax).total;
     const bool census = sa.match.a.census != 0;
-    if (row_smem <= kSupRowSmemMax && sa.match.a.hc >= sup_row_min_rows()) {
+    if (sup_by_rows(sa.match.a.hc, nc, census, row_smem)) {
         const void *fn = census ? (const void *)support_match_row_kernel<true>
                                 : (const void *)support_match_row_kernel<false>;
         if ((s = sup_row_smem_attr(fn, row_smem)) != ELAS_OK) return s;
         if (census)
-            support_match_row_kernel<true><<<lattice_row_grid(sa.match.a.hc), 32 * warps_per_block, row_smem, st>>>(
+            support_match_row_kernel<true><<<dim3(sa.match.a.hc, nseg), 32 * warps_per_block, row_smem, st>>>(
                 sa.match);
         else
-            support_match_row_kernel<false><<<lattice_row_grid(sa.match.a.hc), 32 * warps_per_block, row_smem, st>>>(
+            support_match_row_kernel<false><<<dim3(sa.match.a.hc, nseg), 32 * warps_per_block, row_smem, st>>>(
                 sa.match);
         if ((s = launch_status("support_match_row_kernel")) != ELAS_OK) return s;
     } else {
@@ -704,6 +725,12 @@ elas_status launch_support_b(const SupportTables &t, const SupportStage *host, c
     vmap_clear(m_rows, pairs.stride);
     vmap_clear(m_lg, pairs.stride);
     size_t cons_smem = 0;
+    long long rows[2] = {0, 0}, cand[2] = {0, 0};
+    for (int i = 0; i < pairs.n; ++i) {
+        const SupportArgs &a = slot_entry(host, pairs.stride, pairs.slot[i]).match.a;
+        rows[a.census ? 1 : 0] += a.hc;
+        cand[a.census ? 1 : 0] += (long long)a.wc * a.hc;
+    }
     for (int i = 0; i < pairs.n; ++i) {
         const int slot = pairs.slot[i];
         const SupportStage &h = slot_entry(host, pairs.stride, slot);
@@ -711,8 +738,9 @@ elas_status launch_support_b(const SupportTables &t, const SupportStage *host, c
             return fail(ELAS_ERR_INVALID_ARG, "pair %d has no lattice candidate", i);
         const int c = h.match.a.census ? 1 : 0;
         vmap_add(m_match[c], slot, support_match_grid(h.match, match_warps));
-        vmap_add(m_krows[c], slot, lattice_row_grid(h.red.hc));
-        row_smem[c] = max(row_smem[c], sup_row_smem(h.match.a.wc, h.match.a.dmin, h.match.a.dmax).total);
+        const int wc = h.match.a.wc, nseg = sup_row_segments(wc, cand[c]);
+        vmap_add(m_krows[c], slot, dim3(h.red.hc, nseg));
+        row_smem[c] = max(row_smem[c], sup_row_smem((wc + nseg - 1) / nseg, h.match.a.dmin, h.match.a.dmax).total);
         red_smem = max(red_smem, red_smem_bytes(h.red.wc, h.red.maxd, h.red.g.gw, h.red.g.nw));
         vmap_add(m_cons, slot, consistency_grid(h.cons));
         vmap_add(m_rows, slot, lattice_row_grid(h.red.hc));
@@ -724,7 +752,7 @@ elas_status launch_support_b(const SupportTables &t, const SupportStage *host, c
     elas_status s;
     for (int c = 0; c < 2; ++c) {
         if (m_match[c].n == 0) continue;
-        if (row_smem[c] <= kSupRowSmemMax && vmap_total(m_krows[c]) >= sup_row_min_rows()) {
+        if (sup_by_rows(rows[c], cand[c], c != 0, row_smem[c])) {
             const void *fn = c ? (const void *)support_match_row_kernel_b<true>
                                : (const void *)support_match_row_kernel_b<false>;
             if ((s = sup_row_smem_attr(fn, row_smem[c])) != ELAS_OK) return s;
