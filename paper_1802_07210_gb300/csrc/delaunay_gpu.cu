@@ -1324,14 +1324,17 @@ __device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, 
         k = 1;
         __syncthreads();
     }
+    const bool ring = ordered && sh.quads == 15u;  // a fan already (dt_warp_star)
     if (tid == 0) {
         sh.far = max(fabsf(cand[sh.nearest].x), fabsf(cand[sh.nearest].y)) >= (float)kDtNearMax;
         sh.k = k;
     }
     __syncthreads();
     // points spread over the whole set, so that the first circles are not
-    // far wider than the star's
-    if (tid < kDtSamples) {
+    // far wider than the star's (a point with neighbours all around has none
+    // that wide, and would only step over the samples too: 1920x1080 pass
+    // 124 -> 112 us with this and the circles' regions below)
+    if (tid < kDtSamples && !ring) {
         const int4 q = S.pts[(int)((int64_t)tid * n / kDtSamples)];
         const int dx = q.x - p.x, dy = q.y - p.y, nz = __float_as_int(cand[sh.nearest].w);
         if (q.w && q.z != p.z && q.z != nz && (max(abs(dx), abs(dy)) > R || dx * dx + dy * dy > R * R)) {
@@ -1431,9 +1434,6 @@ __device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, 
             __syncthreads();
             const int nbad = sh.nbad;
             t0 = sh.next;
-            // a whole star in one group: a point inside any circle is inside
-            // that of its own sector
-            const bool sector = !fan && first && t0 >= nt;
             first = false;
             if (nbad == 0 && !ends) continue;
             const DtPt el = dt_point(cand[star.v[0][star.n[0]]]), er = dt_point(cand[star.v[1][star.n[1]]]);
@@ -1513,15 +1513,10 @@ __device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, 
                         // region holds it
                         unsigned need = 0;
                         for (int b = 0; b < nbad; ++b) {
-                            bool in;
-                            if (!sector) {
-                                const float3 g = sh.region[b];
-                                const float dx = qx - g.x, dy = qy - g.y;
-                                in = !(g.z >= 0.0f && dx * dx + dy * dy > g.z * g.z);
-                            } else {
-                                const DtPt u = sh.bad[b].a, v = sh.bad[b].b;
-                                in = u.x * q.y - u.y * q.x >= 0 && v.x * q.y - v.y * q.x <= 0;
-                            }
+                            const float3 g = sh.region[b];
+                            const float dx = qx - g.x, dy = qy - g.y;
+                            const bool in = g.z >= 0.0f ? dx * dx + dy * dy <= g.z * g.z
+                                                        : g.x * qx + g.y * qy >= -1.0f;
                             need |= (unsigned)in << b;
                         }
                         const bool some = t.w && t.z != p.z;
@@ -1529,19 +1524,11 @@ __device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, 
                         if (ends && some)
                             hit = (open_l && el.x * q.y - el.y * q.x > 0) || (open_r && er.x * q.y - er.y * q.x < 0);
                         if (!some) need = 0;
-                        if (hit && sector) need = nbad < 32 ? (1u << nbad) - 1u : 0xFFFFFFFFu;
-                        for (bool all = hit || !sector; need; need &= need - 1) {
+                        for (; need; need &= need - 1) {
                             const int b = __ffs(need) - 1;
                             if (!dt_violates(sh.bad[b], p.z, q)) continue;
                             hit = true;
                             star.state[sh.tri[b] >> 15][sh.tri[b] & 0x7FFF] = kDtHit;
-                            if (!all) {  // now every circle that holds it
-                                all = true;
-                                for (int c = 0; c < nbad; ++c)
-                                    if (c != b && dt_violates(sh.bad[c], p.z, q))
-                                        star.state[sh.tri[c] >> 15][sh.tri[c] & 0x7FFF] = kDtHit;
-                                break;
-                            }
                         }
                         const unsigned m = __ballot_sync(0xFFFFFFFFu, hit);
                         if (!m) continue;
