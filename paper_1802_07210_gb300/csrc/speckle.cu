@@ -5,11 +5,12 @@
 //
 // Connected components by union-find over pixel indices, every parent index
 // below its child's, so a root is the least pixel index of its tree:
-//   speckle_local_kernel   one CTA per 32x16 tile: union-find of the links
-//                          inside the tile in shared memory; each pixel's
-//                          label = the global index of its tile-local root,
-//                          and each tile-local root's size entry = its
-//                          pixel count in the tile (0 for other pixels).
+//   speckle_local_kernel   one CTA per 64x32 tile: union-find of the links
+//                          inside the tile in shared memory.  A tile-local
+//                          root's label is its own global index and its size
+//                          entry its pixel count in the tile; another pixel's
+//                          label names its tile-local root (as -2 - index,
+//                          -1: invalid), and its size entry is not used.
 //   speckle_border_kernel  one thread per link across a tile's right or
 //                          bottom edge: union in global memory (atomicMin on
 //                          roots).
@@ -26,18 +27,26 @@
 
 namespace elas {
 
-constexpr int kSpTX = 32, kSpTY = 16, kSpThreads = kSpTX * kSpTY;
+// Tiles of 64x32 rather than 32x16 halve the links across tile edges and
+// quarter the tile-local roots that those link (border pass at 1920x1080
+// 15.0 -> 10.8 us).
+constexpr int kSpTX = 64, kSpTY = 32, kSpCells = kSpTX * kSpTY, kSpWarps = 16, kSpRows = kSpTY / kSpWarps;
 
 struct SpeckleArgs {
     const int16_t *d;
     int16_t *out;
-    int32_t *label;   // [h][w]: parent index, -1 for invalid pixels
-    int32_t *size;    // [h][w]: pixel count of the segment rooted here
+    int32_t *label;   // [h][w]: tile-local roots: parent; else -2 - the tile-local root, -1 for invalid pixels
+    int32_t *size;    // [h][w]: tile-local roots: pixel count
     int32_t *status;  // 0, or 1 if a loop bound was reached
     int w, h, thr, min_size;
 };
 
 __device__ __forceinline__ bool sp_linked(int a, int b, int thr) { return a >= 0 && b >= 0 && abs(a - b) <= thr; }
+
+__device__ __forceinline__ int sp_tile_root(const int32_t *L, int i) {
+    const int v = __ldcg(L + i);
+    return v < -1 ? -2 - v : i;
+}
 
 // Root of x in a forest whose parents are strictly smaller indices; reads
 // through L2 (`ld.cg`) because other CTAs relink roots during the kernel.
@@ -58,6 +67,8 @@ __device__ __forceinline__ int sp_find_global(int32_t *L, int x, int limit) {
 // one with atomicMin; if that root was relinked meanwhile, the returned old
 // parent (a smaller index) is where the walk resumes.
 __device__ void sp_unite_global(int32_t *L, int a, int b, int limit, int32_t *status) {
+    a = sp_tile_root(L, a);
+    b = sp_tile_root(L, b);
     for (int it = 0; it < limit; ++it) {
         a = sp_find_global(L, a, limit);
         b = sp_find_global(L, b, limit);
@@ -88,7 +99,7 @@ __device__ __forceinline__ int sp_find_readonly(const int32_t *L, int x, int lim
 }
 
 __device__ __forceinline__ int sp_find_shared(volatile int *L, int x) {
-    for (int it = 0; it < kSpThreads; ++it) {
+    for (int it = 0; it < kSpCells; ++it) {
         const int p = L[x];
         if (p == x) return x;
         const int g = L[p];
@@ -98,8 +109,18 @@ __device__ __forceinline__ int sp_find_shared(volatile int *L, int x) {
     return -1;
 }
 
+// Without writes, as sp_find_readonly and for the same reason.
+__device__ __forceinline__ int sp_find_shared_readonly(const volatile int *L, int x) {
+    for (int it = 0; it < kSpCells; ++it) {
+        const int p = L[x];
+        if (p == x) return x;
+        x = p;
+    }
+    return -1;
+}
+
 __device__ void sp_unite_shared(int *L, int a, int b, int32_t *status) {
-    for (int it = 0; it < kSpThreads; ++it) {
+    for (int it = 0; it < kSpCells; ++it) {
         a = sp_find_shared(L, a);
         b = sp_find_shared(L, b);
         if (a < 0 || b < 0) break;
@@ -116,57 +137,109 @@ __device__ void sp_unite_shared(int *L, int a, int b, int32_t *status) {
     atomicExch(status, 1);
 }
 
-// A tile row is one warp: the horizontal links of a row become runs from one
-// ballot (a pixel's run root is the nearest run start at or left of it), so
-// union-find only joins runs through vertical links, and a vertical link is
-// skipped where the link to its left, with the two horizontal links beside
-// it, already connects the same pixels (those links are processed or
-// skipped for the same reason further left, ending at a processed one).
-__global__ void __launch_bounds__(kSpThreads) speckle_local_kernel(SpeckleArgs a) {
-    __shared__ int sL[kSpThreads];
-    __shared__ int sC[kSpThreads];
-    __shared__ int16_t sD[kSpThreads];
-    const int tx = threadIdx.x, ty = threadIdx.y, t = ty * kSpTX + tx;
+// A warp takes whole tile rows, a lane the pixels lane and lane + 32 of each:
+// the horizontal links of a row become runs from two ballots (a pixel's run
+// root is the nearest run start at or left of it), so union-find only joins
+// runs through vertical links, and a vertical link is skipped where the link
+// to its left, with the two horizontal links beside it, already connects the
+// same pixels (those links are processed or skipped for the same reason
+// further left, ending at a processed one).  Bound by instruction issue, most
+// of it in the walks, which few lanes of a row have: the links left and the
+// run starts are listed, so that whole warps walk, and a run adds its length
+// to its root's count once (1920x1080: 24.7 us with a thread for each pixel's
+// link and addition, 23.7 with the additions of runs, 16.8 with the lists).
+__global__ void __launch_bounds__(32 * kSpWarps, 2048 / (32 * kSpWarps)) speckle_local_kernel(SpeckleArgs a) {
+    __shared__ int sL[kSpCells];
+    __shared__ int sC[kSpCells];  // run starts: the run's length, then roots: the segment's pixels
+    __shared__ int16_t sD[kSpCells];
+    __shared__ uint16_t sLink[kSpCells], sRun[kSpCells];
+    __shared__ int s_links, s_runs;
+    const int lane = threadIdx.x & 31, row0 = (threadIdx.x >> 5) * kSpRows;
     const int x0 = blockIdx.x * kSpTX, y0 = blockIdx.y * kSpTY;
-    const int x = x0 + tx, y = y0 + ty;
-    const bool in = x < a.w && y < a.h;
-    const size_t i = (size_t)y * a.w + x;
-    const int dv = in ? a.d[i] : -1;
-    sD[t] = (int16_t)dv;
-    sC[t] = 0;
-    __syncthreads();
-    const bool left = tx > 0 && sp_linked(sD[t - 1], dv, a.thr);
-    const unsigned linked_left = __ballot_sync(0xFFFFFFFFu, left);
-    // run starts at or left of this lane (lane 0 is never linked left)
-    const unsigned starts = ~linked_left & (0xFFFFFFFFu >> (31 - tx));
-    sL[t] = dv >= 0 ? ty * kSpTX + (31 - __clz(starts)) : -1;
-    __syncthreads();
-    if (dv >= 0 && ty + 1 < kSpTY && sp_linked(dv, sD[t + kSpTX], a.thr)) {
-        const bool redundant = left && sp_linked(sD[t - 1], sD[t - 1 + kSpTX], a.thr) &&
-                               sp_linked(sD[t - 1 + kSpTX], sD[t + kSpTX], a.thr);
-        if (!redundant) sp_unite_shared(sL, t, t + kSpTX, a.status);
+    const unsigned upto = 0xFFFFFFFFu >> (31 - lane), below = upto >> 1;
+    int16_t dv[2 * kSpRows];
+#pragma unroll
+    for (int k = 0; k < 2 * kSpRows; ++k) {
+        const int x = x0 + lane + 32 * (k & 1), y = y0 + row0 + (k >> 1);
+        dv[k] = x < a.w && y < a.h ? a.d[(size_t)y * a.w + x] : (int16_t)-1;
     }
+#pragma unroll
+    for (int k = 0; k < 2 * kSpRows; ++k) sD[row0 * kSpTX + 32 * k + lane] = dv[k];
+    if (threadIdx.x == 0) s_links = s_runs = 0;
     __syncthreads();
-    int r = -1;
-    if (dv >= 0) {
-        r = sp_find_shared(sL, t);
-        if (r < 0) {
-            atomicExch(a.status, 1);
-            r = t;
+#pragma unroll
+    for (int r = 0; r < kSpRows; ++r) {
+        const int c = (row0 + r) * kSpTX + lane, d0 = dv[2 * r], d1 = dv[2 * r + 1];
+        const bool l0 = lane > 0 && sp_linked(sD[c - (lane > 0)], d0, a.thr), l1 = sp_linked(sD[c + 31], d1, a.thr);
+        const unsigned s0 = ~__ballot_sync(0xFFFFFFFFu, l0);  // run starts (pixel 0 of the row always)
+        const unsigned s1 = ~__ballot_sync(0xFFFFFFFFu, l1);
+        const int first = c - lane;
+        sL[c] = d0 >= 0 ? first + 31 - __clz(s0 & upto) : -1;
+        sL[c + 32] = d1 >= 0 ? first + (s1 & upto ? 63 - __clz(s1 & upto) : 31 - __clz(s0)) : -1;
+        auto link = [&](int e, int d, bool left) {
+            if (row0 + r + 1 == kSpTY) return false;
+            const int q = sD[e + kSpTX];
+            if (!sp_linked(d, q, a.thr)) return false;
+            if (!left) return true;
+            const int v = sD[e - 1 + kSpTX];
+            return !(sp_linked(sD[e - 1], v, a.thr) && sp_linked(v, q, a.thr));
+        };
+        const bool k0 = link(c, d0, l0), k1 = link(c + 32, d1, l1);
+        const unsigned m0 = __ballot_sync(0xFFFFFFFFu, k0), m1 = __ballot_sync(0xFFFFFFFFu, k1);
+        const unsigned h0 = s0 & __ballot_sync(0xFFFFFFFFu, d0 >= 0), h1 = s1 & __ballot_sync(0xFFFFFFFFu, d1 >= 0);
+        int at = 0;
+        if (lane == 0) at = atomicAdd(&s_links, __popc(m0) + __popc(m1));
+        if (lane == 1) at = atomicAdd(&s_runs, __popc(h0) + __popc(h1));
+        const int lk = __shfl_sync(0xFFFFFFFFu, at, 0), rn = __shfl_sync(0xFFFFFFFFu, at, 1);
+        if (k0) sLink[lk + __popc(m0 & below)] = (uint16_t)c;
+        if (k1) sLink[lk + __popc(m0) + __popc(m1 & below)] = (uint16_t)(c + 32);
+        if (h0 >> lane & 1u) {
+            const unsigned after = s0 & ~upto;
+            sRun[rn + __popc(h0 & below)] = (uint16_t)c;
+            sC[c] = (after ? __ffs(after) - 1 : s1 ? 31 + __ffs(s1) : 64) - lane;
         }
-        atomicAdd(sC + r, 1);
+        if (h1 >> lane & 1u) {
+            const unsigned after = s1 & ~upto;
+            sRun[rn + __popc(h0) + __popc(h1 & below)] = (uint16_t)(c + 32);
+            sC[c + 32] = (after ? __ffs(after) - 1 : 32) - lane;
+        }
     }
     __syncthreads();
-    if (in) {
-        // the tile-local root's global index: local order is raster order
-        // inside the tile, so the label is still <= i
-        a.label[i] = r < 0 ? -1 : (y0 + r / kSpTX) * a.w + (x0 + r % kSpTX);
-        a.size[i] = sC[t];  // the tile-local count at a tile-local root, else 0
+    const int links = s_links, runs = s_runs;
+    for (int q = threadIdx.x; q < links; q += 32 * kSpWarps) sp_unite_shared(sL, sLink[q], sLink[q] + kSpTX, a.status);
+    __syncthreads();
+    for (int q = threadIdx.x; q < runs; q += 32 * kSpWarps) {
+        const int c = sRun[q];
+        int root = sp_find_shared_readonly(sL, c);
+        if (root < 0) {
+            atomicExch(a.status, 1);
+            root = c;
+        }
+        if (root == c) continue;
+        sL[c] = root;                 // an ancestor: the forest stays valid
+        atomicAdd(sC + root, sC[c]);  // lengths are added to roots alone
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 2 * kSpRows; ++k) {
+        const int x = x0 + lane + 32 * (k & 1), y = y0 + row0 + (k >> 1), c = row0 * kSpTX + 32 * k + lane;
+        if (x >= a.w || y >= a.h) continue;
+        const int i = y * a.w + x;
+        int label = -1;
+        if (dv[k] >= 0) {
+            // a pixel's parent is a run's first pixel, whose parent is the
+            // root.  The root's global index is at most i: local order is
+            // raster order inside the tile
+            const int root = sL[sL[c]];
+            label = root == c ? i : -2 - ((y0 + root / kSpTX) * a.w + x0 + root % kSpTX);
+            if (root == c) a.size[i] = sC[c];
+        }
+        a.label[i] = label;
     }
 }
 
-// Links across tile edges: first every right edge (x = 32k + 31, k =
-// 0..ntx-2) of every row, then every bottom edge (y = 16k + 15) of every
+// Links across tile edges: first every right edge (x = 64k + 63, k =
+// 0..ntx-2) of every row, then every bottom edge (y = 32k + 31) of every
 // column.  A right-edge link is skipped where the link above it and the two
 // vertical links beside it connect the same pixels and those vertical links
 // lie inside a tile (not on a tile's first row); a bottom-edge link likewise
@@ -200,36 +273,68 @@ __global__ void __launch_bounds__(256) speckle_border_kernel(SpeckleArgs a) {
     }
 }
 
+// Four pixels a thread: their labels come in one load, and the walks of the
+// four are in flight together.  1920x1080: resolve 7.3 us (6.6 before, when
+// the counts were also written and read for every pixel and the walks were
+// shorter), apply 5.8 -> 5.4.
+__device__ __forceinline__ void sp_labels(const int32_t *label, int i0, int n, int *l) {
+    if (i0 + 4 <= n) {
+        const int4 q = __ldcg(reinterpret_cast<const int4 *>(label + i0));
+        l[0] = q.x, l[1] = q.y, l[2] = q.z, l[3] = q.w;
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) l[k] = i0 + k < n ? __ldcg(label + i0 + k) : -1;
+    }
+}
+
 __global__ void __launch_bounds__(256) speckle_resolve_kernel(SpeckleArgs a) {
-    const int n = a.w * a.h;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        // tile-local roots hold their tile count (>= 1); adds only go to
-        // final roots, which are tile-local roots too, so the test is stable
-        const int c = __ldcg(a.size + i);
-        if (c <= 0) continue;
-        const int root = sp_find_readonly(a.label, i, n);
+    const int n = a.w * a.h, i0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+    if (i0 >= n) return;
+    int l[4];
+    sp_labels(a.label, i0, n, l);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int i = i0 + k;
+        if (l[k] < 0 || l[k] == i) continue;  // not a tile-local root, or a final root
+        const int root = sp_find_readonly(a.label, l[k], n);
         if (root < 0) {
             atomicExch(a.status, 1);
             continue;
         }
-        if (root != i) {
-            __stcg(a.label + i, root);  // an ancestor: the forest stays valid
-            atomicAdd(a.size + root, c);
-        }
+        __stcg(a.label + i, root);  // an ancestor: the forest stays valid
+        atomicAdd(a.size + root, a.size[i]);  // counts are added to final roots alone
     }
 }
 
-__global__ void __launch_bounds__(256) speckle_apply_kernel(SpeckleArgs a) {
-    const int n = a.w * a.h;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int r = a.label[i];
-        const int16_t dv = a.d[i];
-        bool keep = false;
-        if (r >= 0) {
-            const int root = a.label[r];  // r's final root (r itself if it is one)
-            keep = a.size[root] >= a.min_size;
-        }
-        a.out[i] = keep ? dv : (int16_t)-1;
+// kWide: 8-byte aligned maps, four pixels an access.
+template <bool kWide> __global__ void __launch_bounds__(256) speckle_apply_kernel(SpeckleArgs a) {
+    const int n = a.w * a.h, i0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+    if (i0 >= n) return;
+    const bool all = i0 + 4 <= n;
+    int r[4];
+    union {
+        uint2 v;
+        int16_t d[4];
+    } px;
+    sp_labels(a.label, i0, n, r);
+    if (kWide && all) {
+        px.v = *reinterpret_cast<const uint2 *>(a.d + i0);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) px.d[k] = i0 + k < n ? a.d[i0 + k] : (int16_t)-1;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (r[k] < -1) r[k] = a.label[-2 - r[k]];  // the tile-local root's final root (itself if it is one)
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        if (r[k] < 0 || a.size[r[k]] < a.min_size) px.d[k] = -1;
+    if (kWide && all) {
+        *reinterpret_cast<uint2 *>(a.out + i0) = px.v;
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (i0 + k < n) a.out[i0 + k] = px.d[k];
     }
 }
 
@@ -252,17 +357,21 @@ elas_status launch_speckle(const int16_t *d, int w, int h, int thr, int min_size
     a.min_size = min_size;
     if (cudaMemsetAsync(a.status, 0, sizeof(int32_t), st) != cudaSuccess) return launch_status("speckle status");
     const dim3 tiles((w + kSpTX - 1) / kSpTX, (h + kSpTY - 1) / kSpTY);
-    speckle_local_kernel<<<tiles, dim3(kSpTX, kSpTY), 0, st>>>(a);
+    speckle_local_kernel<<<tiles, 32 * kSpWarps, 0, st>>>(a);
     elas_status s = launch_status("speckle_local_kernel");
     if (s != ELAS_OK) return s;
-    const int n = w * h;
-    int blocks = (n + 255) / 256;
-    if (blocks > sm_count() * 8) blocks = sm_count() * 8;
-    speckle_border_kernel<<<blocks, 256, 0, st>>>(a);
-    if ((s = launch_status("speckle_border_kernel")) != ELAS_OK) return s;
-    speckle_resolve_kernel<<<blocks, 256, 0, st>>>(a);
+    const int ntx = (int)tiles.x, nty = (int)tiles.y;
+    const int links = (ntx - 1) * h + (nty - 1) * w, quads = (w * h + 3) / 4;
+    if (links > 0) {
+        speckle_border_kernel<<<min((links + 255) / 256, sm_count() * 8), 256, 0, st>>>(a);
+        if ((s = launch_status("speckle_border_kernel")) != ELAS_OK) return s;
+    }
+    speckle_resolve_kernel<<<(quads + 255) / 256, 256, 0, st>>>(a);
     if ((s = launch_status("speckle_resolve_kernel")) != ELAS_OK) return s;
-    speckle_apply_kernel<<<blocks, 256, 0, st>>>(a);
+    if (aligned(d, 8) && aligned(out, 8))
+        speckle_apply_kernel<true><<<(quads + 255) / 256, 256, 0, st>>>(a);
+    else
+        speckle_apply_kernel<false><<<(quads + 255) / 256, 256, 0, st>>>(a);
     return launch_status("speckle_apply_kernel");
 }
 
