@@ -50,9 +50,57 @@ inline GridGeom grid_geom(int w, int h, const elas_params *p) {
 // Prior table P[0..sradius] from the parameters (host, double precision).
 void prior_table(const elas_params *p, int32_t *P);
 
+// Launch of a kernel that begins with after_previous(): its CTAs may take
+// their places while the last ones of the kernel before it in the stream
+// still run, so the launch's own latency is hidden behind that kernel (the
+// triangulation is nine kernels of 1 to 40 us: 1242x375, both sides one call
+// each, 177 -> 141 us; LR check to speckle removal of 1920x1080 91 -> 82).  A
+// kernel launched without it, a copy or an event waits for the whole kernel
+// as ever.  Under capture it is an ordinary launch: a graph's own edges are as
+// quick (640x480, twenty kernels: 143 us with them, 140 to 150 with early
+// starts).
+template <class... P, class... A>
+inline void launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchAttribute early{};
+    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    early.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &early;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
+        (void)cudaGetLastError();  // the launch reports what is wrong
+        cs = cudaStreamCaptureStatusActive;
+    }
+    cfg.numAttrs = cs == cudaStreamCaptureStatusNone ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);  // errors: launch_status
+}
+
 // ---------------------------------------------------------------------------
 // Device helpers
 // ---------------------------------------------------------------------------
+
+// Lets the next kernel of the stream take its places as soon as every CTA of
+// this one has started.
+__device__ __forceinline__ void let_next_in() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// First statement of a kernel launched by launch_after: waits until the
+// kernel before it in the stream (so, in turn, all before that) is complete
+// and its writes are visible; no global memory is touched earlier.
+__device__ __forceinline__ void after_previous() {
+    let_next_in();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// p, not known to the compiler before this point: a read-only load (__ldg)
+// through it cannot be moved above after_previous().
+template <class T> __device__ __forceinline__ T *settled(T *p) {
+    asm volatile("" : "+l"(p)::"memory");
+    return p;
+}
 
 // Sum of |a_i - b_i| over the 4 bytes of a and b, added to acc.
 __device__ __forceinline__ uint32_t sad4_acc(uint32_t a, uint32_t b, uint32_t acc) {

@@ -65,7 +65,10 @@ __device__ __forceinline__ void dt_points_body(const DtArgs &a, const VB &vb) {
     }
 }
 
-__global__ void dt_points_kernel(DtArgs a) { dt_points_body(a, vb_single()); }
+__global__ void dt_points_kernel(DtArgs a) {
+    after_previous();
+    dt_points_body(a, vb_single());
+}
 __global__ void dt_points_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
     const VB vb = vb_batch(vm);
     dt_points_body(slot_entry(tab, vm.stride, vb.slot), vb);
@@ -133,7 +136,10 @@ __device__ __forceinline__ void dt_cell_scan_body(const DtArgs &a, const VB &vb)
     });
 }
 
-__global__ void __launch_bounds__(1024) dt_cell_scan_kernel(DtArgs a) { dt_cell_scan_body(a, vb_single()); }
+__global__ void __launch_bounds__(1024) dt_cell_scan_kernel(DtArgs a) {
+    after_previous();
+    dt_cell_scan_body(a, vb_single());
+}
 __global__ void __launch_bounds__(1024) dt_cell_scan_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
     const VB vb = vb_batch(vm);
     dt_cell_scan_body(slot_entry(tab, vm.stride, vb.slot), vb);
@@ -150,7 +156,10 @@ __device__ __forceinline__ void dt_scatter_body(const DtArgs &a, const VB &vb) {
     }
 }
 
-__global__ void dt_scatter_kernel(DtArgs a) { dt_scatter_body(a, vb_single()); }
+__global__ void dt_scatter_kernel(DtArgs a) {
+    after_previous();
+    dt_scatter_body(a, vb_single());
+}
 __global__ void dt_scatter_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
     const VB vb = vb_batch(vm);
     dt_scatter_body(slot_entry(tab, vm.stride, vb.slot), vb);
@@ -176,7 +185,10 @@ __device__ __forceinline__ void dt_dedup_body(const DtArgs &a, const VB &vb) {
     }
 }
 
-__global__ void dt_dedup_kernel(DtArgs a) { dt_dedup_body(a, vb_single()); }
+__global__ void dt_dedup_kernel(DtArgs a) {
+    after_previous();
+    dt_dedup_body(a, vb_single());
+}
 __global__ void dt_dedup_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
     const VB vb = vb_batch(vm);
     dt_dedup_body(slot_entry(tab, vm.stride, vb.slot), vb);
@@ -829,7 +841,10 @@ __device__ __forceinline__ void dt_pass1_body(const DtArgs &a, const VB &vb) {
     }
 }
 
-__global__ void __launch_bounds__(kDtWarps * 32, 4) dt_pass1_kernel(const __grid_constant__ DtArgs a) { dt_pass1_body(a, vb_single()); }
+__global__ void __launch_bounds__(kDtWarps * 32, 4) dt_pass1_kernel(const __grid_constant__ DtArgs a) {
+    after_previous();
+    dt_pass1_body(a, vb_single());
+}
 __global__ void __launch_bounds__(kDtWarps * 32, 4) dt_pass1_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
     const VB vb = vb_batch(vm);
     dt_pass1_body(slot_entry(tab, vm.stride, vb.slot), vb);
@@ -1575,6 +1590,7 @@ __device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, 
 // passes leave unused.
 __global__ void __launch_bounds__(kDtBlockThreads, kDtBlocksPerSM) dt_pass_block_kernel(const __grid_constant__ DtArgs a,
                                                                                              int nsides) {
+    after_previous();
     extern __shared__ float4 s_cand[];  // [kDtCacheCap], then the region rows
     __shared__ DtStarShared sh;
     __shared__ int s_item;
@@ -1678,7 +1694,10 @@ __device__ __forceinline__ void dt_tri_scan_body(const DtArgs &a, const VB &vb) 
     if (threadIdx.x == 0) *S.ntri = total > a.cap_tri ? -1 : total;  // -1: the triangulation failed
 }
 
-__global__ void __launch_bounds__(1024) dt_tri_scan_kernel(DtArgs a) { dt_tri_scan_body(a, vb_single()); }
+__global__ void __launch_bounds__(1024) dt_tri_scan_kernel(DtArgs a) {
+    after_previous();
+    dt_tri_scan_body(a, vb_single());
+}
 __global__ void __launch_bounds__(1024) dt_tri_scan_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
     const VB vb = vb_batch(vm);
     dt_tri_scan_body(slot_entry(tab, vm.stride, vb.slot), vb);
@@ -1703,7 +1722,10 @@ __device__ __forceinline__ void dt_emit_body(const DtArgs &a, const VB &vb) {
     }
 }
 
-__global__ void dt_emit_kernel(DtArgs a) { dt_emit_body(a, vb_single()); }
+__global__ void dt_emit_kernel(DtArgs a) {
+    after_previous();
+    dt_emit_body(a, vb_single());
+}
 __global__ void dt_emit_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
     const VB vb = vb_batch(vm);
     dt_emit_body(slot_entry(tab, vm.stride, vb.slot), vb);
@@ -1789,24 +1811,23 @@ elas_status launch_triangulate_device(const int16_t *list, const int32_t *count,
     }
     // counters, cell counts and row extremes of both sides: one kernel
     const int nall = a.gw * a.gh + 1 + 2 * h + kDtCounters;
-    dt_init_kernel<<<dim3((nall + 255) / 256, nsides), 256, 0, st>>>(a);
+    launch_after(dt_init_kernel, dim3((nall + 255) / 256, nsides), 256, 0, st, a);
     const int tb = 256;
     const int pblocks = max(1, min((cap + tb - 1) / tb, sm_count() * 8));
-    dt_points_kernel<<<dim3(pblocks, nsides), tb, 0, st>>>(a);
-    dt_cell_scan_kernel<<<dim3(1, nsides), 1024, 0, st>>>(a);
-    dt_scatter_kernel<<<dim3(pblocks, nsides), tb, 0, st>>>(a);
-    dt_dedup_kernel<<<dim3(pblocks, nsides), tb, 0, st>>>(a);
-    dt_pass1_kernel<<<dim3(max(1, min((cap + kDtWarps - 1) / kDtWarps, sm_count() * 16)), nsides), kDtWarps * 32, 0,
-                      st>>>(a);
+    launch_after(dt_points_kernel, dim3(pblocks, nsides), tb, 0, st, a);
+    launch_after(dt_cell_scan_kernel, dim3(1, nsides), 1024, 0, st, a);
+    launch_after(dt_scatter_kernel, dim3(pblocks, nsides), tb, 0, st, a);
+    launch_after(dt_dedup_kernel, dim3(pblocks, nsides), tb, 0, st, a);
+    launch_after(dt_pass1_kernel, dim3(max(1, min((cap + kDtWarps - 1) / kDtWarps, sm_count() * 16)), nsides), kDtWarps * 32, 0, st, a);
 
     // no middle pass: it would add its longest star's time to the CTA pass's
     // (640x480 115 against 78 us)
     const int smem = kDtCacheCap * (int)sizeof(float4) + 2 * a.gh * (int)sizeof(int);
     if (cudaFuncSetAttribute(dt_pass_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
         return launch_status("dt_pass_block_kernel shared memory attribute");
-    dt_pass_block_kernel<<<sm_count() * kDtBlocksPerSM, kDtBlockThreads, smem, st>>>(a, nsides);
-    dt_tri_scan_kernel<<<dim3(1, nsides), 1024, 0, st>>>(a);
-    dt_emit_kernel<<<dim3(pblocks, nsides), tb, 0, st>>>(a);
+    launch_after(dt_pass_block_kernel, sm_count() * kDtBlocksPerSM, kDtBlockThreads, smem, st, a, nsides);
+    launch_after(dt_tri_scan_kernel, dim3(1, nsides), 1024, 0, st, a);
+    launch_after(dt_emit_kernel, dim3(pblocks, nsides), tb, 0, st, a);
     return launch_status("triangulation kernels");
 }
 
@@ -1829,7 +1850,10 @@ __device__ __forceinline__ void dt_init_body(const DtArgs &a, const VB &vb, int3
     }
 }
 
-__global__ void __launch_bounds__(256) dt_init_kernel(DtArgs a) { dt_init_body(a, vb_single(), nullptr); }
+__global__ void __launch_bounds__(256) dt_init_kernel(DtArgs a) {
+    after_previous();
+    dt_init_body(a, vb_single(), nullptr);
+}
 __global__ void __launch_bounds__(256) dt_init_kernel_b(const DtArgs *__restrict__ tab, VMap vm, int32_t *counter) {
     const VB vb = vb_batch(vm);
     dt_init_body(slot_entry(tab, vm.stride, vb.slot), vb, counter);

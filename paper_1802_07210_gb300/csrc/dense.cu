@@ -68,6 +68,8 @@ constexpr int kRecWords = 4;  // 16-byte words of a stored record: edges, plane,
 // xmin).
 __device__ __forceinline__ TriRec tri_record(const int16_t *__restrict__ list, const int32_t *__restrict__ tri, int t,
                                              int right, int w, int h, TriBox &box) {
+    list = settled(list);
+    tri = settled(tri);
     int i0 = __ldg(tri + 3 * t), i1 = __ldg(tri + 3 * t + 1), i2 = __ldg(tri + 3 * t + 2);
     // canonical vertex order: ascending list index
     if (i1 < i0) { const int q = i0; i0 = i1; i1 = q; }
@@ -157,7 +159,10 @@ __device__ __forceinline__ void raster_setup_body(const RasterArgs &a, const VB 
     }
 }
 
-__global__ void __launch_bounds__(256) raster_setup_kernel(RasterArgs a) { raster_setup_body(a, vb_single()); }
+__global__ void __launch_bounds__(256) raster_setup_kernel(RasterArgs a) {
+    after_previous();
+    raster_setup_body(a, vb_single());
+}
 __global__ void __launch_bounds__(256) raster_setup_kernel_b(const RasterArgs *__restrict__ tab, VMap vm) {
     const VB vb = vb_batch(vm);
     raster_setup_body(slot_entry(tab, vm.stride, vb.slot), vb);
@@ -172,6 +177,7 @@ constexpr int kListPad = 16;  // padding entries (2047) after a candidate list
 // below it, so the list comes out sorted with no per-lane bit loop.
 __device__ __forceinline__ int expand_cell_list(const uint32_t *__restrict__ g, int nw, int dmin, int dmax,
                                                 uint16_t *out, int lane) {
+    g = settled(g);
     const uint32_t below = (1u << lane) - 1u;
     int base = 0;
     for (int w0 = 0; w0 < nw; w0 += 32) {
@@ -218,7 +224,10 @@ __device__ __forceinline__ void raster_list_body(const RasterArgs &a, const VB &
     }
 }
 
-__global__ void __launch_bounds__(256) raster_list_kernel(RasterArgs a) { raster_list_body(a, vb_single()); }
+__global__ void __launch_bounds__(256) raster_list_kernel(RasterArgs a) {
+    after_previous();
+    raster_list_body(a, vb_single());
+}
 __global__ void __launch_bounds__(256) raster_list_kernel_b(const RasterArgs *__restrict__ tab, VMap vm) {
     const VB vb = vb_batch(vm);
     raster_list_body(slot_entry(tab, vm.stride, vb.slot), vb);
@@ -289,7 +298,10 @@ __device__ __forceinline__ void raster_draw_body(const RasterArgs &a, const VB &
     }
 }
 
-__global__ void __launch_bounds__(256) raster_draw_kernel(RasterArgs a) { raster_draw_body(a, vb_single()); }
+__global__ void __launch_bounds__(256) raster_draw_kernel(RasterArgs a) {
+    after_previous();
+    raster_draw_body(a, vb_single());
+}
 __global__ void __launch_bounds__(256) raster_draw_kernel_b(const RasterArgs *__restrict__ tab, VMap vm) {
     const VB vb = vb_batch(vm);
     raster_draw_body(slot_entry(tab, vm.stride, vb.slot), vb);
@@ -449,6 +461,7 @@ __device__ __forceinline__ void cell_body(const CellArgs &a, const VB &vb) {
 }
 
 template <bool CENSUS, bool GLIST> __global__ void __launch_bounds__(1024, 2) cell_kernel(CellArgs a) {
+    let_next_in();
     cell_body<1, CENSUS, GLIST>(a, vb_single());
 }
 
@@ -607,9 +620,9 @@ static int raster_setup_blocks(const RasterArgs &a, int cap_blocks) {
 
 // Prior maps of one or two meshes.
 static elas_status raster_meshes(const RasterArgs &a, cudaStream_t st) {
-    raster_setup_kernel<<<dim3(raster_setup_blocks(a, sm_count() * 4), a.nsides), 256, 0, st>>>(a);
-    raster_list_kernel<<<dim3(raster_setup_blocks(a, sm_count() * 4), a.nsides), 256, 0, st>>>(a);
-    raster_draw_kernel<<<dim3(sm_count() * 4, a.nsides), 256, 0, st>>>(a);
+    launch_after(raster_setup_kernel, dim3(raster_setup_blocks(a, sm_count() * 4), a.nsides), 256, 0, st, a);
+    launch_after(raster_list_kernel, dim3(raster_setup_blocks(a, sm_count() * 4), a.nsides), 256, 0, st, a);
+    launch_after(raster_draw_kernel, dim3(sm_count() * 4, a.nsides), 256, 0, st, a);
     return launch_status("plane prior kernels");
 }
 

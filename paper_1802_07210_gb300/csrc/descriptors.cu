@@ -261,6 +261,7 @@ __device__ __forceinline__ void descriptor_body(const DescArgs &a, const VB &vb,
 }
 
 __global__ void __launch_bounds__(32 * kDescWarps) descriptor_kernel(DescArgs a, int rows) {
+    let_next_in();
     descriptor_body(a, vb_single(), rows);
 }
 
@@ -393,6 +394,7 @@ template <int W, int NW> __device__ __forceinline__ void census_body(const Censu
 }
 
 template <int W, int NW> __global__ void __launch_bounds__(32 * kCensusTH) census_kernel(CensusArgs a) {
+    let_next_in();
     census_body<W, NW>(a, vb_single());
 }
 template <int W, int NW>

@@ -79,7 +79,10 @@ __device__ __forceinline__ void lr_check_body(const LrArgs &a, const VB &vb) {
         lr_check_row<1>(a, row, sL, sR);
 }
 
-__global__ void __launch_bounds__(256, 8) lr_check_kernel(LrArgs a) { lr_check_body(a, vb_single()); }
+__global__ void __launch_bounds__(256, 8) lr_check_kernel(LrArgs a) {
+    after_previous();
+    lr_check_body(a, vb_single());
+}
 __global__ void __launch_bounds__(256, 8) lr_check_kernel_b(const LrArgs *__restrict__ tab, VMap vm) {
     const VB vb = vb_batch(vm);
     lr_check_body(slot_entry(tab, vm.stride, vb.slot), vb);
@@ -156,7 +159,10 @@ __device__ __forceinline__ void post_pass_body(const PostArgs &a, const VB &vb) 
     a.out[(size_t)v * w + u] = res;
 }
 
-__global__ void __launch_bounds__(256) post_pass_kernel(PostArgs a) { post_pass_body(a, vb_single()); }
+__global__ void __launch_bounds__(256) post_pass_kernel(PostArgs a) {
+    after_previous();
+    post_pass_body(a, vb_single());
+}
 __global__ void __launch_bounds__(256) post_pass_kernel_b(const PostArgs *__restrict__ tab, VMap vm) {
     const VB vb = vb_batch(vm);
     post_pass_body(slot_entry(tab, vm.stride, vb.slot), vb);
@@ -319,7 +325,10 @@ __device__ __forceinline__ void fused_post_body(const FusedPostArgs &a, const VB
     }
 }
 
-__global__ void __launch_bounds__(256) fused_post_kernel(FusedPostArgs a) { fused_post_body(a, vb_single()); }
+__global__ void __launch_bounds__(256) fused_post_kernel(FusedPostArgs a) {
+    after_previous();
+    fused_post_body(a, vb_single());
+}
 __global__ void __launch_bounds__(256) fused_post_kernel_b(const FusedPostArgs *__restrict__ tab, VMap vm) {
     const VB vb = vb_batch(vm);
     fused_post_body(slot_entry(tab, vm.stride, vb.slot), vb);
@@ -352,7 +361,7 @@ elas_status launch_lr_check(int16_t *dL, int16_t *dR, int w, int h, int thr, uin
     const size_t smem = lr_smem(w);
     elas_status s = lr_smem_attr((const void *)lr_check_kernel, smem);
     if (s != ELAS_OK) return s;
-    lr_check_kernel<<<h, 256, smem, st>>>(LrArgs{dL, dR, w, h, thr, maskL, maskR});
+    launch_after(lr_check_kernel, h, 256, smem, st, LrArgs{dL, dR, w, h, thr, maskL, maskR});
     return launch_status("lr_check_kernel");
 }
 
@@ -386,13 +395,13 @@ dim3 post_grid(int w, int h) { return dim3((w + 31) / 32, (h + 7) / 8); }
 
 elas_status launch_post(const int16_t *d, int w, int h, const elas_params *p, float *out, void *ws, cudaStream_t st) {
     if (post_fusable(p)) {
-        fused_post_kernel<<<fused_post_grid(w, h), 256, 0, st>>>(fused_post_args(d, w, h, p, out));
+        launch_after(fused_post_kernel, fused_post_grid(w, h), 256, 0, st, fused_post_args(d, w, h, p, out));
         return launch_status("fused_post_kernel");
     }
     PostArgs passes[4];
     const int np = post_passes(d, w, h, p, out, ws, passes);
     for (int i = 0; i < np; ++i) {
-        post_pass_kernel<<<post_grid(w, h), dim3(32, 8), 0, st>>>(passes[i]);
+        launch_after(post_pass_kernel, post_grid(w, h), dim3(32, 8), 0, st, passes[i]);
         elas_status s = launch_status("post_pass_kernel");
         if (s != ELAS_OK) return s;
     }
@@ -558,6 +567,8 @@ __global__ void __launch_bounds__(256) median3_kernel(const int16_t *__restrict_
                                                       int16_t *__restrict__ out) {
     // a row holds the pixels x0 - 2 .. x0 + kMed3TX + 1
     __shared__ uint32_t s[kMed3TY + 2][kMed3W];
+    after_previous();
+    d = settled(d);
     const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
     const int x0 = blockIdx.x * kMed3TX, y0 = blockIdx.y * kMed3TY;
     if (kWide) {
@@ -656,9 +667,9 @@ extern "C" elas_status elas_median(const int16_t *d, int32_t w, int32_t h, int32
     if (radius == 1) {
         const dim3 tiles((w + kMed3TX - 1) / kMed3TX, (h + kMed3TY - 1) / kMed3TY);
         if (w % 2 == 0 && aligned(d, 4) && aligned(out, 4))
-            median3_kernel<true><<<tiles, 256, 0, to_stream(stream)>>>(d, w, h, out);
+            launch_after(median3_kernel<true>, tiles, 256, 0, to_stream(stream), d, w, h, out);
         else
-            median3_kernel<false><<<tiles, 256, 0, to_stream(stream)>>>(d, w, h, out);
+            launch_after(median3_kernel<false>, tiles, 256, 0, to_stream(stream), d, w, h, out);
         return launch_status("median3_kernel");
     }
     const dim3 grid((w + kMedTX - 1) / kMedTX, (h + kMedTY - 1) / kMedTY);

@@ -149,6 +149,7 @@ __device__ void sp_unite_shared(int *L, int a, int b, int32_t *status) {
 // to its root's count once (1920x1080: 24.7 us with a thread for each pixel's
 // link and addition, 23.7 with the additions of runs, 16.8 with the lists).
 __global__ void __launch_bounds__(32 * kSpWarps, 2048 / (32 * kSpWarps)) speckle_local_kernel(SpeckleArgs a) {
+    after_previous();
     __shared__ int sL[kSpCells];
     __shared__ int sC[kSpCells];  // run starts: the run's length, then roots: the segment's pixels
     __shared__ int16_t sD[kSpCells];
@@ -247,6 +248,7 @@ __global__ void __launch_bounds__(32 * kSpWarps, 2048 / (32 * kSpWarps)) speckle
 // rests on a link one row up or one column left, so the chain ends at a
 // processed link and no component loses a connection.
 __global__ void __launch_bounds__(256) speckle_border_kernel(SpeckleArgs a) {
+    after_previous();
     const int ntx = (a.w + kSpTX - 1) / kSpTX, nty = (a.h + kSpTY - 1) / kSpTY;
     const int nr = (ntx - 1) * a.h, nb = (nty - 1) * a.w;
     const int n = a.w * a.h, w = a.w, thr = a.thr;
@@ -288,6 +290,7 @@ __device__ __forceinline__ void sp_labels(const int32_t *label, int i0, int n, i
 }
 
 __global__ void __launch_bounds__(256) speckle_resolve_kernel(SpeckleArgs a) {
+    after_previous();
     const int n = a.w * a.h, i0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
     if (i0 >= n) return;
     int l[4];
@@ -308,6 +311,7 @@ __global__ void __launch_bounds__(256) speckle_resolve_kernel(SpeckleArgs a) {
 
 // kWide: 8-byte aligned maps, four pixels an access.
 template <bool kWide> __global__ void __launch_bounds__(256) speckle_apply_kernel(SpeckleArgs a) {
+    after_previous();
     const int n = a.w * a.h, i0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
     if (i0 >= n) return;
     const bool all = i0 + 4 <= n;
@@ -357,21 +361,21 @@ elas_status launch_speckle(const int16_t *d, int w, int h, int thr, int min_size
     a.min_size = min_size;
     if (cudaMemsetAsync(a.status, 0, sizeof(int32_t), st) != cudaSuccess) return launch_status("speckle status");
     const dim3 tiles((w + kSpTX - 1) / kSpTX, (h + kSpTY - 1) / kSpTY);
-    speckle_local_kernel<<<tiles, 32 * kSpWarps, 0, st>>>(a);
+    launch_after(speckle_local_kernel, tiles, 32 * kSpWarps, 0, st, a);
     elas_status s = launch_status("speckle_local_kernel");
     if (s != ELAS_OK) return s;
     const int ntx = (int)tiles.x, nty = (int)tiles.y;
     const int links = (ntx - 1) * h + (nty - 1) * w, quads = (w * h + 3) / 4;
     if (links > 0) {
-        speckle_border_kernel<<<min((links + 255) / 256, sm_count() * 8), 256, 0, st>>>(a);
+        launch_after(speckle_border_kernel, min((links + 255) / 256, sm_count() * 8), 256, 0, st, a);
         if ((s = launch_status("speckle_border_kernel")) != ELAS_OK) return s;
     }
-    speckle_resolve_kernel<<<(quads + 255) / 256, 256, 0, st>>>(a);
+    launch_after(speckle_resolve_kernel, (quads + 255) / 256, 256, 0, st, a);
     if ((s = launch_status("speckle_resolve_kernel")) != ELAS_OK) return s;
     if (aligned(d, 8) && aligned(out, 8))
-        speckle_apply_kernel<true><<<(quads + 255) / 256, 256, 0, st>>>(a);
+        launch_after(speckle_apply_kernel<true>, (quads + 255) / 256, 256, 0, st, a);
     else
-        speckle_apply_kernel<false><<<(quads + 255) / 256, 256, 0, st>>>(a);
+        launch_after(speckle_apply_kernel<false>, (quads + 255) / 256, 256, 0, st, a);
     return launch_status("speckle_apply_kernel");
 }
 

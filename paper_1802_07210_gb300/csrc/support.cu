@@ -123,8 +123,8 @@ __device__ __forceinline__ int warp_best_disparity(const uint4 *__restrict__ oth
 
 template <bool CENSUS> __device__ __forceinline__ void support_match_body(const MatchArgs &m, const VB &vb) {
     const SupportArgs &a = m.a;
-    const uint4 *__restrict__ dL = m.dL;
-    const uint4 *__restrict__ dR = m.dR;
+    const uint4 *__restrict__ dL = settled(m.dL);
+    const uint4 *__restrict__ dR = settled(m.dR);
     const int warp = (vb.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     const int w = a.w, wc = a.wc;
@@ -152,6 +152,7 @@ template <bool CENSUS> __device__ __forceinline__ void support_match_body(const 
 }
 
 template <bool CENSUS> __global__ void __launch_bounds__(512) support_match_kernel(MatchArgs m) {
+    after_previous();
     support_match_body<CENSUS>(m, vb_single());
 }
 
@@ -189,8 +190,8 @@ __host__ __device__ __forceinline__ SupRowSmem sup_row_smem(int nc, int dmin, in
 
 template <bool CENSUS> __device__ __forceinline__ void support_match_row_body(const MatchArgs &m, const VB &vb) {
     const SupportArgs &a = m.a;
-    const uint4 *__restrict__ dL = m.dL;
-    const uint4 *__restrict__ dR = m.dR;
+    const uint4 *__restrict__ dL = settled(m.dL);
+    const uint4 *__restrict__ dR = settled(m.dR);
     const int w = a.w, wc = a.wc, step = a.step, dmin = a.dmin, dmax = a.dmax;
     const int ic = vb.x, v = ic * step;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
@@ -308,6 +309,7 @@ template <bool CENSUS> __device__ __forceinline__ void support_match_row_body(co
 }
 
 template <bool CENSUS> __global__ void __launch_bounds__(512) support_match_row_kernel(MatchArgs m) {
+    after_previous();
     support_match_row_body<CENSUS>(m, vb_single());
 }
 // Batched launches: one launch per cost kind among the pairs.
@@ -367,6 +369,7 @@ __device__ __forceinline__ void consistency_body(const ConsArgs &c, const VB &vb
 }
 
 __global__ void __launch_bounds__(kConsTX *kConsTY) consistency_kernel(ConsArgs c) {
+    after_previous();
     consistency_body(c, vb_single());
 }
 __global__ void __launch_bounds__(kConsTX *kConsTY) consistency_kernel_b(const ConsArgs *__restrict__ tab, VMap vm) {
@@ -493,6 +496,7 @@ __device__ __forceinline__ void redundancy_grid_body(const RedArgs &ra, const VB
 }
 
 __global__ void __launch_bounds__(128) redundancy_grid_kernel(RedArgs ra, int staged) {
+    after_previous();
     redundancy_grid_body(ra, vb_single(), staged != 0);
 }
 __global__ void __launch_bounds__(128) redundancy_grid_kernel_b(const RedArgs *__restrict__ tab, VMap vm, int staged) {
@@ -540,7 +544,10 @@ __device__ __forceinline__ void compact_rows_body(const CompactArgs &ca, const V
     if (ic == hc - 1 && tid == 0) *ca.count = ca.keep_every > 1 ? (base + ca.keep_every - 1) / ca.keep_every : base;
 }
 
-__global__ void __launch_bounds__(128) compact_rows_kernel(CompactArgs ca) { compact_rows_body(ca, vb_single()); }
+__global__ void __launch_bounds__(128) compact_rows_kernel(CompactArgs ca) {
+    after_previous();
+    compact_rows_body(ca, vb_single());
+}
 
 // Grid vectors of a down-sampled list (the masks were cleared by the
 // consistency kernel): each point ORs its {d-1, d, d+1} bits into the 3x3
@@ -562,7 +569,10 @@ __device__ __forceinline__ void list_grid_body(const ListGridArgs &a, const VB &
         }
     }
 }
-__global__ void __launch_bounds__(128) list_grid_kernel(ListGridArgs a) { list_grid_body(a, vb_single()); }
+__global__ void __launch_bounds__(128) list_grid_kernel(ListGridArgs a) {
+    after_previous();
+    list_grid_body(a, vb_single());
+}
 __global__ void __launch_bounds__(128) list_grid_kernel_b(const ListGridArgs *__restrict__ tab, VMap vm) {
     const VB vb = vb_batch(vm);
     list_grid_body(slot_entry(tab, vm.stride, vb.slot), vb);
@@ -695,36 +705,34 @@ elas_status launch_support(const uint8_t *descL, const uint8_t *descR, int w, in
                                 : (const void *)support_match_row_kernel<false>;
         if ((s = sup_row_smem_attr(fn, row_smem)) != ELAS_OK) return s;
         if (census)
-            support_match_row_kernel<true><<<dim3(sa.match.a.hc, nseg), 32 * warps_per_block, row_smem, st>>>(
-                sa.match);
+            launch_after(support_match_row_kernel<true>, dim3(sa.match.a.hc, nseg), 32 * warps_per_block, row_smem, st, sa.match);
         else
-            support_match_row_kernel<false><<<dim3(sa.match.a.hc, nseg), 32 * warps_per_block, row_smem, st>>>(
-                sa.match);
+            launch_after(support_match_row_kernel<false>, dim3(sa.match.a.hc, nseg), 32 * warps_per_block, row_smem, st, sa.match);
         if ((s = launch_status("support_match_row_kernel")) != ELAS_OK) return s;
     } else {
         const dim3 grid = support_match_grid(sa.match, warps_per_block);
         if (census)
-            support_match_kernel<true><<<grid, 32 * warps_per_block, 0, st>>>(sa.match);
+            launch_after(support_match_kernel<true>, grid, 32 * warps_per_block, 0, st, sa.match);
         else
-            support_match_kernel<false><<<grid, 32 * warps_per_block, 0, st>>>(sa.match);
+            launch_after(support_match_kernel<false>, grid, 32 * warps_per_block, 0, st, sa.match);
         if ((s = launch_status("support_match_kernel")) != ELAS_OK) return s;
     }
     const size_t smem = consistency_smem(sa.cons.r);
     if ((s = consistency_smem_attr((const void *)consistency_kernel, smem)) != ELAS_OK) return s;
-    consistency_kernel<<<consistency_grid(sa.cons), dim3(kConsTX, kConsTY), smem, st>>>(sa.cons);
+    launch_after(consistency_kernel, consistency_grid(sa.cons), dim3(kConsTX, kConsTY), smem, st, sa.cons);
     if ((s = launch_status("consistency_kernel")) != ELAS_OK) return s;
     size_t red_smem = red_smem_bytes(sa.red.wc, sa.red.maxd, sa.red.g.gw, sa.red.g.nw);
     const int red_staged = red_smem <= kRedSmemMax;
     if (!red_staged) red_smem = 0;
     if ((s = red_smem_attr((const void *)redundancy_grid_kernel, red_smem)) != ELAS_OK) return s;
-    redundancy_grid_kernel<<<lattice_row_grid(sa.red.hc), 128, red_smem, st>>>(sa.red, red_staged);
+    launch_after(redundancy_grid_kernel, lattice_row_grid(sa.red.hc), 128, red_smem, st, sa.red, red_staged);
     if ((s = launch_status("redundancy_grid_kernel")) != ELAS_OK) return s;
-    compact_rows_kernel<<<lattice_row_grid(sa.compact.hc), 128, 0, st>>>(sa.compact);
+    launch_after(compact_rows_kernel, lattice_row_grid(sa.compact.hc), 128, 0, st, sa.compact);
     if ((s = launch_status("compact_rows_kernel")) != ELAS_OK) return s;
     if (sa.compact.keep_every <= 1) return ELAS_OK;
     int blocks = (sa.lg.cap + 127) / 128;
     if (blocks > sm_count() * 4) blocks = sm_count() * 4;
-    list_grid_kernel<<<blocks, 128, 0, st>>>(sa.lg);
+    launch_after(list_grid_kernel, blocks, 128, 0, st, sa.lg);
     return launch_status("list_grid_kernel");
 }
 
