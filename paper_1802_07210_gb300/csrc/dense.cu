@@ -13,12 +13,12 @@
 // raster_list_kernel   one thread per triangle: the chunks after the first
 //                      of a box go to the mesh's list of extra units (one
 //                      atomicAdd per triangle of more than one chunk);
-// raster_draw_kernel   half a warp per unit (grid-stride; unit t < ntri is
-//                      the first chunk of triangle t, the rest come from the
-//                      list), its lanes on 32 pixels of the box at a time: a
+// raster_draw_kernel   16 lanes per unit, 8 in batches (grid-stride; unit t <
+//                      ntri is the first chunk of triangle t, the rest come
+//                      from the list), each on every 16th (8th) pixel: a
 //                      pixel owned by the triangle (at most one owner: the
 //                      top-left rule) takes clamp(floor(plane + 0.5)).  A
-//                      full list makes the warp of a triangle's first chunk
+//                      full list makes the lanes of a triangle's first chunk
 //                      draw the whole box instead.
 // cell_kernel          one CTA per grid-vector cell (G x G pixels, which share
 //                      one candidate mask) and per reference image.  It
@@ -234,32 +234,54 @@ __global__ void __launch_bounds__(256) raster_list_kernel_b(const RasterArgs *__
 }
 
 // Lanes per unit in the draw kernel.  Boxes hold about 65 pixels, so a warp
-// per unit spent most of its instructions on the unit's constants; two units
-// a warp share them, and the edge functions step along with the pixel (64 x
-// 1242x375 prior stage 0.617 -> 0.531 ms, 1920x1080 63 -> 55 us; eight lanes
-// are as good in batches but slower at one 640x480 pair, 24 against 22 us).
-constexpr int kDrawLanes = 16;
+// per unit spent most of its instructions on the unit's constants; several
+// units a warp share them, and the edge functions step along with the pixel.
+// In batches, bound by instruction issue, eight lanes are the fewest
+// instructions (64 x 1242x375 with 4, 8 and 16 lanes: 334, 318 and 344 us;
+// about 500 with a warp per unit); one pair's units are too few to fill the chip with eight lanes
+// each (640x480 8.8 us against 7.5, 1920x1080 32.0 against 32.5).
+constexpr int kDrawLanes = 16, kDrawLanesBatch = 8;
 
-// Pixels [p0, p1) of the box of record r (row-major in the box), kDrawLanes
-// at a time across the unit's lanes.
+// Pixels [p0, p1) of the box of record r (row-major in the box), LANES at a
+// time across the unit's lanes.
+template <int LANES>
 __device__ __forceinline__ void raster_span(const RasterArgs &a, const RasterSide &S, const TriRec &r, const int4 &b,
                                             int p0, int p1, int lane) {
     const int bw = b.y - b.x + 1;
     int p = p0 + lane;
-    int y = b.z + p / bw, x = b.x + (p - (p / bw) * bw);
-    const int dy = kDrawLanes / bw, dx = kDrawLanes - dy * bw;
+    // p / bw and LANES / bw by one reciprocal: a quotient is at most the
+    // 16383 rows of an image, so it is off by less than one, which the
+    // remainder shows (two integer divisions a lane were a fifth of the
+    // kernel: 64 x 1242x375 with 16 lanes 418 -> 344 us)
+    const float inv = __fdividef(1.0f, (float)bw);
+    auto divide = [&](int n, int &rem) {
+        int q = (int)((float)n * inv);
+        rem = n - q * bw;
+        if (rem < 0) {
+            --q;
+            rem += bw;
+        } else if (rem >= bw) {
+            ++q;
+            rem -= bw;
+        }
+        return q;
+    };
+    int x, dx;
+    int y = b.z + divide(p, x);
+    x += b.x;
+    const int dy = divide(LANES, dx);
     // the edge functions step along with the pixel
     int e0 = r.A[0] * x + r.B[0] * y + r.C[0], e1 = r.A[1] * x + r.B[1] * y + r.C[1],
         e2 = r.A[2] * x + r.B[2] * y + r.C[2];
     const int s0 = r.A[0] * dx + r.B[0] * dy, s1 = r.A[1] * dx + r.B[1] * dy, s2 = r.A[2] * dx + r.B[2] * dy;
     const int w0 = r.B[0] - r.A[0] * bw, w1 = r.B[1] - r.A[1] * bw, w2 = r.B[2] - r.A[2] * bw;
-    for (; p < p1; p += kDrawLanes) {
+    for (; p < p1; p += LANES) {
         if (min(e0, min(e1, e2)) > 0) {
             const float t1 = __fmul_rn(r.fa, __int2float_rn(x));
             const float t2 = __fmul_rn(r.fb, __int2float_rn(y));
             const float mu = __fadd_rn(__fadd_rn(t1, t2), r.fc);
-            const int dp = __float2int_rz(floorf(__fadd_rn(mu, 0.5f)));
-            S.dplane[(size_t)y * a.w + x] = (int16_t)min(max(dp, a.dmin), a.dmax);
+            const int dp = __float2int_rd(__fadd_rn(mu, 0.5f));
+            S.dplane[y * a.w + x] = (int16_t)min(max(dp, a.dmin), a.dmax);
         }
         x += dx;
         y += dy;
@@ -276,10 +298,10 @@ __device__ __forceinline__ void raster_span(const RasterArgs &a, const RasterSid
     }
 }
 
-__device__ __forceinline__ void raster_draw_body(const RasterArgs &a, const VB &vb) {
+template <int LANES> __device__ __forceinline__ void raster_draw_body(const RasterArgs &a, const VB &vb) {
     const RasterSide &S = a.s[vb.y];
-    const int lane = threadIdx.x & (kDrawLanes - 1);
-    const int gid = (vb.x * blockDim.x + threadIdx.x) / kDrawLanes, ngroups = vb.gx * blockDim.x / kDrawLanes;
+    const int lane = threadIdx.x & (LANES - 1);
+    const int gid = (vb.x * blockDim.x + threadIdx.x) / LANES, ngroups = vb.gx * blockDim.x / LANES;
     const int ntri = side_ntri(S);
     const unsigned long long nextra = *S.nunits;
     const bool whole = nextra > (unsigned long long)a.unit_cap;  // the list is incomplete
@@ -294,17 +316,17 @@ __device__ __forceinline__ void raster_draw_body(const RasterArgs &a, const VB &
         const int4 b = S.rec[kRecWords * (size_t)t + 3];
         if (b.y < b.x || b.w < b.z) continue;
         const int area = (b.y - b.x + 1) * (b.w - b.z + 1);
-        raster_span(a, S, load_rec(S.rec, t), b, c * kUnitPx, whole ? area : min(area, (c + 1) * kUnitPx), lane);
+        raster_span<LANES>(a, S, load_rec(S.rec, t), b, c * kUnitPx, whole ? area : min(area, (c + 1) * kUnitPx), lane);
     }
 }
 
 __global__ void __launch_bounds__(256) raster_draw_kernel(RasterArgs a) {
     after_previous();
-    raster_draw_body(a, vb_single());
+    raster_draw_body<kDrawLanes>(a, vb_single());
 }
 __global__ void __launch_bounds__(256) raster_draw_kernel_b(const RasterArgs *__restrict__ tab, VMap vm) {
     const VB vb = vb_batch(vm);
-    raster_draw_body(slot_entry(tab, vm.stride, vb.slot), vb);
+    raster_draw_body<kDrawLanesBatch>(slot_entry(tab, vm.stride, vb.slot), vb);
 }
 
 
@@ -540,7 +562,7 @@ template <int TPP> __global__ void __launch_bounds__(kFusedThreads, 4) dense_fus
     grid.sync();
     for (int b = blockIdx.x; b < vmap_total(f.draw); b += nb) {
         const VB vb = vb_at(f.draw, b);
-        raster_draw_body(slot_entry(f.rtab, f.draw.stride, vb.slot), vb);
+        raster_draw_body<kDrawLanesBatch>(slot_entry(f.rtab, f.draw.stride, vb.slot), vb);
     }
     grid.sync();
     for (int b = blockIdx.x; b < vmap_total(f.cells[0]); b += nb) fused_cells<TPP, false>(f, f.cells[0], b);
