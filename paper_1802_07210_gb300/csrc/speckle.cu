@@ -5,7 +5,7 @@
 //
 // Connected components by union-find over pixel indices, every parent index
 // below its child's, so a root is the least pixel index of its tree:
-//   speckle_local_kernel   one CTA per 64x32 tile: union-find of the links
+//   speckle_local_kernel   one CTA per 64x32 or 64x16 tile: union-find of the links
 //                          inside the tile in shared memory.  A tile-local
 //                          root's label is its own global index and its size
 //                          entry its pixel count in the tile; another pixel's
@@ -27,10 +27,12 @@
 
 namespace elas {
 
-// Tiles of 64x32 rather than 32x16 halve the links across tile edges and
-// quarter the tile-local roots that those link (border pass at 1920x1080
-// 15.0 -> 10.8 us).
-constexpr int kSpTX = 64, kSpTY = 32, kSpCells = kSpTX * kSpTY, kSpWarps = 16, kSpRows = kSpTY / kSpWarps;
+// Tiles of 64 x TY pixels, 16 warps each.  Taller tiles have fewer links
+// across edges and fewer tile-local roots that those link, shorter ones more
+// CTAs, each with less to walk: 32 rows from a tile for every SM on, else 16
+// (local and border pass: 1920x1080 27.0 us with 32 rows, 29.2 with 16;
+// 320x240 11.8 and 10.9; with 32x16 tiles 39 and 10.9).
+constexpr int kSpTX = 64, kSpWarps = 16, kSpMaxCells = kSpTX * 32;
 
 struct SpeckleArgs {
     const int16_t *d;
@@ -99,7 +101,7 @@ __device__ __forceinline__ int sp_find_readonly(const int32_t *L, int x, int lim
 }
 
 __device__ __forceinline__ int sp_find_shared(volatile int *L, int x) {
-    for (int it = 0; it < kSpCells; ++it) {
+    for (int it = 0; it < kSpMaxCells; ++it) {
         const int p = L[x];
         if (p == x) return x;
         const int g = L[p];
@@ -111,7 +113,7 @@ __device__ __forceinline__ int sp_find_shared(volatile int *L, int x) {
 
 // Without writes, as sp_find_readonly and for the same reason.
 __device__ __forceinline__ int sp_find_shared_readonly(const volatile int *L, int x) {
-    for (int it = 0; it < kSpCells; ++it) {
+    for (int it = 0; it < kSpMaxCells; ++it) {
         const int p = L[x];
         if (p == x) return x;
         x = p;
@@ -120,7 +122,7 @@ __device__ __forceinline__ int sp_find_shared_readonly(const volatile int *L, in
 }
 
 __device__ void sp_unite_shared(int *L, int a, int b, int32_t *status) {
-    for (int it = 0; it < kSpCells; ++it) {
+    for (int it = 0; it < kSpMaxCells; ++it) {
         a = sp_find_shared(L, a);
         b = sp_find_shared(L, b);
         if (a < 0 || b < 0) break;
@@ -148,7 +150,9 @@ __device__ void sp_unite_shared(int *L, int a, int b, int32_t *status) {
 // run starts are listed, so that whole warps walk, and a run adds its length
 // to its root's count once (1920x1080: 24.7 us with a thread for each pixel's
 // link and addition, 23.7 with the additions of runs, 16.8 with the lists).
+template <int TY>
 __global__ void __launch_bounds__(32 * kSpWarps, 2048 / (32 * kSpWarps)) speckle_local_kernel(SpeckleArgs a) {
+    constexpr int kSpTY = TY, kSpCells = kSpTX * TY, kSpRows = TY / kSpWarps;
     after_previous();
     __shared__ int sL[kSpCells];
     __shared__ int sC[kSpCells];  // run starts: the run's length, then roots: the segment's pixels
@@ -240,14 +244,14 @@ __global__ void __launch_bounds__(32 * kSpWarps, 2048 / (32 * kSpWarps)) speckle
 }
 
 // Links across tile edges: first every right edge (x = 64k + 63, k =
-// 0..ntx-2) of every row, then every bottom edge (y = 32k + 31) of every
+// 0..ntx-2) of every row, then every bottom edge (y = TY k + TY - 1) of every
 // column.  A right-edge link is skipped where the link above it and the two
 // vertical links beside it connect the same pixels and those vertical links
 // lie inside a tile (not on a tile's first row); a bottom-edge link likewise
 // with the link to its left and horizontal links inside a tile.  Each skip
 // rests on a link one row up or one column left, so the chain ends at a
 // processed link and no component loses a connection.
-__global__ void __launch_bounds__(256) speckle_border_kernel(SpeckleArgs a) {
+template <int kSpTY> __global__ void __launch_bounds__(256) speckle_border_kernel(SpeckleArgs a) {
     after_previous();
     const int ntx = (a.w + kSpTX - 1) / kSpTX, nty = (a.h + kSpTY - 1) / kSpTY;
     const int nr = (ntx - 1) * a.h, nb = (nty - 1) * a.w;
@@ -275,70 +279,30 @@ __global__ void __launch_bounds__(256) speckle_border_kernel(SpeckleArgs a) {
     }
 }
 
-// Four pixels a thread: their labels come in one load, and the walks of the
-// four are in flight together.  1920x1080: resolve 7.3 us (6.6 before, when
-// the counts were also written and read for every pixel and the walks were
-// shorter), apply 5.8 -> 5.4.
-__device__ __forceinline__ void sp_labels(const int32_t *label, int i0, int n, int *l) {
-    if (i0 + 4 <= n) {
-        const int4 q = __ldcg(reinterpret_cast<const int4 *>(label + i0));
-        l[0] = q.x, l[1] = q.y, l[2] = q.z, l[3] = q.w;
-    } else {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) l[k] = i0 + k < n ? __ldcg(label + i0 + k) : -1;
-    }
-}
-
 __global__ void __launch_bounds__(256) speckle_resolve_kernel(SpeckleArgs a) {
     after_previous();
-    const int n = a.w * a.h, i0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
-    if (i0 >= n) return;
-    int l[4];
-    sp_labels(a.label, i0, n, l);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int i = i0 + k;
-        if (l[k] < 0 || l[k] == i) continue;  // not a tile-local root, or a final root
-        const int root = sp_find_readonly(a.label, l[k], n);
+    const int n = a.w * a.h;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const int l = __ldcg(a.label + i);
+        if (l < 0 || l == i) continue;  // not a tile-local root, or a final root
+        const int root = sp_find_readonly(a.label, l, n);
         if (root < 0) {
             atomicExch(a.status, 1);
             continue;
         }
-        __stcg(a.label + i, root);  // an ancestor: the forest stays valid
+        __stcg(a.label + i, root);            // an ancestor: the forest stays valid
         atomicAdd(a.size + root, a.size[i]);  // counts are added to final roots alone
     }
 }
 
-// kWide: 8-byte aligned maps, four pixels an access.
-template <bool kWide> __global__ void __launch_bounds__(256) speckle_apply_kernel(SpeckleArgs a) {
+__global__ void __launch_bounds__(256) speckle_apply_kernel(SpeckleArgs a) {
     after_previous();
-    const int n = a.w * a.h, i0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
-    if (i0 >= n) return;
-    const bool all = i0 + 4 <= n;
-    int r[4];
-    union {
-        uint2 v;
-        int16_t d[4];
-    } px;
-    sp_labels(a.label, i0, n, r);
-    if (kWide && all) {
-        px.v = *reinterpret_cast<const uint2 *>(a.d + i0);
-    } else {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) px.d[k] = i0 + k < n ? a.d[i0 + k] : (int16_t)-1;
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-        if (r[k] < -1) r[k] = a.label[-2 - r[k]];  // the tile-local root's final root (itself if it is one)
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-        if (r[k] < 0 || a.size[r[k]] < a.min_size) px.d[k] = -1;
-    if (kWide && all) {
-        *reinterpret_cast<uint2 *>(a.out + i0) = px.v;
-    } else {
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if (i0 + k < n) a.out[i0 + k] = px.d[k];
+    const int n = a.w * a.h;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        int r = a.label[i];
+        const int16_t dv = a.d[i];
+        if (r < -1) r = a.label[-2 - r];  // the tile-local root's final root (itself if it is one)
+        a.out[i] = r >= 0 && a.size[r] >= a.min_size ? dv : (int16_t)-1;
     }
 }
 
@@ -360,22 +324,22 @@ elas_status launch_speckle(const int16_t *d, int w, int h, int thr, int min_size
     a.thr = thr;
     a.min_size = min_size;
     if (cudaMemsetAsync(a.status, 0, sizeof(int32_t), st) != cudaSuccess) return launch_status("speckle status");
-    const dim3 tiles((w + kSpTX - 1) / kSpTX, (h + kSpTY - 1) / kSpTY);
-    launch_after(speckle_local_kernel, tiles, 32 * kSpWarps, 0, st, a);
+    const int ntx = (w + kSpTX - 1) / kSpTX;
+    const int ty = ntx * ((h + 31) / 32) >= sm_count() ? 32 : 16, nty = (h + ty - 1) / ty;
+    launch_after(ty == 32 ? speckle_local_kernel<32> : speckle_local_kernel<16>, dim3(ntx, nty), 32 * kSpWarps, 0, st,
+                 a);
     elas_status s = launch_status("speckle_local_kernel");
     if (s != ELAS_OK) return s;
-    const int ntx = (int)tiles.x, nty = (int)tiles.y;
-    const int links = (ntx - 1) * h + (nty - 1) * w, quads = (w * h + 3) / 4;
+    const int cap = sm_count() * 8, links = (ntx - 1) * h + (nty - 1) * w;
     if (links > 0) {
-        launch_after(speckle_border_kernel, min((links + 255) / 256, sm_count() * 8), 256, 0, st, a);
+        launch_after(ty == 32 ? speckle_border_kernel<32> : speckle_border_kernel<16>, min((links + 255) / 256, cap),
+                     256, 0, st, a);
         if ((s = launch_status("speckle_border_kernel")) != ELAS_OK) return s;
     }
-    launch_after(speckle_resolve_kernel, (quads + 255) / 256, 256, 0, st, a);
+    const int blocks = min((w * h + 255) / 256, cap);
+    launch_after(speckle_resolve_kernel, blocks, 256, 0, st, a);
     if ((s = launch_status("speckle_resolve_kernel")) != ELAS_OK) return s;
-    if (aligned(d, 8) && aligned(out, 8))
-        launch_after(speckle_apply_kernel<true>, (quads + 255) / 256, 256, 0, st, a);
-    else
-        launch_after(speckle_apply_kernel<false>, (quads + 255) / 256, 256, 0, st, a);
+    launch_after(speckle_apply_kernel, blocks, 256, 0, st, a);
     return launch_status("speckle_apply_kernel");
 }
 

@@ -38,8 +38,8 @@ def _map(w, h, holes, top=60, seed=0):
     return d
 
 
-# sizes around the 64x16 and 64x32 tiles, even and odd widths
-FILTER_SIZES = [(1, 1), (2, 1), (63, 15), (64, 16), (65, 17), (66, 31), (128, 32), (129, 33), (190, 65)]
+# sizes around the 64x16 and (from 152 tiles on) 64x32 tiles, even and odd widths
+FILTER_SIZES = [(1, 1), (2, 1), (63, 15), (64, 16), (65, 17), (66, 31), (128, 32), (129, 33), (190, 65), (1217, 257)]
 
 
 @pytest.mark.parametrize("size", FILTER_SIZES)
