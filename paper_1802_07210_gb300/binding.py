@@ -17,8 +17,11 @@ from ._lib import (BatchConfig, ElasError, Params, PipelineStats, ServerConfig, 
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    # the current stream's handle without a Stream object around it: 3 us less
+    # a call (descriptors and support points of 1013x547: 91 -> 69 us)
+    if stream is None:
+        return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+    return C.c_void_p(stream.cuda_stream)
 
 
 def _dev(t, dtype, name, shape=None):
