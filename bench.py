@@ -50,11 +50,11 @@ METRIC = "Mpix/s & pairs/s at 640x480 D=256; p50/p99 served latency vs per-pair 
 WORKLOADS = {"vga_640": (synth.VGA_640, 2), "small_320": (synth.SMALL_320, 1),
              "kitti_1242": (synth.KITTI_1242, 3)}
 # kernels of one plain step: descriptors 1; support 4 (match, consistency,
-# redundancy + grids, compaction); triangulation 10 (init, points, cell scan,
-# scatter, dedup, group pass, CTA pass, triangle scan, emit, emit big); plane
+# redundancy + grids, compaction); triangulation 9 (init, points, cell scan,
+# scatter, dedup, warp pass, CTA pass, triangle scan, emit); plane
 # prior 3 (setup, extra-unit list, draw); dense 1; LR 1; post-processing 1
 # (fused) or 0.  No memsets.
-KERNELS_PER_STEP = {True: 21, False: 20}
+KERNELS_PER_STEP = {True: 20, False: 19}
 STAGES = ("descriptors", "support", "triangulation", "plane_prior", "dense_argmin", "lr_post")
 # bytes a dense launch must move at least: both descriptor images read once
 # (32 B/px), the two prior maps read (4 B/px), the two maps written (4 B/px)
@@ -342,7 +342,7 @@ def run_batch_section(B, torch, dev, stream, flush, steps, npairs, distinct, pea
             "ms_per_batch": t_b, "pairs_per_s": npairs / (t_b * 1e-3), "mpix_per_s": npairs * w * h / (t_b * 1e-3) / 1e6,
             "plain_ms_per_batch": t_p, "plain_pairs_per_s": npairs / (t_p * 1e-3),
             "speedup_vs_plain": t_p / t_b, "tuned": tuned, "stages_ms": stage, "support_points_first": nsup[:4],
-            "launches_per_batch": 21, "graph": True,
+            "launches_per_batch": 20, "graph": True,
             "l2": "flushed before every timed batch", "roofline_dense": roof}
 
 

@@ -54,7 +54,7 @@ void prior_table(const elas_params *p, int32_t *P);
 // their places while the last ones of the kernel before it in the stream
 // still run, so the launch's own latency is hidden behind that kernel (the
 // triangulation is nine kernels of 1 to 40 us: 1242x375, both sides one call
-// each, 177 -> 141 us; LR check to speckle removal of 1920x1080 91 -> 82).  A
+// each, 180 -> 151 us; LR check to speckle removal of 1920x1080 91 -> 80).  A
 // kernel launched without it, a copy or an event waits for the whole kernel
 // as ever.  Under capture it is an ordinary launch: a graph's own edges are as
 // quick (640x480, twenty kernels: 143 us with them, 140 to 150 with early

@@ -22,10 +22,10 @@
 // counts, and within a star counter-clockwise from the nearest neighbour (an
 // open star then clockwise from it).
 //
-// One step of the earlier design (4 or 16 lanes per star, the whole star,
-// 64-bit key comparisons, one region scan per step of a wide star) against
-// this one: 640x480 172 -> 96 us, 1920x1080 590 -> 276 us, 64 x 1242x375
-// 3.44 -> 1.82 ms for all triangulation kernels.
+// The earlier design (4 or 16 lanes per star, the whole star, 64-bit key
+// comparisons, one region scan per step of a wide star) against this one, all
+// triangulation kernels: 640x480 172 -> 69 us, 1920x1080 590 -> 207 us,
+// 64 x 1242x375 3.44 -> 1.33 ms.
 #include "launch.cuh"
 
 namespace elas {
@@ -784,7 +784,9 @@ __device__ __forceinline__ bool dt_warp_star(const DtArgs &a, const DtSide &S, c
 }
 
 // Warp pass: one warp per point, the candidates within 24 pixels (16 or 8
-// where there are more than 64).  Bound by instruction issue.
+// where there are more than 64).  Bound by instruction issue; 64 x 1242x375
+// 685 us for 0.77 M stars, 640x480 10 (whole stars by 4 or 16 lanes each: 1,590
+// and 47), 1920x1080 67.
 __device__ __forceinline__ void dt_pass1_body(const DtArgs &a, const VB &vb) {
     constexpr int kRows = 2 * kDtRadius / kDtCell + 1;  // cell rows (and columns) the disc's square meets
     static_assert(2 * kDtRadius % kDtCell == 0, "the square of a disc spans kRows rows wherever it lies");
@@ -911,6 +913,12 @@ __global__ void __launch_bounds__(kDtWarpsM * 32, 7) dt_pass2_kernel_b(const DtA
 // with a stride, which finds points that shrink the circles to a small part
 // of it.  A full cache keeps only the star's own vertices and goes on with
 // the whole star (its region can only shrink, so that ends).
+//
+// Bound by the latency of the stars' own chains (a step over the cache is
+// about 800 cycles, two warps of the CTA at work; a scan 5,000 to 20,000) and,
+// from several thousand stars on, by issue: 640x480 94 -> 38 us with 1,050
+// stars, one for each resident CTA, the longest 39 us; 1920x1080 5,500 stars,
+// 110 us; 64 x 1242x375 after the middle pass 920 -> 325 us.
 constexpr int kDtRadiusC = 48;
 constexpr int kDtSamples = 64;     // points of the whole set cached too
 constexpr int kDtCacheCap = 1024;   // cached points (16 KB)
@@ -1821,7 +1829,7 @@ elas_status launch_triangulate_device(const int16_t *list, const int32_t *count,
     launch_after(dt_pass1_kernel, dim3(max(1, min((cap + kDtWarps - 1) / kDtWarps, sm_count() * 16)), nsides), kDtWarps * 32, 0, st, a);
 
     // no middle pass: it would add its longest star's time to the CTA pass's
-    // (640x480 115 against 78 us)
+    // (640x480 38 us alone, 37 + 37 with it; 1920x1080 126 and 52 + 74)
     const int smem = kDtCacheCap * (int)sizeof(float4) + 2 * a.gh * (int)sizeof(int);
     if (cudaFuncSetAttribute(dt_pass_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
         return launch_status("dt_pass_block_kernel shared memory attribute");

@@ -3,12 +3,13 @@
 // one-hot masks, Sec. VI.D) and raster-order compaction.
 //
 // Kernels, in launch order:
-//   support_match_row_kernel  one CTA per lattice row: warps hold 32 right
-//                           windows each and walk the row's candidates
+//   support_match_row_kernel  (batches and one large pair: sup_by_rows) one
+//                           CTA per lattice row or part of one: warps hold 32
+//                           right windows each and walk the candidates
 //                           (below); the re-match is one warp per candidate.
-//   support_match_kernel    (rows too wide for the row kernel's shared
-//                           memory) one warp per lattice candidate; lanes
-//                           stride the disparity range, each lane keeps
+//   support_match_kernel    (too few rows, or rows too wide for the row
+//                           kernel's shared memory) one warp per lattice
+//                           candidate; lanes stride the disparity range, each lane keeps
 //                           (best, second) and the warp merges them with two
 //                           min-reductions; the right-to-left re-match runs
 //                           in the same warp.
@@ -17,11 +18,12 @@
 //                           the grid-vector masks.
 //   redundancy_grid_kernel  one lattice row per CTA: four directional scans
 //                           over the rows within maxd (staged in shared
-//                           memory), atomicOr of the {d-1,d,d+1} bits of every
-//                           surviving point into the 3x3 cells around it (in
-//                           shared memory, then one global atomic per word;
-//                           OR is order free, so the masks are
-//                           deterministic), and the row's point count.
+//                           memory), the {d-1,d,d+1} bits of every surviving
+//                           point for the 3x3 cells around it (its own cell
+//                           in shared memory, the others by widening each
+//                           word on its way to the grid; OR is order free, so
+//                           the masks are deterministic), and the row's point
+//                           count.
 //   compact_rows_kernel     one lattice row per CTA: offset = points in the
 //                           rows above, ballot-based placement; raster order.
 #include "launch.cuh"
