@@ -2,7 +2,8 @@
 their tiles and of the rules, against the oracle: support matching by parts of
 lattice rows, the 3x3 median and small-segment removal (word accesses or not),
 the LR check (one or two pixels an access), the fused post-processing tile and
-the prior of triangles much larger than the units they are drawn in."""
+the prior of triangles much larger than the units they are drawn in, and chains
+of calls whose kernels start early."""
 import numpy as np
 import pytest
 
@@ -180,3 +181,49 @@ def test_prior_of_few_large_triangles(n, right):
     exp = oracle.plane_prior(lst, tri, w, h, prm, right=right)
     out = _B().elas_plane_prior(dev(lst), dev(tri), w, h, prm, right=right)
     np.testing.assert_array_equal(host(out), exp)
+
+
+def _calls(B, L, R, prm, stream=None):
+    """Every single-stage call of a pair after the other, as a program without
+    the pipeline makes them (capacities in place of counts: no copy to the host)."""
+    dl, dr = B.elas_descriptors(L, R, stream=stream)
+    s = B.elas_support_points(dl, dr, prm, stream=stream)
+    h, w = L.shape
+    tri = [B.elas_triangulate_device(s["list"], s["count"], w, h, right, stream=stream) for right in (False, True)]
+    d = B.elas_dense_argmin(dl, dr, dict(prm, flags=2), stream=stream)
+    dR = B.elas_dense_argmin(dl, dr, dict(prm, flags=2), right=True, stream=stream)
+    B.elas_lr_check(d, dR, 2, masks=False, stream=stream)
+    post = B.elas_postprocess(d, prm, stream=stream)
+    return [s["d_can"], s["count"], s["grid_L"], s["grid_R"], tri[0][1], tri[1][1], d, dR, post,
+            B.elas_median(d, 1, stream=stream), B.elas_speckle(d, 1, 20, stream=stream)]
+
+
+def test_chains_of_calls_on_streams_and_captured():
+    """The calls' kernels may take their places before the one ahead of them
+    ends: chains over changing inputs, queued without a stop on one stream, on
+    two streams in turn and replayed from a graph, give what a chain with a
+    synchronisation after it gives."""
+    B = _B()
+    prm = dict(disp_max=47, ipol_gap_width=3, filter_adaptive_mean=1)
+    pairs = [tuple(dev(a) for a in _support(203 + 64 * k, 117, prm)) for k in range(3)]
+    alone = []
+    for L, R in pairs:
+        alone.append([t.clone() for t in _calls(B, L, R, prm)])
+        torch.cuda.synchronize()
+    got = [(k % 3, _calls(B, *pairs[k % 3], prm)) for k in range(24)]
+    side = [torch.cuda.Stream(), torch.cuda.Stream()]
+    torch.cuda.synchronize()
+    for k in range(24):
+        with torch.cuda.stream(side[k % 2]):
+            got.append((k % 3, _calls(B, *pairs[k % 3], prm)))
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=side[0]):
+        out = _calls(B, *pairs[1], prm, stream=side[0])
+    for _ in range(3):
+        g.replay()
+    torch.cuda.synchronize()
+    got.append((1, out))
+    for k, res in got:
+        for a, b in zip(res, alone[k]):
+            np.testing.assert_array_equal(host(a), host(b))
