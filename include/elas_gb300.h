@@ -272,7 +272,9 @@ elas_status elas_triangulate(const int16_t *list, int32_t n, int32_t right, int3
  * indices, coincident right-image points keep the lowest index).  Each point
  * builds its own star by exact gift-wrapping among its neighbours, certified
  * by the circumdisc test; uncertified stars are redone with a larger radius.
- * list: device int16 [cap][3] with 0 <= v < h (u - d may be negative);
+ * list: device int16 [cap][3] with 0 <= v < h (u - d may be negative), the
+ * points' extents X and Y with X^2 + Y^2 < 2^31 (else *ntri = -1; any list of
+ * an image and disparities up to 1,023 meets it);
  * count: device int32, number of points (<= cap); right: 0 = (u, v),
  * 1 = (u - d, v).  Outputs on the device: tri int32
  * [cap_tri][3] (counter-clockwise, each triangle once, deterministic order),

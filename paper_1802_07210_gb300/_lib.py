@@ -132,6 +132,7 @@ SIGNATURES = {
     "elas_server_inject_alloc_failures": (C.c_int, [_P, _I]),
     "elas_server_destroy": (None, [_P]),
     "elas_probe_sad16": (C.c_int, [_I, _I, _I, _I, _P, _P]),
+    "elas_probe_triangulate_pool": (C.c_int, [_P, _P, _I, _I, _I, _I, _P, _I, _P, _P, _Z, _I, _P]),
 }
 
 _lib = None

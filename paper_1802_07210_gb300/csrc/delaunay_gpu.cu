@@ -26,11 +26,30 @@
 // comparisons, one region scan per step of a wide star) against this one, all
 // triangulation kernels: 640x480 172 -> 69 us, 1920x1080 590 -> 207 us,
 // 64 x 1242x375 3.44 -> 1.33 ms.
+#include <climits>
+
 #include "launch.cuh"
+#include "elas_probe.h"
 
 namespace elas {
 
 constexpr int kDtCell = 16;
+
+// Bits of DtSide::err.  Pool and range: the triangulation fails (ntri = -1).
+constexpr int kDtErrPool = 4;    // the pool has no room for a fan
+constexpr int kDtErrOrder = 8;   // the list is not in raster order
+constexpr int kDtErrBox = 16;    // a point lies outside the box below
+constexpr int kDtErrRange = 32;  // the points lie too far apart for the integer steps
+
+// The integer steps are exact, and so the stars agree with one another, while
+// X^2 + Y^2 < 2^31 for the extents X and Y of the points: |N| = |c.(c - e)| and
+// |c|^2 are at most that, D at most X Y.  Points inside this box meet it, and
+// it holds every point of an image and its disparities; the extents are only
+// taken (dt_cell_scan_body) when a point lies outside.
+constexpr int kDtBoxX0 = -8192, kDtBoxX1 = 32767, kDtBoxY0 = -4096, kDtBoxY1 = 17407;
+static_assert((int64_t)(kDtBoxX1 - kDtBoxX0) * (kDtBoxX1 - kDtBoxX0) +
+                      (int64_t)(kDtBoxY1 - kDtBoxY0) * (kDtBoxY1 - kDtBoxY0) < (int64_t)1 << 31,
+              "points of the box meet the integer steps' range");
 
 __device__ __forceinline__ int dt_ncell(const DtArgs &a) { return a.gw * a.gh; }
 
@@ -52,7 +71,8 @@ __device__ __forceinline__ void dt_points_body(const DtArgs &a, const VB &vb) {
         S.X[i] = x;
         S.Y[i] = v;
         S.owned[i] = 0;
-        if (i > 0 && a.list[3 * i - 2] > v) atomicOr(S.err, 8);  // not in raster order
+        if (i > 0 && a.list[3 * i - 2] > v) atomicOr(S.err, kDtErrOrder);
+        if (x < kDtBoxX0 || x > kDtBoxX1 || v < kDtBoxY0 || v > kDtBoxY1) atomicOr(S.err, kDtErrBox);
         atomicAdd(S.cell_cnt + dt_cell(a, x, v), 1);
         // the lanes of one image row (a run of the raster-ordered list) take
         // its extremes with one atomic each
@@ -126,14 +146,37 @@ template <class Put> __device__ __forceinline__ int dt_block_scan(const int32_t 
     return total;
 }
 
+// Sets kDtErrRange when the points' extents are beyond the integer steps.
+__device__ __noinline__ void dt_check_extents(const DtSide &S, int n) {
+    __shared__ int s_ext[4];
+    if (threadIdx.x < 4) s_ext[threadIdx.x] = threadIdx.x & 1 ? INT_MIN : INT_MAX;
+    __syncthreads();
+    int x0 = INT_MAX, x1 = INT_MIN, y0 = INT_MAX, y1 = INT_MIN;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        x0 = min(x0, S.X[i]);
+        x1 = max(x1, S.X[i]);
+        y0 = min(y0, S.Y[i]);
+        y1 = max(y1, S.Y[i]);
+    }
+    atomicMin(&s_ext[0], x0);
+    atomicMax(&s_ext[1], x1);
+    atomicMin(&s_ext[2], y0);
+    atomicMax(&s_ext[3], y1);
+    __syncthreads();
+    const int64_t ex = (int64_t)s_ext[1] - s_ext[0], ey = (int64_t)s_ext[3] - s_ext[2];
+    if (threadIdx.x == 0 && ex * ex + ey * ey >= (int64_t)1 << 31) atomicOr(S.err, kDtErrRange);
+}
+
 // One CTA per side: where each cell's points start; entry ncell is the total
 // (its own count stays 0).  The arrays are padded to 16 bytes.
 __device__ __forceinline__ void dt_cell_scan_body(const DtArgs &a, const VB &vb) {
     const DtSide &S = a.s[vb.y];
+    const int err = *S.err;  // in flight during the scan
     dt_block_scan(S.cell_cnt, dt_ncell(a) + 1, [&](int i, const int4 &before) {
         *reinterpret_cast<int4 *>(S.cell_start + i) = before;
         *reinterpret_cast<int4 *>(S.cell_fill + i) = before;
     });
+    if (err & kDtErrBox) dt_check_extents(S, min(max(*a.count, 0), a.cap));
 }
 
 __global__ void __launch_bounds__(1024) dt_cell_scan_kernel(DtArgs a) {
@@ -148,10 +191,11 @@ __global__ void __launch_bounds__(1024) dt_cell_scan_kernel_b(const DtArgs *__re
 __device__ __forceinline__ void dt_scatter_body(const DtArgs &a, const VB &vb) {
     const DtSide S = vb.y ? a.s[1] : a.s[0];
     const int n = min(max(*a.count, 0), a.cap);
+    const int alive = !(*S.err & kDtErrRange);  // else no point has a star: every queue stays empty
     for (int i = vb.x * blockDim.x + threadIdx.x; i < n; i += vb.gx * blockDim.x) {
         const int x = S.X[i], y = S.Y[i];
         const int k = atomicAdd(S.cell_fill + dt_cell(a, x, y), 1);
-        S.pts[k] = make_int4(x, y, i, 1);
+        S.pts[k] = make_int4(x, y, i, alive);
         S.slot[i] = k;
     }
 }
@@ -658,6 +702,20 @@ __device__ __forceinline__ bool dt_wide_step(const DtArgs &a, const DtSide &S, c
 // vertex r of the fan (0 when it is none of its vertices).
 __device__ __forceinline__ int dt_fan_pos(int t, int m, int r) { return t >= r ? t - r : t + m - r; }
 
+// Room in the pool for the m > kDtSlots owned triangles of point pz (one
+// thread): their first entry, which the point's slots then name, or -1 when
+// there is none and the triangulation fails.  Stars that agree own fewer than
+// two triangles a point in all, which the pool holds.
+__device__ __forceinline__ int dt_pool_room(const DtSide &S, int pz, int m) {
+    const int base = atomicAdd(S.npool, m);
+    if (base < 0 || m > S.pool_cap - base) {
+        atomicOr(S.err, kDtErrPool);
+        return -1;
+    }
+    S.slots[(size_t)pz * kDtSlots] = make_int2(base, 0);
+    return base;
+}
+
 // The owned triangles of a star whose vertices sit one per lane: a[0..na]
 // counter-clockwise from the first vertex, b[0..nb] clockwise from it.
 __device__ __forceinline__ void dt_warp_write(const DtSide &S, int pz, int lane, bool fan, int va, int vb, int na,
@@ -677,11 +735,10 @@ __device__ __forceinline__ void dt_warp_write(const DtSide &S, int pz, int lane,
     int2 *out = S.slots + (size_t)pz * kDtSlots;
     if (m > kDtSlots) {
         int base = 0;
-        if (lane == 0) {
-            base = atomicAdd(S.npool, m);
-            *out = make_int2(base, 0);
-        }
-        out = S.pool + __shfl_sync(0xFFFFFFFFu, base, 0);
+        if (lane == 0) base = dt_pool_room(S, pz, m);
+        base = __shfl_sync(0xFFFFFFFFu, base, 0);
+        if (base < 0) return;
+        out = S.pool + base;
     }
     if (oa) out[pa] = make_int2(va, va1);
     if (ob) out[pb] = make_int2(vb1, vb);
@@ -795,7 +852,7 @@ __device__ __forceinline__ void dt_pass1_body(const DtArgs &a, const VB &vb) {
     const int n = min(max(*a.count, 0), a.cap);
     const int lane = threadIdx.x & 31;
     float4 *list = s_list[threadIdx.x >> 5];
-    const bool ordered = !(*S.err & 8);
+    const bool ordered = !(*S.err & kDtErrOrder);
     for (int j = vb.x * kDtWarps + (threadIdx.x >> 5); j < n; j += vb.gx * kDtWarps) {
         const int4 p = S.pts[j];
         if (!p.w) continue;
@@ -859,7 +916,7 @@ __device__ __forceinline__ void dt_pass2_body(const DtArgs &a, const VB &vb) {
     const DtSide &S = a.s[vb.y];
     const int lane = threadIdx.x & 31;
     float4 *list = s_list[threadIdx.x >> 5];
-    const bool ordered = !(*S.err & 8);
+    const bool ordered = !(*S.err & kDtErrOrder);
     const int njobs = *S.npending;
     for (int j = vb.x * kDtWarpsM + (threadIdx.x >> 5); j < njobs; j += vb.gx * kDtWarpsM) {
         const int at = S.pending[j];
@@ -1232,11 +1289,10 @@ __device__ __forceinline__ void dt_block_write(const DtSide &S, int pz, bool fan
     int2 *out = S.slots + (size_t)pz * kDtSlots;
     if (m > kDtSlots) {
         int base = 0;
-        if (lane == 0) {
-            base = atomicAdd(S.npool, m);
-            *out = make_int2(base, 0);
-        }
-        out = S.pool + __shfl_sync(0xFFFFFFFFu, base, 0);
+        if (lane == 0) base = dt_pool_room(S, pz, m);
+        base = __shfl_sync(0xFFFFFFFFu, base, 0);
+        if (base < 0) return;
+        out = S.pool + base;
     }
     int done = 0;
     for (int t0 = 0; t0 < nt; t0 += 32) {
@@ -1302,11 +1358,9 @@ __device__ __noinline__ void dt_block_star_all(const DtSide &S, const int4 &p, i
             m = written;
             out = S.slots + (size_t)p.z * kDtSlots;
             if (m > kDtSlots) {
-                if (threadIdx.x == 0) {
-                    sh.total = atomicAdd(S.npool, m);
-                    *out = make_int2(sh.total, 0);
-                }
+                if (threadIdx.x == 0) sh.total = dt_pool_room(S, p.z, m);
                 __syncthreads();
+                if (sh.total < 0) return;
                 out = S.pool + sh.total;
             }
         }
@@ -1619,7 +1673,7 @@ __global__ void __launch_bounds__(kDtBlockThreads, kDtBlocksPerSM) dt_pass_block
         const int side = two ? (item & 1) : (nq0 > nq1 ? 0 : 1);
         const int idx = two ? (item >> 1) : item - m;
         const DtSide &S = a.s[side];
-        dt_block_item(a, S, S.pending[idx], n, !(*S.err & 8), s_cand, r_start, r_start + a.gh, sh);
+        dt_block_item(a, S, S.pending[idx], n, !(*S.err & kDtErrOrder), s_cand, r_start, r_start + a.gh, sh);
     }
 }
 
@@ -1689,7 +1743,7 @@ __global__ void __launch_bounds__(kDtBlockThreads, kDtBlocksPerSM)
         const DtSide &S = a.s[lo % nsides];
         const int n = min(max(*a.count, 0), a.cap);
         const int at = (second ? S.pending2 : S.pending)[item - s_pre[lo]];
-        dt_block_item(a, S, at, n, !(*S.err & 8), s_cand, r_start, r_start + a.gh, sh);
+        dt_block_item(a, S, at, n, !(*S.err & kDtErrOrder), s_cand, r_start, r_start + a.gh, sh);
     }
 }
 
@@ -1699,7 +1753,8 @@ __device__ __forceinline__ void dt_tri_scan_body(const DtArgs &a, const VB &vb) 
     const int total = dt_block_scan(S.owned, min(max(*a.count, 0), a.cap), [&](int i, const int4 &before) {
         *reinterpret_cast<int4 *>(S.offset + i) = before;
     });
-    if (threadIdx.x == 0) *S.ntri = total > a.cap_tri ? -1 : total;  // -1: the triangulation failed
+    const bool failed = total > a.cap_tri || *S.err & (kDtErrPool | kDtErrRange);
+    if (threadIdx.x == 0) *S.ntri = failed ? -1 : total;
 }
 
 __global__ void __launch_bounds__(1024) dt_tri_scan_kernel(DtArgs a) {
@@ -1760,6 +1815,8 @@ size_t dt_side_bytes(int cap, int w, int h) {
            2 * align_up(c * 4, 256) + 2 * align_up((size_t)h * 4, 256) + align_up(kDtCounters * 4, 256);
 }
 
+static int dt_pool_cap(int cap) { return 2 * (cap > 0 ? cap : 1); }  // a mesh has fewer than 2n triangles
+
 static DtSide dt_carve(void *ws, int cap, int w, int h) {
     int gw, gh;
     dt_geom(w, h, gw, gh);
@@ -1782,7 +1839,8 @@ static DtSide dt_carve(void *ws, int cap, int w, int h) {
     s.owned = reinterpret_cast<int32_t *>(take(c * 4));
     s.offset = reinterpret_cast<int32_t *>(take(c * 4));
     s.slots = reinterpret_cast<int2 *>(take(c * kDtSlots * 8));
-    s.pool = reinterpret_cast<int2 *>(take(2 * c * 8));  // a mesh has fewer than 2n triangles
+    s.pool = reinterpret_cast<int2 *>(take((size_t)dt_pool_cap(cap) * 8));
+    s.pool_cap = dt_pool_cap(cap);
     s.pending = reinterpret_cast<int32_t *>(take(c * 4));
     s.pending2 = reinterpret_cast<int32_t *>(take(c * 4));
     s.rowmin = reinterpret_cast<int32_t *>(take((size_t)h * 4));
@@ -1801,7 +1859,7 @@ __global__ void __launch_bounds__(256) dt_init_kernel(DtArgs a);
 // Triangulates one or both sides.  sides[i] = right flag; tri/ntri per side.
 elas_status launch_triangulate_device(const int16_t *list, const int32_t *count, int cap, int w, int h, int nsides,
                                       const int *rights, int32_t *const *tri, int32_t *const *ntri, int cap_tri,
-                                      void *ws, cudaStream_t st) {
+                                      void *ws, cudaStream_t st, int pool_cap) {
     DtArgs a{};
     a.list = list;
     a.count = count;
@@ -1816,6 +1874,7 @@ elas_status launch_triangulate_device(const int16_t *list, const int32_t *count,
         a.s[i].right = rights[i];
         a.s[i].tri = tri[i];
         a.s[i].ntri = ntri[i];
+        if (pool_cap >= 0) a.s[i].pool_cap = min(pool_cap, a.s[i].pool_cap);
     }
     // counters, cell counts and row extremes of both sides: one kernel
     const int nall = a.gw * a.gh + 1 + 2 * h + kDtCounters;
@@ -1952,11 +2011,11 @@ extern "C" size_t elas_triangulate_device_workspace_bytes(int32_t cap, int32_t w
     return elas::triangulate_device_workspace(cap, w, h, 1);
 }
 
-extern "C" elas_status elas_triangulate_device(const int16_t *list, const int32_t *count, int32_t cap, int32_t w,
-                                               int32_t h, int32_t right, int32_t *tri, int32_t cap_tri,
-                                               int32_t *ntri, void *workspace, size_t workspace_bytes,
-                                               elas_stream stream) {
-    using namespace elas;
+namespace elas {
+// The C entry; pool_cap >= 0: room for only so many triangles of large fans.
+static elas_status triangulate_entry(const int16_t *list, const int32_t *count, int32_t cap, int32_t w, int32_t h,
+                                     int32_t right, int32_t *tri, int32_t cap_tri, int32_t *ntri, void *workspace,
+                                     size_t workspace_bytes, int32_t pool_cap, elas_stream stream) {
     if (w < 1 || h < 1 || w > 16383 || h > 16383) return fail(ELAS_ERR_INVALID_ARG, "image size %dx%d", w, h);
     if (!list || !count || !tri || !ntri || !workspace) return fail(ELAS_ERR_INVALID_ARG, "NULL buffer");
     if (cap < 0 || cap_tri < 2 * cap + 8)
@@ -1969,5 +2028,23 @@ extern "C" elas_status elas_triangulate_device(const int16_t *list, const int32_
     int32_t *tris[1] = {tri};
     int32_t *nts[1] = {ntri};
     return launch_triangulate_device(list, count, cap, w, h, 1, rights, tris, nts, cap_tri, workspace,
-                                     to_stream(stream));
+                                     to_stream(stream), pool_cap);
+}
+}  // namespace elas
+
+extern "C" elas_status elas_triangulate_device(const int16_t *list, const int32_t *count, int32_t cap, int32_t w,
+                                               int32_t h, int32_t right, int32_t *tri, int32_t cap_tri,
+                                               int32_t *ntri, void *workspace, size_t workspace_bytes,
+                                               elas_stream stream) {
+    return elas::triangulate_entry(list, count, cap, w, h, right, tri, cap_tri, ntri, workspace, workspace_bytes, -1,
+                                   stream);
+}
+
+extern "C" elas_status elas_probe_triangulate_pool(const int16_t *list, const int32_t *count, int32_t cap, int32_t w,
+                                                   int32_t h, int32_t right, int32_t *tri, int32_t cap_tri,
+                                                   int32_t *ntri, void *workspace, size_t workspace_bytes,
+                                                   int32_t pool, elas_stream stream) {
+    if (pool < 0) return elas::fail(ELAS_ERR_INVALID_ARG, "pool of %d triangles", pool);
+    return elas::triangulate_entry(list, count, cap, w, h, right, tri, cap_tri, ntri, workspace, workspace_bytes, pool,
+                                   stream);
 }

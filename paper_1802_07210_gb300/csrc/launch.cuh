@@ -36,7 +36,7 @@ elas_status launch_dense_both(const uint8_t *descL, const uint8_t *descR, int w,
 size_t triangulate_device_workspace(int cap, int w, int h, int nsides);
 elas_status launch_triangulate_device(const int16_t *list, const int32_t *count, int cap, int w, int h, int nsides,
                                       const int *rights, int32_t *const *tri, int32_t *const *ntri, int cap_tri,
-                                      void *ws, cudaStream_t st);
+                                      void *ws, cudaStream_t st, int pool_cap = -1);
 elas_status launch_lr_check(int16_t *dL, int16_t *dR, int w, int h, int thr, uint8_t *maskL, uint8_t *maskR,
                             cudaStream_t st);
 size_t post_workspace(int w, int h);

@@ -108,7 +108,8 @@ struct DtSide {
     int32_t *owned;            // [cap] triangles owned (lowest-index vertex)
     int32_t *offset;           // [cap] exclusive scan of owned
     int2 *slots;               // [cap][kDtSlots] owned triangles (the other two vertices), or where they are in pool
-    int2 *pool;                // [2 * cap] the owned triangles of larger fans
+    int2 *pool;                // [pool_cap] the owned triangles of larger fans
+    int32_t pool_cap;          // 2 * cap
     int32_t *npool;            // pool entries taken
     int32_t *pending;          // [cap] points queued by the warp pass
     int32_t *npending;         // queue length
@@ -118,7 +119,7 @@ struct DtSide {
     int32_t *rowmin, *rowmax;  // [h] extreme x of the points of each image row
     int32_t *tri;              // output [cap_tri][3]
     int32_t *ntri;             // output count
-    int32_t *err;              // bit 3: the list is not in raster order
+    int32_t *err;              // kDtErr* bits
 };
 
 struct DtArgs {
