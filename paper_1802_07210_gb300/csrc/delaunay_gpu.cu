@@ -1800,6 +1800,11 @@ __global__ void dt_emit_kernel_b(const DtArgs *__restrict__ tab, VMap vm) {
 
 constexpr int kDtCounters = 5;  // err, npending, npending2, nwork, npool
 
+// Dynamic shared memory of the CTA pass for images of up to gh cell rows.
+static constexpr int dt_block_smem(int gh) { return kDtCacheCap * (int)sizeof(float4) + 2 * gh * (int)sizeof(int); }
+static_assert(dt_block_smem(16384 / kDtCell) + sizeof(DtStarShared) + (2 * kMaxBatch + 2) * sizeof(int) <= kSmemNoLeave,
+              "the CTA pass needs no leave for its shared memory at any size");
+
 static void dt_geom(int w, int h, int &gw, int &gh) {
     gw = (w + kDtCell - 1) / kDtCell;
     gh = (h + kDtCell - 1) / kDtCell;
@@ -1889,9 +1894,7 @@ elas_status launch_triangulate_device(const int16_t *list, const int32_t *count,
 
     // no middle pass: it would add its longest star's time to the CTA pass's
     // (640x480 38 us alone, 37 + 37 with it; 1920x1080 126 and 52 + 74)
-    const int smem = kDtCacheCap * (int)sizeof(float4) + 2 * a.gh * (int)sizeof(int);
-    if (cudaFuncSetAttribute(dt_pass_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-        return launch_status("dt_pass_block_kernel shared memory attribute");
+    const int smem = dt_block_smem(a.gh);
     launch_after(dt_pass_block_kernel, sm_count() * kDtBlocksPerSM, kDtBlockThreads, smem, st, a, nsides);
     launch_after(dt_tri_scan_kernel, dim3(1, nsides), 1024, 0, st, a);
     launch_after(dt_emit_kernel, dim3(pblocks, nsides), tb, 0, st, a);
@@ -1962,9 +1965,7 @@ elas_status launch_triangulate_b(const DtArgs *tab, const DtArgs *host, const VM
         vmap_add(m_grp2, slot, dim3(vmap_share(a.cap, caps, sm_count() * 7 * 4 / nsides), nsides));
         max_gh = max(max_gh, a.gh);
     }
-    const int smem = kDtCacheCap * (int)sizeof(float4) + 2 * max_gh * (int)sizeof(int);
-    if (cudaFuncSetAttribute(dt_pass_block_kernel_b, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-        return launch_status("dt_pass_block_kernel_b shared memory attribute");
+    const int smem = dt_block_smem(max_gh);
     dt_init_kernel_b<<<vmap_total(m_init), 256, 0, st>>>(tab, m_init, counter);
     dt_points_kernel_b<<<vmap_total(m_pts), 256, 0, st>>>(tab, m_pts);
     dt_cell_scan_kernel_b<<<vmap_total(m_scan), 1024, 0, st>>>(tab, m_scan);

@@ -8,6 +8,19 @@
 
 namespace elas {
 
+// Dynamic shared memory of a launch of fn: `smem` bytes, at most `most` in any
+// launch of it.  Above the 48 KB that need no leave, the attribute is set to
+// `most`, the same in every call: it is state of the device that all threads
+// share, and with each call's own size a thread could lower it between
+// another's call and launch.
+constexpr size_t kSmemNoLeave = 48 * 1024, kSmemBlockMax = 227 * 1024;
+inline elas_status allow_smem(const void *fn, size_t smem, size_t most, const char *what) {
+    if (smem > kSmemNoLeave && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                    (int)(smem > most ? smem : most)) != cudaSuccess)
+        return launch_status(what);
+    return ELAS_OK;
+}
+
 // ---- one pair per launch ----------------------------------------------------
 elas_status launch_descriptors(const uint8_t *imgL, const uint8_t *imgR, int w, int h, int pitch, uint8_t *descL,
                                uint8_t *descR, cudaStream_t st);

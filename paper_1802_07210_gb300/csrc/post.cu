@@ -350,10 +350,7 @@ size_t post_workspace(int w, int h) { return 2 * align_up((size_t)w * h * sizeof
 size_t lr_smem(int w) { return 2 * (size_t)((w + 7) & ~7) * sizeof(int16_t); }
 
 static elas_status lr_smem_attr(const void *fn, size_t smem) {
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return launch_status("lr_check smem attribute");
-    return ELAS_OK;
+    return allow_smem(fn, smem, lr_smem(16383), "lr_check smem attribute");  // the widest map
 }
 
 elas_status launch_lr_check(int16_t *dL, int16_t *dR, int w, int h, int thr, uint8_t *maskL, uint8_t *maskR,

@@ -632,20 +632,15 @@ elas_status support_args(const uint8_t *descL, const uint8_t *descR, int w, int 
 size_t consistency_smem(int r) { return (size_t)(kConsTX + 2 * r) * (kConsTY + 2 * r) * sizeof(int16_t); }
 
 static elas_status consistency_smem_attr(const void *fn, size_t smem) {
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return launch_status("consistency_kernel shared memory attribute");
-    return ELAS_OK;
+    // a window that needs more than a CTA can have is refused
+    return allow_smem(fn, smem, kSmemBlockMax, "consistency_kernel shared memory attribute");
 }
 
 // Shared memory of the staged redundancy filter; more runs it unstaged.
 constexpr size_t kRedSmemMax = 96 * 1024;
 
 static elas_status red_smem_attr(const void *fn, size_t smem) {
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return launch_status("redundancy_grid_kernel shared memory attribute");
-    return ELAS_OK;
+    return allow_smem(fn, smem, kRedSmemMax, "redundancy_grid_kernel shared memory attribute");
 }
 
 // Shared memory of the row-organised matcher; wider rows take the
@@ -670,10 +665,7 @@ inline int sup_row_segments(int wc, long long all) {
 }
 
 static elas_status sup_row_smem_attr(const void *fn, size_t smem) {
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return launch_status("support_match_row_kernel shared memory attribute");
-    return ELAS_OK;
+    return allow_smem(fn, smem, kSupRowSmemMax, "support_match_row_kernel shared memory attribute");
 }
 
 dim3 support_match_grid(const MatchArgs &m, int warps) {
