@@ -95,8 +95,10 @@ __device__ __forceinline__ void after_previous() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// p, not known to the compiler before this point: a read-only load (__ldg)
-// through it cannot be moved above after_previous().
+// p, not known to the compiler before this point: a read-only load (__ldg, or
+// one that a `const __restrict__` pointer allows) through it cannot be moved
+// above after_previous().  Every such pointer of a kernel launched by
+// launch_after goes through this.
 template <class T> __device__ __forceinline__ T *settled(T *p) {
     asm volatile("" : "+l"(p)::"memory");
     return p;

@@ -123,7 +123,7 @@ __device__ __forceinline__ void store_rec(int4 *__restrict__ rec, int t, const T
     o[3] = make_int4(b.xmin, b.xmax, b.ymin, b.ymax);
 }
 
-__device__ __forceinline__ TriRec load_rec(const int4 *__restrict__ rec, int t) {
+__device__ __forceinline__ TriRec load_rec(const int4 *rec, int t) {
     const int4 p = rec[kRecWords * (size_t)t], q = rec[kRecWords * (size_t)t + 1], u = rec[kRecWords * (size_t)t + 2];
     TriRec r;
     r.A[0] = p.x, r.A[1] = p.y, r.A[2] = p.z, r.B[0] = p.w;
