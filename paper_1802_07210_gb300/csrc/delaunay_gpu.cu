@@ -706,7 +706,7 @@ __device__ __forceinline__ int dt_fan_pos(int t, int m, int r) { return t >= r ?
 // thread): their first entry, which the point's slots then name, or -1 when
 // there is none and the triangulation fails.  Stars that agree own fewer than
 // two triangles a point in all, which the pool holds.
-__device__ __forceinline__ int dt_pool_room(const DtSide &S, int pz, int m) {
+__device__ __noinline__ int dt_pool_room(const DtSide &S, int pz, int m) {
     const int base = atomicAdd(S.npool, m);
     if (base < 0 || m > S.pool_cap - base) {
         atomicOr(S.err, kDtErrPool);
