@@ -368,6 +368,9 @@ __device__ __forceinline__ int dt_champion(bool in, int at, Get get, Own own, Be
 // One wrap step by a warp over points given as integers by get(0..k-1)
 // (coordinate differences below 2^14.5; the keys' rounding to FP32 and the
 // division leave a relative error below 2^-20).  The winner's position in at.
+// Four points in flight, and no second walk while a lane's second least key
+// lies outside the band: an apex of 3,000 neighbours takes 29.8 ms, 66.8
+// without (the earlier pass with twice the threads 54.1).
 template <class Get>
 __device__ __forceinline__ bool dt_step_int(Get get, int k, int lane, const DtPt &e, int pz, int side, DtPt &w,
                                             int &at) {
@@ -375,22 +378,28 @@ __device__ __forceinline__ bool dt_step_int(Get get, int k, int lane, const DtPt
         const int D = side * (e.x * q.y - e.y * q.x), N = q.x * q.x + q.y * q.y - (e.x * q.x + e.y * q.y);
         return D > 0 ? dt_div((float)N, (float)D) : kDtInf;
     };
-    float f1 = kDtInf;
-    for (int c = lane; c < k; c += 32) f1 = fminf(f1, key(get(c)));
+    float f1 = kDtInf, f2 = kDtInf;  // least and second least key of the lane
+    int c1 = -1;
+#pragma unroll 4
+    for (int c = lane; c < k; c += 32) {
+        const float f = key(get(c));
+        f2 = fminf(f2, fmaxf(f1, f));
+        if (f < f1) {
+            f1 = f;
+            c1 = c;
+        }
+    }
     const float fm = dt_warp_min(f1);
     if (fm == kDtInf) return false;
     const float thr = fm + 0x1p-17f * fabsf(fm);
     const bool in = f1 <= thr;
-    int c1 = -1;
-    if (in) {  // this lane's exact best of the band
-        DtPt bq{0, 0, 0};
+    if (in && f2 <= thr) {  // several of this lane's candidates: its exact best
+        DtPt bq = get(c1);
         for (int c = lane; c < k; c += 32) {
             const DtPt q = get(c);
-            if (key(q) > thr) continue;
-            if (c1 < 0 || dt_beats(e, pz, bq, q, side)) {
-                c1 = c;
-                bq = q;
-            }
+            if (c == c1 || key(q) > thr || !dt_beats(e, pz, bq, q, side)) continue;
+            c1 = c;
+            bq = q;
         }
     }
     at = dt_champion(
