@@ -227,3 +227,25 @@ def test_chains_of_calls_on_streams_and_captured():
     for k, res in got:
         for a, b in zip(res, alone[k]):
             np.testing.assert_array_equal(host(a), host(b))
+
+
+@pytest.mark.parametrize("size", [(65, 49), (97, 71), (200, 30)])
+@pytest.mark.parametrize("gap", [6, 7, 8, 9, 10, 11, 13, 15, 16])
+@pytest.mark.parametrize("mean", [0, 1])
+def test_wide_gaps(size, gap, mean):
+    """Holes of every length around the gap width, along rows and columns, the search in steps
+    (up to 7) and in fours (from 8 on).  The tolerance is test_fused_post_tiles's."""
+    w, h = size
+    prm = dict(ipol_gap_width=gap, filter_adaptive_mean=mean)
+    rng = np.random.default_rng(gap)
+    d = _map(w, h, 0.05)
+    for k in range(60):
+        x, y, n = rng.integers(0, w), rng.integers(0, h), rng.integers(max(1, gap - 3), gap + 3)
+        if k % 2:
+            d[y, x:x + n] = -1
+        else:
+            d[y:y + n, x:x + 3] = -1
+    exp = oracle.postprocess(d, prm)
+    out = host(_B().elas_postprocess(dev(d), prm))
+    assert np.abs(out - exp).max() <= (1e-4 if mean else 0)
+    assert ((out < 0) == (exp < 0)).all()
