@@ -249,3 +249,29 @@ def test_wide_gaps(size, gap, mean):
     out = host(_B().elas_postprocess(dev(d), prm))
     assert np.abs(out - exp).max() <= (1e-4 if mean else 0)
     assert ((out < 0) == (exp < 0)).all()
+
+
+@pytest.mark.parametrize("size", [(20, 1500), (100, 700), (700, 100), (641, 479)])
+@pytest.mark.parametrize("shape", ["comb", "comb_top", "comb_right", "snake", "rings"])
+def test_speckle_long_segments(size, shape):
+    """Segments that run through many tiles and meet at one end, so that the links across the
+    tiles' edges form long chains."""
+    B = _B()
+    w, h = size
+    d = np.full((h, w), -1, np.int16)
+    if shape == "comb":
+        d[:, ::2], d[-1] = 5, 5
+    elif shape == "comb_top":
+        d[:, ::2], d[0] = 5, 5
+    elif shape == "comb_right":
+        d[::2], d[:, -1] = 5, 5
+    elif shape == "snake":
+        d[::2], d[1::4, -1], d[3::4, 0] = 5, 5, 5
+    else:
+        y, x = np.mgrid[:h, :w]
+        d[np.minimum(np.minimum(x, w - 1 - x), np.minimum(y, h - 1 - y)) % 2 == 0] = 5
+    for least in (10, w * h // 3):
+        for _ in range(3):
+            out, st = B.elas_speckle(dev(d), 1, least, with_status=True)
+            np.testing.assert_array_equal(host(out), oracle.speckle(d, 1, least))
+            assert int(host(st)[0]) == 0
