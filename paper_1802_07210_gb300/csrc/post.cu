@@ -300,6 +300,13 @@ __device__ __forceinline__ void fused_post_body(const FusedPostArgs &a, const VB
     const int PX = TX + 2 * H, PY = TY + 2 * H;  // tile pitch and rows
     const int x0 = vb.x * TX - H, y0 = vb.y * TY - H;
     const int tid = threadIdx.x, nth = blockDim.x;
+    if (H == 0) {  // no pass: the map as floats
+        for (int i = tid; i < TX * TY; i += nth) {
+            const int gx = x0 + i % TX, gy = y0 + i / TX;
+            if (gx < w && gy < h) a.out[(size_t)gy * w + gx] = (float)a.d[(size_t)gy * w + gx];
+        }
+        return;
+    }
     const RowSplit full(PX), inner(PX - 2 * g);
     for (int i = tid; i < PX * PY; i += nth) {
         int yy, xx;

@@ -275,3 +275,15 @@ def test_speckle_long_segments(size, shape):
             out, st = B.elas_speckle(dev(d), 1, least, with_status=True)
             np.testing.assert_array_equal(host(out), oracle.speckle(d, 1, least))
             assert int(host(st)[0]) == 0
+
+
+@pytest.mark.parametrize("size", [(1, 1), (31, 23), (33, 25), (640, 41)])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_post_without_passes(size, offset):
+    """Neither gap interpolation nor means: the map's own values as floats."""
+    B = _B()
+    w, h = size
+    d = _map(w, h, 0.2)
+    d[d < 0] = np.random.default_rng(3).choice([-1, -2, -300], (d < 0).sum())
+    out = host(B.elas_postprocess(_at(d, offset), dict(ipol_gap_width=0, filter_adaptive_mean=0)))
+    np.testing.assert_array_equal(out, d.astype(np.float32))
