@@ -877,11 +877,14 @@ elas_status launch_dense_b(const DenseTables &t, const DenseStage *host, const V
         const long long px = (long long)r.w * r.h;
         const int nt = raster_max_ntri(r), all = sm_count() * 8 * 4 / 2;
         // no more CTAs than two 16-byte stores of the fill a thread, or one for
-        // every 256 triangles
+        // every 256 triangles; a launch of few triangles one for every 64, up
+        // to one set of resident CTAs (prior of one 640x480 pair 29.3 us with
+        // a CTA count by pair, 31.3 without this, 27.2 with it)
         const int by_pixels = (int)min((long long)vmap_share(px, pixels, all), px / 4096 + 1);
         vmap_add(m_setup, slot, dim3(by_pixels, r.nsides));
         vmap_add(m_list, slot, dim3(by_pixels, r.nsides));
-        vmap_add(m_draw, slot, dim3(min(vmap_share(nt, tris, all), nt / 256 + 1), r.nsides));
+        const int one_set = min(vmap_share(nt, tris, sm_count() * (fused ? 4 : 8) / 2), nt / 64 + 1);
+        vmap_add(m_draw, slot, dim3(min(vmap_share(nt, tris, all), max(nt / 256 + 1, one_set)), r.nsides));
         vmap_add(m_cell[d.cell.census ? 1 : 0], slot, cell_grid(d.cell, 2));
         threads = max(threads, cell_threads(d.cell.G, tpp, ppt));
     }
