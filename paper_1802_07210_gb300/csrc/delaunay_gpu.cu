@@ -14,9 +14,9 @@
 //   1. Warp pass: one warp per point, the points within 24 pixels from a
 //      16-pixel grid; a star counts when the circles of its triangles fit
 //      that disc (2r <= R, so no farther point can matter), 93-95 % of them.
-//   2. Middle pass (batches): the others again, with 64 pixels.
+//   2. Middle pass (batches): the others again, with 48 pixels.
 //   3. CTA pass: one CTA per star left (the hull, the rims of empty areas):
-//      the star over the points within 64 pixels, then scans of the cells
+//      the star over the points within 48 pixels, then scans of the cells
 //      that its wide circles meet until they are empty (dt_block_item).
 // The output order is deterministic: an exclusive scan of the per-point
 // counts, and within a star counter-clockwise from the nearest neighbour (an
@@ -25,7 +25,8 @@
 // The earlier design (4 or 16 lanes per star, the whole star, 64-bit key
 // comparisons, one region scan per step of a wide star) against this one, all
 // triangulation kernels: 640x480 172 -> 69 us, 1920x1080 590 -> 207 us,
-// 64 x 1242x375 3.44 -> 1.33 ms.
+// 64 x 1242x375 3.44 -> 1.33 ms.  Sound with the limits below: the extents
+// that the integer steps hold, and the room in the pool.
 #include <climits>
 
 #include "launch.cuh"
@@ -1594,9 +1595,8 @@ __device__ __forceinline__ void dt_block_item(const DtArgs &a, const DtSide &S, 
                         if (j0 + kDtBlockThreads * stride < all) next = load(j0 + (kDtBlockThreads + lane) * stride);
                         const DtPt q{t.x - p.x, t.y - p.y, t.z};
                         const float qx = (float)q.x, qy = (float)q.y;
-                        // the circles that need the exact test: the one in
-                        // whose sector the point lies, or all whose padded
-                        // region holds it
+                        // the circles that need the exact test: all whose
+                        // padded region holds the point
                         unsigned need = 0;
                         for (int b = 0; b < nbad; ++b) {
                             const float3 g = sh.region[b];

@@ -108,6 +108,8 @@ def _dense_block(x0, y0, nx, ny, rng, keep):
     return [(x0 + i, y0 + j, int(rng.integers(0, 8))) for j in range(ny) for i in range(nx) if rng.random() < keep]
 
 
+# The limits of the lists today are kDtNearCap (64 candidates of a warp) and kDtCacheCap (1,024
+# cached points); the two figures below are those of an earlier build, and the cases pass both.
 @pytest.mark.parametrize("case", ["fan17", "fan255", "fan256", "fan700", "unordered", "every_pixel", "far_blocks",
                                   "one_row_apart"])
 def test_star_list_limits(case):
