@@ -46,7 +46,7 @@ constexpr int kDtErrRange = 32;  // the points lie too far apart for the integer
 // X^2 + Y^2 < 2^31 for the extents X and Y of the points: |N| = |c.(c - e)| and
 // |c|^2 are at most that, D at most X Y.  Points inside this box meet it, and
 // it holds every point of an image and its disparities; the extents are only
-// taken (dt_cell_scan_body) when a point lies outside.
+// taken (dt_scatter_body) when a point lies outside.
 constexpr int kDtBoxX0 = -8192, kDtBoxX1 = 32767, kDtBoxY0 = -4096, kDtBoxY1 = 17407;
 static_assert((int64_t)(kDtBoxX1 - kDtBoxX0) * (kDtBoxX1 - kDtBoxX0) +
                       (int64_t)(kDtBoxY1 - kDtBoxY0) * (kDtBoxY1 - kDtBoxY0) < (int64_t)1 << 31,
@@ -147,37 +147,14 @@ template <class Put> __device__ __forceinline__ int dt_block_scan(const int32_t 
     return total;
 }
 
-// Sets kDtErrRange when the points' extents are beyond the integer steps.
-__device__ __noinline__ void dt_check_extents(const DtSide &S, int n) {
-    __shared__ int s_ext[4];
-    if (threadIdx.x < 4) s_ext[threadIdx.x] = threadIdx.x & 1 ? INT_MIN : INT_MAX;
-    __syncthreads();
-    int x0 = INT_MAX, x1 = INT_MIN, y0 = INT_MAX, y1 = INT_MIN;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        x0 = min(x0, S.X[i]);
-        x1 = max(x1, S.X[i]);
-        y0 = min(y0, S.Y[i]);
-        y1 = max(y1, S.Y[i]);
-    }
-    atomicMin(&s_ext[0], x0);
-    atomicMax(&s_ext[1], x1);
-    atomicMin(&s_ext[2], y0);
-    atomicMax(&s_ext[3], y1);
-    __syncthreads();
-    const int64_t ex = (int64_t)s_ext[1] - s_ext[0], ey = (int64_t)s_ext[3] - s_ext[2];
-    if (threadIdx.x == 0 && ex * ex + ey * ey >= (int64_t)1 << 31) atomicOr(S.err, kDtErrRange);
-}
-
 // One CTA per side: where each cell's points start; entry ncell is the total
 // (its own count stays 0).  The arrays are padded to 16 bytes.
 __device__ __forceinline__ void dt_cell_scan_body(const DtArgs &a, const VB &vb) {
     const DtSide &S = a.s[vb.y];
-    const int err = *S.err;  // in flight during the scan
     dt_block_scan(S.cell_cnt, dt_ncell(a) + 1, [&](int i, const int4 &before) {
         *reinterpret_cast<int4 *>(S.cell_start + i) = before;
         *reinterpret_cast<int4 *>(S.cell_fill + i) = before;
     });
-    if (err & kDtErrBox) dt_check_extents(S, min(max(*a.count, 0), a.cap));
 }
 
 __global__ void __launch_bounds__(1024) dt_cell_scan_kernel(DtArgs a) {
@@ -189,16 +166,38 @@ __global__ void __launch_bounds__(1024) dt_cell_scan_kernel_b(const DtArgs *__re
     dt_cell_scan_body(slot_entry(tab, vm.stride, vb.slot), vb);
 }
 
+// Sets kDtErrRange when the points' extents are beyond the integer steps.
+__device__ __noinline__ void dt_check_extents(const int32_t *X, const int32_t *Y, int n, int32_t *err) {
+    __shared__ int s_ext[4];
+    if (threadIdx.x < 4) s_ext[threadIdx.x] = threadIdx.x & 1 ? INT_MIN : INT_MAX;
+    __syncthreads();
+    int x0 = INT_MAX, x1 = INT_MIN, y0 = INT_MAX, y1 = INT_MIN;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        x0 = min(x0, X[i]);
+        x1 = max(x1, X[i]);
+        y0 = min(y0, Y[i]);
+        y1 = max(y1, Y[i]);
+    }
+    atomicMin(&s_ext[0], x0);
+    atomicMax(&s_ext[1], x1);
+    atomicMin(&s_ext[2], y0);
+    atomicMax(&s_ext[3], y1);
+    __syncthreads();
+    const int64_t ex = (int64_t)s_ext[1] - s_ext[0], ey = (int64_t)s_ext[3] - s_ext[2];
+    if (threadIdx.x == 0 && ex * ex + ey * ey >= (int64_t)1 << 31) atomicOr(err, kDtErrRange);
+}
+
 __device__ __forceinline__ void dt_scatter_body(const DtArgs &a, const VB &vb) {
     const DtSide S = vb.y ? a.s[1] : a.s[0];
     const int n = min(max(*a.count, 0), a.cap);
-    const int alive = !(*S.err & kDtErrRange);  // else no point has a star: every queue stays empty
+    const int err = vb.x == 0 ? *S.err : 0;
     for (int i = vb.x * blockDim.x + threadIdx.x; i < n; i += vb.gx * blockDim.x) {
         const int x = S.X[i], y = S.Y[i];
         const int k = atomicAdd(S.cell_fill + dt_cell(a, x, y), 1);
-        S.pts[k] = make_int4(x, y, i, alive);
+        S.pts[k] = make_int4(x, y, i, 1);
         S.slot[i] = k;
     }
+    if (err & kDtErrBox) dt_check_extents(S.X, S.Y, n, S.err);
 }
 
 __global__ void dt_scatter_kernel(DtArgs a) {
@@ -712,23 +711,12 @@ __device__ __forceinline__ bool dt_wide_step(const DtArgs &a, const DtSide &S, c
 // vertex r of the fan (0 when it is none of its vertices).
 __device__ __forceinline__ int dt_fan_pos(int t, int m, int r) { return t >= r ? t - r : t + m - r; }
 
-// Room in the pool for the m > kDtSlots owned triangles of point pz (one
-// thread): their first entry, which the point's slots then name, or -1 when
-// there is none and the triangulation fails.  Stars that agree own fewer than
-// two triangles a point in all, which the pool holds.
-__device__ __noinline__ int dt_pool_room(const DtSide &S, int pz, int m) {
-    const int base = atomicAdd(S.npool, m);
-    if (base < 0 || m > S.pool_cap - base) {
-        atomicOr(S.err, kDtErrPool);
-        return -1;
-    }
-    S.slots[(size_t)pz * kDtSlots] = make_int2(base, 0);
-    return base;
-}
-
 // The owned triangles of a star whose vertices sit one per lane: a[0..na]
-// counter-clockwise from the first vertex, b[0..nb] clockwise from it.
-__device__ __forceinline__ void dt_warp_write(const DtSide &S, int pz, int lane, bool fan, int va, int vb, int na,
+// counter-clockwise from the first vertex, b[0..nb] clockwise from it.  False:
+// more than the point's slots hold, which the CTA pass takes to the pool (the
+// pool's bound in this function took the middle pass of 64 x 1242x375 from 230
+// to 241 us).
+__device__ __forceinline__ bool dt_warp_write(const DtSide &S, int pz, int lane, bool fan, int va, int vb, int na,
                                               int nb, int nnz) {
     const int va1 = __shfl_down_sync(0xFFFFFFFFu, va, 1), vb1 = __shfl_down_sync(0xFFFFFFFFu, vb, 1);
     const bool oa = lane < na && pz < va && pz < va1, ob = lane < nb && pz < vb && pz < vb1;
@@ -742,17 +730,12 @@ __device__ __forceinline__ void dt_warp_write(const DtSide &S, int pz, int lane,
         pa = dt_fan_pos(mb + lane, m, r);
         pb = dt_fan_pos(mb - 1 - lane, m, r);
     }
+    if (m > kDtSlots) return false;
     int2 *out = S.slots + (size_t)pz * kDtSlots;
-    if (m > kDtSlots) {
-        int base = 0;
-        if (lane == 0) base = dt_pool_room(S, pz, m);
-        base = __shfl_sync(0xFFFFFFFFu, base, 0);
-        if (base < 0) return;
-        out = S.pool + base;
-    }
     if (oa) out[pa] = make_int2(va, va1);
     if (ob) out[pb] = make_int2(vb1, vb);
     if (lane == 0) S.owned[pz] = m;
+    return true;
 }
 
 // One star by a warp over the candidates within R of p; true if it came out
@@ -846,8 +829,7 @@ __device__ __forceinline__ bool dt_warp_star(const DtArgs &a, const DtSide &S, c
         }
         if (__any_sync(0xFFFFFFFFu, bad)) return false;
     }
-    dt_warp_write(S, p.z, lane, fan, va, vb, na, nb, __float_as_int(nn.w));
-    return true;
+    return dt_warp_write(S, p.z, lane, fan, va, vb, na, nb, __float_as_int(nn.w));
 }
 
 // Warp pass: one warp per point, the candidates within 24 pixels (16 or 8
@@ -862,10 +844,12 @@ __device__ __forceinline__ void dt_pass1_body(const DtArgs &a, const VB &vb) {
     const int n = min(max(*a.count, 0), a.cap);
     const int lane = threadIdx.x & 31;
     float4 *list = s_list[threadIdx.x >> 5];
-    const bool ordered = !(*S.err & kDtErrOrder);
+    const int err = *S.err;
+    const bool ordered = !(err & kDtErrOrder);
     for (int j = vb.x * kDtWarps + (threadIdx.x >> 5); j < n; j += vb.gx * kDtWarps) {
         const int4 p = S.pts[j];
-        if (!p.w) continue;
+        // out of range: no star is built, the later passes find empty queues
+        if (!p.w || (err & kDtErrRange)) continue;
         const int cx0 = min(a.gw - 1, max(0, p.x - kDtRadius) / kDtCell);
         const int cx1 = min(a.gw - 1, max(0, p.x + kDtRadius) / kDtCell);
         const int cy0 = max(0, p.y - kDtRadius) / kDtCell, cy1 = min(a.gh - 1, (p.y + kDtRadius) / kDtCell);
@@ -1269,6 +1253,20 @@ __device__ __forceinline__ void dt_star_tri(const DtStarList &star, const float4
     const uint16_t *v = t < na ? star.v[0] + t : star.v[1] + (t - na);
     a = cand[v[t < na ? 0 : 1]];
     b = cand[v[t < na ? 1 : 0]];
+}
+
+// Room in the pool for the m > kDtSlots owned triangles of point pz (one
+// thread): their first entry, which the point's slots then name, or -1 when
+// there is none and the triangulation fails.  Stars that agree own fewer than
+// two triangles a point in all, which the pool holds.
+__device__ __noinline__ int dt_pool_room(const DtSide &S, int pz, int m) {
+    const int base = atomicAdd(S.npool, m);
+    if (base < 0 || m > S.pool_cap - base) {
+        atomicOr(S.err, kDtErrPool);
+        return -1;
+    }
+    S.slots[(size_t)pz * kDtSlots] = make_int2(base, 0);
+    return base;
 }
 
 // Writes the owned triangles of a star (warp 0).

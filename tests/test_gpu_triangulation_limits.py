@@ -52,7 +52,7 @@ def _pool_bytes(ws, cap, h):
 
 @pytest.mark.parametrize("fan", [26, 255, 700])
 def test_pool_without_room(fan):
-    """An apex that sees every point of a distant row, wrapped by a warp (26), by a CTA over its
+    """An apex that sees every point of a distant row, certain to a warp (26), wrapped by a CTA over its
     cached points and by a CTA over all points (more vertices than its lists hold)."""
     if fan == 26:  # the points of a half ring within a warp's 24 pixels that the apex sees
         ring = [(x, y) for y in range(1, 25) for x in range(-24, 25) if 22 * 22 <= x * x + y * y <= 24 * 24]
