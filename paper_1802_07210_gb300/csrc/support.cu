@@ -404,7 +404,7 @@ __host__ __device__ __forceinline__ size_t red_smem_bytes(int wc, int maxd, int 
 __device__ __forceinline__ void redundancy_grid_body(const RedArgs &ra, const VB &vb, bool staged) {
     extern __shared__ __align__(16) unsigned char s_red[];
     __shared__ int s_cnt[4];
-    const int16_t *__restrict__ con = settled(ra.con);
+    const int16_t *con = ra.con;
     const int wc = ra.wc, hc = ra.hc, maxd = ra.maxd;
     const GridArgs g = ra.g;
     const int ic = vb.x, tid = threadIdx.x, nth = blockDim.x;
